@@ -1,9 +1,12 @@
-"""ctypes binding of libxnor.so: argument marshalling only.
+"""Binding of libxnor.so: argument marshalling only.
 
 Each function has the name and argument order of the C entry point it
 forwards to (see include/xnor.h) and takes torch CUDA tensors where the C call
-takes device pointers.  Nothing here computes: a missing or unloadable library
-raises, there is no fallback.
+takes device pointers.  The calls that launch kernels convert their arguments in
+the native module _pymarshal (csrc/pymarshal.cpp: about 1 us a call against 10 us
+through ctypes, where a small layer's kernels take as long); queries go through
+ctypes.  Nothing here computes: a missing or unloadable library raises, there is
+no fallback.
 """
 import ctypes
 import os
@@ -56,11 +59,27 @@ class XnorError(RuntimeError):
 
 
 _lib = None
+# Entry points whose arguments the native module converts, in the order its bind() takes them.
+_MARSHALLED = ["binarize_weights", "binactiv", "conv2d_forward", "shortcut_conv1x1",
+               "conv2d_forward_binactiv", "binactiv_finish", "maxpool2d", "binactiv_kbit",
+               "conv2d_forward_kbit", "bwn_prepare_input", "bwn_conv2d_forward",
+               "binarize_weights_transposed", "binary_gradient_backward"]
+
+
+class _Unloaded:
+    """Stands for the native module until the first call loads it."""
+
+    def __getattr__(self, name):
+        load()
+        return getattr(_m, name)
+
+
+_m = _Unloaded()
 
 
 def load():
     """Load libxnor.so (built in-tree by paper_1603_05279_b200.build)."""
-    global _lib
+    global _lib, _m
     if _lib is not None:
         return _lib
     if not os.path.exists(LIB_PATH):
@@ -126,7 +145,13 @@ def load():
     lib.xnor_binary_gradient_backward.argtypes = [vp, vp, vp, ctypes.POINTER(xnor_conv_desc), vp, vp, vp, vp]
     lib.xnor_measure_peaks.restype = ci
     lib.xnor_measure_peaks.argtypes = [ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_double), vp]
-    _lib = lib
+    try:
+        from . import _pymarshal
+    except ImportError as e:
+        raise ImportError("_pymarshal.so is not built: run `python -m paper_1603_05279_b200.build` "
+                          "(%s)" % e) from e
+    _pymarshal.bind([ctypes.cast(getattr(lib, "xnor_" + n), vp).value for n in _MARSHALLED])
+    _lib, _m = lib, _pymarshal
     return lib
 
 
@@ -212,27 +237,22 @@ def xnor_conv2d_binactiv_parts(d):
 
 def xnor_conv2d_forward_binactiv(x_packed, w_packed, alpha, K, residual, d, out, next_scale,
                                  next_shift, x_packed_next, A_parts, stream=None):
-    _check(load().xnor_conv2d_forward_binactiv(
-        _ptr(x_packed, torch.int32), _ptr(w_packed, torch.int32), _ptr(alpha, torch.float32),
-        _ptr(K, torch.float32), _ptr(residual, torch.float32) if residual is not None else None,
-        ctypes.byref(d), _ptr(out, torch.float32) if out is not None else None,
-        _ptr(next_scale, torch.float32) if next_scale is not None else None,
-        _ptr(next_shift, torch.float32) if next_shift is not None else None,
-        _ptr(x_packed_next, torch.int32), _ptr(A_parts, torch.float32), _stream(stream)),
-        "xnor_conv2d_forward_binactiv")
+    s = _m.conv2d_forward_binactiv(x_packed, w_packed, alpha, K, residual, d, out, next_scale,
+                                   next_shift, x_packed_next, A_parts, stream)
+    if s:
+        raise XnorError(s, "xnor_conv2d_forward_binactiv")
 
 
 def xnor_binactiv_finish(A_parts, parts, d_next, A, K, stream=None):
-    _check(load().xnor_binactiv_finish(_ptr(A_parts, torch.float32), int(parts), ctypes.byref(d_next),
-                                       _ptr(A, torch.float32), _ptr(K, torch.float32), _stream(stream)),
-           "xnor_binactiv_finish")
+    s = _m.binactiv_finish(A_parts, int(parts), d_next, A, K, stream)
+    if s:
+        raise XnorError(s, "xnor_binactiv_finish")
 
 
 def xnor_maxpool2d(x, k, stride, pad, relu, out, stream=None):
-    N, C, H, W = x.shape
-    _check(load().xnor_maxpool2d(_ptr(x, torch.float32), N, C, H, W, int(k), int(stride), int(pad),
-                                 1 if relu else 0, _ptr(out, torch.float32), _stream(stream)),
-           "xnor_maxpool2d")
+    s = _m.maxpool2d(x, int(k), int(stride), int(pad), 1 if relu else 0, out, stream)
+    if s:
+        raise XnorError(s, "xnor_maxpool2d")
 
 
 def xnor_selftest_wait_timeout(stream=None):
@@ -241,34 +261,28 @@ def xnor_selftest_wait_timeout(stream=None):
 
 
 def xnor_binarize_weights(w, w_packed, alpha, stream=None):
-    C_out, C_in, k_h, k_w = w.shape
-    _check(load().xnor_binarize_weights(_ptr(w, torch.float32), C_out, C_in, k_h, k_w,
-                                        _ptr(w_packed, torch.int32), _ptr(alpha, torch.float32),
-                                        _stream(stream)), "xnor_binarize_weights")
+    s = _m.binarize_weights(w, w_packed, alpha, stream)
+    if s:
+        raise XnorError(s, "xnor_binarize_weights")
 
 
 def xnor_binactiv(x, bn_scale, bn_shift, d, x_packed, A, K, stream=None):
-    _check(load().xnor_binactiv(_ptr(x, torch.float32), _ptr(bn_scale, torch.float32),
-                                _ptr(bn_shift, torch.float32), ctypes.byref(d),
-                                _ptr(x_packed, torch.int32), _ptr(A, torch.float32),
-                                _ptr(K, torch.float32), _stream(stream)), "xnor_binactiv")
+    s = _m.binactiv(x, bn_scale, bn_shift, d, x_packed, A, K, stream)
+    if s:
+        raise XnorError(s, "xnor_binactiv")
 
 
 def xnor_binactiv_kbit(x, bn_scale, bn_shift, d, kbits, x_planes, A, K, stream=None):
-    _check(load().xnor_binactiv_kbit(_ptr(x, torch.float32), _ptr(bn_scale, torch.float32),
-                                     _ptr(bn_shift, torch.float32), ctypes.byref(d), int(kbits),
-                                     _ptr(x_planes, torch.int32), _ptr(A, torch.float32),
-                                     _ptr(K, torch.float32), _stream(stream)), "xnor_binactiv_kbit")
+    s = _m.binactiv_kbit(x, bn_scale, bn_shift, d, int(kbits), x_planes, A, K, stream)
+    if s:
+        raise XnorError(s, "xnor_binactiv_kbit")
 
 
 def xnor_conv2d_forward_kbit(x_planes, kbits, w_packed, alpha, K, residual, d, out, acc_out=None,
                              stream=None):
-    _check(load().xnor_conv2d_forward_kbit(_ptr(x_planes, torch.int32), int(kbits),
-                                           _ptr(w_packed, torch.int32), _ptr(alpha, torch.float32),
-                                           _ptr(K, torch.float32), _ptr(residual, torch.float32),
-                                           ctypes.byref(d), _ptr(out, torch.float32),
-                                           _ptr(acc_out, torch.int32), _stream(stream)),
-           "xnor_conv2d_forward_kbit")
+    s = _m.conv2d_forward_kbit(x_planes, int(kbits), w_packed, alpha, K, residual, d, out, acc_out, stream)
+    if s:
+        raise XnorError(s, "xnor_conv2d_forward_kbit")
 
 
 def xnor_measure_peaks(stream=None):
@@ -283,17 +297,15 @@ def xnor_bwn_input_elems(d):
 
 
 def xnor_bwn_prepare_input(x, bn_scale, bn_shift, d, x_stream, stream=None):
-    _check(load().xnor_bwn_prepare_input(_ptr(x, torch.float32), _ptr(bn_scale, torch.float32),
-                                         _ptr(bn_shift, torch.float32), ctypes.byref(d),
-                                         _ptr(x_stream, torch.bfloat16), _stream(stream)),
-           "xnor_bwn_prepare_input")
+    s = _m.bwn_prepare_input(x, bn_scale, bn_shift, d, x_stream, stream)
+    if s:
+        raise XnorError(s, "xnor_bwn_prepare_input")
 
 
 def xnor_bwn_conv2d_forward(x_stream, w_packed, alpha, residual, d, out, stream=None):
-    _check(load().xnor_bwn_conv2d_forward(_ptr(x_stream, torch.bfloat16), _ptr(w_packed, torch.int32),
-                                          _ptr(alpha, torch.float32), _ptr(residual, torch.float32),
-                                          ctypes.byref(d), _ptr(out, torch.float32), _stream(stream)),
-           "xnor_bwn_conv2d_forward")
+    s = _m.bwn_conv2d_forward(x_stream, w_packed, alpha, residual, d, out, stream)
+    if s:
+        raise XnorError(s, "xnor_bwn_conv2d_forward")
 
 
 def xnor_bgrad_stream_elems(d):
@@ -302,18 +314,15 @@ def xnor_bgrad_stream_elems(d):
 
 def xnor_binarize_weights_transposed(w, wT_packed, stream=None):
     """w fp32 [C_out][C_in][k_h][k_w] -> sign bits for the backward convolution (alloc_weights_transposed)."""
-    Co, C, kh, kw = w.shape
-    _check(load().xnor_binarize_weights_transposed(_ptr(w, torch.float32), Co, C, kh, kw,
-                                                   _ptr(wT_packed, torch.int32), _stream(stream)),
-           "xnor_binarize_weights_transposed")
+    s = _m.binarize_weights_transposed(w, wT_packed, stream)
+    if s:
+        raise XnorError(s, "xnor_binarize_weights_transposed")
 
 
 def xnor_binary_gradient_backward(g, wT_packed, alpha, d, gmax, g_stream, grad_in, stream=None):
-    _check(load().xnor_binary_gradient_backward(_ptr(g, torch.float32), _ptr(wT_packed, torch.int32),
-                                                _ptr(alpha, torch.float32), ctypes.byref(d),
-                                                _ptr(gmax, torch.float32), _ptr(g_stream, torch.bfloat16),
-                                                _ptr(grad_in, torch.float32), _stream(stream)),
-           "xnor_binary_gradient_backward")
+    s = _m.binary_gradient_backward(g, wT_packed, alpha, d, gmax, g_stream, grad_in, stream)
+    if s:
+        raise XnorError(s, "xnor_binary_gradient_backward")
 
 
 def alloc_weights_transposed(C_out, C_in, k_h, k_w, device="cuda"):
@@ -346,19 +355,15 @@ def xnor_binactiv_static(x, bn_scale, bn_shift, d, x_packed, K, stream=None):
 
 
 def xnor_conv2d_forward(x_packed, w_packed, alpha, K, residual, d, out, acc_out=None, stream=None):
-    _check(load().xnor_conv2d_forward(_ptr(x_packed, torch.int32), _ptr(w_packed, torch.int32),
-                                      _ptr(alpha, torch.float32), _ptr(K, torch.float32),
-                                      _ptr(residual, torch.float32), ctypes.byref(d),
-                                      _ptr(out, torch.float32), _ptr(acc_out, torch.int32),
-                                      _stream(stream)), "xnor_conv2d_forward")
+    s = _m.conv2d_forward(x_packed, w_packed, alpha, K, residual, d, out, acc_out, stream)
+    if s:
+        raise XnorError(s, "xnor_conv2d_forward")
 
 
 def xnor_shortcut_conv1x1(x, w, stride, out, stream=None):
-    N, C_in, H, W = x.shape
-    C_out = w.shape[0]
-    _check(load().xnor_shortcut_conv1x1(_ptr(x, torch.float32), _ptr(w, torch.float32), N, C_in,
-                                        H, W, C_out, int(stride), _ptr(out, torch.float32),
-                                        _stream(stream)), "xnor_shortcut_conv1x1")
+    s = _m.shortcut_conv1x1(x, w, int(stride), out, stream)
+    if s:
+        raise XnorError(s, "xnor_shortcut_conv1x1")
 
 
 # ---- buffer helpers (allocation only; torch owns the memory) -------------------------------
