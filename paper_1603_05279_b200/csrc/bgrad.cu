@@ -17,6 +17,7 @@ namespace {
 // integer atomicMax: exact and independent of the order of arrival.  NaN is skipped.
 __global__ void __launch_bounds__(256)
 grad_max_kernel(const float *__restrict__ g, size_t per_image, int vec4, float *__restrict__ gmax) {
+  stream_order();
   const float *gi = g + (size_t)blockIdx.y * per_image;
   float m = 0.0f;
   if (vec4) {
@@ -45,6 +46,7 @@ grad_max_kernel(const float *__restrict__ g, size_t per_image, int vec4, float *
 __global__ void __launch_bounds__(256)
 binarize_weights_transposed_kernel(const float *__restrict__ w, int Co, int C, int kh, int kw,
                                    int CwT, uint32_t *__restrict__ wT_packed) {
+  stream_order();
   const int lane = threadIdx.x & 31;
   const int taps = kh * kw, nwords = taps * CwT, npad = (nwords + 1) & ~1;
   const long long total = (long long)C * npad;
@@ -75,8 +77,7 @@ cudaError_t launch_grad_max(const float *g, int N, size_t per_image, float *gmax
   const size_t cap = (per_image + 4095) / 4096;
   const unsigned bx = (unsigned)std::max<size_t>(1, std::min(want, cap));
   const int vec4 = (per_image % 4 == 0) ? 1 : 0;     // then every image starts on a 16-byte boundary
-  grad_max_kernel<<<dim3(bx, (unsigned)N), 256, 0, st>>>(g, per_image, vec4, gmax);
-  return cudaGetLastError();
+  return launch_kernel(grad_max_kernel, dim3(bx, (unsigned)N), 256, 0, st, 1, g, per_image, vec4, gmax);
 }
 
 cudaError_t launch_binarize_weights_transposed(const float *w, int Co, int C, int kh, int kw,
@@ -84,8 +85,7 @@ cudaError_t launch_binarize_weights_transposed(const float *w, int Co, int C, in
   const int CwT = (Co + 31) / 32;
   const long long total = (long long)C * ((kh * kw * CwT + 1) & ~1);
   const unsigned grid = (unsigned)std::min<long long>((total + 7) / 8, 4096);
-  binarize_weights_transposed_kernel<<<grid, 256, 0, st>>>(w, Co, C, kh, kw, CwT, wT_packed);
-  return cudaGetLastError();
+  return launch_kernel(binarize_weights_transposed_kernel, dim3(grid), 256, 0, st, 1, w, Co, C, kh, kw, CwT, wT_packed);
 }
 
 }  // namespace xnor

@@ -41,6 +41,7 @@ binactiv_pack_kernel(const float *__restrict__ x, const float *__restrict__ scal
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int pgl = warp / G, g = warp - pgl * G;
   const bool active = pgl < PG;
+  stream_order();
   if (kHasBN) {
     for (int c = threadIdx.x; c < Cw * 32; c += 32 * kWarps)
       bn[c] = c < C ? make_float2(__ldg(scale + c), __ldg(shift + c)) : make_float2(0.0f, 0.0f);
@@ -288,6 +289,9 @@ binactiv_image_kernel(const __grid_constant__ ImgParams P) {
     mbar_init(cbar, kImgWarps);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  stream_order();
+  if (producer) {
     // the first copies start before the rest of the block has set up: every buffer is free
     for (; q < total && q < P.nbuf; ++q) issue_chunk();
   }
@@ -474,6 +478,7 @@ template <int KS>
 __global__ void __launch_bounds__(256)
 box_filter_kernel(const float *__restrict__ A, int H, int W, int kh, int kw, int stride, int pad,
                   int Ho, int Wo, int valid_taps, float *__restrict__ K) {
+  stream_order();
   const int i = blockIdx.x * 256 + threadIdx.x;
   if (i >= Ho * Wo) return;
   const int oy = i / Wo, ox = i - oy * Wo;
@@ -594,8 +599,7 @@ cudaError_t launch_image_variant(const ImgParams &ip, int sms, size_t smem, cuda
   }
   const long long resident = (long long)per_sm * sms;
   const unsigned grid = (unsigned)(ip.N < resident ? ip.N : resident);
-  binactiv_image_kernel<kHasBN, KS, kKbit><<<grid, kImgThreads, smem, st>>>(ip);
-  return cudaGetLastError();
+  return launch_kernel(binactiv_image_kernel<kHasBN, KS, kKbit>, dim3(grid), kImgThreads, smem, st, 1, ip);
 }
 
 void fill_img_params(ImgParams &ip, const float *x, const float *scale, const float *shift,
@@ -692,12 +696,11 @@ cudaError_t launch_binactiv(const float *x, const float *scale, const float *shi
   }
   const long long resident = (long long)per_sm * sms;
   const unsigned grid = (unsigned)(nbatches < resident ? nbatches : resident);
-#define XNOR_PACK(BN, V16) binactiv_pack_kernel<BN, V16><<<grid, 32 * kWarps, smem, st>>>( \
+#define XNOR_PACK(BN, V16) launch_kernel(binactiv_pack_kernel<BN, V16>, dim3(grid), 32 * kWarps, smem, st, 1, \
       x, scale, shift, total_pix, g.C, g.H * g.W, g.Cw, G, PG, x_packed, A)
-  if (scale) { if (v16) XNOR_PACK(true, true); else XNOR_PACK(true, false); }
-  else { if (v16) XNOR_PACK(false, true); else XNOR_PACK(false, false); }
+  const cudaError_t e = scale ? (v16 ? XNOR_PACK(true, true) : XNOR_PACK(true, false))
+                              : (v16 ? XNOR_PACK(false, true) : XNOR_PACK(false, false));
 #undef XNOR_PACK
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return launch_box_filter(A, g, K, st);
 }
@@ -707,15 +710,9 @@ cudaError_t launch_box_filter(const float *A, const ConvGeom &g, float *K, cudaS
   const dim3 kgrid((unsigned)((g.Ho * g.Wo + 255) / 256), (unsigned)g.N);
   const int ks = g.kh == g.kw ? g.kh : 0;
   const int valid = (g.flags & XNOR_FLAG_K_VALID_TAPS) ? 1 : 0;
-#define XNOR_BOX(KS) box_filter_kernel<KS><<<kgrid, 256, 0, st>>>(A, g.H, g.W, g.kh, g.kw, g.stride, \
-                                                                g.pad, g.Ho, g.Wo, valid, K)
-  if (ks == 1) XNOR_BOX(1);
-  else if (ks == 3) XNOR_BOX(3);
-  else if (ks == 5) XNOR_BOX(5);
-  else if (ks == 7) XNOR_BOX(7);
-  else XNOR_BOX(0);
-#undef XNOR_BOX
-  return cudaGetLastError();
+  const auto kern = ks == 1 ? box_filter_kernel<1> : ks == 3 ? box_filter_kernel<3> : ks == 5 ? box_filter_kernel<5>
+                    : ks == 7 ? box_filter_kernel<7> : box_filter_kernel<0>;
+  return launch_kernel(kern, kgrid, 256, 0, st, 1, A, g.H, g.W, g.kh, g.kw, g.stride, g.pad, g.Ho, g.Wo, valid, K);
 }
 
 
@@ -724,6 +721,7 @@ namespace {
 // A[i] = (part 0 + part 1 + ...)[i] / C, the parts added in index order.
 __global__ void __launch_bounds__(256)
 sum_parts_kernel(const float *__restrict__ parts, int nparts, size_t n, float C, float *__restrict__ A) {
+  stream_order();
   for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (size_t)gridDim.x * 256) {
     float s = 0.0f;
     for (int p = 0; p < nparts; ++p) s += __ldg(parts + (size_t)p * n + i);
@@ -737,8 +735,7 @@ cudaError_t launch_binactiv_finish(const float *A_part, int parts, const ConvGeo
                                    float *K, cudaStream_t st) {
   const size_t n = (size_t)g.N * g.H * g.W;
   const unsigned grid = (unsigned)std::min<size_t>((n + 255) / 256, (size_t)sm_count_of_current_device() * 8);
-  sum_parts_kernel<<<grid, 256, 0, st>>>(A_part, parts, n, (float)g.C, A);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_kernel(sum_parts_kernel, dim3(grid), 256, 0, st, 1, A_part, parts, n, (float)g.C, A);
   if (e != cudaSuccess) return e;
   return launch_box_filter(A, g, K, st);
 }
@@ -759,6 +756,7 @@ binactiv_pack_kbit_kernel(const float *__restrict__ x, const float *__restrict__
                           const float *__restrict__ shift, long long total_pix, int C, int HW, int Cw,
                           int kbits, uint32_t *__restrict__ x_planes, float *__restrict__ A) {
   __shared__ float tau[128];                 // tau[j], j = 1 .. 2^k - 1; tau[0] unused
+  stream_order();
   const int levels = (1 << kbits) - 1;
   for (int j = 1 + threadIdx.x; j <= levels; j += blockDim.x)
     tau[j] = (float)((double)(2 * j - 1) / (double)levels - 1.0);
@@ -828,9 +826,8 @@ cudaError_t launch_binactiv_kbit(const float *x, const float *scale, const float
   const long long total_pix = (long long)g.N * g.H * g.W;
   const long long nblocks = ((total_pix + 31) / 32 + 7) / 8;
   const unsigned grid = (unsigned)std::min<long long>(nblocks, 8ll * sm_count_of_current_device());
-  binactiv_pack_kbit_kernel<<<grid, 256, 0, st>>>(x, scale, shift, total_pix, g.C, g.H * g.W, g.Cw,
-                                                  kbits, x_planes, A);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_kernel(binactiv_pack_kbit_kernel, dim3(grid), 256, 0, st, 1, x, scale, shift, total_pix, g.C, g.H * g.W,
+                                g.Cw, kbits, x_planes, A);
   if (e != cudaSuccess) return e;
   return launch_box_filter(A, g, K, st);
 }

@@ -13,6 +13,7 @@ binarize_weights_kernel(const float *__restrict__ w, int Co, int C, int taps, in
                         uint32_t *__restrict__ w_packed, float *__restrict__ alpha) {
   extern __shared__ uint32_t words[];  // [taps][Cw]
   __shared__ double red[kThreads / 32];
+  stream_order();
   const int co = blockIdx.x;
   const int n = C * taps;
   const int nwords = taps * Cw;
@@ -55,8 +56,7 @@ cudaError_t launch_binarize_weights(const float *w, int Co, int C, int kh, int k
   const int taps = kh * kw, Cw = (C + 31) / 32;
   const size_t smem = (size_t)taps * Cw * sizeof(uint32_t);
   if (smem > 48 * 1024) return cudaErrorInvalidValue;
-  binarize_weights_kernel<<<Co, kThreads, smem, st>>>(w, Co, C, taps, Cw, w_packed, alpha);
-  return cudaGetLastError();
+  return launch_kernel(binarize_weights_kernel, dim3((unsigned)Co), kThreads, smem, st, 1, w, Co, C, taps, Cw, w_packed, alpha);
 }
 
 }  // namespace xnor

@@ -26,6 +26,7 @@ binconv_popc_kernel(const uint32_t *__restrict__ xp, const uint32_t *__restrict_
                     const float *__restrict__ alpha, const float *__restrict__ K,
                     const float *residual, PopcParams P, EpiOpts epi, float *out, int32_t *acc_out) {
   extern __shared__ uint32_t smem[];
+  stream_order();
   const int taps = P.kh * P.kw;
   uint32_t *patch = smem;                       // [cwc][PP]
   uint32_t *wts = smem + (size_t)P.cwc * P.PP;  // [TF][taps][cwc]
@@ -161,8 +162,7 @@ cudaError_t launch_binconv_popc(const uint32_t *xp, const uint32_t *wp, const fl
     attr_set = true;
   }
   const dim3 grid((unsigned)(g.N * P.tiles_per_image), (unsigned)((g.Co + TF - 1) / TF));
-  binconv_popc_kernel<<<grid, kThreads, smem, st>>>(xp, wp, alpha, K, residual, P, epi, out, acc_out);
-  return cudaGetLastError();
+  return launch_kernel(binconv_popc_kernel, grid, kThreads, smem, st, 1, xp, wp, alpha, K, residual, P, epi, out, acc_out);
 }
 
 }  // namespace xnor

@@ -1137,16 +1137,6 @@ binconv_tc_kernel(const __grid_constant__ TcParams P) {
     *S.abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // per-filter vectors of the epilogue, zero beyond C_out (one global round trip per CTA
-  // instead of one per 16 columns drained); alpha carries the call's extra output factor
-  // (1 except in the passes of a k-bit convolution; a product with 1 is exact)
-  for (int i = tid; i < P.vec_len; i += kThreads) {
-    reinterpret_cast<float *>(smem + P.off_vec)[i] = i < P.Co ? __fmul_rn(__ldg(P.alpha + i), P.out_scale) : 0.0f;
-    if (kFuse && P.nscale != nullptr) {
-      reinterpret_cast<float *>(smem + P.off_vec)[P.vec_len + i] = i < P.Co ? __ldg(P.nscale + i) : 0.0f;
-      reinterpret_cast<float *>(smem + P.off_vec)[2 * P.vec_len + i] = i < P.Co ? __ldg(P.nshift + i) : 0.0f;
-    }
-  }
   if (warp == kMmaWarp) {
     if (kPair) {
       // the same warp of both CTAs of the pair allocates, at the same shared-memory offset
@@ -1172,6 +1162,18 @@ binconv_tc_kernel(const __grid_constant__ TcParams P) {
       asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1};"
                    ::"r"(taddr + 8u * k), "r"(one) : "memory");
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+  }
+  // everything up to here overlaps the end of the kernel before this one
+  stream_order();
+  // per-filter vectors of the epilogue, zero beyond C_out (one global round trip per CTA
+  // instead of one per 16 columns drained); alpha carries the call's extra output factor
+  // (1 except in the passes of a k-bit convolution; a product with 1 is exact)
+  for (int i = tid; i < P.vec_len; i += kThreads) {
+    reinterpret_cast<float *>(smem + P.off_vec)[i] = i < P.Co ? __fmul_rn(__ldg(P.alpha + i), P.out_scale) : 0.0f;
+    if (kFuse && P.nscale != nullptr) {
+      reinterpret_cast<float *>(smem + P.off_vec)[P.vec_len + i] = i < P.Co ? __ldg(P.nscale + i) : 0.0f;
+      reinterpret_cast<float *>(smem + P.off_vec)[2 * P.vec_len + i] = i < P.Co ? __ldg(P.nshift + i) : 0.0f;
+    }
   }
   tc_fence_before();
   __syncthreads();
@@ -1416,19 +1418,8 @@ Plan plan_variant_uncached(const ConvGeom &g, TcVariant v, bool fuse) {
 
 template <bool kRes, bool kPair, bool kFuse>
 cudaError_t launch_variant(const Plan &pl, unsigned units, cudaStream_t st) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kPair ? 2 * units : units);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = pl.smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = kPair ? 2 : 1;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, binconv_tc_kernel<kRes, kPair, kFuse>, pl.P);
+  return launch_kernel(binconv_tc_kernel<kRes, kPair, kFuse>, dim3(kPair ? 2 * units : units), kThreads, pl.smem, st,
+                       kPair ? 2u : 1u, pl.P);
 }
 
 }  // namespace
@@ -1555,6 +1546,7 @@ namespace {
 __global__ void wait_timeout_selftest_kernel() {
   __shared__ __align__(8) uint64_t bar;
   __shared__ volatile int abort_flag;
+  stream_order();
   if (threadIdx.x == 0) {
     mbar_init(smem_u32(&bar), 1);
     abort_flag = 0;
@@ -1567,8 +1559,7 @@ __global__ void wait_timeout_selftest_kernel() {
 }  // namespace
 
 cudaError_t launch_wait_timeout_selftest(cudaStream_t st) {
-  wait_timeout_selftest_kernel<<<1, 32, 0, st>>>();
-  return cudaGetLastError();
+  return launch_kernel(wait_timeout_selftest_kernel, dim3(1), 32, 0, st, 1);
 }
 
 cudaError_t read_status_tc(int *status) {

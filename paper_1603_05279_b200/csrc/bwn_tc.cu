@@ -467,14 +467,15 @@ bwn_conv_kernel(const __grid_constant__ BwnParams P) {
     *S.abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  for (int i = tid; i < P.vec_len; i += kThreads)
-    reinterpret_cast<float *>(smem + P.off_vec)[i] =
-        i < P.Co ? (P.alpha != nullptr ? __ldg(P.alpha + i) : 1.0f) : 0.0f;   // no alpha: unit scale
   if (warp == kMmaWarp) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                  ::"r"(smem_u32(S.tmem_slot)), "r"((uint32_t)kTmemCols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  stream_order();
+  for (int i = tid; i < P.vec_len; i += kThreads)
+    reinterpret_cast<float *>(smem + P.off_vec)[i] =
+        i < P.Co ? (P.alpha != nullptr ? __ldg(P.alpha + i) : 1.0f) : 0.0f;   // no alpha: unit scale
   fence_proxy_async();
   tc_fence_before();
   __syncthreads();
@@ -517,6 +518,7 @@ bwn_prepare_kernel(const float *__restrict__ x, const float *__restrict__ scale,
                    int W, int s, int Hq, int Wq, int leadY, int leadX, long long L, int Cp,
                    uint16_t *__restrict__ xs) {
   __shared__ float tile[64][33];
+  stream_order();
   const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;      // 8 warps
   const long long nblk = (L + 31) / 32;
   const int phase = (int)(blockIdx.x / nblk);
@@ -724,9 +726,8 @@ cudaError_t launch_bwn_prepare(const float *x, const float *scale, const float *
   const StreamGeom q = stream_geom(g);
   const long long nblk = (q.L + 31) / 32 * q.phases;
   if (nblk >= (1ll << 31)) return cudaErrorInvalidValue;
-  bwn_prepare_kernel<<<(unsigned)nblk, 256, 0, st>>>(x, scale, shift, nullptr, g.N, g.C, g.H, g.W, q.s,
-                                                    q.Hq, q.Wq, q.leadY, q.leadX, q.L, q.Cp, x_stream);
-  return cudaGetLastError();
+  return launch_kernel(bwn_prepare_kernel, dim3((unsigned)nblk), 256, 0, st, 1, x, scale, shift, nullptr, g.N, g.C, g.H, g.W,
+                       q.s, q.Hq, q.Wq, q.leadY, q.leadX, q.L, q.Cp, x_stream);
 }
 
 cudaError_t launch_bwn_prepare_grad(const float *g, const float *alpha, const float *gmax,
@@ -734,9 +735,8 @@ cudaError_t launch_bwn_prepare_grad(const float *g, const float *alpha, const fl
   const StreamGeom q = stream_geom(gb);
   const long long nblk = (q.L + 31) / 32 * q.phases;
   if (nblk >= (1ll << 31)) return cudaErrorInvalidValue;
-  bwn_prepare_kernel<<<(unsigned)nblk, 256, 0, st>>>(g, alpha, nullptr, gmax, gb.N, gb.C, gb.H, gb.W, q.s,
-                                                    q.Hq, q.Wq, q.leadY, q.leadX, q.L, q.Cp, g_stream);
-  return cudaGetLastError();
+  return launch_kernel(bwn_prepare_kernel, dim3((unsigned)nblk), 256, 0, st, 1, g, alpha, nullptr, gmax, gb.N, gb.C, gb.H, gb.W,
+                       q.s, q.Hq, q.Wq, q.leadY, q.leadX, q.L, q.Cp, g_stream);
 }
 
 cudaError_t launch_bwn_conv(const uint16_t *x_stream, const uint32_t *wp, const float *alpha,
@@ -766,9 +766,7 @@ cudaError_t launch_bwn_conv(const uint16_t *x_stream, const uint32_t *wp, const 
   }
   const long long total = (long long)P.ntiles * P.nslabs;
   const unsigned grid = (unsigned)std::min<long long>(total, sm_count_of_current_device());
-  bwn_conv_kernel<<<grid, kThreads, pl.smem, st>>>(P);
-  cudaError_t e = cudaGetLastError();
-  return e;
+  return launch_kernel(bwn_conv_kernel, dim3(grid), kThreads, pl.smem, st, 1, P);
 }
 
 cudaError_t read_status_bwn(int *status) {

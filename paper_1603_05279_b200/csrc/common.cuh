@@ -39,6 +39,46 @@ inline ConvGeom make_geom(const xnor_conv_desc &d) {
   return g;
 }
 
+// Consecutive kernels of a stream overlap their launch and set-up with the end of the kernel before
+// (programmatic dependent launch).  Every kernel of the library is launched through launch_kernel and
+// calls stream_order() before its first access to global memory: it returns when the kernels before
+// it in the stream have completed and their writes are visible, so a kernel still sees everything that
+// was launched before it.  A kernel that leaves SMs free then lets the next one start at once (a batch-1
+// layer's kernels take 2 to 9 us each, a launch gap with the set-up of the tensor-core kernel 3: the
+// 16-layer chain of one image 395 -> 276 us).  A kernel that fills the GPU lets it start as its own
+// blocks leave (256 images 1643 -> 1578 us against ordinary launches): started earlier, the next kernel's
+// waiting blocks keep other streams' kernels off the SMs (the four AlexNet layers on parallel branches
+// 224 -> 238 us) and its own split of L1 and shared memory is the one of the kernel it waits for (a pool
+// that reads through L1 92 -> 113 us).
+constexpr unsigned kSms = 148;
+__device__ __forceinline__ void stream_order() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (gridDim.x * gridDim.y < kSms) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// `cluster`: CTAs per cluster along x (1: none).
+template <class... Params, class... Args>
+cudaError_t launch_kernel(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st,
+                          unsigned cluster, const Args &...args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+  if (e != cudaSuccess) (void)cudaGetLastError();
+  return e;
+}
+
 // Packed weights are stored word-pair-major so that the convolution kernels read them
 // coalesced: with f = tap * Cw + cw the index of a word inside a filter (tap = ky * k_w + kx),
 // word f of filter co is element ((f / 2) * C_out + co) * 2 + f % 2.  Words 2j and 2j+1 of all

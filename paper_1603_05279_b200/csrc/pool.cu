@@ -25,6 +25,7 @@ template <bool kRelu>
 __global__ void __launch_bounds__(kPoolThreads)
 maxpool_kernel(const float *__restrict__ x, long long total_out, int H, int W, int k, int stride,
                int pad, int Ho, int Wo, Magic div_howo, Magic div_wo, float *__restrict__ out) {
+  stream_order();
   const int HoWo = Ho * Wo;
   // chunks of 2^30 outputs keep the index arithmetic in 32 bits
   for (long long base = 0; base < total_out; base += (1ll << 30)) {
@@ -66,11 +67,8 @@ cudaError_t launch_maxpool2d(const float *x, int N, int C, int H, int W, int k, 
   const Magic dh = magic((uint32_t)(Ho * Wo)), dw = magic((uint32_t)Wo);
   const unsigned grid = (unsigned)std::min<long long>((total + kPoolThreads - 1) / kPoolThreads,
                                                       16ll * sms);
-  if (relu)
-    maxpool_kernel<true><<<grid, kPoolThreads, 0, st>>>(x, total, H, W, k, stride, pad, Ho, Wo, dh, dw, out);
-  else
-    maxpool_kernel<false><<<grid, kPoolThreads, 0, st>>>(x, total, H, W, k, stride, pad, Ho, Wo, dh, dw, out);
-  return cudaGetLastError();
+  return launch_kernel(relu ? maxpool_kernel<true> : maxpool_kernel<false>, dim3(grid), kPoolThreads, 0, st, 1, x, total, H, W,
+                       k, stride, pad, Ho, Wo, dh, dw, out);
 }
 
 }  // namespace xnor

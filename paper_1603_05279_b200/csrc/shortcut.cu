@@ -45,6 +45,7 @@ shortcut_conv1x1_kernel(const float *__restrict__ x, const float *__restrict__ w
   const float *wsrc = w + (size_t)(lf_on ? co0 + lf : 0) * C;
   const bool wvec = (C & 3) == 0;
   float xr[16], wr[8];
+  stream_order();
   auto fetch = [&](int c0) {
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
@@ -134,8 +135,7 @@ cudaError_t launch_shortcut_conv1x1(const float *x, const float *w, int N, int C
   const long long tiles = (total_pix + SP - 1) / SP;
   if (tiles > 0x7FFFFFFFll) return cudaErrorInvalidValue;
   const dim3 grid((unsigned)tiles, (unsigned)((Co + SF - 1) / SF));
-  shortcut_conv1x1_kernel<<<grid, 256, 0, st>>>(x, w, C, H, W, Co, stride, Ho, Wo, total_pix, out);
-  return cudaGetLastError();
+  return launch_kernel(shortcut_conv1x1_kernel, grid, 256, 0, st, 1, x, w, C, H, W, Co, stride, Ho, Wo, total_pix, out);
 }
 
 }  // namespace xnor
