@@ -4,8 +4,11 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "umma_common.cuh"
 
 namespace xnor {
+
+__device__ int g_status_pool = 0;
 
 namespace {
 
@@ -17,10 +20,113 @@ __device__ __forceinline__ uint32_t fast_div(uint32_t n, Magic g) {
   return (uint32_t)(((uint64_t)n * g.m) >> (31 + g.s));
 }
 
-// A thread per output (consecutive threads = consecutive outputs of a plane, so stores are
-// coalesced); its window comes through the read-only cache, where the overlapping windows of
-// neighbouring outputs meet, so HBM sees each input element once.  (A variant that staged
-// whole planes in shared memory first was measured slower: 1.9 against 2.3-2.5 TB/s.)
+struct PoolParams {
+  const float *x;
+  float *out;
+  long long planes;              // N * C
+  int H, W, k, stride, pad, Ho, Wo;
+  Magic div_howo, div_wo;
+  int per_chunk;                 // planes per chunk: a multiple of 4, so that chunks start on 16 bytes
+  uint32_t chunk_bytes;          // shared memory of a chunk's planes
+};
+
+// Maximum over the window whose corner is (iy, ix) of plane t in shared memory.
+// KS > 0: windows of KS x KS wholly inside the plane.
+template <int KS>
+__device__ __forceinline__ float window_max(const PoolParams &P, const float *t, int iy, int ix) {
+  if constexpr (KS > 0) {
+    const float *r = t + iy * P.W + ix;
+    float m = r[0];
+#pragma unroll
+    for (int ky = 0; ky < KS; ++ky)
+#pragma unroll
+      for (int kx = 0; kx < KS; ++kx)
+        if (ky + kx > 0) m = fmaxf(m, r[ky * P.W + kx]);
+    return m;
+  } else {
+    const int y0 = max(iy, 0), y1 = min(iy + P.k, P.H), x0 = max(ix, 0), x1 = min(ix + P.k, P.W);
+    float m = t[y0 * P.W + x0];
+    for (int y = y0; y < y1; ++y)
+      for (int x = x0; x < x1; ++x) m = fmaxf(m, t[y * P.W + x]);
+    return m;
+  }
+}
+
+// Planes are streamed through shared memory: a chunk is a few whole planes, contiguous in memory and
+// 16-byte aligned, and comes in with one bulk copy; kBufs chunks per block in flight.  HBM bounds it.
+constexpr int kBufs = 4;
+template <bool kRelu, int KS>
+__global__ void __launch_bounds__(kPoolThreads) maxpool_stream_kernel(const PoolParams P) {
+  using namespace umma;
+  extern __shared__ __align__(128) uint8_t smem[];
+  __shared__ __align__(8) uint64_t full[kBufs];
+  __shared__ volatile int abort_flag;
+  const int tid = threadIdx.x;
+  const uint32_t base = smem_u32(smem);
+  const int HW = P.H * P.W, HoWo = P.Ho * P.Wo;
+  const long long nchunks = (P.planes + P.per_chunk - 1) / P.per_chunk;
+  if (tid == 0) {
+    for (int i = 0; i < kBufs; ++i) mbar_init(smem_u32(&full[i]), 1);
+    abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  stream_order();
+  // thread 0: chunk c into buffer b; the tensor's last floats (its size need not be a multiple of
+  // four) by plain loads
+  auto fetch = [&](long long c, int b) {
+    const long long p0 = c * P.per_chunk, np = min((long long)P.per_chunk, P.planes - p0);
+    const uint32_t floats = (uint32_t)np * (uint32_t)HW, bulk = floats & ~3u, dst = base + (uint32_t)b * P.chunk_bytes;
+    const float *src = P.x + (size_t)p0 * HW;
+    for (uint32_t i = bulk; i < floats; ++i) reinterpret_cast<float *>(smem + (size_t)b * P.chunk_bytes)[i] = __ldg(src + i);
+    const uint32_t bar = smem_u32(&full[b]);
+    if (bulk) {
+      mbar_arrive_expect_tx(bar, bulk * 4u);
+      bulk_copy_g2s(dst, src, bulk * 4u, bar);
+    } else {
+      mbar_arrive(bar);
+    }
+  };
+  long long next = blockIdx.x;
+  int pending = 0;                       // copies started and not yet waited for
+  if (tid == 0)
+    for (int b = 0; b < kBufs - 1 && next < nchunks; ++b, next += gridDim.x, ++pending) fetch(next, b);
+  int b = 0;
+  uint32_t ph = 0u;
+  bool ok = true;
+  for (long long c = blockIdx.x; c < nchunks; c += gridDim.x) {
+    // the buffer filled now is the one every thread left before the last __syncthreads
+    if (tid == 0 && next < nchunks) {
+      fence_proxy_async();
+      fetch(next, b == 0 ? kBufs - 1 : b - 1);
+      next += gridDim.x;
+      ++pending;
+    }
+    ok = mbar_wait(smem_u32(&full[b]), ph, &abort_flag, &g_status_pool);
+    if (__syncthreads_or(!ok)) break;
+    --pending;
+    const long long p0 = c * P.per_chunk;
+    const uint32_t count = (uint32_t)min((long long)P.per_chunk, P.planes - p0) * (uint32_t)HoWo;
+    const float *chunk = reinterpret_cast<const float *>(smem + (size_t)b * P.chunk_bytes);
+    float *out = P.out + (size_t)p0 * HoWo;
+    for (uint32_t i = tid; i < count; i += kPoolThreads) {
+      const uint32_t pl = fast_div(i, P.div_howo), r = i - pl * (uint32_t)HoWo, oy = fast_div(r, P.div_wo), ox = r - oy * (uint32_t)P.Wo;
+      const float m = window_max<KS>(P, chunk + (size_t)pl * HW, (int)oy * P.stride - P.pad, (int)ox * P.stride - P.pad);
+      __stcs(out + i, kRelu ? fmaxf(m, 0.0f) : m);
+    }
+    if (++b == kBufs) { b = 0; ph ^= 1u; }
+    __syncthreads();
+  }
+  // gave up: the copies in flight must land before the block's shared memory is released
+  if (tid == 0)
+    for (; pending > 0; --pending) {
+      for (int i = 0; i < (1 << 20) && !mbar_try(smem_u32(&full[b]), ph); ++i) {}
+      if (++b == kBufs) { b = 0; ph ^= 1u; }
+    }
+}
+
+// A thread per output, its window through the read-only cache: planes too large to stage, and calls
+// too small to be worth it.
 template <bool kRelu>
 __global__ void __launch_bounds__(kPoolThreads)
 maxpool_kernel(const float *__restrict__ x, long long total_out, int H, int W, int k, int stride,
@@ -49,6 +155,18 @@ maxpool_kernel(const float *__restrict__ x, long long total_out, int H, int W, i
   }
 }
 
+template <bool kRelu, int KS>
+cudaError_t launch_stream(const PoolParams &P, unsigned grid, size_t smem, cudaStream_t st) {
+  static bool attr_flags[64] = {};
+  bool &attr_set = attr_done_for_current_device(attr_flags);
+  if (!attr_set) {
+    cudaError_t e = cudaFuncSetAttribute(maxpool_stream_kernel<kRelu, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024);
+    if (e != cudaSuccess) { (void)cudaGetLastError(); return e; }
+    attr_set = true;
+  }
+  return launch_kernel(maxpool_stream_kernel<kRelu, KS>, dim3(grid), kPoolThreads, smem, st, 1, P);
+}
+
 }  // namespace
 
 cudaError_t launch_maxpool2d(const float *x, int N, int C, int H, int W, int k, int stride, int pad,
@@ -65,10 +183,39 @@ cudaError_t launch_maxpool2d(const float *x, int N, int C, int H, int W, int k, 
     return g;
   };
   const Magic dh = magic((uint32_t)(Ho * Wo)), dw = magic((uint32_t)Wo);
+  // Streamed when chunks of at least four planes and at most 24 KB exist, enough of them for several
+  // rounds of every block (two blocks per SM, four chunks each).  AlexNet's 3x3/2 pool of conv2's
+  // output (235 MB): 92 us with a thread per output, bounded by its nine global loads, 57 us streamed (4.1 TB/s).
+  const size_t four = 16 * (size_t)H * W;
+  if (four <= 24 * 1024) {
+    PoolParams P;
+    P.x = x; P.out = out; P.planes = (long long)N * C;
+    P.H = H; P.W = W; P.k = k; P.stride = stride; P.pad = pad; P.Ho = Ho; P.Wo = Wo;
+    P.div_howo = dh; P.div_wo = dw;
+    P.per_chunk = 4 * (int)std::max<size_t>(1, 16 * 1024 / four);
+    P.chunk_bytes = (uint32_t)(((size_t)P.per_chunk * H * W * 4 + 127) / 128 * 128);
+    const long long nchunks = (P.planes + P.per_chunk - 1) / P.per_chunk;
+    if (nchunks >= 4ll * sms) {
+      const unsigned grid = (unsigned)std::min<long long>(nchunks, 2ll * sms);
+      const size_t smem = (size_t)kBufs * P.chunk_bytes;
+      // windows that never leave the plane: no clipping
+      const bool inside = pad == 0;
+      if (inside && k == 3) return relu ? launch_stream<true, 3>(P, grid, smem, st) : launch_stream<false, 3>(P, grid, smem, st);
+      if (inside && k == 2) return relu ? launch_stream<true, 2>(P, grid, smem, st) : launch_stream<false, 2>(P, grid, smem, st);
+      return relu ? launch_stream<true, 0>(P, grid, smem, st) : launch_stream<false, 0>(P, grid, smem, st);
+    }
+  }
   const unsigned grid = (unsigned)std::min<long long>((total + kPoolThreads - 1) / kPoolThreads,
                                                       16ll * sms);
   return launch_kernel(relu ? maxpool_kernel<true> : maxpool_kernel<false>, dim3(grid), kPoolThreads, 0, st, 1, x, total, H, W,
                        k, stride, pad, Ho, Wo, dh, dw, out);
+}
+
+cudaError_t read_status_pool(int *status) {
+  cudaError_t e = cudaMemcpyFromSymbol(status, g_status_pool, sizeof(int));
+  const int zero = 0;
+  if (e == cudaSuccess && *status != 0) e = cudaMemcpyToSymbol(g_status_pool, &zero, sizeof(int));
+  return e;
 }
 
 }  // namespace xnor
