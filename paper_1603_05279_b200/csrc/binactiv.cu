@@ -19,6 +19,11 @@ __device__ __forceinline__ uint32_t smem_addr(const void *p) {
   return (uint32_t)__cvta_generic_to_shared(p);
 }
 
+// Decision point tau_j of q_k: the level index is at least j exactly when y >= tau_j.
+__host__ __device__ constexpr float decision_point(int j, int kbits) {
+  return (float)((double)(2 * j - 1) / (double)((1 << kbits) - 1) - 1.0);
+}
+
 // Persistent blocks of 8 warps.  A task is (group of 32 consecutive pixels, flat over n,h,w;
 // 32-channel word): lane = pixel, so one channel of a task is a contiguous 128-byte run of
 // x.  The G warps of a pixel group take words g, g + G, ...; a block works on 8 / G pixel
@@ -28,16 +33,26 @@ __device__ __forceinline__ uint32_t smem_addr(const void *p) {
 // bandwidth needs) do not depend on how the compiler schedules loads against their uses.
 // Packed words are staged and written as contiguous runs; A is reduced over the warps of a
 // pixel group in a fixed order.
-template <bool kHasBN, bool kVec16>
+// kBits: 1 = sign bits; 2 = two bit planes of the level index (decision points in registers); 0 = any
+// number of planes (bisection over the decision points in shared memory); see "BinActiv with k-bit
+// activations" below.  x_packed is then [kbits][N][H][W][Cw].
+template <bool kHasBN, bool kVec16, int kBits>
 __global__ void __launch_bounds__(32 * kWarps)
 binactiv_pack_kernel(const float *__restrict__ x, const float *__restrict__ scale,
                      const float *__restrict__ shift, long long total_pix, int C, int HW, int Cw,
-                     int G, int PG, uint32_t *__restrict__ x_packed, float *__restrict__ A) {
+                     int G, int PG, int kbits, uint32_t *__restrict__ x_packed, float *__restrict__ A) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
+  const int nplanes = kBits > 0 ? kBits : kbits;
+  const int plane_words = PG * kPix * Cw;                  // staged words of a bit plane
+  const size_t out_words = (size_t)total_pix * Cw;         // words of a bit plane of the tensor
+  __shared__ float tau[kBits == 0 ? 128 : 1];
+  constexpr float t1 = decision_point(1, 2), t2 = decision_point(2, 2), t3 = decision_point(3, 2);
+  if (kBits == 0)
+    for (int j = 1 + threadIdx.x; j < (1 << kbits); j += 32 * kWarps) tau[j] = decision_point(j, kbits);
   float *stage = reinterpret_cast<float *>(smem_raw);                      // [warp][buf][32][32]
   float2 *bn = reinterpret_cast<float2 *>(stage + kWarps * kBufsPerWarp * kTileFloats);  // [Cw*32]
-  uint32_t *words = reinterpret_cast<uint32_t *>(bn + (kHasBN ? Cw * 32 : 0));  // [PG][32][Cw]
-  float *sabs = reinterpret_cast<float *>(words + PG * kPix * Cw);          // [PG][G][32]
+  uint32_t *words = reinterpret_cast<uint32_t *>(bn + (kHasBN ? Cw * 32 : 0));  // [planes][PG][32][Cw]
+  float *sabs = reinterpret_cast<float *>(words + nplanes * plane_words);   // [PG][G][32]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int pgl = warp / G, g = warp - pgl * G;
   const bool active = pgl < PG;
@@ -119,9 +134,27 @@ binactiv_pack_kernel(const float *__restrict__ x, const float *__restrict__ scal
       const int cw = g + k * G;
       const int c0 = cw * 32;
       const float *t = my_stage + buf * kTileFloats + lane;
-      uint32_t word = 0u;
+      uint32_t word = 0u, word2 = 0u;
       float part = 0.0f;
-      if (live) {
+      if (kBits == 0) {
+        // any number of planes: the words are built in shared memory
+        float p0 = 0.0f, p1 = 0.0f;
+        uint32_t *w = words + (pgl * kPix + lane) * Cw + cw;
+        for (int pl = 0; pl < nplanes; ++pl) w[pl * plane_words] = 0u;
+        if (live) {
+          const int nc = min(32, C - c0);
+          for (int j = 0; j < nc; ++j) {
+            float y = t[j * kPix];
+            if (kHasBN) y = __fmaf_rn(bn[c0 + j].x, y, bn[c0 + j].y);
+            if (j & 1) p1 += fabsf(y); else p0 += fabsf(y);
+            int idx = 0;                       // the largest index whose decision point is <= y
+            for (int b = nplanes - 1; b >= 0; --b)
+              if (y >= tau[idx + (1 << b)]) idx += 1 << b;
+            for (int pl = 0; pl < nplanes; ++pl) w[pl * plane_words] |= (uint32_t)((idx >> pl) & 1) << j;
+          }
+          part = p0 + p1;
+        }
+      } else if (live) {
         const float2 *ss = bn + c0;
         if (c0 + 32 <= C) {
           // two interleaved sums keep the additions from forming one long dependent chain
@@ -133,8 +166,17 @@ binactiv_pack_kernel(const float *__restrict__ x, const float *__restrict__ scal
               y0 = __fmaf_rn(ss[j].x, y0, ss[j].y);
               y1 = __fmaf_rn(ss[j + 1].x, y1, ss[j + 1].y);
             }
-            if (y0 >= 0.0f) word |= 1u << j;
-            if (y1 >= 0.0f) word |= 2u << j;
+            if (kBits == 1) {
+              if (y0 >= 0.0f) word |= 1u << j;
+              if (y1 >= 0.0f) word |= 2u << j;
+            } else {
+              // bit 1 of the index: y >= tau_2; bit 0: the parity of how many comparisons hold
+              const bool b0 = y0 >= t2, b1 = y1 >= t2;
+              if (b0 ? y0 >= t3 : y0 >= t1) word |= 1u << j;
+              if (b1 ? y1 >= t3 : y1 >= t1) word |= 2u << j;
+              if (b0) word2 |= 1u << j;
+              if (b1) word2 |= 2u << j;
+            }
             p0 += fabsf(y0);
             p1 += fabsf(y1);
           }
@@ -143,13 +185,20 @@ binactiv_pack_kernel(const float *__restrict__ x, const float *__restrict__ scal
           for (int j = 0; c0 + j < C; ++j) {
             float y = t[j * kPix];
             if (kHasBN) y = __fmaf_rn(ss[j].x, y, ss[j].y);
-            if (y >= 0.0f) word |= 1u << j;
+            if (kBits == 1) {
+              if (y >= 0.0f) word |= 1u << j;
+            } else {
+              const bool b = y >= t2;
+              if (b ? y >= t3 : y >= t1) word |= 1u << j;
+              if (b) word2 |= 1u << j;
+            }
             part += fabsf(y);
           }
         }
       }
       asum += part;
-      words[(pgl * kPix + lane) * Cw + cw] = word;
+      if (kBits > 0) words[(pgl * kPix + lane) * Cw + cw] = word;
+      if (kBits == 2) words[plane_words + (pgl * kPix + lane) * Cw + cw] = word2;
       __syncwarp();                      // every lane is done reading the tile before it is refilled
       issue(fb, fk, buf); advance_fetch();                   // refill the tile just consumed
       buf ^= 1;
@@ -161,9 +210,11 @@ binactiv_pack_kernel(const float *__restrict__ x, const float *__restrict__ scal
       long long npix = total_pix - gp0;
       if (npix > kPix) npix = kPix;
       if (npix > 0) {
-        uint32_t *dst = x_packed + (size_t)gp0 * Cw;
-        const uint32_t *srcw = words + pgl * kPix * Cw;
-        for (int i = lane; i < (int)npix * Cw; i += 32) dst[i] = srcw[i];
+        for (int pl = 0; pl < nplanes; ++pl) {
+          uint32_t *dst = x_packed + pl * out_words + (size_t)gp0 * Cw;
+          const uint32_t *srcw = words + pl * plane_words + pgl * kPix * Cw;
+          for (int i = lane; i < (int)npix * Cw; i += 32) dst[i] = srcw[i];
+        }
       }
       __syncwarp();
       continue;
@@ -179,8 +230,10 @@ binactiv_pack_kernel(const float *__restrict__ x, const float *__restrict__ scal
     const long long bp0 = batch * PG * kPix;
     long long npix = total_pix - bp0;
     if (npix > PG * kPix) npix = PG * kPix;
-    uint32_t *dst = x_packed + (size_t)bp0 * Cw;
-    for (int i = threadIdx.x; i < (int)npix * Cw; i += 32 * kWarps) dst[i] = words[i];
+    for (int pl = 0; pl < nplanes; ++pl) {
+      uint32_t *dst = x_packed + pl * out_words + (size_t)bp0 * Cw;
+      for (int i = threadIdx.x; i < (int)npix * Cw; i += 32 * kWarps) dst[i] = words[pl * plane_words + i];
+    }
     __syncthreads();
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -524,24 +577,24 @@ constexpr size_t kPackSmemMax = 100 * 1024;      // three blocks per SM
 
 struct PackPlan { int G, PG; size_t smem; };
 
-size_t pack_smem(int Cw, bool bn, int G, int PG) {
+size_t pack_smem(int Cw, bool bn, int G, int PG, int planes) {
   return (size_t)kWarps * kBufsPerWarp * kTileFloats * sizeof(float) +
-         (bn ? (size_t)Cw * 32 * sizeof(float2) : 0) + (size_t)PG * kPix * Cw * sizeof(uint32_t) +
+         (bn ? (size_t)Cw * 32 * sizeof(float2) : 0) + (size_t)planes * PG * kPix * Cw * sizeof(uint32_t) +
          (size_t)PG * G * kPix * sizeof(float);
 }
 
 // With enough pixel groups to fill the GPU every warp packs whole pixel groups on its own
 // (G = 1); otherwise, or when the staged words of eight pixel groups do not fit shared
 // memory (many channels), the channel words of a pixel group are spread over the warps.
-bool pack_plan(const ConvGeom &g, bool bn, PackPlan *pl) {
+bool pack_plan(const ConvGeom &g, bool bn, PackPlan *pl, int planes = 1) {
   const long long total_pix = (long long)g.N * g.H * g.W;
   const long long ngroups = (total_pix + kPix - 1) / kPix;
   const int Gs = g.Cw < kWarps ? g.Cw : kWarps;
   int G = ngroups >= 2048 ? 1 : Gs;
-  if (pack_smem(g.Cw, bn, G, kWarps / G) > kPackSmemMax) G = Gs;
+  if (pack_smem(g.Cw, bn, G, kWarps / G, planes) > kPackSmemMax) G = Gs;
   pl->G = G;
   pl->PG = kWarps / G;
-  pl->smem = pack_smem(g.Cw, bn, G, pl->PG);
+  pl->smem = pack_smem(g.Cw, bn, G, pl->PG, planes);
   return pl->smem <= kPackSmemMax;
 }
 
@@ -650,10 +703,49 @@ bool binactiv_supported(const ConvGeom &g, bool has_bn) {
   return g.N <= 65535 && pack_plan(g, has_bn, &pl);
 }
 
+namespace {
+
+template <bool kHasBN, bool kVec16, int kBits>
+cudaError_t launch_pack_variant(const float *x, const float *scale, const float *shift, const ConvGeom &g,
+                                const PackPlan &pl, int kbits, uint32_t *x_packed, float *A, cudaStream_t st) {
+  const auto kern = binactiv_pack_kernel<kHasBN, kVec16, kBits>;
+  static bool attr_flags[64] = {};
+  bool &attr_set = attr_done_for_current_device(attr_flags);
+  if (!attr_set) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPackSmemMax);
+    if (e != cudaSuccess) { (void)cudaGetLastError(); return e; }
+    attr_set = true;
+  }
+  const long long total_pix = (long long)g.N * g.H * g.W;
+  const long long nbatches = ((total_pix + kPix - 1) / kPix + pl.PG - 1) / pl.PG;
+  // persistent grid: as many blocks as are resident at once (the shared-memory split the driver picks
+  // for this kernel decides whether two or three fit an SM), so that no block waits for a second wave
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kWarps, pl.smem) != cudaSuccess || per_sm < 1) {
+    (void)cudaGetLastError();
+    per_sm = 2;
+  }
+  const long long resident = (long long)per_sm * sm_count_of_current_device();
+  const unsigned grid = (unsigned)(nbatches < resident ? nbatches : resident);
+  return launch_kernel(kern, dim3(grid), 32 * kWarps, pl.smem, st, 1, x, scale, shift, total_pix, g.C, g.H * g.W, g.Cw, pl.G,
+                       pl.PG, kbits, x_packed, A);
+}
+
+template <int kBits>
+cudaError_t launch_pack(const float *x, const float *scale, const float *shift, const ConvGeom &g, const PackPlan &pl,
+                        int kbits, uint32_t *x_packed, float *A, cudaStream_t st) {
+  const bool v16 = ((g.H * g.W) & 3) == 0;
+  if (scale) return v16 ? launch_pack_variant<true, true, kBits>(x, scale, shift, g, pl, kbits, x_packed, A, st)
+                        : launch_pack_variant<true, false, kBits>(x, scale, shift, g, pl, kbits, x_packed, A, st);
+  return v16 ? launch_pack_variant<false, true, kBits>(x, scale, shift, g, pl, kbits, x_packed, A, st)
+             : launch_pack_variant<false, false, kBits>(x, scale, shift, g, pl, kbits, x_packed, A, st);
+}
+
+}  // namespace
+
 cudaError_t launch_binactiv(const float *x, const float *scale, const float *shift,
                             const ConvGeom &g, uint32_t *x_packed, float *A, float *K,
                             cudaStream_t st) {
-  const long long total_pix = (long long)g.N * g.H * g.W;
   PackPlan pl;
   if (g.N > 65535 || !pack_plan(g, scale != nullptr, &pl)) return cudaErrorInvalidValue;
   const int sms = sm_count_of_current_device();
@@ -664,43 +756,7 @@ cudaError_t launch_binactiv(const float *x, const float *scale, const float *shi
       return launch_binactiv_image(ip, scale != nullptr, sms, st);
     }
   }
-  const int G = pl.G, PG = pl.PG;
-  const size_t smem = pl.smem;
-  static bool attr_flags[64] = {};
-  bool &attr_set = attr_done_for_current_device(attr_flags);
-  if (!attr_set) {
-    cudaError_t e = cudaSuccess;
-    const void *kernels[4] = {(const void *)binactiv_pack_kernel<true, true>,
-                              (const void *)binactiv_pack_kernel<true, false>,
-                              (const void *)binactiv_pack_kernel<false, true>,
-                              (const void *)binactiv_pack_kernel<false, false>};
-    for (int i = 0; i < 4 && e == cudaSuccess; ++i)
-      e = cudaFuncSetAttribute(kernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPackSmemMax);
-    if (e != cudaSuccess) { (void)cudaGetLastError(); return e; }
-    attr_set = true;
-  }
-  const long long nbatches = ((total_pix + kPix - 1) / kPix + PG - 1) / PG;
-  const bool v16 = ((g.H * g.W) & 3) == 0;
-  // persistent grid: as many blocks as are resident at once (the shared-memory split the driver
-  // picks for this kernel decides whether two or three fit an SM), so that no block waits for
-  // a second wave
-  const void *kern = scale ? (v16 ? (const void *)binactiv_pack_kernel<true, true>
-                                  : (const void *)binactiv_pack_kernel<true, false>)
-                           : (v16 ? (const void *)binactiv_pack_kernel<false, true>
-                                  : (const void *)binactiv_pack_kernel<false, false>);
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kWarps, smem) != cudaSuccess ||
-      per_sm < 1) {
-    (void)cudaGetLastError();
-    per_sm = 2;
-  }
-  const long long resident = (long long)per_sm * sms;
-  const unsigned grid = (unsigned)(nbatches < resident ? nbatches : resident);
-#define XNOR_PACK(BN, V16) launch_kernel(binactiv_pack_kernel<BN, V16>, dim3(grid), 32 * kWarps, smem, st, 1, \
-      x, scale, shift, total_pix, g.C, g.H * g.W, g.Cw, G, PG, x_packed, A)
-  const cudaError_t e = scale ? (v16 ? XNOR_PACK(true, true) : XNOR_PACK(true, false))
-                              : (v16 ? XNOR_PACK(false, true) : XNOR_PACK(false, false));
-#undef XNOR_PACK
+  const cudaError_t e = launch_pack<1>(x, scale, shift, g, pl, 1, x_packed, A, st);
   if (e != cudaSuccess) return e;
   return launch_box_filter(A, g, K, st);
 }
@@ -822,6 +878,16 @@ cudaError_t launch_binactiv_kbit(const float *x, const float *scale, const float
       fill_img_params(ip, x, scale, shift, g, x_planes, A, K);
       return launch_binactiv_image(ip, scale != nullptr, sms, st);
     }
+  }
+  // The pipelined pack kernel with k bit planes per tile (128x28x28, 256 images, k = 2: 30 us, the
+  // simple kernel below 127); the simple one where the staged words do not fit shared memory.
+  PackPlan pl;
+  if (pack_plan(g, scale != nullptr, &pl, kbits)) {
+    cudaError_t e = kbits == 1 ? launch_pack<1>(x, scale, shift, g, pl, 1, x_planes, A, st)
+                    : kbits == 2 ? launch_pack<2>(x, scale, shift, g, pl, 2, x_planes, A, st)
+                                 : launch_pack<0>(x, scale, shift, g, pl, kbits, x_planes, A, st);
+    if (e != cudaSuccess) return e;
+    return launch_box_filter(A, g, K, st);
   }
   const long long total_pix = (long long)g.N * g.H * g.W;
   const long long nblocks = ((total_pix + 31) / 32 + 7) / 8;
