@@ -975,12 +975,12 @@ __device__ bool epilogue_role(const TcParams &P, const Smem &S, long long i0, in
 #pragma unroll
           for (int j = 0; j < 16; ++j) v[j] = fmaxf(v[j], 0.0f);
         }
-        // one address per store, each one multiply-add from the one before; streaming stores
-        // (the output is not read again by this kernel: evict-first keeps the L2 for the inputs;
-        // 6-8 % on the ResNet layers run back to back, nothing on a whole step)
+        // one address per store, each one multiply-add from the one before.  (Evict-first stores gain
+        // 6-8 % on the ResNet layers run back to back, but the next layer's BinActiv or pool, which
+        // starts with what was written last, then finds less of it in the L2.)
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
-          if (in_bounds(obase + (size_t)(co + j) * HoWo < out_elems, 7)) __stcs(op, v[j]);
+          if (in_bounds(obase + (size_t)(co + j) * HoWo < out_elems, 7)) *op = v[j];
           op += howo;
         }
       } else if (co + 16 <= P.Co && with_res) {
@@ -995,7 +995,7 @@ __device__ bool epilogue_role(const TcParams &P, const Smem &S, long long i0, in
 #pragma unroll
           for (int jj = 0; jj < 4; ++jj) {
             const float v = __fmul_rn(__fmul_rn(__int_as_float(r[j4 * 4 + jj]), kv), a4[jj]) + res[j4 * 4 + jj];
-            if (in_bounds((size_t)(op - P.out) < out_elems, 8)) __stcs(op, relu ? fmaxf(v, 0.0f) : v);
+            if (in_bounds((size_t)(op - P.out) < out_elems, 8)) *op = relu ? fmaxf(v, 0.0f) : v;
             op += howo;
           }
         }

@@ -72,10 +72,12 @@ __global__ void __launch_bounds__(kPoolThreads) maxpool_stream_kernel(const Pool
   }
   __syncthreads();
   stream_order();
+  // from the end to the start: the last part of what the convolution wrote is still in the L2
+  auto place = [&](long long c) { return nchunks - 1 - c; };
   // thread 0: chunk c into buffer b; the tensor's last floats (its size need not be a multiple of
   // four) by plain loads
   auto fetch = [&](long long c, int b) {
-    const long long p0 = c * P.per_chunk, np = min((long long)P.per_chunk, P.planes - p0);
+    const long long p0 = place(c) * P.per_chunk, np = min((long long)P.per_chunk, P.planes - p0);
     const uint32_t floats = (uint32_t)np * (uint32_t)HW, bulk = floats & ~3u, dst = base + (uint32_t)b * P.chunk_bytes;
     const float *src = P.x + (size_t)p0 * HW;
     for (uint32_t i = bulk; i < floats; ++i) reinterpret_cast<float *>(smem + (size_t)b * P.chunk_bytes)[i] = __ldg(src + i);
@@ -105,7 +107,7 @@ __global__ void __launch_bounds__(kPoolThreads) maxpool_stream_kernel(const Pool
     ok = mbar_wait(smem_u32(&full[b]), ph, &abort_flag, &g_status_pool);
     if (__syncthreads_or(!ok)) break;
     --pending;
-    const long long p0 = c * P.per_chunk;
+    const long long p0 = place(c) * P.per_chunk;
     const uint32_t count = (uint32_t)min((long long)P.per_chunk, P.planes - p0) * (uint32_t)HoWo;
     const float *chunk = reinterpret_cast<const float *>(smem + (size_t)b * P.chunk_bytes);
     float *out = P.out + (size_t)p0 * HoWo;
@@ -184,8 +186,8 @@ cudaError_t launch_maxpool2d(const float *x, int N, int C, int H, int W, int k, 
   };
   const Magic dh = magic((uint32_t)(Ho * Wo)), dw = magic((uint32_t)Wo);
   // Streamed when chunks of at least four planes and at most 24 KB exist, enough of them for several
-  // rounds of every block (two blocks per SM, four chunks each).  AlexNet's 3x3/2 pool of conv2's
-  // output (235 MB): 92 us with a thread per output, bounded by its nine global loads, 57 us streamed (4.1 TB/s).
+  // rounds of every block (as many blocks per SM as fit, four chunks each).  AlexNet's 3x3/2 pool of conv2's
+  // output (235 MB): 92 us with a thread per output, bounded by its nine global loads, 47 us streamed (5 TB/s).
   const size_t four = 16 * (size_t)H * W;
   if (four <= 24 * 1024) {
     PoolParams P;
@@ -196,8 +198,9 @@ cudaError_t launch_maxpool2d(const float *x, int N, int C, int H, int W, int k, 
     P.chunk_bytes = (uint32_t)(((size_t)P.per_chunk * H * W * 4 + 127) / 128 * 128);
     const long long nchunks = (P.planes + P.per_chunk - 1) / P.per_chunk;
     if (nchunks >= 4ll * sms) {
-      const unsigned grid = (unsigned)std::min<long long>(nchunks, 2ll * sms);
       const size_t smem = (size_t)kBufs * P.chunk_bytes;
+      const long long per_sm = std::min<long long>(6, (long long)(227 * 1024 / (smem + 2048)));
+      const unsigned grid = (unsigned)std::min<long long>(nchunks, per_sm * sms);
       // windows that never leave the plane: no clipping
       const bool inside = pad == 0;
       if (inside && k == 3) return relu ? launch_stream<true, 3>(P, grid, smem, st) : launch_stream<false, 3>(P, grid, smem, st);
