@@ -1,0 +1,89 @@
+"""GPU parity of kernels that a size selects and the other files' shapes do not reach: the streamed
+pooling, every tile of the projection shortcut, the pipelined k-bit pack kernel with each number of
+planes, the box filter with four outputs per thread.  Edges of tiles, remainders, ragged tensors."""
+import numpy as np
+import pytest
+import torch
+
+import paper_1603_05279_b200 as X
+from test_gpu_options import _index_of_planes
+from util import GuardSet, assert_close, dev, host
+
+pytestmark = pytest.mark.gpu
+
+
+def rng(seed):
+    return np.random.Generator(np.random.Philox(seed))
+
+
+# (N, C, H, W, k, stride, pad): a last chunk of one plane and a tensor that is not a multiple of four
+# floats; several planes per chunk; clipped windows; the largest planes that are streamed
+@pytest.mark.parametrize("relu", [False, True])
+@pytest.mark.parametrize("case", [(197, 193, 9, 7, 2, 2, 0), (150, 256, 13, 13, 3, 2, 0),
+                                  (10, 256, 27, 27, 3, 2, 1), (3, 805, 38, 40, 5, 3, 2)])
+def test_streamed_maxpool_is_exact(oracle, case, relu):
+    N, C, H, W, k, s, p = case
+    x = rng(sum(case)).standard_normal((N, C, H, W)).astype(np.float32)
+    want = oracle.maxpool2d(x, k, s, p, relu=relu)
+    gs = GuardSet()
+    out = gs.new("out", want.shape)
+    X.xnor_maxpool2d(dev(x), k, s, p, relu, out)
+    X.xnor_check_device()
+    gs.check()
+    assert np.array_equal(host(out), want)
+
+
+# large, middle and small tiles; channel, filter and pixel tails; planes of odd size
+@pytest.mark.parametrize("case", [(64, 64, 28, 28, 130, 1), (40, 70, 57, 55, 96, 2), (16, 128, 28, 28, 256, 2),
+                                  (5, 70, 15, 13, 90, 1), (2, 256, 14, 14, 512, 2), (1, 33, 9, 9, 40, 2)])
+def test_shortcut_tiles(oracle, case):
+    N, C, H, W, Co, s = case
+    g = rng(sum(case))
+    x = g.standard_normal((N, C, H, W)).astype(np.float32)
+    w = (0.05 * g.standard_normal((Co, C))).astype(np.float32)
+    gs = GuardSet()
+    out = gs.new("out", (N, Co, (H - 1) // s + 1, (W - 1) // s + 1))
+    X.xnor_shortcut_conv1x1(dev(x), dev(w), s, out)
+    gs.check()
+    assert_close(host(out), oracle.shortcut_conv1x1(x, w.reshape(Co, C, 1, 1), s), "shortcut")
+
+
+# one warp per pixel group and groups shared by warps; channel tails; 16- and 4-byte copies
+@pytest.mark.parametrize("kbits", [2, 3, 7])
+@pytest.mark.parametrize("case", [(90, 40, 28, 28, 3, 1), (2, 300, 10, 14, 5, 2), (3, 70, 9, 11, 3, 1)])
+def test_kbit_pack(oracle, case, kbits):
+    N, C, H, W, k, p = case
+    g = rng(sum(case) + kbits)
+    x = (0.6 * g.standard_normal((N, C, H, W))).astype(np.float32)
+    scale = (1.0 + 0.2 * g.standard_normal(C)).astype(np.float32)
+    shift = (0.2 * g.standard_normal(C)).astype(np.float32)
+    d = X.make_desc(N, C, H, W, 8, k, k, 1, p)
+    gs = GuardSet()
+    planes = gs.new("x_planes", (kbits, N, H, W, (C + 31) // 32), torch.int32)
+    _, A0, K0 = X.alloc_binactiv(d)
+    A, K = gs.like("A", A0), gs.like("K", K0)
+    X.xnor_binactiv_kbit(dev(x), dev(scale), dev(shift), d, kbits, planes, A, K)
+    gs.check()
+    y = oracle.bn_affine(x, scale, shift)
+    codes = 2 * _index_of_planes(host(planes), C) - (2 ** kbits - 1)
+    assert np.array_equal(codes, oracle.quantize_k(y, kbits).astype(np.int64))
+    A_or = oracle.channel_abs_mean(y)
+    assert_close(host(A), A_or, "A")
+    assert_close(host(K), oracle.box_filter(A_or, k, k, 1, p), "K")
+
+
+@pytest.mark.parametrize("valid", [False, True])
+@pytest.mark.parametrize("case", [(190, 2, 56, 56, 3, 1), (260, 2, 55, 44, 5, 2), (230, 1, 51, 48, 5, 0),
+                                  (330, 1, 37, 50, 3, 0)])
+def test_box_filter_rows(oracle, case, valid):
+    N, C, H, W, k, p = case
+    x = rng(sum(case)).standard_normal((N, C, H, W)).astype(np.float32)
+    d = X.make_desc(N, C, H, W, 8, k, k, 1, p, X.XNOR_FLAG_K_VALID_TAPS if valid else 0)
+    gs = GuardSet()
+    xp, A, K = (gs.like(n, t) for n, t in zip(("x_packed", "A", "K"), X.alloc_binactiv(d)))
+    X.xnor_binactiv(dev(x), None, None, d, xp, A, K)
+    gs.check()
+    A_or = oracle.channel_abs_mean(x)
+    assert_close(host(A), A_or, "A")
+    want = oracle.box_filter_valid_taps(A_or, k, k, 1, p) if valid else oracle.box_filter(A_or, k, k, 1, p)
+    assert_close(host(K), want, "K")
