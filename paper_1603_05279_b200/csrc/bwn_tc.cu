@@ -3,26 +3,28 @@
 //
 // The inputs are rounded once to bfloat16 and laid out as the "pixel stream" the XNOR kernel
 // uses (every input row preceded by lead zero pixels, every image by lead zero rows, one
-// stream per stride phase), but materialised in memory with the padding written as zeros:
-//   x_stream  bf16 [phases][L][Cp],  L = N*Hq*Wq stream positions, Cp = C rounded up to 32.
+// stream per stride phase), but materialised in memory with the padding written as zeros, one plane
+// per eight channels:
+//   x_stream  bf16 [phases][Cp / 8][L][8],  L = N*Hq*Wq stream positions, Cp = C rounded up to 32;
+// plane 4 w + q holds channels 32 w + 4 q + i and 32 w + 16 + 4 q + i (i = 0..3) at elements 2 i and
+// 2 i + 1 (the order in which a packed word of filter signs expands with two operations per register).
 // With GEMM row m = stream position of an output pixel, tap (ky,kx) reads position
 // m + shift(ky,kx) of one phase: a CTA fetches the ppix = 128 + halo positions a tile touches
-// ONCE, with one TMA tile copy per phase and group of 8 channels (box = 8 channels x ppix
-// positions): shared memory then holds [channel group][position][16 bytes], the no-swizzle
-// K-major operand layout, and every tap's A operand is that patch at a shifted start address.
-// Positions beyond the tensor read as zeros (TMA bounds fill).
+// ONCE, one contiguous bulk copy per plane: shared memory then holds [plane][position][16 bytes], the
+// no-swizzle K-major operand layout, and every tap's A operand is that patch at a shifted start address.
+// (With the channels innermost in memory a patch came in as 16-byte pieces of a tiled tensor copy.)
 //
 // B operand: the packed sign words of a slab of NT filters, expanded by producer warps into
 // +-1 bfloat16 rows in a ring of stages (one K-step of 16 channels = two 16-byte pieces of a
 // filter row).  tcgen05.mma kind::f16 (bf16 x bf16, fp32 accumulation in tensor memory): every
 // product is +-x exactly; only the fp32 accumulation rounds.
 //
-// Roles (576 threads, persistent, one CTA per SM, items = (pixel tile, filter slab) in tile-major
+// Roles (832 threads, persistent, one CTA per SM, items = (pixel tiles, filter slab) in tile-major
 // order, a contiguous range per CTA): warps 0-7 epilogue (D * alpha (+ residual) -> NCHW; two
 // warps per quarter of the lanes, taking alternate groups of 16 columns), warp 8 issues the MMAs,
-// warp 9 issues the TMA copies, warps 10-17 expand weights.  Every wait is
-// bounded; on expiry the CTA records XNOR_ERR_TIMEOUT, stops, and frees its tensor memory.
-#include <cuda.h>
+// warp 9 issues the bulk copies, warps 10-25 expand weights (two groups of eight, alternate stages).
+// Every wait is bounded; on expiry the CTA records XNOR_ERR_TIMEOUT, stops, and frees its tensor memory.
+#include <cuda_bf16.h>
 
 #include <algorithm>
 
@@ -40,8 +42,8 @@ using namespace umma;
 constexpr int kEpiWarps = 8;          // two per quarter of the tensor-memory lanes
 constexpr int kMmaWarp = 8;
 constexpr int kTmaWarp = 9;
-constexpr int kWgtWarp0 = 10, kWgtWarps = 8;
-constexpr int kThreads = 32 * (kWgtWarp0 + kWgtWarps);   // 576: 18 warps, 112 registers each
+constexpr int kWgtWarp0 = 10, kWgtGroups = 2, kWgtWarps = 8;     // groups of eight warps
+constexpr int kThreads = 32 * (kWgtWarp0 + kWgtGroups * kWgtWarps);   // 832: 26 warps, 72 registers each
 constexpr int kTileM = 128;
 constexpr int kTmemCols = 512;
 constexpr int kMaxAcc = 4;
@@ -51,21 +53,21 @@ constexpr int kMaxTaps = 121;
 constexpr size_t kCtrlBytes = 1024;
 constexpr size_t kSmemMax = 232448 - 1024;
 
-struct alignas(64) BwnParams {
-  CUtensorMap tmap;            // x_stream as {8 channels, Cp/8 groups, L positions, phases}
+struct BwnParams {
+  const uint8_t *xs;           // x_stream
   const uint32_t *wp;
   const float *alpha, *residual;
   float *out;
   int N, C, H, W, Co, kh, kw, stride, pad, Ho, Wo, Cw;
-  int Cp, cpt;                 // channels padded to 32; K-steps per tap = Cp / 16 (even)
+  int Cp;                      // channels padded to 32
   int Hq, Wq, leadY, leadX;
   long long L;
-  int ntiles, nslabs, NT, nacc, ppix, npb, stages, mps, nsteps, ntaps, phases;
+  int ntiles, nslabs, NT, nacc, ppix, npb, stages, ntaps, phases;
+  int nwords, wps;             // packed words per filter row; words per weight stage
   int tpi;                     // pixel tiles per work item (1 or 2): every weight stage then serves
                                // tpi MMAs, so the filter rows are expanded once per tpi * 128 pixels;
                                // ntiles counts items' worth of tiles (groups of tpi stream tiles)
-  int nload, box_pos;          // TMA copies per operand plane of a patch and their extent in positions
-  int rows_mod, grp_steps;
+  int rows_mod;
   uint32_t plane_bytes, phase_bytes, patch_bytes, stage_bytes;
   uint32_t off_vec, off_ring, off_patch;
   int vec_len;
@@ -108,17 +110,6 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint32_t a_lo, uint32
 __device__ __forceinline__ void commit_one(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                ::"r"(bar) : "memory");
-}
-
-// TMA tile copy global -> shared of one operand plane of a patch: box {8, 1, ppix, 1} at
-// coordinates {0, group, pos, phase}; its bytes complete on `bar`.  The innermost coordinate
-// is 0, so the copy starts on a 16-byte boundary whatever `pos` is.
-__device__ __forceinline__ void tma_load_plane(uint32_t dst, const CUtensorMap *tmap, int group,
-                                               int pos, int phase, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
-      "[%0], [%1, {%2, %3, %4, %5}], [%6];"
-      ::"r"(dst), "l"(tmap), "r"(0), "r"(group), "r"(pos), "r"(phase), "r"(bar) : "memory");
 }
 
 __device__ __forceinline__ float4 lds_f4(uint32_t addr) {
@@ -164,12 +155,12 @@ __device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatil
 // ------------------------------------------------------------------ MMA issuer (one thread)
 __device__ void mma_loop(const BwnParams &P, const Smem &S, long long i0, long long i1,
                          uint32_t tmem_base) {
-  const int nst = (P.nsteps + P.mps - 1) / P.mps;
+  const int nst = (P.nwords + P.wps - 1) / P.wps;
   const uint32_t b_lbo = (uint32_t)P.NT * 16u;
   const uint32_t desc_hi = (128u >> 4) | (1u << 14);      // 128 B between 8-row groups; version
   const uint32_t a_lbo_hi = (P.plane_bytes >> 4) << 16;    // the K-step's second piece: next plane
   const uint32_t b_lo0 = ((S.ring & 0x3FFFFu) >> 4) | ((b_lbo >> 4) << 16);
-  const uint32_t b_step = (2u * b_lbo) >> 4;
+  const uint32_t b_step = (2u * b_lbo) >> 4;               // next K-step
   const uint32_t a_step = (2u * P.plane_bytes) >> 4;       // next 16 channels of the same tap
   const uint32_t stage_step = P.stage_bytes >> 4;
   int ws = 0, pb = 0, ab = 0;
@@ -188,24 +179,26 @@ __device__ void mma_loop(const BwnParams &P, const Smem &S, long long i0, long l
     if (!ok) break;
     tc_fence_after();
     const uint32_t d_tmem = tmem_base + (uint32_t)(ab * P.tpi * P.NT);
-    int tap = 0, c16 = 0;                    // K-step j = tap * cpt + c16
+    int tap = 0, cw = 0;                     // word f = tap * Cw + cw: two K-steps
+    uint32_t acc = 0u;
     for (int st = 0; st < nst && ok; ++st) {
-      const int j0 = st * P.mps;
-      const int nj = min(P.mps, P.nsteps - j0);
       ok = mbar_wait(S.wfull + 8u * ws, wph, S.abort_flag, &g_status_bwn);
       if (!ok) break;
-      tc_fence_after();
-      const uint32_t b_lo = b_lo0 + (uint32_t)ws * stage_step;
-      for (int jj = 0; jj < nj; ++jj) {
-        const uint32_t a_lo = ((patch_lo + P.tap_lo[tap] + (uint32_t)c16 * a_step) & 0x3FFFu) | a_lbo_hi;
-        umma_bf16(d_tmem, a_lo, desc_hi, b_lo + (uint32_t)jj * b_step, desc_hi, P.idesc,
-                  (j0 + jj) == 0 ? 0u : 1u);
-        // the item's second pixel tile: the same patch 128 positions (128 x 16 bytes) further,
-        // the same filter rows, the next accumulator
+      uint32_t b_lo = b_lo0 + (uint32_t)ws * stage_step;
+      const int nw = min(P.wps, P.nwords - st * P.wps);
+#pragma unroll 1
+      for (int i = 0; i < nw; ++i) {
+        const uint32_t a = ((patch_lo + P.tap_lo[tap] + (uint32_t)cw * (2u * a_step)) & 0x3FFFu) | a_lbo_hi;
+        umma_bf16(d_tmem, a, desc_hi, b_lo, desc_hi, P.idesc, acc);
+        // the item's second pixel tile: the same patch 128 positions (128 x 16 bytes) further, the
+        // same filter rows, the next accumulator
+        if (P.tpi == 2) umma_bf16(d_tmem + (uint32_t)P.NT, a + (uint32_t)kTileM, desc_hi, b_lo, desc_hi, P.idesc, acc);
+        umma_bf16(d_tmem, a + a_step, desc_hi, b_lo + b_step, desc_hi, P.idesc, 1u);
         if (P.tpi == 2)
-          umma_bf16(d_tmem + (uint32_t)P.NT, a_lo + (uint32_t)kTileM, desc_hi,
-                    b_lo + (uint32_t)jj * b_step, desc_hi, P.idesc, (j0 + jj) == 0 ? 0u : 1u);
-        if (++c16 == P.cpt) { c16 = 0; ++tap; }
+          umma_bf16(d_tmem + (uint32_t)P.NT, a + a_step + (uint32_t)kTileM, desc_hi, b_lo + b_step, desc_hi, P.idesc, 1u);
+        acc = 1u;
+        b_lo += 2u * b_step;
+        if (++cw == P.Cw) { cw = 0; ++tap; }
       }
       commit_one(S.wempty + 8u * ws);
       if (++ws == P.stages) { ws = 0; wph ^= 1u; }
@@ -226,29 +219,34 @@ __device__ __forceinline__ void mma_role(const BwnParams &P, const Smem &S, long
   __syncwarp();
 }
 
-// ------------------------------------------------------------------ TMA producer (one warp)
+// ------------------------------------------------------------------ patch producer (one warp)
 __device__ void tma_role(const BwnParams &P, const Smem &S, long long i0, long long i1, int lane) {
   const int tile0 = (int)(i0 / P.nslabs);
   const uint32_t npatches = (uint32_t)((i1 - 1) / P.nslabs) - (uint32_t)tile0 + 1u;
+  const int nplanes = P.phases * (P.Cp / 8);
   bool ok = true;
   uint32_t started = 0;
   for (uint32_t seq = 0; seq < npatches && ok; ++seq) {
     const uint32_t pb = seq % (uint32_t)P.npb, use = seq / (uint32_t)P.npb;
     ok = wait_warp(S.pempty + 8u * pb, (use & 1u) ^ 1u, S.abort_flag);
     if (!ok) break;
-    if (lane == 0) {
-      const uint32_t bar = S.pfull + 8u * pb;
-      const uint32_t dst = S.patch + pb * P.patch_bytes;
-      mbar_arrive_expect_tx(bar, P.patch_bytes);
-      const int pos = (tile0 + (int)seq) * P.tpi * kTileM;
-      const int ngroups = P.Cp / 8;
-      for (int ph = 0; ph < P.phases; ++ph)
-        for (int g8 = 0; g8 < ngroups; ++g8)
-          for (int ld = 0; ld < P.nload; ++ld)
-            tma_load_plane(dst + (uint32_t)ph * P.phase_bytes + (uint32_t)g8 * P.plane_bytes +
-                               (uint32_t)(ld * P.box_pos) * 16u,
-                           &P.tmap, g8, pos + ld * P.box_pos, ph, bar);
+    // positions of the patch inside the stream; those beyond it are the padding below and right of the
+    // last image: zeros
+    const long long pos = (long long)(tile0 + (int)seq) * P.tpi * kTileM;
+    const uint32_t bytes = (uint32_t)min((long long)P.ppix, P.L - pos) * 16u;
+    const uint32_t bar = S.pfull + 8u * pb, dst = S.patch + pb * P.patch_bytes;
+    if (bytes < P.plane_bytes) {
+      for (int pl = 0; pl < nplanes; ++pl)
+        for (uint32_t b = bytes + (uint32_t)lane * 16u; b < P.plane_bytes; b += 512u)
+          sts128(dst + (uint32_t)pl * P.plane_bytes + b, 0u, 0u, 0u, 0u);
+      fence_proxy_async();
+      __syncwarp();
     }
+    if (lane == 0) mbar_arrive_expect_tx(bar, bytes * (uint32_t)nplanes);
+    __syncwarp();
+    for (int pl = lane; pl < nplanes; pl += 32)
+      bulk_copy_g2s(dst + (uint32_t)pl * P.plane_bytes, P.xs + ((size_t)pl * (size_t)P.L + (size_t)pos) * 16u, bytes, bar);
+    __syncwarp();
     started = seq + 1u;
   }
   if (!ok && started > 0u) {
@@ -261,87 +259,65 @@ __device__ void tma_role(const BwnParams &P, const Smem &S, long long i0, long l
   }
 }
 
-// ------------------------------------------------------------------ weight producers (8 warps)
-// Byte kByte of a packed word (eight sign bits, a set bit is +1) -> eight bfloat16 values +-1
-// (0x3F80 / 0xBF80), channel 2i in the low half of register i.  `inv` is the complemented word:
-// its bit is the sign bit of the value.  Four operations per register, all shifts constant.
-template <int kByte>
-__device__ __forceinline__ void expand_byte(uint32_t inv, uint32_t v[4]) {
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    constexpr int base = 8 * kByte;
-    const int p = base + 2 * i;                         // bit of the low value; p + 1 of the high one
-    const uint32_t lo = p <= 15 ? (inv << (15 - p)) : (inv >> (p - 15));
-    const uint32_t hi = inv << (30 - p);
-    v[i] = 0x3F803F80u | (lo & 0x8000u) | (hi & 0x80000000u);
-  }
+// ------------------------------------------------------------------ weight producers (16 warps)
+// A packed word (32 sign bits, a set bit is +1) -> 16 registers of two bfloat16 +-1 (0x3F80 / 0xBF80):
+// register r holds channel r in its low half and channel r + 16 in its high one, so that a shift brings
+// both signs to their places: two operations per register.  `inv` is the complemented word.
+__device__ __forceinline__ uint32_t expand_pair(uint32_t inv, int r) {
+  return ((r <= 15 ? inv << (15 - r) : inv) & 0x80008000u) | 0x3F803F80u;
 }
 
-// A stage holds mps K-steps (mps / 2 packed words) of NT filter rows: piece (2 jj + half) of
-// NT x 16 bytes.  K-step j is bits 16 (j & 1) .. + 15 of packed word j >> 1 of the filter (the
-// channels are padded to whole words), so a word expands to four consecutive pieces.  Thread
-// mapping: row = wt % rows_mod, the 256 / rows_mod groups split the words of a stage (at most
-// two words per thread and stage).  The words of the NEXT stage are fetched before the current
-// one is expanded: the filters are re-read (from L2) for every work item.
-__device__ void weight_role(const BwnParams &P, const Smem &S, long long i0, long long i1, int wt,
-                            int lane) {
-  constexpr int kMaxWords = 2;
-  const int nst = (P.nsteps + P.mps - 1) / P.mps;
-  const int wps = P.mps >> 1, nwords = P.nsteps >> 1;   // words per stage, per filter row
-  const int row = wt % P.rows_mod, grp = wt / P.rows_mod;
-  const int wpt = P.grp_steps;                          // words per thread and stage (1 or 2)
-  const bool grp_on = grp * wpt < wps && row < P.NT;
+// A stage holds wps packed words of NT filter rows: word i in pieces 4 i .. 4 i + 3 of NT x 16 bytes (two
+// K-steps).  Two groups of eight warps take alternate stages of the sequence over all items; a thread
+// expands one word of one row per stage.  Its words of the next two stages are fetched ahead: the
+// filters are re-read (from L2) for every work item.
+__device__ void weight_role(const BwnParams &P, const Smem &S, long long i0, long long i1, int wt, int lane) {
+  const int nst = (P.nwords + P.wps - 1) / P.wps;
+  const int group = wt / (32 * kWgtWarps), t = wt - group * (32 * kWgtWarps);
+  const int row = t % P.rows_mod, wl = t / P.rows_mod;  // row of the slab, word of the stage
   const uint32_t b_lbo = (uint32_t)P.NT * 16u;
-  auto fetch = [&](int st, int co, uint32_t w[kMaxWords]) {
-#pragma unroll
-    for (int u = 0; u < kMaxWords; ++u) {
-      const int wl = grp * wpt + u, f = st * wps + wl;
-      w[u] = 0u;
-      if (grp_on && u < wpt && wl < wps && f < nwords && co < P.Co)
-        w[u] = __ldg(P.wp + packed_weight_index(P.Co, co, f));
+  const bool on = row < P.NT && wl < P.wps;
+  struct Cursor { long long it; int st, slab; };
+  auto advance = [&](Cursor &c, int by) {
+    c.st += by;
+    while (c.st >= nst) {
+      c.st -= nst;
+      ++c.it;
+      if (++c.slab == P.nslabs) c.slab = 0;
     }
   };
-  int ws = 0;
-  uint32_t wph = 1u;
-  bool ok = true;
-  int slab = (int)(i0 % P.nslabs);
-  uint32_t cur[kMaxWords], nxt[kMaxWords];
-  fetch(0, slab * P.NT + row, cur);
-  for (long long it = i0; it < i1 && ok; ++it) {
-    int nslab = slab + 1;
-    if (nslab == P.nslabs) nslab = 0;
-    for (int st = 0; st < nst && ok; ++st) {
-      // the stage after this one: the next of this item, or the first of the next item
+  auto fetch = [&](const Cursor &c) {
+    const int f = c.st * P.wps + wl, co = c.slab * P.NT + row;
+    return on && c.it < i1 && f < P.nwords && co < P.Co ? __ldg(P.wp + packed_weight_index(P.Co, co, f)) : 0u;
+  };
+  Cursor c{i0, 0, (int)(i0 % P.nslabs)};
+  advance(c, group);
+  Cursor ahead = c;
+  uint32_t cur = fetch(ahead);
+  advance(ahead, kWgtGroups);
+  uint32_t nxt = fetch(ahead);
+  uint32_t ws = (uint32_t)group, wph = 1u;             // stages >= groups (host)
+  const uint32_t off = (uint32_t)row * 16u + (uint32_t)(4 * wl) * b_lbo;
+#pragma unroll 1
+  while (c.it < i1) {
+    advance(ahead, kWgtGroups);
+    const uint32_t nxt2 = fetch(ahead);
+    if (!mbar_wait_relaxed(S.wempty + 8u * ws, wph, S.abort_flag, &g_status_bwn, 50)) return;
+    if (on) {
+      const uint32_t inv = ~cur, a = S.ring + ws * P.stage_bytes + off;
 #pragma unroll
-      for (int u = 0; u < kMaxWords; ++u) nxt[u] = 0u;
-      if (st + 1 < nst) fetch(st + 1, slab * P.NT + row, nxt);
-      else if (it + 1 < i1) fetch(0, nslab * P.NT + row, nxt);
-      ok = mbar_wait_relaxed(S.wempty + 8u * ws, wph, S.abort_flag, &g_status_bwn, 50);
-      if (!ok) break;
-      if (grp_on) {
-        const uint32_t stage = S.ring + (uint32_t)ws * P.stage_bytes + (uint32_t)row * 16u;
-#pragma unroll
-        for (int u = 0; u < kMaxWords; ++u) {
-          const int wl = grp * wpt + u;
-          if (u < wpt && wl < wps && st * wps + wl < nwords) {
-            const uint32_t inv = ~cur[u];
-            const uint32_t a = stage + (uint32_t)(4 * wl) * b_lbo;       // pieces 4 wl .. 4 wl + 3
-            uint32_t v[4];
-            expand_byte<0>(inv, v); sts128(a, v[0], v[1], v[2], v[3]);
-            expand_byte<1>(inv, v); sts128(a + b_lbo, v[0], v[1], v[2], v[3]);
-            expand_byte<2>(inv, v); sts128(a + 2u * b_lbo, v[0], v[1], v[2], v[3]);
-            expand_byte<3>(inv, v); sts128(a + 3u * b_lbo, v[0], v[1], v[2], v[3]);
-          }
-        }
-      }
-      fence_proxy_async();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(S.wfull + 8u * ws);
-      if (++ws == P.stages) { ws = 0; wph ^= 1u; }
-#pragma unroll
-      for (int u = 0; u < kMaxWords; ++u) cur[u] = nxt[u];
+      for (int q = 0; q < 4; ++q)
+        sts128(a + (uint32_t)q * b_lbo, expand_pair(inv, 4 * q), expand_pair(inv, 4 * q + 1), expand_pair(inv, 4 * q + 2),
+               expand_pair(inv, 4 * q + 3));
     }
-    slab = nslab;
+    fence_proxy_async();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(S.wfull + 8u * ws);
+    ws += kWgtGroups;
+    if (ws >= (uint32_t)P.stages) { ws -= (uint32_t)P.stages; wph ^= 1u; }
+    advance(c, kWgtGroups);
+    cur = nxt;
+    nxt = nxt2;
   }
 }
 
@@ -391,17 +367,14 @@ __device__ void epilogue_role(const BwnParams &P, const Smem &S, long long i0, l
     const Pix px = decode(tile * P.tpi + tt);
     const bool last_tile = tt + 1 == P.tpi;
     const uint32_t t_acc = t_lane + (uint32_t)((ab * P.tpi + tt) * P.NT);
-    int32_t nx[16], cur[16];
-    tmem_ld16(t_acc + (uint32_t)(e * 16), nx);
+    int32_t cur[16];
 #pragma unroll 1
     for (int k = 0; k < nk; ++k) {
       const int b = e + 2 * k;
-      tmem_wait16(nx);
-#pragma unroll
-      for (int j = 0; j < 16; ++j) cur[j] = nx[j];
-      if (k + 1 < nk) {
-        tmem_ld16(t_acc + (uint32_t)((b + 2) * 16), nx);
-      } else if (last_tile) {                    // last load of the item done: release its accumulators
+      __syncwarp();
+      tmem_ld16(t_acc + (uint32_t)(b * 16), cur);
+      tmem_wait16(cur);
+      if (k + 1 == nk && last_tile) {            // last load of the item done: release its accumulators
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(S.aempty + 8u * ab);
@@ -499,80 +472,80 @@ bwn_conv_kernel(const __grid_constant__ BwnParams P) {
 }
 
 // ------------------------------------------------------------------ input preparation
-// fp32 NCHW (after the optional BatchNorm affine) -> bf16 stream [phase][position][Cp], zeros at
-// padding positions and in channels C .. Cp - 1.  A block handles 32 consecutive stream
-// positions of one phase, 64 channels at a time: reads run along the positions (consecutive
-// input pixels, eight loads per thread in flight), writes along the channels (a lane packs two
-// channels, a warp writes the 128 bytes of a position); the transposition goes through shared
-// memory.
-__device__ __forceinline__ uint32_t bf16_rne(float v) {
-  // round to nearest even on the bit pattern (NaN and infinity pass through truncated)
-  uint32_t u = __float_as_uint(v);
-  if ((u & 0x7F800000u) != 0x7F800000u) u += 0x7FFFu + ((u >> 16) & 1u);
-  return u >> 16;
-}
+// fp32 NCHW (after the optional BatchNorm affine) -> the bf16 stream, zeros at padding positions and in
+// channels C .. Cp - 1.  Thread = stream position, kPrepPlanes planes of eight channels: every load of a
+// warp runs along consecutive input pixels, every store is 512 contiguous bytes, nothing is transposed.
+// HBM bounds it.
+constexpr int kPrepPlanes = 4;                // planes per block: one group of 32 channels
 
+template <bool kGrad>
 __global__ void __launch_bounds__(256)
 bwn_prepare_kernel(const float *__restrict__ x, const float *__restrict__ scale,
-                   const float *__restrict__ shift, const float *__restrict__ gmax, int N, int C, int H,
-                   int W, int s, int Hq, int Wq, int leadY, int leadX, long long L, int Cp,
-                   uint16_t *__restrict__ xs) {
-  __shared__ float tile[64][33];
+                   const float *__restrict__ shift, const float *__restrict__ gmax, int C, int H,
+                   int W, int s, int Hq, int Wq, int leadY, int leadX, long long L, int Cp, int ngroups,
+                   uint4 *__restrict__ xs) {
   stream_order();
-  const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;      // 8 warps
-  const long long nblk = (L + 31) / 32;
-  const int phase = (int)(blockIdx.x / nblk);
-  const long long m0 = (long long)(blockIdx.x - phase * nblk) * 32;
+  const int phase = (int)(blockIdx.y / (unsigned)ngroups), grp = (int)blockIdx.y - phase * ngroups;
+  const long long m = (long long)blockIdx.x * 256 + threadIdx.x;
+  if (m >= L) return;
   const int py = phase / s, px = phase - py * s;
-  // this lane's stream position for the reads
-  const long long m = m0 + lane;
-  bool real = m < L;
-  size_t src = 0;
-  float gm = 0.0f;             // gradient mode: the scale of this position's image
-  if (real) {
-    const long long r = m / Wq;
-    const int c = (int)(m - r * Wq);
-    const long long n = r / Hq;
-    if (gmax != nullptr) gm = __ldg(gmax + n);
-    const int ry = (int)(r - n * Hq);
-    const int iy = (ry - leadY) * s + py, ix = (c - leadX) * s + px;
-    real = ry >= leadY && c >= leadX && iy < H && ix < W;
-    src = ((size_t)n * C * H + iy) * W + ix;
-  }
+  const uint32_t mu = (uint32_t)m, r = mu / (uint32_t)Wq, c = mu - r * (uint32_t)Wq, n = r / (uint32_t)Hq;   // L < 2^31
+  const int ry = (int)(r - n * (uint32_t)Hq);
+  const int iy = (ry - leadY) * s + py, ix = ((int)c - leadX) * s + px;
+  const bool real = ry >= leadY && (int)c >= leadX && iy < H && ix < W;
   const size_t plane = (size_t)H * W;
-  uint32_t *dst = reinterpret_cast<uint32_t *>(xs + ((size_t)phase * L + m0) * Cp);   // Cp is even
-  for (int c0 = 0; c0 < Cp; c0 += 64) {
-    // warp wy reads channels c0 + wy, + 8, ..., + 56 of the 32 positions
-    float v[8];
+  const int c0 = grp * 32;
+  const float *src = x + ((size_t)n * C + c0) * plane + (size_t)iy * W + ix;
+  const float gm = kGrad && real ? __ldg(gmax + n) : 0.0f;    // the scale of this position's image
+  uint4 *dst = xs + ((size_t)(phase * (Cp / 8) + grp * kPrepPlanes) * (size_t)L + (size_t)m);
+  const bool whole = c0 + 32 <= C;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int ch = c0 + wy + 8 * q;
-      v[q] = (real && ch < C) ? __ldg(x + src + (size_t)ch * plane) : 0.0f;
+  for (int q = 0; q < kPrepPlanes; ++q) {
+    float v[8];                               // channels c0 + 4 q + i, then c0 + 16 + 4 q + i
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int ch = 4 * q + (j & 3) + 16 * (j >> 2);
+      v[j] = real && (whole || c0 + ch < C) ? __ldg(src + (size_t)ch * plane) : 0.0f;
     }
+    // the factors of the eight channels: four consecutive ones per load
+    float sc[8], sh[8];
+    if (scale != nullptr && whole) {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int ch = c0 + wy + 8 * q;
-      if (gmax != nullptr) {
-        // binarised gradient (Section 3.2, "Binary Gradient"): sign(g) scaled by the image's
-        // max|g| and, here, by the filter's alpha (`scale`), the product formed in fp32
-        if (real && ch < C) v[q] = v[q] >= 0.0f ? __fmul_rn(gm, __ldg(scale + ch)) : -__fmul_rn(gm, __ldg(scale + ch));
-      } else if (scale != nullptr && real && ch < C) {
-        v[q] = __fmaf_rn(__ldg(scale + ch), v[q], __ldg(shift + ch));
+      for (int h = 0; h < 2; ++h) {
+        const float4 a = __ldg(reinterpret_cast<const float4 *>(scale + c0 + 16 * h + 4 * q));
+        sc[4 * h] = a.x; sc[4 * h + 1] = a.y; sc[4 * h + 2] = a.z; sc[4 * h + 3] = a.w;
+        if (!kGrad) {
+          const float4 b = __ldg(reinterpret_cast<const float4 *>(shift + c0 + 16 * h + 4 * q));
+          sh[4 * h] = b.x; sh[4 * h + 1] = b.y; sh[4 * h + 2] = b.z; sh[4 * h + 3] = b.w;
+        }
       }
-      tile[wy + 8 * q][lane] = v[q];
-    }
-    __syncthreads();
-    // warp wy writes positions wy, wy + 8, ...: lane = channels c0 + 2 lane, + 1
-    if (c0 + 2 * lane < Cp) {
+    } else if (scale != nullptr) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int pos = wy + 8 * q;
-        if (m0 + pos < L)
-          dst[((size_t)pos * Cp + c0) / 2 + lane] =
-              bf16_rne(tile[2 * lane][pos]) | (bf16_rne(tile[2 * lane + 1][pos]) << 16);
+      for (int j = 0; j < 8; ++j) {
+        const int ch = c0 + 4 * q + (j & 3) + 16 * (j >> 2);
+        sc[j] = ch < C ? __ldg(scale + ch) : 0.0f;
+        sh[j] = !kGrad && ch < C ? __ldg(shift + ch) : 0.0f;
       }
     }
-    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      if (!real) continue;                    // padding stays zero
+      if (kGrad) {
+        // binarised gradient (Section 3.2, "Binary Gradient"): sign(g) scaled by the image's max|g| and,
+        // here, by the filter's alpha (`scale`), the product formed in fp32
+        const float p = __fmul_rn(gm, sc[j]);
+        v[j] = v[j] >= 0.0f ? p : -p;
+      } else if (scale != nullptr) {
+        v[j] = __fmaf_rn(sc[j], v[j], sh[j]);
+      }
+    }
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const __nv_bfloat162 b = __floats2bfloat162_rn(v[i], v[i + 4]);       // to nearest even
+      w[i] = *reinterpret_cast<const uint32_t *>(&b);
+    }
+    dst[(size_t)q * (size_t)L] = make_uint4(w[0], w[1], w[2], w[3]);
   }
 }
 
@@ -606,28 +579,6 @@ StreamGeom stream_geom(const ConvGeom &g) {
   return q;
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
-                                  const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
-                                  const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// The driver's tensor-map encoder, looked up through the runtime (no link-time dependency on
-// the driver library).
-EncodeTiledFn encode_tiled_fn() {
-  static EncodeTiledFn fn = nullptr;
-  if (fn == nullptr) {
-    void *p = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &qres) != cudaSuccess ||
-        qres != cudaDriverEntryPointSuccess) {
-      (void)cudaGetLastError();
-      return nullptr;
-    }
-    fn = reinterpret_cast<EncodeTiledFn>(p);
-  }
-  return fn;
-}
-
 BwnPlan make_plan(const ConvGeom &g) {
   BwnPlan pl{};
   pl.ok = false;
@@ -636,50 +587,48 @@ BwnPlan make_plan(const ConvGeom &g) {
   const StreamGeom q = stream_geom(g);
   P.N = g.N; P.C = g.C; P.H = g.H; P.W = g.W; P.Co = g.Co; P.kh = g.kh; P.kw = g.kw;
   P.stride = g.stride; P.pad = g.pad; P.Ho = g.Ho; P.Wo = g.Wo; P.Cw = g.Cw;
-  P.Cp = q.Cp; P.cpt = q.Cp / 16;
+  P.Cp = q.Cp;
   P.Hq = q.Hq; P.Wq = q.Wq; P.leadY = q.leadY; P.leadX = q.leadX; P.L = q.L;
   P.phases = q.phases;
   P.ntaps = g.kh * g.kw;
-  P.nsteps = P.ntaps * P.cpt;
+  P.nwords = P.ntaps * g.Cw;
   const int halo = (q.dymax - q.dymin) * q.Wq + (q.dxmax - q.dxmin);
-  if ((kTileM + halo + 7) / 8 * 8 > 256) return pl;        // a tile's window: at most one TMA box
+  if ((kTileM + halo + 7) / 8 * 8 > 256) return pl;
   if (q.L + 4 * kTileM + 256 >= (1ll << 31)) return pl;
   // filter slabs: as few as fit two accumulators into the tensor-memory columns
   const int max_nt = 128;
   P.nslabs = (g.Co + max_nt - 1) / max_nt;
   P.NT = ((g.Co + P.nslabs - 1) / P.nslabs + 15) / 16 * 16;
-  // weight stages: rows_mod threads cover the rows, the other groups split a stage's K-steps
+  // weight stages: rows_mod threads of a group of warps cover the rows of a word
   int ntp = 16;
   while (ntp < P.NT) ntp *= 2;
   P.rows_mod = ntp;
-  const int groups = std::max(1, 32 * kWgtWarps / ntp);    // >= 2: slabs hold at most 128 filters
-  P.mps = 8;                                               // K-steps per stage = 4 packed words per row
-  P.grp_steps = std::max(1, (P.mps / 2) / groups);         // words per thread and stage: 2 or 1
-  P.stage_bytes = (uint32_t)P.mps * (uint32_t)P.NT * 32u;
+  P.wps = std::min(4, 32 * kWgtWarps / ntp);               // a word per thread: 2 (128 filters) or 4
+  P.stage_bytes = (uint32_t)P.wps * (uint32_t)P.NT * 64u;
   P.off_vec = (uint32_t)((kCtrlBytes + 127) / 128 * 128);
   P.vec_len = (g.Co + 15) / 16 * 16 + 256;
   P.off_ring = (uint32_t)((P.off_vec + (size_t)P.vec_len * 4 + 127) / 128 * 128);
   // Two pixel tiles per work item when their common window (256 + halo positions) fits beside two
   // weight stages: the expansion of the filter rows, which bounds the kernel, is then shared by
-  // two MMAs.  The window is fetched with one or two TMA copies per operand plane (box <= 256).
+  // two MMAs.
   const int stream_tiles = (int)((q.L + kTileM - 1) / kTileM);
   for (P.tpi = (kTmemCols / P.NT >= 2 && stream_tiles >= 2) ? 2 : 1; P.tpi >= 1; --P.tpi) {
     P.ppix = (P.tpi * kTileM + halo + 7) / 8 * 8;
-    P.nload = P.ppix > 256 ? 2 : 1;
-    if (P.nload == 2) P.ppix = (P.ppix + 15) / 16 * 16;   // two boxes of a multiple of 8 positions
-    P.box_pos = P.ppix / P.nload;
     P.plane_bytes = (uint32_t)P.ppix * 16u;
     P.phase_bytes = P.plane_bytes * (uint32_t)(P.Cp / 8);
     P.patch_bytes = P.phase_bytes * (uint32_t)P.phases;
-    if (P.off_ring + 2 * (size_t)P.stage_bytes + P.patch_bytes <= kSmemMax) break;
+    if (P.off_ring + (P.tpi == 2 ? 4 : 2) * (size_t)P.stage_bytes + P.patch_bytes <= kSmemMax) break;
   }
   if (P.tpi < 1) return pl;
   P.ntiles = (stream_tiles + P.tpi - 1) / P.tpi;
   P.nacc = std::max(1, std::min(kMaxAcc, kTmemCols / (P.NT * P.tpi)));
   const size_t avail = kSmemMax - P.off_ring;
-  int stages = 2, npb = 1;
   auto fits = [&](int st, int pb) { return (size_t)st * P.stage_bytes + (size_t)pb * P.patch_bytes <= avail; };
-  while (stages < 4 && fits(stages + 1, npb)) ++stages;
+  // a second patch buffer hides the patch copies behind the MMAs and comes before more than three stages
+  // (each group of weight warps needs one)
+  int stages = 2, npb = 1;
+  if (!fits(stages, npb)) return pl;
+  while (stages < 3 && fits(stages + 1, npb)) ++stages;
   while (npb < 2 && fits(stages, npb + 1)) ++npb;
   while (stages < kMaxStages && fits(stages + 1, npb)) ++stages;
   while (npb < kMaxPatchBufs && fits(stages, npb + 1)) ++npb;
@@ -721,22 +670,29 @@ size_t bwn_stream_elems(const ConvGeom &g) {
   return (size_t)q.phases * (size_t)q.L * (size_t)q.Cp;
 }
 
+namespace {
+
+template <bool kGrad>
+cudaError_t launch_prepare(const float *x, const float *scale, const float *shift, const float *gmax, const ConvGeom &g,
+                           uint16_t *x_stream, cudaStream_t st) {
+  const StreamGeom q = stream_geom(g);
+  const int ngroups = q.Cp / 32;
+  if (q.L >= (1ll << 31) || (long long)ngroups * q.phases > 65535) return cudaErrorInvalidValue;
+  const dim3 grid((unsigned)((q.L + 255) / 256), (unsigned)(ngroups * q.phases));
+  return launch_kernel(bwn_prepare_kernel<kGrad>, grid, 256, 0, st, 1, x, scale, shift, gmax, g.C, g.H, g.W, q.s, q.Hq, q.Wq,
+                       q.leadY, q.leadX, q.L, q.Cp, ngroups, reinterpret_cast<uint4 *>(x_stream));
+}
+
+}  // namespace
+
 cudaError_t launch_bwn_prepare(const float *x, const float *scale, const float *shift,
                                const ConvGeom &g, uint16_t *x_stream, cudaStream_t st) {
-  const StreamGeom q = stream_geom(g);
-  const long long nblk = (q.L + 31) / 32 * q.phases;
-  if (nblk >= (1ll << 31)) return cudaErrorInvalidValue;
-  return launch_kernel(bwn_prepare_kernel, dim3((unsigned)nblk), 256, 0, st, 1, x, scale, shift, nullptr, g.N, g.C, g.H, g.W,
-                       q.s, q.Hq, q.Wq, q.leadY, q.leadX, q.L, q.Cp, x_stream);
+  return launch_prepare<false>(x, scale, shift, nullptr, g, x_stream, st);
 }
 
 cudaError_t launch_bwn_prepare_grad(const float *g, const float *alpha, const float *gmax,
                                     const ConvGeom &gb, uint16_t *g_stream, cudaStream_t st) {
-  const StreamGeom q = stream_geom(gb);
-  const long long nblk = (q.L + 31) / 32 * q.phases;
-  if (nblk >= (1ll << 31)) return cudaErrorInvalidValue;
-  return launch_kernel(bwn_prepare_kernel, dim3((unsigned)nblk), 256, 0, st, 1, g, alpha, nullptr, gmax, gb.N, gb.C, gb.H, gb.W,
-                       q.s, q.Hq, q.Wq, q.leadY, q.leadX, q.L, q.Cp, g_stream);
+  return launch_prepare<true>(g, alpha, nullptr, gmax, gb, g_stream, st);
 }
 
 cudaError_t launch_bwn_conv(const uint16_t *x_stream, const uint32_t *wp, const float *alpha,
@@ -744,16 +700,7 @@ cudaError_t launch_bwn_conv(const uint16_t *x_stream, const uint32_t *wp, const 
   BwnPlan pl = make_plan(g);
   if (!pl.ok) return cudaErrorInvalidValue;
   BwnParams &P = pl.P;
-  EncodeTiledFn encode = encode_tiled_fn();
-  if (encode == nullptr) return cudaErrorNotSupported;
-  const cuuint64_t dims[4] = {8, (cuuint64_t)(P.Cp / 8), (cuuint64_t)P.L, (cuuint64_t)P.phases};
-  const cuuint64_t strides[3] = {16, (cuuint64_t)P.Cp * 2, (cuuint64_t)P.L * P.Cp * 2};
-  const cuuint32_t box[4] = {8, 1, (cuuint32_t)P.box_pos, 1};
-  const cuuint32_t estr[4] = {1, 1, 1, 1};
-  if (encode(&P.tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<uint16_t *>(x_stream), dims,
-             strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-    return cudaErrorInvalidValue;
+  P.xs = reinterpret_cast<const uint8_t *>(x_stream);
   P.wp = wp; P.alpha = alpha; P.residual = residual; P.out = out;
   P.relu = (g.flags & XNOR_FLAG_RELU) ? 1 : 0;
   static bool attr_flags[64] = {};
