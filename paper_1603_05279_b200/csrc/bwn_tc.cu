@@ -19,10 +19,12 @@
 // filter row).  tcgen05.mma kind::f16 (bf16 x bf16, fp32 accumulation in tensor memory): every
 // product is +-x exactly; only the fp32 accumulation rounds.
 //
-// Roles (832 threads, persistent, one CTA per SM, items = (pixel tiles, filter slab) in tile-major
+// Roles (768 threads, persistent, one CTA per SM, items = (pixel tiles, filter slab) in tile-major
 // order, a contiguous range per CTA): warps 0-7 epilogue (D * alpha (+ residual) -> NCHW; two
 // warps per quarter of the lanes, taking alternate groups of 16 columns), warp 8 issues the MMAs,
-// warp 9 issues the bulk copies, warps 10-25 expand weights (two groups of eight, alternate stages).
+// warp 12 the bulk copies, and the twelve warps 9-11, 13-15, 17-19, 21-23 expand weights (three groups of
+// four, every third stage each).  Warp w runs on scheduler w % 4: the expansion stays off scheduler 0,
+// whose instruction cache then holds the loop of the issuing thread, the path everything waits for.
 // Every wait is bounded; on expiry the CTA records XNOR_ERR_TIMEOUT, stops, and frees its tensor memory.
 #include <cuda_bf16.h>
 
@@ -41,9 +43,9 @@ using namespace umma;
 
 constexpr int kEpiWarps = 8;          // two per quarter of the tensor-memory lanes
 constexpr int kMmaWarp = 8;
-constexpr int kTmaWarp = 9;
-constexpr int kWgtWarp0 = 10, kWgtGroups = 2, kWgtWarps = 8;     // groups of eight warps
-constexpr int kThreads = 32 * (kWgtWarp0 + kWgtGroups * kWgtWarps);   // 832: 26 warps, 72 registers each
+constexpr int kTmaWarp = 12;
+constexpr int kWgtGroups = 3, kWgtWarps = 4;     // groups of four warps
+constexpr int kThreads = 768;                    // 24 warps, 80 registers each
 constexpr int kTileM = 128;
 constexpr int kTmemCols = 512;
 constexpr int kMaxAcc = 4;
@@ -73,7 +75,7 @@ struct BwnParams {
   int vec_len;
   uint32_t idesc;
   int relu;
-  uint32_t tap_lo[kMaxTaps];   // per tap: start of its A operand inside a patch, in 16-byte units
+  uint32_t tap_lo[kMaxTaps + 1];   // per tap: start of its A operand inside a patch, in 16-byte units
   uint32_t div_wq_m, div_hq_m;
   int div_wq_s, div_hq_s;
 };
@@ -180,6 +182,7 @@ __device__ void mma_loop(const BwnParams &P, const Smem &S, long long i0, long l
     tc_fence_after();
     const uint32_t d_tmem = tmem_base + (uint32_t)(ab * P.tpi * P.NT);
     int tap = 0, cw = 0;                     // word f = tap * Cw + cw: two K-steps
+    uint32_t a = (patch_lo + P.tap_lo[0]) | a_lbo_hi;    // addresses stay below 2^18: no carry into the offset
     uint32_t acc = 0u;
     for (int st = 0; st < nst && ok; ++st) {
       ok = mbar_wait(S.wfull + 8u * ws, wph, S.abort_flag, &g_status_bwn);
@@ -188,7 +191,6 @@ __device__ void mma_loop(const BwnParams &P, const Smem &S, long long i0, long l
       const int nw = min(P.wps, P.nwords - st * P.wps);
 #pragma unroll 1
       for (int i = 0; i < nw; ++i) {
-        const uint32_t a = ((patch_lo + P.tap_lo[tap] + (uint32_t)cw * (2u * a_step)) & 0x3FFFu) | a_lbo_hi;
         umma_bf16(d_tmem, a, desc_hi, b_lo, desc_hi, P.idesc, acc);
         // the item's second pixel tile: the same patch 128 positions (128 x 16 bytes) further, the
         // same filter rows, the next accumulator
@@ -198,7 +200,8 @@ __device__ void mma_loop(const BwnParams &P, const Smem &S, long long i0, long l
           umma_bf16(d_tmem + (uint32_t)P.NT, a + a_step + (uint32_t)kTileM, desc_hi, b_lo + b_step, desc_hi, P.idesc, 1u);
         acc = 1u;
         b_lo += 2u * b_step;
-        if (++cw == P.Cw) { cw = 0; ++tap; }
+        a += 2u * a_step;
+        if (++cw == P.Cw) { cw = 0; ++tap; a = (patch_lo + P.tap_lo[tap]) | a_lbo_hi; }
       }
       commit_one(S.wempty + 8u * ws);
       if (++ws == P.stages) { ws = 0; wph ^= 1u; }
@@ -259,7 +262,7 @@ __device__ void tma_role(const BwnParams &P, const Smem &S, long long i0, long l
   }
 }
 
-// ------------------------------------------------------------------ weight producers (16 warps)
+// ------------------------------------------------------------------ weight producers (12 warps)
 // A packed word (32 sign bits, a set bit is +1) -> 16 registers of two bfloat16 +-1 (0x3F80 / 0xBF80):
 // register r holds channel r in its low half and channel r + 16 in its high one, so that a shift brings
 // both signs to their places: two operations per register.  `inv` is the complemented word.
@@ -268,15 +271,14 @@ __device__ __forceinline__ uint32_t expand_pair(uint32_t inv, int r) {
 }
 
 // A stage holds wps packed words of NT filter rows: word i in pieces 4 i .. 4 i + 3 of NT x 16 bytes (two
-// K-steps).  Two groups of eight warps take alternate stages of the sequence over all items; a thread
-// expands one word of one row per stage.  Its words of the next two stages are fetched ahead: the
-// filters are re-read (from L2) for every work item.
-__device__ void weight_role(const BwnParams &P, const Smem &S, long long i0, long long i1, int wt, int lane) {
+// K-steps).  The groups of four warps take the stages of the sequence over all items in turn; a thread
+// expands up to two words of one row per stage.  Its words of the group's next stage are fetched ahead:
+// the filters are re-read (from L2) for every work item.
+__device__ void weight_role(const BwnParams &P, const Smem &S, long long i0, long long i1, int group, int t, int lane) {
+  constexpr int kU = 2;
   const int nst = (P.nwords + P.wps - 1) / P.wps;
-  const int group = wt / (32 * kWgtWarps), t = wt - group * (32 * kWgtWarps);
-  const int row = t % P.rows_mod, wl = t / P.rows_mod;  // row of the slab, word of the stage
+  const int row = t % P.rows_mod, sub = t / P.rows_mod, subs = 32 * kWgtWarps / P.rows_mod;   // words sub, sub + subs of a stage
   const uint32_t b_lbo = (uint32_t)P.NT * 16u;
-  const bool on = row < P.NT && wl < P.wps;
   struct Cursor { long long it; int st, slab; };
   auto advance = [&](Cursor &c, int by) {
     c.st += by;
@@ -286,38 +288,43 @@ __device__ void weight_role(const BwnParams &P, const Smem &S, long long i0, lon
       if (++c.slab == P.nslabs) c.slab = 0;
     }
   };
-  auto fetch = [&](const Cursor &c) {
-    const int f = c.st * P.wps + wl, co = c.slab * P.NT + row;
-    return on && c.it < i1 && f < P.nwords && co < P.Co ? __ldg(P.wp + packed_weight_index(P.Co, co, f)) : 0u;
+  auto fetch = [&](const Cursor &c, uint32_t w[kU]) {
+    const int co = c.slab * P.NT + row;
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int wl = sub + u * subs, f = c.st * P.wps + wl;
+      w[u] = row < P.NT && wl < P.wps && c.it < i1 && f < P.nwords && co < P.Co ? __ldg(P.wp + packed_weight_index(P.Co, co, f)) : 0u;
+    }
   };
   Cursor c{i0, 0, (int)(i0 % P.nslabs)};
   advance(c, group);
-  Cursor ahead = c;
-  uint32_t cur = fetch(ahead);
-  advance(ahead, kWgtGroups);
-  uint32_t nxt = fetch(ahead);
+  uint32_t cur[kU], nxt[kU];
+  fetch(c, cur);
   uint32_t ws = (uint32_t)group, wph = 1u;             // stages >= groups (host)
-  const uint32_t off = (uint32_t)row * 16u + (uint32_t)(4 * wl) * b_lbo;
+  const uint32_t off = (uint32_t)row * 16u + (uint32_t)(4 * sub) * b_lbo;
 #pragma unroll 1
   while (c.it < i1) {
-    advance(ahead, kWgtGroups);
-    const uint32_t nxt2 = fetch(ahead);
+    advance(c, kWgtGroups);
+    fetch(c, nxt);
     if (!mbar_wait_relaxed(S.wempty + 8u * ws, wph, S.abort_flag, &g_status_bwn, 50)) return;
-    if (on) {
-      const uint32_t inv = ~cur, a = S.ring + ws * P.stage_bytes + off;
+    const uint32_t a = S.ring + ws * P.stage_bytes + off;
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        sts128(a + (uint32_t)q * b_lbo, expand_pair(inv, 4 * q), expand_pair(inv, 4 * q + 1), expand_pair(inv, 4 * q + 2),
-               expand_pair(inv, 4 * q + 3));
+    for (int u = 0; u < kU; ++u) {
+      if (row < P.NT && sub + u * subs < P.wps) {
+        const uint32_t inv = ~cur[u], au = a + (uint32_t)(4 * u * subs) * b_lbo;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          sts128(au + (uint32_t)q * b_lbo, expand_pair(inv, 4 * q), expand_pair(inv, 4 * q + 1), expand_pair(inv, 4 * q + 2),
+                 expand_pair(inv, 4 * q + 3));
+      }
     }
     fence_proxy_async();
     __syncwarp();
     if (lane == 0) mbar_arrive(S.wfull + 8u * ws);
     ws += kWgtGroups;
     if (ws >= (uint32_t)P.stages) { ws -= (uint32_t)P.stages; wph ^= 1u; }
-    advance(c, kWgtGroups);
-    cur = nxt;
-    nxt = nxt2;
+#pragma unroll
+    for (int u = 0; u < kU; ++u) cur[u] = nxt[u];
   }
 }
 
@@ -462,7 +469,10 @@ bwn_conv_kernel(const __grid_constant__ BwnParams P) {
     if (warp < kEpiWarps) epilogue_role(P, S, i0, i1, tmem_base, warp & 3, warp >> 2, lane);
     else if (warp == kMmaWarp) mma_role(P, S, i0, i1, tmem_base);
     else if (warp == kTmaWarp) tma_role(P, S, i0, i1, lane);
-    else weight_role(P, S, i0, i1, tid - 32 * kWgtWarp0, lane);
+    else if ((warp & 3) != 0) {
+      const int wi = ((warp >> 2) - 2) * 3 + (warp & 3) - 1;           // 0 .. 11
+      weight_role(P, S, i0, i1, wi / kWgtWarps, 32 * (wi % kWgtWarps) + lane, lane);
+    }
   }
   tc_fence_before();
   __syncthreads();
@@ -603,8 +613,6 @@ BwnPlan make_plan(const ConvGeom &g) {
   int ntp = 16;
   while (ntp < P.NT) ntp *= 2;
   P.rows_mod = ntp;
-  P.wps = std::min(4, 32 * kWgtWarps / ntp);               // a word per thread: 2 (128 filters) or 4
-  P.stage_bytes = (uint32_t)P.wps * (uint32_t)P.NT * 64u;
   P.off_vec = (uint32_t)((kCtrlBytes + 127) / 128 * 128);
   P.vec_len = (g.Co + 15) / 16 * 16 + 256;
   P.off_ring = (uint32_t)((P.off_vec + (size_t)P.vec_len * 4 + 127) / 128 * 128);
@@ -612,23 +620,28 @@ BwnPlan make_plan(const ConvGeom &g) {
   // weight stages: the expansion of the filter rows, which bounds the kernel, is then shared by
   // two MMAs.
   const int stream_tiles = (int)((q.L + kTileM - 1) / kTileM);
+  const int wps_max = std::min(4, 2 * 32 * kWgtWarps / ntp);   // two words per thread: 2 (128 filters) or 4
+  auto stage_of = [&](int wps) { P.wps = wps; P.stage_bytes = (uint32_t)wps * (uint32_t)P.NT * 64u; };
   for (P.tpi = (kTmemCols / P.NT >= 2 && stream_tiles >= 2) ? 2 : 1; P.tpi >= 1; --P.tpi) {
     P.ppix = (P.tpi * kTileM + halo + 7) / 8 * 8;
     P.plane_bytes = (uint32_t)P.ppix * 16u;
     P.phase_bytes = P.plane_bytes * (uint32_t)(P.Cp / 8);
     P.patch_bytes = P.phase_bytes * (uint32_t)P.phases;
-    if (P.off_ring + (P.tpi == 2 ? 4 : 2) * (size_t)P.stage_bytes + P.patch_bytes <= kSmemMax) break;
+    // a stage per group of weight warps at least: shorter ones where the patch leaves little room
+    stage_of(wps_max);
+    while (P.tpi == 1 && P.wps > 1 && P.off_ring + kWgtGroups * (size_t)P.stage_bytes + P.patch_bytes > kSmemMax)
+      stage_of(P.wps / 2);
+    if (P.off_ring + (P.tpi == 2 ? 4 : kWgtGroups) * (size_t)P.stage_bytes + P.patch_bytes <= kSmemMax) break;
   }
   if (P.tpi < 1) return pl;
   P.ntiles = (stream_tiles + P.tpi - 1) / P.tpi;
   P.nacc = std::max(1, std::min(kMaxAcc, kTmemCols / (P.NT * P.tpi)));
   const size_t avail = kSmemMax - P.off_ring;
   auto fits = [&](int st, int pb) { return (size_t)st * P.stage_bytes + (size_t)pb * P.patch_bytes <= avail; };
-  // a second patch buffer hides the patch copies behind the MMAs and comes before more than three stages
-  // (each group of weight warps needs one)
-  int stages = 2, npb = 1;
+  // a second patch buffer hides the patch copies behind the MMAs and comes before more stages than one
+  // per group of weight warps
+  int stages = kWgtGroups, npb = 1;
   if (!fits(stages, npb)) return pl;
-  while (stages < 3 && fits(stages + 1, npb)) ++stages;
   while (npb < 2 && fits(stages, npb + 1)) ++npb;
   while (stages < kMaxStages && fits(stages + 1, npb)) ++stages;
   while (npb < kMaxPatchBufs && fits(stages, npb + 1)) ++npb;
