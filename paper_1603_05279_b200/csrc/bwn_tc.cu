@@ -155,60 +155,79 @@ __device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatil
 }
 
 // ------------------------------------------------------------------ MMA issuer (one thread)
+// kTpi: pixel tiles per item.  The thread's instruction latencies are on the path of everything else
+// (an MMA takes 64 cycles), so what can be is kept in registers, a stage's barrier is polled before the
+// MMAs of the stage before it, and two words are issued in straight-line code.
+template <int kTpi>
 __device__ void mma_loop(const BwnParams &P, const Smem &S, long long i0, long long i1,
                          uint32_t tmem_base) {
-  const int nst = (P.nwords + P.wps - 1) / P.wps;
-  const uint32_t b_lbo = (uint32_t)P.NT * 16u;
-  const uint32_t desc_hi = (128u >> 4) | (1u << 14);      // 128 B between 8-row groups; version
+  const int wps = P.wps, nwords = P.nwords, Cw = P.Cw, nslabs = P.nslabs;
+  const uint32_t NT = (uint32_t)P.NT, idesc = P.idesc, stages = (uint32_t)P.stages;
+  const uint32_t b_lbo = NT * 16u;
+  const uint32_t hi = (128u >> 4) | (1u << 14);           // 128 B between 8-row groups; version
   const uint32_t a_lbo_hi = (P.plane_bytes >> 4) << 16;    // the K-step's second piece: next plane
   const uint32_t b_lo0 = ((S.ring & 0x3FFFFu) >> 4) | ((b_lbo >> 4) << 16);
   const uint32_t b_step = (2u * b_lbo) >> 4;               // next K-step
   const uint32_t a_step = (2u * P.plane_bytes) >> 4;       // next 16 channels of the same tap
   const uint32_t stage_step = P.stage_bytes >> 4;
-  int ws = 0, pb = 0, ab = 0;
-  uint32_t wph = 0, pph = 0, aph = 1u;
-  int slab = (int)(i0 % P.nslabs);
-  bool ok = true, new_tile = true;
+  uint32_t ws = 0u, wph = 0u, pph = 0u, aph = 1u;
+  int pb = 0, ab = 0;
+  int slab = (int)(i0 % nslabs);
+  bool new_tile = true, ready = false;
   uint32_t patch_lo = 0;
   const uint32_t nitems = (uint32_t)(i1 - i0);
-  for (uint32_t it = 0; it < nitems && ok; ++it) {
+  for (uint32_t it = 0; it < nitems; ++it) {
     if (new_tile) {
-      ok = mbar_wait(S.pfull + 8u * pb, pph, S.abort_flag, &g_status_bwn);
-      if (!ok) break;
-      patch_lo = ((S.patch + (uint32_t)pb * P.patch_bytes) & 0x3FFFFu) >> 4;
+      if (!mbar_wait(S.pfull + 8u * pb, pph, S.abort_flag, &g_status_bwn)) return;
+      patch_lo = (((S.patch + (uint32_t)pb * P.patch_bytes) & 0x3FFFFu) >> 4) | a_lbo_hi;
     }
-    ok = mbar_wait(S.aempty + 8u * ab, aph, S.abort_flag, &g_status_bwn);
-    if (!ok) break;
+    if (!mbar_wait(S.aempty + 8u * ab, aph, S.abort_flag, &g_status_bwn)) return;
     tc_fence_after();
-    const uint32_t d_tmem = tmem_base + (uint32_t)(ab * P.tpi * P.NT);
-    int tap = 0, cw = 0;                     // word f = tap * Cw + cw: two K-steps
-    uint32_t a = (patch_lo + P.tap_lo[0]) | a_lbo_hi;    // addresses stay below 2^18: no carry into the offset
-    uint32_t acc = 0u;
-    for (int st = 0; st < nst && ok; ++st) {
-      ok = mbar_wait(S.wfull + 8u * ws, wph, S.abort_flag, &g_status_bwn);
-      if (!ok) break;
-      uint32_t b_lo = b_lo0 + (uint32_t)ws * stage_step;
-      const int nw = min(P.wps, P.nwords - st * P.wps);
+    const uint32_t d0 = tmem_base + (uint32_t)(ab * kTpi) * NT, d1 = d0 + NT;
+    // word f = tap * Cw + cw is two K-steps; addresses stay below 2^18: no carry into the offset field
+    int tap = 0, cw = 0;
+    uint32_t a = patch_lo + P.tap_lo[0], a_next = patch_lo + P.tap_lo[1], acc = 0u;
+    auto next_word = [&]() {
+      const uint32_t cur = a;
+      a += 2u * a_step;
+      if (++cw == Cw) { cw = 0; a = a_next; ++tap; a_next = patch_lo + P.tap_lo[min(tap + 1, kMaxTaps)]; }
+      return cur;
+    };
+    // a K-step's MMAs: the item's second pixel tile is the same patch 128 positions (128 x 16 bytes)
+    // further, the same filter rows, the next accumulator
+    auto step = [&](uint32_t av, uint32_t b, uint32_t accumulate) {
+      umma_bf16(d0, av, hi, b, hi, idesc, accumulate);
+      if (kTpi == 2) umma_bf16(d1, av + (uint32_t)kTileM, hi, b, hi, idesc, accumulate);
+    };
+    for (int left = nwords; left > 0; left -= wps) {
+      if (!ready && !mbar_wait(S.wfull + 8u * ws, wph, S.abort_flag, &g_status_bwn)) return;
+      uint32_t b = b_lo0 + ws * stage_step;
+      uint32_t nws = ws + 1u, nph = wph;
+      if (nws == stages) { nws = 0u; nph ^= 1u; }
+      ready = mbar_try(S.wfull + 8u * nws, nph);
+      int n = min(wps, left);
 #pragma unroll 1
-      for (int i = 0; i < nw; ++i) {
-        umma_bf16(d_tmem, a, desc_hi, b_lo, desc_hi, P.idesc, acc);
-        // the item's second pixel tile: the same patch 128 positions (128 x 16 bytes) further, the
-        // same filter rows, the next accumulator
-        if (P.tpi == 2) umma_bf16(d_tmem + (uint32_t)P.NT, a + (uint32_t)kTileM, desc_hi, b_lo, desc_hi, P.idesc, acc);
-        umma_bf16(d_tmem, a + a_step, desc_hi, b_lo + b_step, desc_hi, P.idesc, 1u);
-        if (P.tpi == 2)
-          umma_bf16(d_tmem + (uint32_t)P.NT, a + a_step + (uint32_t)kTileM, desc_hi, b_lo + b_step, desc_hi, P.idesc, 1u);
+      for (; n >= 2; n -= 2) {
+        const uint32_t a0 = next_word(), a1 = next_word();
+        step(a0, b, acc);
+        step(a0 + a_step, b + b_step, 1u);
+        step(a1, b + 2u * b_step, 1u);
+        step(a1 + a_step, b + 3u * b_step, 1u);
         acc = 1u;
-        b_lo += 2u * b_step;
-        a += 2u * a_step;
-        if (++cw == P.Cw) { cw = 0; ++tap; a = (patch_lo + P.tap_lo[tap]) | a_lbo_hi; }
+        b += 4u * b_step;
+      }
+      if (n > 0) {
+        const uint32_t a0 = next_word();
+        step(a0, b, acc);
+        step(a0 + a_step, b + b_step, 1u);
+        acc = 1u;
       }
       commit_one(S.wempty + 8u * ws);
-      if (++ws == P.stages) { ws = 0; wph ^= 1u; }
+      ws = nws;
+      wph = nph;
     }
-    if (!ok) break;
     new_tile = false;
-    if (++slab == P.nslabs) { slab = 0; new_tile = true; }
+    if (++slab == nslabs) { slab = 0; new_tile = true; }
     commit_one(S.afull + 8u * ab);
     if (new_tile || it + 1 == nitems) commit_one(S.pempty + 8u * pb);
     if (new_tile) { if (++pb == P.npb) { pb = 0; pph ^= 1u; } }
@@ -218,7 +237,10 @@ __device__ void mma_loop(const BwnParams &P, const Smem &S, long long i0, long l
 
 __device__ __forceinline__ void mma_role(const BwnParams &P, const Smem &S, long long i0, long long i1,
                                          uint32_t tmem_base) {
-  if (elect_one()) mma_loop(P, S, i0, i1, tmem_base);
+  if (elect_one()) {
+    if (P.tpi == 2) mma_loop<2>(P, S, i0, i1, tmem_base);
+    else mma_loop<1>(P, S, i0, i1, tmem_base);
+  }
   __syncwarp();
 }
 
