@@ -21,10 +21,10 @@
 //
 // Roles (768 threads, persistent, one CTA per SM, items = (pixel tiles, filter slab) in tile-major
 // order, a contiguous range per CTA): warps 0-7 epilogue (D * alpha (+ residual) -> NCHW; two
-// warps per quarter of the lanes, taking alternate groups of 16 columns), warp 8 issues the MMAs,
+// warps per quarter of the lanes, taking alternate groups of 16 columns), warps 8 and 16 issue the MMAs,
 // warp 12 the bulk copies, and the twelve warps 9-11, 13-15, 17-19, 21-23 expand weights (three groups of
 // four, every third stage each).  Warp w runs on scheduler w % 4: the expansion stays off scheduler 0,
-// whose instruction cache then holds the loop of the issuing thread, the path everything waits for.
+// whose instruction cache then holds the loop of the issuing threads, the path everything waits for.
 // Every wait is bounded; on expiry the CTA records XNOR_ERR_TIMEOUT, stops, and frees its tensor memory.
 #include <cuda_bf16.h>
 
@@ -42,7 +42,7 @@ namespace {
 using namespace umma;
 
 constexpr int kEpiWarps = 8;          // two per quarter of the tensor-memory lanes
-constexpr int kMmaWarp = 8;
+constexpr int kMmaWarp = 8, kMma2Warp = 16;
 constexpr int kTmaWarp = 12;
 constexpr int kWgtGroups = 3, kWgtWarps = 4;     // groups of four warps
 constexpr int kThreads = 768;                    // 24 warps, 80 registers each
@@ -155,12 +155,12 @@ __device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatil
 }
 
 // ------------------------------------------------------------------ MMA issuer (one thread)
-// kTpi: pixel tiles per item.  The thread's instruction latencies are on the path of everything else
-// (an MMA takes 64 cycles), so what can be is kept in registers, a stage's barrier is polled before the
-// MMAs of the stage before it, and two words are issued in straight-line code.
-template <int kTpi>
+// Issues the MMAs of pixel tile `which` of every item: the items' second tile has a warp of its own (one
+// thread issues an MMA in 60 to 85 cycles beside the other roles, the tensor core takes 64; both read the
+// same filter rows, into different accumulators).  What can be is kept in registers, a stage's barrier
+// is polled before the MMAs of the stage before it, and two words are issued in straight-line code.
 __device__ void mma_loop(const BwnParams &P, const Smem &S, long long i0, long long i1,
-                         uint32_t tmem_base) {
+                         uint32_t tmem_base, uint32_t which) {
   const int wps = P.wps, nwords = P.nwords, Cw = P.Cw, nslabs = P.nslabs;
   const uint32_t NT = (uint32_t)P.NT, idesc = P.idesc, stages = (uint32_t)P.stages;
   const uint32_t b_lbo = NT * 16u;
@@ -179,11 +179,12 @@ __device__ void mma_loop(const BwnParams &P, const Smem &S, long long i0, long l
   for (uint32_t it = 0; it < nitems; ++it) {
     if (new_tile) {
       if (!mbar_wait(S.pfull + 8u * pb, pph, S.abort_flag, &g_status_bwn)) return;
-      patch_lo = (((S.patch + (uint32_t)pb * P.patch_bytes) & 0x3FFFFu) >> 4) | a_lbo_hi;
+      // the second tile is the same patch 128 positions (128 x 16 bytes) further
+      patch_lo = ((((S.patch + (uint32_t)pb * P.patch_bytes) & 0x3FFFFu) >> 4) + which * (uint32_t)kTileM) | a_lbo_hi;
     }
     if (!mbar_wait(S.aempty + 8u * ab, aph, S.abort_flag, &g_status_bwn)) return;
     tc_fence_after();
-    const uint32_t d0 = tmem_base + (uint32_t)(ab * kTpi) * NT, d1 = d0 + NT;
+    const uint32_t d_tmem = tmem_base + ((uint32_t)(ab * P.tpi) + which) * NT;
     // word f = tap * Cw + cw is two K-steps; addresses stay below 2^18: no carry into the offset field
     int tap = 0, cw = 0;
     uint32_t a = patch_lo + P.tap_lo[0], a_next = patch_lo + P.tap_lo[1], acc = 0u;
@@ -193,11 +194,8 @@ __device__ void mma_loop(const BwnParams &P, const Smem &S, long long i0, long l
       if (++cw == Cw) { cw = 0; a = a_next; ++tap; a_next = patch_lo + P.tap_lo[min(tap + 1, kMaxTaps)]; }
       return cur;
     };
-    // a K-step's MMAs: the item's second pixel tile is the same patch 128 positions (128 x 16 bytes)
-    // further, the same filter rows, the next accumulator
     auto step = [&](uint32_t av, uint32_t b, uint32_t accumulate) {
-      umma_bf16(d0, av, hi, b, hi, idesc, accumulate);
-      if (kTpi == 2) umma_bf16(d1, av + (uint32_t)kTileM, hi, b, hi, idesc, accumulate);
+      umma_bf16(d_tmem, av, hi, b, hi, idesc, accumulate);
     };
     for (int left = nwords; left > 0; left -= wps) {
       if (!ready && !mbar_wait(S.wfull + 8u * ws, wph, S.abort_flag, &g_status_bwn)) return;
@@ -236,11 +234,8 @@ __device__ void mma_loop(const BwnParams &P, const Smem &S, long long i0, long l
 }
 
 __device__ __forceinline__ void mma_role(const BwnParams &P, const Smem &S, long long i0, long long i1,
-                                         uint32_t tmem_base) {
-  if (elect_one()) {
-    if (P.tpi == 2) mma_loop<2>(P, S, i0, i1, tmem_base);
-    else mma_loop<1>(P, S, i0, i1, tmem_base);
-  }
+                                         uint32_t tmem_base, uint32_t which) {
+  if (elect_one()) mma_loop(P, S, i0, i1, tmem_base, which);
   __syncwarp();
 }
 
@@ -456,14 +451,14 @@ bwn_conv_kernel(const __grid_constant__ BwnParams P) {
   if (tid == 0) {
     for (int i = 0; i < kMaxStages; ++i) {
       mbar_init(S.wfull + 8u * i, kWgtWarps);
-      mbar_init(S.wempty + 8u * i, 1);
+      mbar_init(S.wempty + 8u * i, (uint32_t)P.tpi);           // a commit of every issuing warp
     }
     for (int i = 0; i < kMaxPatchBufs; ++i) {
       mbar_init(S.pfull + 8u * i, 1);
-      mbar_init(S.pempty + 8u * i, 1);
+      mbar_init(S.pempty + 8u * i, (uint32_t)P.tpi);
     }
     for (int i = 0; i < kMaxAcc; ++i) {
-      mbar_init(S.afull + 8u * i, 1);
+      mbar_init(S.afull + 8u * i, (uint32_t)P.tpi);
       mbar_init(S.aempty + 8u * i, kEpiWarps);
     }
     *S.abort_flag = 0;
@@ -489,7 +484,8 @@ bwn_conv_kernel(const __grid_constant__ BwnParams P) {
   const long long i1 = total * (blockIdx.x + 1) / gridDim.x;
   if (i0 < i1) {
     if (warp < kEpiWarps) epilogue_role(P, S, i0, i1, tmem_base, warp & 3, warp >> 2, lane);
-    else if (warp == kMmaWarp) mma_role(P, S, i0, i1, tmem_base);
+    else if (warp == kMmaWarp) mma_role(P, S, i0, i1, tmem_base, 0u);
+    else if (warp == kMma2Warp) { if (P.tpi == 2) mma_role(P, S, i0, i1, tmem_base, 1u); }
     else if (warp == kTmaWarp) tma_role(P, S, i0, i1, lane);
     else if ((warp & 3) != 0) {
       const int wi = ((warp >> 2) - 2) * 3 + (warp & 3) - 1;           // 0 .. 11
