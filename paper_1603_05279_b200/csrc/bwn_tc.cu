@@ -507,13 +507,20 @@ bwn_conv_kernel(const __grid_constant__ BwnParams P) {
 constexpr int kPrepPlanes = 4;                // planes per block: one group of 32 channels
 
 template <bool kGrad>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 6)
 bwn_prepare_kernel(const float *__restrict__ x, const float *__restrict__ scale,
                    const float *__restrict__ shift, const float *__restrict__ gmax, int C, int H,
                    int W, int s, int Hq, int Wq, int leadY, int leadX, long long L, int Cp, int ngroups,
                    uint4 *__restrict__ xs) {
   stream_order();
   const int phase = (int)(blockIdx.y / (unsigned)ngroups), grp = (int)blockIdx.y - phase * ngroups;
+  __shared__ __align__(16) float factor[2][32];            // scale and shift of the block's channels
+  if (threadIdx.x < 32 && scale != nullptr) {
+    const int ch = grp * 32 + threadIdx.x;
+    factor[0][threadIdx.x] = ch < C ? __ldg(scale + ch) : 0.0f;
+    factor[1][threadIdx.x] = !kGrad && ch < C ? __ldg(shift + ch) : 0.0f;
+  }
+  __syncthreads();
   const long long m = (long long)blockIdx.x * 256 + threadIdx.x;
   if (m >= L) return;
   const int py = phase / s, px = phase - py * s;
@@ -535,24 +542,14 @@ bwn_prepare_kernel(const float *__restrict__ x, const float *__restrict__ scale,
       const int ch = 4 * q + (j & 3) + 16 * (j >> 2);
       v[j] = real && (whole || c0 + ch < C) ? __ldg(src + (size_t)ch * plane) : 0.0f;
     }
-    // the factors of the eight channels: four consecutive ones per load
     float sc[8], sh[8];
-    if (scale != nullptr && whole) {
+    if (scale != nullptr) {
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const float4 a = __ldg(reinterpret_cast<const float4 *>(scale + c0 + 16 * h + 4 * q));
+        const float4 a = *reinterpret_cast<const float4 *>(&factor[0][16 * h + 4 * q]);
+        const float4 b = *reinterpret_cast<const float4 *>(&factor[1][16 * h + 4 * q]);
         sc[4 * h] = a.x; sc[4 * h + 1] = a.y; sc[4 * h + 2] = a.z; sc[4 * h + 3] = a.w;
-        if (!kGrad) {
-          const float4 b = __ldg(reinterpret_cast<const float4 *>(shift + c0 + 16 * h + 4 * q));
-          sh[4 * h] = b.x; sh[4 * h + 1] = b.y; sh[4 * h + 2] = b.z; sh[4 * h + 3] = b.w;
-        }
-      }
-    } else if (scale != nullptr) {
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int ch = c0 + 4 * q + (j & 3) + 16 * (j >> 2);
-        sc[j] = ch < C ? __ldg(scale + ch) : 0.0f;
-        sh[j] = !kGrad && ch < C ? __ldg(shift + ch) : 0.0f;
+        sh[4 * h] = b.x; sh[4 * h + 1] = b.y; sh[4 * h + 2] = b.z; sh[4 * h + 3] = b.w;
       }
     }
 #pragma unroll
