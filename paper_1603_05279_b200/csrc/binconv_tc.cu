@@ -35,10 +35,12 @@
 //  are +-{2, 1, 0.5, 0.5} for r = 0..3, weights +-{0.5, 1, 2, 2}: every product
 //  is the product of the two signs.
 //
-//  Roles (512 threads, one CTA per SM, CTAs loop over work items = (pixel
-//  tile, filter slab)): warps 0-3 epilogue (tensor memory -> registers ->
-//  coalesced NCHW stores of D * K * alpha (+ residual)), warp 4 issues the
-//  MMAs, warps 5-12 expand weights, warps 13-15 expand activation patches.
+//  Roles (one CTA per SM, CTAs loop over work items = (pixel tile, filter slab)): warps 0-3 epilogue
+//  (tensor memory -> registers -> coalesced NCHW stores of D * K * alpha (+ residual)), warp 4 issues the
+//  MMAs.  Resident schedule (512 threads): warps 5-12 expand weights, warps 13-15 expand activation
+//  patches.  Streaming schedule (768 threads): twelve warps expand weights and three patches, none of
+//  them on scheduler 0 (warp w runs on scheduler w % 4), whose instruction cache then holds the loop of
+//  the issuing thread, the path everything waits for.
 //  Accumulators are multi-buffered in tensor memory so the epilogue of one
 //  item overlaps the MMAs of the next.  Every wait is bounded: on expiry the
 //  CTA records XNOR_ERR_TIMEOUT in a device status word, stops, frees its
@@ -101,18 +103,19 @@ constexpr int kEpiWarps = 4;
 constexpr int kMmaWarp = 4;
 constexpr int kWgtWarp0 = 5, kWgtWarps = 8;
 constexpr int kPatWarp0 = 13, kPatWarps = 3;
-constexpr int kThreads = 32 * (kPatWarp0 + kPatWarps);     // 512: 16 warps, 128 registers each
+constexpr int kThreadsRes = 32 * (kPatWarp0 + kPatWarps);   // 512: 16 warps, 128 registers each
+// streaming: weight warps in groups of four, patch warps behind them (see the kernel's role table)
+constexpr int kStreamGroups = 3, kGroupWarps = 4, kThreadsStream = 768;   // 24 warps, 80 registers each
 constexpr int kTileM = 128;          // stream positions per tile = tensor-memory lanes
 constexpr int kTmemCols = 512;
 constexpr int kSfCol = 480;          // columns [480, 512): unit block scales
 constexpr int kMaxAccCols = 480;
 constexpr int kMaxAcc = 4;           // accumulator buffers
-constexpr int kMaxStages = 6;         // ring stages of the streaming schedule
+constexpr int kMaxStages = 8;         // ring stages of the streaming schedule
 constexpr int kMaxBarStages = 32;    // stage barriers (the resident schedule has one stage per mps K-steps of a row)
 constexpr int kEpiSplitMax = 3;      // warps per lane quarter in the resident epilogue
 constexpr int kMaxPatchBufs = 4;
 constexpr int kMaxRaw = 6;            // raw buffers: up to 2 for each of up to 3 subgroups of patch warps
-constexpr int kPatUnits = 2;         // patch units a warp works on together
 constexpr int kMaxSteps = 800;       // K-steps (MMAs) per work item (< 1024: swap_mask)
 constexpr size_t kCtrlBytes = 1024;
 constexpr size_t kSmemMax = 232448 - 1024;
@@ -140,6 +143,7 @@ struct TcParams {
   uint32_t patch_bytes, stage_bytes;
   int rows_mod, grp_steps;     // weight-thread mapping (see weight producer)
   uint32_t off_ring, off_patch, off_raw;  // byte offsets in dynamic shared memory
+  uint32_t off_tab;            // streaming: descriptor words of the K-steps in shared memory (0: read from here)
   uint32_t off_vec;            // per-filter vectors staged for the epilogue: alpha, then (fused)
   int vec_len;                 // the next layer's scale and shift; vec_len floats each
   uint32_t raw_bytes;          // size of a raw buffer: the packed input rows a patch can touch
@@ -355,6 +359,7 @@ struct Smem {
   uint32_t *tmem_slot;
   volatile int *abort_flag;
   uint32_t ring, patch, raw;                              // shared-space byte addresses
+  uint32_t tab;                                           // descriptor words (streaming)
   uint32_t alpha, nscale, nshift;                         // staged per-filter vectors
   uint32_t rank;                                          // CTA rank in its pair (0 = issues the MMAs)
 };
@@ -376,6 +381,7 @@ __device__ __forceinline__ Smem carve(uint8_t *smem, const TcParams &P) {
   s.ring = base + P.off_ring;
   s.patch = base + P.off_patch;
   s.raw = base + P.off_raw;
+  s.tab = base + P.off_tab;
   s.alpha = base + P.off_vec;
   s.nscale = s.alpha + 4u * (uint32_t)P.vec_len;
   s.nshift = s.nscale + 4u * (uint32_t)P.vec_len;
@@ -422,11 +428,10 @@ __device__ __forceinline__ void issue_item_flat(const TcParams &P, uint32_t d_tm
   }
 }
 
-// kRes: resident schedule.  The stage barriers are then waited for only before the first item
-// (the CTA stays on one slab, which stays in shared memory) and never released.
-template <bool kRes, bool kPair>
-__device__ void mma_loop(const TcParams &P, const Smem &S, long long i0, long long i1,
-                         uint32_t tmem_base) {
+// Resident schedule.  The stage barriers are waited for only before the first item (the CTA stays on one
+// slab, which stays in shared memory) and never released.
+template <bool kPair>
+__device__ void mma_resident(const TcParams &P, const Smem &S, uint32_t tmem_base) {
   const uint32_t tmem_sf = tmem_base + (uint32_t)kSfCol;
   const int nst = (P.nsteps + P.mps - 1) / P.mps;
   const uint32_t b_lbo = (uint32_t)P.NTh * 16u;
@@ -435,66 +440,109 @@ __device__ void mma_loop(const TcParams &P, const Smem &S, long long i0, long lo
   const uint32_t b_lo0 = ((S.ring & 0x3FFFFu) >> 4) | ((b_lbo >> 4) << 16);   // stage 0, K-step 0
   const uint32_t b_step = (2u * b_lbo) >> 4;                                   // next K-step
   const uint32_t stage_step = P.stage_bytes >> 4;
-  int ws = 0, pb = 0, ab = 0;
-  uint32_t wph = 0, pph = 0;
+  int pb = 0, ab = 0;
+  uint32_t pph = 0;
   uint32_t aph = 1u;                     // parity to wait for on the accumulator's empty barrier
-  // streaming: items [i0, i1), item = tile * nslabs + slab; resident: the unit's own tiles of
-  // its slab (see ResSched), one patch per item
-  const ResSched R = res_sched(P.ntiles, P.nslabs, kPair);
-  int slab = kRes ? 0 : (int)(i0 % P.nslabs);
-  bool ok = true, new_tile = true;
-  uint32_t patch_lo = 0;                 // patch address in descriptor units
-  const uint32_t nitems = kRes ? R.total() : (uint32_t)(i1 - i0);
-  for (uint32_t it = 0; it < nitems && ok; ++it) {
-    if (new_tile) {
-      ok = mbar_wait(S.pfull + 8u * pb, pph, S.abort_flag, &g_status_tc);
-      if (!ok) break;
-      patch_lo = ((S.patch + (uint32_t)pb * P.patch_bytes) & 0x3FFFFu) >> 4;
-    }
-    const bool wait_stages = !kRes || it == 0;
-    ok = mbar_wait(S.aempty + 8u * ab, aph, S.abort_flag, &g_status_tc);
-    if (!ok) break;
+  const uint32_t nitems = res_sched(P.ntiles, P.nslabs, kPair).total();       // one patch per item
+  for (uint32_t it = 0; it < nitems; ++it) {
+    if (!mbar_wait(S.pfull + 8u * pb, pph, S.abort_flag, &g_status_tc)) return;
+    const uint32_t patch_lo = ((S.patch + (uint32_t)pb * P.patch_bytes) & 0x3FFFFu) >> 4;   // in descriptor units
+    if (!mbar_wait(S.aempty + 8u * ab, aph, S.abort_flag, &g_status_tc)) return;
     tc_fence_after();
     const uint32_t d_tmem = tmem_base + (uint32_t)(ab * P.NT);
-    if (kRes) ws = 0;
-    if (kRes && !wait_stages) issue_item_flat<kPair>(P, d_tmem, patch_lo, desc_hi, b_lo0, b_step, tmem_sf);
-    else
-    for (int st = 0; st < nst && ok; ++st) {
-      const int j0 = st * P.mps;
-      const int nj = min(P.mps, P.nsteps - j0);
-      const uint32_t b_lo = b_lo0 + (uint32_t)ws * stage_step;
-      const uint32_t first = st == 0 ? 0u : 1u;     // the first MMA of an item overwrites
-      if (wait_stages) {
-        ok = mbar_wait(S.wfull + 8u * ws, wph, S.abort_flag, &g_status_tc);
-        if (!ok) break;
-        tc_fence_after();
-      }
-      if (nj == 4) issue_stage<4, kPair>(P, j0, d_tmem, patch_lo, desc_hi, b_lo, desc_hi, b_step, tmem_sf, first);
-      else if (nj == 2) issue_stage<2, kPair>(P, j0, d_tmem, patch_lo, desc_hi, b_lo, desc_hi, b_step, tmem_sf, first);
-      else if (nj == 8) issue_stage<8, kPair>(P, j0, d_tmem, patch_lo, desc_hi, b_lo, desc_hi, b_step, tmem_sf, first);
-      else {
-        for (int jj = 0; jj < nj; ++jj)
-          umma_issue<kPair>(d_tmem, P.adesc_lo[j0 + jj] + patch_lo, desc_hi,
-                            b_lo + (uint32_t)jj * b_step, desc_hi, P.idesc, tmem_sf,
-                            jj == 0 ? first : 1u);
-      }
-      if (!kRes) umma_commit_to<kPair>(S.wempty + 8u * ws);
-      if (++ws == P.stages) { ws = 0; if (!kRes) wph ^= 1u; }
-    }
-    if (!ok) break;
-    if (kRes) {
-      // every item has its own patch
-      umma_commit_to<kPair>(S.afull + 8u * ab);
-      umma_commit_to<kPair>(S.pempty + 8u * pb);
-      if (++pb == P.npb) { pb = 0; pph ^= 1u; }
+    if (it > 0) {
+      issue_item_flat<kPair>(P, d_tmem, patch_lo, desc_hi, b_lo0, b_step, tmem_sf);
     } else {
-      // next item: same tile (next slab) or the next tile
-      new_tile = false;
-      if (++slab == P.nslabs) { slab = 0; new_tile = true; }
-      umma_commit_to<kPair>(S.afull + 8u * ab);
-      if (new_tile || it + 1 == nitems) umma_commit_to<kPair>(S.pempty + 8u * pb);
-      if (new_tile) { if (++pb == P.npb) { pb = 0; pph ^= 1u; } }
+      for (int st = 0; st < nst; ++st) {
+        const int j0 = st * P.mps;
+        const int nj = min(P.mps, P.nsteps - j0);
+        const uint32_t b_lo = b_lo0 + (uint32_t)st * stage_step;
+        const uint32_t first = st == 0 ? 0u : 1u;     // the first MMA of an item overwrites
+        if (!mbar_wait(S.wfull + 8u * st, 0u, S.abort_flag, &g_status_tc)) return;
+        tc_fence_after();
+        if (nj == 4) issue_stage<4, kPair>(P, j0, d_tmem, patch_lo, desc_hi, b_lo, desc_hi, b_step, tmem_sf, first);
+        else if (nj == 2) issue_stage<2, kPair>(P, j0, d_tmem, patch_lo, desc_hi, b_lo, desc_hi, b_step, tmem_sf, first);
+        else if (nj == 8) issue_stage<8, kPair>(P, j0, d_tmem, patch_lo, desc_hi, b_lo, desc_hi, b_step, tmem_sf, first);
+        else {
+          for (int jj = 0; jj < nj; ++jj)
+            umma_issue<kPair>(d_tmem, P.adesc_lo[j0 + jj] + patch_lo, desc_hi,
+                              b_lo + (uint32_t)jj * b_step, desc_hi, P.idesc, tmem_sf,
+                              jj == 0 ? first : 1u);
+        }
+      }
     }
+    umma_commit_to<kPair>(S.afull + 8u * ab);
+    umma_commit_to<kPair>(S.pempty + 8u * pb);
+    if (++pb == P.npb) { pb = 0; pph ^= 1u; }
+    if (++ab == P.nacc) { ab = 0; aph ^= 1u; }
+  }
+}
+
+// Streaming schedule: items [i0, i1), item = tile * nslabs + slab, so that a patch serves all slabs of
+// its tile.  The thread's instruction latencies are on the path of everything else (an MMA takes 64
+// cycles): constants in registers, the patch descriptors four at a time from shared memory, the next
+// stage's barrier polled before this stage's MMAs are issued.
+template <bool kPair>
+__device__ void mma_stream(const TcParams &P, const Smem &S, long long i0, long long i1, uint32_t tmem_base) {
+  const uint32_t sf = tmem_base + (uint32_t)kSfCol, idesc = P.idesc, stages = (uint32_t)P.stages;
+  const int nsteps = P.nsteps, mps = P.mps, nslabs = P.nslabs;
+  const uint32_t b_lbo = (uint32_t)P.NTh * 16u;
+  const uint32_t hi = (128u >> 4) | (1u << 14);
+  const uint32_t b_lo0 = ((S.ring & 0x3FFFFu) >> 4) | ((b_lbo >> 4) << 16);
+  const uint32_t b_step = (2u * b_lbo) >> 4, stage_step = P.stage_bytes >> 4;
+  const bool table = P.off_tab != 0u;
+  uint32_t ws = 0u, wph = 0u, pph = 0u, aph = 1u, patch_lo = 0u;
+  int pb = 0, ab = 0, slab = (int)(i0 % nslabs);
+  bool new_tile = true, ready = false;
+  const uint32_t nitems = (uint32_t)(i1 - i0);
+  for (uint32_t it = 0; it < nitems; ++it) {
+    if (new_tile) {
+      if (!mbar_wait(S.pfull + 8u * pb, pph, S.abort_flag, &g_status_tc)) return;
+      patch_lo = ((S.patch + (uint32_t)pb * P.patch_bytes) & 0x3FFFFu) >> 4;
+    }
+    if (!mbar_wait(S.aempty + 8u * ab, aph, S.abort_flag, &g_status_tc)) return;
+    tc_fence_after();
+    const uint32_t d_tmem = tmem_base + (uint32_t)(ab * P.NT);
+    uint32_t acc = 0u;                           // the first MMA of an item overwrites
+    for (int j0 = 0; j0 < nsteps; j0 += mps) {
+      if (!ready && !mbar_wait(S.wfull + 8u * ws, wph, S.abort_flag, &g_status_tc)) return;
+      uint32_t b = b_lo0 + ws * stage_step;
+      uint32_t nws = ws + 1u, nph = wph;
+      if (nws == stages) { nws = 0u; nph ^= 1u; }
+      ready = mbar_try(S.wfull + 8u * nws, nph);
+      int n = min(mps, nsteps - j0), j = j0;
+#pragma unroll 1
+      for (; n >= 4; n -= 4, j += 4) {
+        uint32_t x[4];
+        if (table) {
+          lds128(S.tab + (uint32_t)j * 4u, x);   // mps is 4 or 8 here: 16-byte aligned
+        } else {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) x[i] = P.adesc_lo[j + i];
+        }
+        umma_issue<kPair>(d_tmem, x[0] + patch_lo, hi, b, hi, idesc, sf, acc);
+        umma_issue<kPair>(d_tmem, x[1] + patch_lo, hi, b + b_step, hi, idesc, sf, 1u);
+        umma_issue<kPair>(d_tmem, x[2] + patch_lo, hi, b + 2u * b_step, hi, idesc, sf, 1u);
+        umma_issue<kPair>(d_tmem, x[3] + patch_lo, hi, b + 3u * b_step, hi, idesc, sf, 1u);
+        acc = 1u;
+        b += 4u * b_step;
+      }
+#pragma unroll 1
+      for (; n > 0; --n, ++j) {
+        umma_issue<kPair>(d_tmem, P.adesc_lo[j] + patch_lo, hi, b, hi, idesc, sf, acc);
+        acc = 1u;
+        b += b_step;
+      }
+      umma_commit_to<kPair>(S.wempty + 8u * ws);
+      ws = nws;
+      wph = nph;
+    }
+    // next item: same tile (next slab) or the next tile
+    new_tile = false;
+    if (++slab == nslabs) { slab = 0; new_tile = true; }
+    umma_commit_to<kPair>(S.afull + 8u * ab);
+    if (new_tile || it + 1 == nitems) umma_commit_to<kPair>(S.pempty + 8u * pb);
+    if (new_tile) { if (++pb == P.npb) { pb = 0; pph ^= 1u; } }
     if (++ab == P.nacc) { ab = 0; aph ^= 1u; }
   }
 }
@@ -502,7 +550,10 @@ __device__ void mma_loop(const TcParams &P, const Smem &S, long long i0, long lo
 template <bool kRes, bool kPair>
 __device__ __forceinline__ void mma_role(const TcParams &P, const Smem &S, long long i0, long long i1,
                                          uint32_t tmem_base) {
-  if (elect_one()) mma_loop<kRes, kPair>(P, S, i0, i1, tmem_base);
+  if (elect_one()) {
+    if constexpr (kRes) mma_resident<kPair>(P, S, tmem_base);
+    else mma_stream<kPair>(P, S, i0, i1, tmem_base);
+  }
   __syncwarp();
 }
 
@@ -646,6 +697,82 @@ __device__ __forceinline__ bool weight_dispatch(const TcParams &P, const Smem &S
   return weight_role_swap<1>(P, S, nitems, slab0, wph0, wt, lane);
 }
 
+// ---- streaming schedule: twelve warps
+// The groups of four warps fill the stages of the sequence over all items in turn: with every warp on
+// every stage the expansion was bound by its latency (one instruction in 10 to 15 cycles per warp next
+// to the other roles, barriers and bookkeeping per stage).  A thread expands four units of a stage, a
+// unit being one K-step of one row: row t % rows_mod and every (128 / rows_mod)-th K-step, or rows t and
+// t + 128 of two K-steps.  The packed words of its next stage are fetched ahead.
+__device__ void weight_stream(const TcParams &P, const Smem &S, long long i0, long long i1, int group, int t, int lane) {
+  constexpr int kU = 4;
+  const int nst = (P.nsteps + P.mps - 1) / P.mps;
+  const bool tall = P.rows_mod > 32 * kGroupWarps;
+  const int row = tall ? t : t & (P.rows_mod - 1), sub = tall ? 0 : t / P.rows_mod, subs = tall ? 1 : 32 * kGroupWarps / P.rows_mod;
+  const uint32_t lbo = (uint32_t)P.NTh * 16u;
+  const int nplain = P.row_words >> 1;              // K-steps j < nplain have both words
+  const bool special = P.any_swap || (P.row_words & 1) != 0;
+  const uint2 *wp2 = reinterpret_cast<const uint2 *>(P.wp);
+  auto row_of = [&](int u) { return tall ? row + 32 * kGroupWarps * (u & 1) : row; };
+  auto step_of = [&](int u) { return tall ? u >> 1 : sub + u * subs; };
+  struct Cursor { long long it; int st, slab; };
+  auto advance = [&](Cursor &c, int by) {
+    c.st += by;
+    while (c.st >= nst) {
+      c.st -= nst;
+      ++c.it;
+      if (++c.slab == P.nslabs) c.slab = 0;
+    }
+  };
+  auto fetch = [&](const Cursor &c, uint2 w[kU]) {
+    const int co0 = c.slab * P.NT + (int)S.rank * P.NTh;
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int r = row_of(u), js = step_of(u), j = c.st * P.mps + js;
+      w[u] = c.it < i1 && r < P.NTh && co0 + r < P.Co && js < P.mps && j < P.nsteps ? __ldg(wp2 + (size_t)j * P.Co + (co0 + r))
+                                                                                    : make_uint2(0u, 0u);
+    }
+  };
+  Cursor c{i0, 0, (int)(i0 % P.nslabs)};
+  advance(c, group);
+  uint2 cur[kU], nxt[kU];
+  fetch(c, cur);
+  uint32_t ws = (uint32_t)group, wph = 1u;           // stages >= groups (host)
+#pragma unroll 1
+  while (c.it < i1) {
+    const int j0 = c.st * P.mps;
+    advance(c, kStreamGroups);
+    fetch(c, nxt);
+    if (!mbar_wait_relaxed(S.wempty + 8u * ws, wph, S.abort_flag, &g_status_tc, XNOR_SLEEP_WGT)) return;
+    const uint32_t stage = S.ring + ws * P.stage_bytes;
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int r = row_of(u), js = step_of(u);
+      if (r < P.NTh && js < P.mps) {
+        uint32_t v0[4], v1[4], sw = 0u;
+        expand_signs<false>(cur[u].x, v0);
+        expand_signs<false>(cur[u].y, v1);
+        if (special) {
+          const int j = j0 + js;
+          if ((P.swap_mask[(j >> 5) & 31] >> (j & 31)) & 1u) sw = lbo;
+          if (j >= nplain) v1[0] = v1[1] = v1[2] = v1[3] = 0u;       // the row's lone last word: its partner is 0
+        }
+        const uint32_t a = stage + (uint32_t)js * (2u * lbo) + (uint32_t)r * 16u;
+        if (in_bounds(a >= S.ring && a + lbo + 16u <= S.ring + (uint32_t)P.stages * P.stage_bytes, 13)) {
+          sts128(a + sw, v0[0], v0[1], v0[2], v0[3]);
+          sts128(a + lbo - sw, v1[0], v1[1], v1[2], v1[3]);
+        }
+      }
+    }
+    fence_proxy_async();
+    __syncwarp();
+    if (lane == 0) { if (P.pair) mbar_arrive_cluster(S.wfull + 8u * ws, 0u); else mbar_arrive(S.wfull + 8u * ws); }
+    ws += (uint32_t)kStreamGroups;
+    if (ws >= (uint32_t)P.stages) { ws -= (uint32_t)P.stages; wph ^= 1u; }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) cur[u] = nxt[u];
+  }
+}
+
 // ------------------------------------------------------------------ patch producers
 // A group of P.pat_group warps (the three patch warps) builds the CTA's patches one after the
 // other, all warps on the same patch: units of (32 stream positions, phase plane, up to 4 channel words) are dealt round
@@ -681,6 +808,7 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
   const int npass = (P.ppix + 31) >> 5;
   const int nunits = npass * phases * ngrp;
 
+  constexpr int kPatUnits = kRes ? 2 : 1;                 // patch units a warp works on together (registers)
   auto tile_of = [&](uint32_t seq) {
     if (!kRes) return tile0 + (int)seq;
     uint32_t sl, t;
@@ -1108,9 +1236,10 @@ __device__ bool epilogue_role(const TcParams &P, const Smem &S, long long i0, in
 }
 
 template <bool kRes, bool kPair, bool kFuse>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kRes ? kThreadsRes : kThreadsStream, 1)
 binconv_tc_kernel(const __grid_constant__ TcParams P) {
   extern __shared__ __align__(128) uint8_t smem[];
+  constexpr int kThreads = kRes ? kThreadsRes : kThreadsStream;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const Smem S = carve(smem, P);
 
@@ -1119,7 +1248,7 @@ binconv_tc_kernel(const __grid_constant__ TcParams P) {
     // waits for them); the MMA warp's commits reach the consumer barriers of both CTAs.
     constexpr uint32_t kCtas = kPair ? 2u : 1u;
     for (int i = 0; i < kMaxBarStages; ++i) {
-      mbar_init(S.wfull + 8u * i, (uint32_t)P.wgt_warps * kCtas);
+      mbar_init(S.wfull + 8u * i, (uint32_t)(kRes ? P.wgt_warps : kGroupWarps) * kCtas);
       mbar_init(S.wempty + 8u * i, 1);
     }
     for (int i = 0; i < kMaxPatchBufs; ++i) {
@@ -1168,6 +1297,8 @@ binconv_tc_kernel(const __grid_constant__ TcParams P) {
   // per-filter vectors of the epilogue, zero beyond C_out (one global round trip per CTA
   // instead of one per 16 columns drained); alpha carries the call's extra output factor
   // (1 except in the passes of a k-bit convolution; a product with 1 is exact)
+  if (!kRes && P.off_tab != 0u)
+    for (int i = tid; i < P.nsteps; i += kThreads) reinterpret_cast<uint32_t *>(smem + P.off_tab)[i] = P.adesc_lo[i];
   for (int i = tid; i < P.vec_len; i += kThreads) {
     reinterpret_cast<float *>(smem + P.off_vec)[i] = i < P.Co ? __fmul_rn(__ldg(P.alpha + i), P.out_scale) : 0.0f;
     if (kFuse && P.nscale != nullptr) {
@@ -1191,12 +1322,18 @@ binconv_tc_kernel(const __grid_constant__ TcParams P) {
   if (kRes ? R.total() > 0u : i0 < i1) {
     const int wt = tid - 32 * kWgtWarp0;
     if (warp == kMmaWarp) { if (S.rank == 0) mma_role<kRes, kPair>(P, S, i0, i1, tmem_base); }
-    else if (warp >= kPatWarp0) patch_role<kRes>(P, S, i0, i1, warp - kPatWarp0, lane);
-    else if (!kRes) {
+    else if constexpr (!kRes) {
+      // warps 5-7, 9-11, 13-15, 17-19 expand weights, 21-23 patches; 8, 12, 16, 20 (scheduler 0) rest
+      const int wi = ((warp >> 2) - 1) * 3 + (warp & 3) - 1;
       if (warp < kEpiWarps)
         epilogue_role<false, kFuse>(P, S, i0, 0, 0, 0, (uint32_t)(i1 - i0), 0, tmem_base, warp, 0, lane);
-      else weight_dispatch(P, S, i1 - i0, (int)(i0 % P.nslabs), 1u, wt, lane);
-    } else {
+      else if ((warp & 3) == 0) {}
+      else if (wi < kStreamGroups * kGroupWarps)
+        weight_stream(P, S, i0, i1, wi / kGroupWarps, 32 * (wi % kGroupWarps) + lane, lane);
+      else patch_role<false>(P, S, i0, i1, wi - kStreamGroups * kGroupWarps, lane);
+    }
+    else if (warp >= kPatWarp0) patch_role<kRes>(P, S, i0, i1, warp - kPatWarp0, lane);
+    else {
       // Slab visits of this CTA in order.  The weight warps expand the slab, then every
       // worker warp drains its share of the visit's items.
       const bool wgt = warp >= kWgtWarp0;
@@ -1345,10 +1482,19 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse = false) {
     P.NTh = pair ? P.NT / 2 : P.NT;
     P.wgt_warps = kWgtWarps;
     P.pat_group = kPatWarps;
-    plan_stage(P);
-    if (!fits(2, 1, 1)) return pl;
-    // at least 2 stages and 1 patch; then patches up to 3, stages up to 6, one more patch
-    stages = 2; npb = 1;
+    // stages of four units per thread of a group of warps (see weight_stream), shorter ones where the
+    // patch leaves little room; a stage per group at least
+    P.rows_mod = 16;
+    while (P.rows_mod < P.NTh) P.rows_mod *= 2;
+    const int subs = 32 * kGroupWarps / P.rows_mod;
+    P.mps = subs == 0 ? 2 : std::min(8, 4 * subs);
+    while (P.mps > 4 && P.nsteps < 3 * P.mps) P.mps /= 2;   // short items: smaller stages start sooner
+    auto stage = [&](int mps) { P.mps = mps; P.stage_bytes = (uint32_t)mps * (uint32_t)P.NTh * 32u; };
+    stage(P.mps);
+    while (P.mps > 1 && !fits(kStreamGroups, 1, 1)) stage(P.mps / 2);
+    if (!fits(kStreamGroups, 1, 1)) return pl;
+    // at least 3 stages and 1 patch; then patches up to 3, stages up to 8, one more patch
+    stages = kStreamGroups; npb = 1;
     while (stages < 4 && fits(stages + 1, npb, 1)) ++stages;
     while (npb < 3 && fits(stages, npb + 1, 1)) ++npb;
     while (stages < kMaxStages && fits(stages + 1, npb, 2)) ++stages;
@@ -1361,11 +1507,16 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse = false) {
   P.epi_split = std::min(kEpiSplitMax, P.NT / (fuse ? 32 : 16));
   if (fuse && (g.Co & 31) != 0) return pl;          // whole words of the next layer's input
   P.stages = stages; P.npb = npb;
+  P.off_tab = 0u;
   // small patches: every patch warp builds whole patches on its own, three at a time
   P.pat_sub = subgroups(npb);
   P.off_patch = P.off_ring + (uint32_t)stages * P.stage_bytes;
   P.off_raw = P.off_patch + (uint32_t)npb * P.patch_bytes;
   pl.smem = (size_t)P.off_raw + (size_t)(P.pat_sub * P.nraw) * P.raw_bytes;
+  if (!P.resident && pl.smem + (size_t)P.nsteps * 4 + 16 <= kSmemMax) {       // the descriptor table, where it fits
+    P.off_tab = (uint32_t)((pl.smem + 15) / 16 * 16);
+    pl.smem = (size_t)P.off_tab + (size_t)P.nsteps * 4;
+  }
   // block-scaled instruction descriptor: e2m1 x e2m1, ue8m0 scales, M = 128 (256 for a
   // pair), N = NT
   P.idesc = (1u << 7) | (1u << 10) | ((uint32_t)(P.NT >> 3) << 17) | (1u << 23) |
@@ -1418,7 +1569,7 @@ Plan plan_variant_uncached(const ConvGeom &g, TcVariant v, bool fuse) {
 
 template <bool kRes, bool kPair, bool kFuse>
 cudaError_t launch_variant(const Plan &pl, unsigned units, cudaStream_t st) {
-  return launch_kernel(binconv_tc_kernel<kRes, kPair, kFuse>, dim3(kPair ? 2 * units : units), kThreads, pl.smem, st,
+  return launch_kernel(binconv_tc_kernel<kRes, kPair, kFuse>, dim3(kPair ? 2 * units : units), kRes ? kThreadsRes : kThreadsStream, pl.smem, st,
                        kPair ? 2u : 1u, pl.P);
 }
 
