@@ -105,7 +105,8 @@ constexpr int kWgtWarp0 = 5, kWgtWarps = 8;
 constexpr int kPatWarp0 = 13, kPatWarps = 3;
 constexpr int kThreadsRes = 32 * (kPatWarp0 + kPatWarps);   // 512: 16 warps, 128 registers each
 // streaming: weight warps in groups of four, patch warps behind them (see the kernel's role table)
-constexpr int kStreamGroups = 3, kGroupWarps = 4, kThreadsStream = 768;   // 24 warps, 80 registers each
+constexpr int kLongItem = 64;         // streaming: K-steps of an item that count as many
+constexpr int kGroupWarps = 4, kThreadsStream = 768;   // 24 warps, 80 registers each
 constexpr int kTileM = 128;          // stream positions per tile = tensor-memory lanes
 constexpr int kTmemCols = 512;
 constexpr int kSfCol = 480;          // columns [480, 512): unit block scales
@@ -171,6 +172,7 @@ struct TcParams {
   float *A_part;                     // fp32 [nslabs * epi_split][N][Ho][Wo]: partial sums of |y|
   int Cw_next;                       // ceil(C_out / 32)
   int resident;                // 1: resident schedule (stages = all stages of a slab)
+  int wgt_groups;              // streaming: groups of four warps that expand weights, 3 or 2
   int epi_split;               // warps per lane quarter that drain an accumulator
   int any_swap;                // some bit of swap_mask is set
   uint32_t div_wq_m, div_hq_m; // multipliers and shifts of the exact divisions by Wq and Hq
@@ -460,7 +462,11 @@ __device__ void mma_resident(const TcParams &P, const Smem &S, uint32_t tmem_bas
         const uint32_t first = st == 0 ? 0u : 1u;     // the first MMA of an item overwrites
         if (!mbar_wait(S.wfull + 8u * st, 0u, S.abort_flag, &g_status_tc)) return;
         tc_fence_after();
-        if (nj == 4) issue_stage<4, kPair>(P, j0, d_tmem, patch_lo, desc_hi, b_lo, desc_hi, b_step, tmem_sf, first);
+        if (nj > 8 && (nj & 3) == 0) {            // small problems (see make_plan)
+          for (int jj = 0; jj < nj; jj += 4)
+            issue_stage<4, kPair>(P, j0 + jj, d_tmem, patch_lo, desc_hi, b_lo + (uint32_t)jj * b_step, desc_hi, b_step, tmem_sf,
+                                  jj == 0 ? first : 1u);
+        } else if (nj == 4) issue_stage<4, kPair>(P, j0, d_tmem, patch_lo, desc_hi, b_lo, desc_hi, b_step, tmem_sf, first);
         else if (nj == 2) issue_stage<2, kPair>(P, j0, d_tmem, patch_lo, desc_hi, b_lo, desc_hi, b_step, tmem_sf, first);
         else if (nj == 8) issue_stage<8, kPair>(P, j0, d_tmem, patch_lo, desc_hi, b_lo, desc_hi, b_step, tmem_sf, first);
         else {
@@ -700,76 +706,75 @@ __device__ __forceinline__ bool weight_dispatch(const TcParams &P, const Smem &S
 // ---- streaming schedule: twelve warps
 // The groups of four warps fill the stages of the sequence over all items in turn: with every warp on
 // every stage the expansion was bound by its latency (one instruction in 10 to 15 cycles per warp next
-// to the other roles, barriers and bookkeeping per stage).  A thread expands four units of a stage, a
-// unit being one K-step of one row: row t % rows_mod and every (128 / rows_mod)-th K-step, or rows t and
-// t + 128 of two K-steps.  The packed words of its next stage are fetched ahead.
-__device__ void weight_stream(const TcParams &P, const Smem &S, long long i0, long long i1, int group, int t, int lane) {
+// to the other roles, barriers and bookkeeping per stage).  A thread expands up to four K-steps of one
+// row of a stage: row t % rows_mod, every (128 / rows_mod)-th K-step.  What bounds the loop is its number
+// of instructions, so nothing in it is predicated: rows beyond C_out and K-steps beyond the last re-read
+// an existing word (their columns are never stored, their K-steps never issued), and a word of the next
+// stage is loaded into the register of the one just expanded.
+template <bool kSpecial>
+__device__ void weight_stream(const TcParams &P, const Smem &S, uint32_t nitems, int slab0, int group, int t, int lane) {
   constexpr int kU = 4;
   const int nst = (P.nsteps + P.mps - 1) / P.mps;
-  const bool tall = P.rows_mod > 32 * kGroupWarps;
-  const int row = tall ? t : t & (P.rows_mod - 1), sub = tall ? 0 : t / P.rows_mod, subs = tall ? 1 : 32 * kGroupWarps / P.rows_mod;
-  const uint32_t lbo = (uint32_t)P.NTh * 16u;
-  const int nplain = P.row_words >> 1;              // K-steps j < nplain have both words
-  const bool special = P.any_swap || (P.row_words & 1) != 0;
+  const int subs = 32 * kGroupWarps / P.rows_mod, row = t & (P.rows_mod - 1), sub = t / P.rows_mod;
+  const int nu = max(1, P.mps / subs);               // K-steps of this thread in a stage
+  const bool on = row < P.NTh && sub < P.mps;
+  const uint32_t lbo = (uint32_t)P.NTh * 16u, lstep = (uint32_t)subs * 2u * lbo, gstep = (uint32_t)(subs * P.Co);
+  const uint32_t last = (uint32_t)(P.nsteps * P.Co) - 1u;
+  const int nplain = P.row_words >> 1;               // K-steps j < nplain have both words
+  const int row_co = (int)S.rank * P.NTh + row;
+  const uint32_t row_off = (uint32_t)row * 16u + (uint32_t)sub * 2u * lbo;
   const uint2 *wp2 = reinterpret_cast<const uint2 *>(P.wp);
-  auto row_of = [&](int u) { return tall ? row + 32 * kGroupWarps * (u & 1) : row; };
-  auto step_of = [&](int u) { return tall ? u >> 1 : sub + u * subs; };
-  struct Cursor { long long it; int st, slab; };
-  auto advance = [&](Cursor &c, int by) {
-    c.st += by;
-    while (c.st >= nst) {
-      c.st -= nst;
-      ++c.it;
-      if (++c.slab == P.nslabs) c.slab = 0;
+  uint32_t it = 0u;
+  int st = group, slab = slab0;
+  auto settle = [&]() {
+    while (st >= nst) {
+      st -= nst;
+      ++it;
+      if (++slab == P.nslabs) slab = 0;
     }
   };
-  auto fetch = [&](const Cursor &c, uint2 w[kU]) {
-    const int co0 = c.slab * P.NT + (int)S.rank * P.NTh;
+  auto offset = [&]() { return (uint32_t)((st * P.mps + sub) * P.Co + min(slab * P.NT + row_co, P.Co - 1)); };
+  settle();
+  uint2 w[kU];
+  uint32_t off = offset();
 #pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const int r = row_of(u), js = step_of(u), j = c.st * P.mps + js;
-      w[u] = c.it < i1 && r < P.NTh && co0 + r < P.Co && js < P.mps && j < P.nsteps ? __ldg(wp2 + (size_t)j * P.Co + (co0 + r))
-                                                                                    : make_uint2(0u, 0u);
-    }
-  };
-  Cursor c{i0, 0, (int)(i0 % P.nslabs)};
-  advance(c, group);
-  uint2 cur[kU], nxt[kU];
-  fetch(c, cur);
+  for (int u = 0; u < kU; ++u) w[u] = __ldg(wp2 + min(off + (uint32_t)u * gstep, last));
   uint32_t ws = (uint32_t)group, wph = 1u;           // stages >= groups (host)
 #pragma unroll 1
-  while (c.it < i1) {
-    const int j0 = c.st * P.mps;
-    advance(c, kStreamGroups);
-    fetch(c, nxt);
+  while (it < nitems) {
+    const int j0 = st * P.mps + sub;
+    st += P.wgt_groups;
+    settle();
+    off = offset();
     if (!mbar_wait_relaxed(S.wempty + 8u * ws, wph, S.abort_flag, &g_status_tc, XNOR_SLEEP_WGT)) return;
-    const uint32_t stage = S.ring + ws * P.stage_bytes;
+    if (on) {
+      uint32_t a = S.ring + ws * P.stage_bytes + row_off;
 #pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const int r = row_of(u), js = step_of(u);
-      if (r < P.NTh && js < P.mps) {
-        uint32_t v0[4], v1[4], sw = 0u;
-        expand_signs<false>(cur[u].x, v0);
-        expand_signs<false>(cur[u].y, v1);
-        if (special) {
-          const int j = j0 + js;
-          if ((P.swap_mask[(j >> 5) & 31] >> (j & 31)) & 1u) sw = lbo;
-          if (j >= nplain) v1[0] = v1[1] = v1[2] = v1[3] = 0u;       // the row's lone last word: its partner is 0
-        }
-        const uint32_t a = stage + (uint32_t)js * (2u * lbo) + (uint32_t)r * 16u;
-        if (in_bounds(a >= S.ring && a + lbo + 16u <= S.ring + (uint32_t)P.stages * P.stage_bytes, 13)) {
-          sts128(a + sw, v0[0], v0[1], v0[2], v0[3]);
-          sts128(a + lbo - sw, v1[0], v1[1], v1[2], v1[3]);
+      for (int u = 0; u < kU; ++u) {
+        if (u < nu) {
+          uint32_t v0[4], v1[4], sw = 0u;
+          expand_signs<false>(w[u].x, v0);
+          expand_signs<false>(w[u].y, v1);
+          w[u] = __ldg(wp2 + min(off, last));
+          if (kSpecial) {
+            const int j = j0 + u * subs;
+            if ((P.swap_mask[(j >> 5) & 31] >> (j & 31)) & 1u) sw = lbo;
+            if (j >= nplain) v1[0] = v1[1] = v1[2] = v1[3] = 0u;       // the row's lone last word: its partner is 0
+          }
+          if (in_bounds(a >= S.ring && a + lbo + 16u <= S.ring + (uint32_t)P.stages * P.stage_bytes, 13)) {
+            sts128(a + sw, v0[0], v0[1], v0[2], v0[3]);
+            sts128(a + lbo - sw, v1[0], v1[1], v1[2], v1[3]);
+          }
+          a += lstep;
+          off += gstep;
         }
       }
     }
     fence_proxy_async();
     __syncwarp();
     if (lane == 0) { if (P.pair) mbar_arrive_cluster(S.wfull + 8u * ws, 0u); else mbar_arrive(S.wfull + 8u * ws); }
-    ws += (uint32_t)kStreamGroups;
+    ws += (uint32_t)P.wgt_groups;
     if (ws >= (uint32_t)P.stages) { ws -= (uint32_t)P.stages; wph ^= 1u; }
-#pragma unroll
-    for (int u = 0; u < kU; ++u) cur[u] = nxt[u];
   }
 }
 
@@ -993,7 +998,7 @@ __device__ bool epilogue_role(const TcParams &P, const Smem &S, long long i0, in
                               int tstep, uint32_t nitems, long long k0, uint32_t tmem_base,
                               int quarter, int e, int lane) {
   const int b_end = P.NT / 16;
-  const int esplit = kRes ? P.epi_split : 1;
+  const int esplit = P.epi_split;
   // the k-th group of this warp: groups e, e + esplit, ... or, fused, the two groups of the
   // pairs e, e + esplit, ...
   const int units = kFuse ? b_end / 2 : b_end;
@@ -1261,7 +1266,7 @@ binconv_tc_kernel(const __grid_constant__ TcParams P) {
     }
     for (int i = 0; i < kMaxAcc; ++i) {
       mbar_init(S.afull + 8u * i, 1);
-      mbar_init(S.aempty + 8u * i, (kRes ? kEpiWarps * P.epi_split : kEpiWarps) * kCtas);
+      mbar_init(S.aempty + 8u * i, (uint32_t)(kEpiWarps * P.epi_split * kCtas));
     }
     *S.abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1323,14 +1328,19 @@ binconv_tc_kernel(const __grid_constant__ TcParams P) {
     const int wt = tid - 32 * kWgtWarp0;
     if (warp == kMmaWarp) { if (S.rank == 0) mma_role<kRes, kPair>(P, S, i0, i1, tmem_base); }
     else if constexpr (!kRes) {
-      // warps 5-7, 9-11, 13-15, 17-19 expand weights, 21-23 patches; 8, 12, 16, 20 (scheduler 0) rest
-      const int wi = ((warp >> 2) - 1) * 3 + (warp & 3) - 1;
-      if (warp < kEpiWarps)
-        epilogue_role<false, kFuse>(P, S, i0, 0, 0, 0, (uint32_t)(i1 - i0), 0, tmem_base, warp, 0, lane);
+      // warps 5-7, 9-11, ... in this order: weight groups, patch warps; the last four warps drain too
+      // where the epilogue is split
+      const int wi = ((warp >> 2) - 1) * 3 + (warp & 3) - 1 - kGroupWarps * P.wgt_groups;
+      const bool last = warp >= kThreadsStream / 32 - kEpiWarps && P.epi_split == 2;
+      if (warp < kEpiWarps || last)
+        epilogue_role<false, kFuse>(P, S, i0, 0, 0, 0, (uint32_t)(i1 - i0), 0, tmem_base, warp & 3, last ? 1 : 0, lane);
       else if ((warp & 3) == 0) {}
-      else if (wi < kStreamGroups * kGroupWarps)
-        weight_stream(P, S, i0, i1, wi / kGroupWarps, 32 * (wi % kGroupWarps) + lane, lane);
-      else patch_role<false>(P, S, i0, i1, wi - kStreamGroups * kGroupWarps, lane);
+      else if (wi < 0) {
+        const int group = (wi >> 2) + P.wgt_groups, t = 32 * (wi & 3) + lane, slab0 = (int)(i0 % P.nslabs);
+        if (P.any_swap || (P.row_words & 1)) weight_stream<true>(P, S, (uint32_t)(i1 - i0), slab0, group, t, lane);
+        else weight_stream<false>(P, S, (uint32_t)(i1 - i0), slab0, group, t, lane);
+      }
+      else if (wi < kPatWarps) patch_role<false>(P, S, i0, i1, wi, lane);
     }
     else if (warp >= kPatWarp0) patch_role<kRes>(P, S, i0, i1, warp - kPatWarp0, lane);
     else {
@@ -1377,13 +1387,13 @@ struct Plan {
 // Weight-thread mapping and stage size for slabs of NT filters: rows_mod threads cover the
 // rows of a K-step, the other thread groups take other K-steps of the stage; a stage is up to
 // 32 KB of expanded weights.
-void plan_stage(TcParams &P) {
+void plan_stage(TcParams &P, bool few) {
   int ntp = 16;
   while (ntp < P.NTh) ntp *= 2;                         // 16 .. 256
   P.rows_mod = ntp;
   const int groups = std::max(1, 32 * P.wgt_warps / P.rows_mod);   // 1 .. 16
-  P.mps = std::max(2, std::min(8, 1024 / ntp));
-  while (P.mps > 4 && P.nsteps < 3 * P.mps) P.mps /= 2;   // short items: smaller stages start sooner
+  P.mps = std::max(2, std::min(few ? 32 : 8, 1024 / ntp));
+  while (P.mps > 4 && P.nsteps < (few ? 2 : 3) * P.mps) P.mps /= 2;   // short items: smaller stages start sooner
   if (P.mps > 4 * groups) P.mps = 4 * groups;           // a thread expands at most 4 K-steps of a stage
   P.grp_steps = std::max(1, P.mps / groups);            // 4, 4, 2, 1, 1
   P.stage_bytes = (uint32_t)P.mps * (uint32_t)P.NTh * 32u;
@@ -1449,24 +1459,36 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse = false) {
   P.pat_group = kPatWarps;
   // as few slabs as fit two accumulators in the tensor-memory columns
   const int max_nt = pair ? 224 : 240;
-  const int min_slabs = (g.Co + max_nt - 1) / max_nt;
+  int min_slabs = (g.Co + max_nt - 1) / max_nt;
+  // Items for fewer than half the SMs: narrower slabs on up to half of them, a CTA then expands and
+  // drains less (512 channels, 7x7, one image: 15.6 -> 9.4 us; 64 channels, 14x14: 6.7 -> 6.5 us).  With
+  // few K-steps the drain counts most and 16 filters win, else 32.  A small problem fills its one item's
+  // stages in few, large steps (`few` in plan_stage): the latency per stage is what it waits for.
+  const int spread = (int)kSms / 2 / P.ntiles;
+  const bool few = !pair && !fuse && min_slabs <= spread;
+  if (few) {
+    const int width = P.nsteps < 16 ? 16 : 32;
+    min_slabs = std::max(min_slabs, std::min(spread, (g.Co + width - 1) / width));
+  }
   int stages = 0, npb = 0;
   P.resident = 0;
   if (schedule == 0) {
-    // Resident: the widest slab whose expanded rows fit beside two patches.  Every slab
-    // needs its own patch per tile and narrow MMAs re-read the pixel operand more often, so
-    // (measured) slabs below 128 filters pay only when one slab holds all filters.
+    // Resident: the widest slab whose expanded rows fit beside two patches.  Every slab needs its own
+    // patch per tile and narrow MMAs re-read the pixel operand more often.  So (measured) several slabs
+    // pay only from 128 filters (a pair: 96; 512 channels, 7x7, residual: 45.6 -> 34.1 us) and with two
+    // K-steps or more per plane of the patch: kernels of 3x3 and up with stride 1 (128 channels, 28x28,
+    // stride 2: 29.5 us resident, 27.0 streaming).
     for (int ns = min_slabs; ns <= 16 && !P.resident; ++ns) {
-      P.nslabs = ns;
       P.NT = slab_width(g.Co, ns, pair || fuse);
+      P.nslabs = (g.Co + P.NT - 1) / P.NT;
       P.NTh = pair ? P.NT / 2 : P.NT;
-      if (P.NT < 128 && ns > 1) break;
+      if (P.nslabs > 1 && !few && (P.NT < (pair ? 96 : 128) || P.nsteps < 2 * P.nplanes)) break;
       // (Lending four of the weight warps to the patch builders where a pixel has many channel
       // words was the better split while the drain loop was longer; since its trimming twelve
       // draining warps win on every layer measured: conv4 50.4 -> 48.1 us, conv5 39.4 -> 37.3.)
       P.wgt_warps = kWgtWarps;
       P.pat_group = kPatWarps;
-      plan_stage(P);
+      plan_stage(P, few);
       const int nst = (P.nsteps + P.mps - 1) / P.mps;
       if (nst <= kMaxBarStages && fits(nst, 2, 1)) {
         P.resident = 1;
@@ -1477,24 +1499,29 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse = false) {
     }
   }
   if (!P.resident) {
-    P.nslabs = min_slabs;
-    P.NT = slab_width(g.Co, P.nslabs, pair || fuse);
+    P.NT = slab_width(g.Co, std::max(min_slabs, (g.Co + 127) / 128), pair || fuse);
+    P.nslabs = (g.Co + P.NT - 1) / P.NT;
     P.NTh = pair ? P.NT / 2 : P.NT;
     P.wgt_warps = kWgtWarps;
     P.pat_group = kPatWarps;
     // stages of four units per thread of a group of warps (see weight_stream), shorter ones where the
     // patch leaves little room; a stage per group at least
+    if (P.NTh > 32 * kGroupWarps) return pl;             // a thread expands one row
     P.rows_mod = 16;
     while (P.rows_mod < P.NTh) P.rows_mod *= 2;
     const int subs = 32 * kGroupWarps / P.rows_mod;
-    P.mps = subs == 0 ? 2 : std::min(8, 4 * subs);
+    P.mps = std::min(8, 4 * subs);
     while (P.mps > 4 && P.nsteps < 3 * P.mps) P.mps /= 2;   // short items: smaller stages start sooner
+    // Long items are bound by the expansion, short ones by the epilogue: two warps per quarter of the
+    // lanes in place of a weight group (1024 channels, 1x1: 27.2 -> 25.6 us; 512 channels, 3x3, 72 K-steps:
+    // 32.8 -> 34.7 us).
+    P.wgt_groups = P.nsteps < kLongItem && !fuse ? 2 : 3;
     auto stage = [&](int mps) { P.mps = mps; P.stage_bytes = (uint32_t)mps * (uint32_t)P.NTh * 32u; };
     stage(P.mps);
-    while (P.mps > 1 && !fits(kStreamGroups, 1, 1)) stage(P.mps / 2);
-    if (!fits(kStreamGroups, 1, 1)) return pl;
+    while (P.mps > 1 && !fits(P.wgt_groups, 1, 1)) stage(P.mps / 2);
+    if (!fits(P.wgt_groups, 1, 1)) return pl;
     // at least 3 stages and 1 patch; then patches up to 3, stages up to 8, one more patch
-    stages = kStreamGroups; npb = 1;
+    stages = P.wgt_groups; npb = 1;
     while (stages < 4 && fits(stages + 1, npb, 1)) ++stages;
     while (npb < 3 && fits(stages, npb + 1, 1)) ++npb;
     while (stages < kMaxStages && fits(stages + 1, npb, 2)) ++stages;
@@ -1504,7 +1531,7 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse = false) {
   P.nacc = std::max(1, std::min(kMaxAcc, kMaxAccCols / P.NT));
   // worker warps per quarter of the lanes in the resident schedule: the four epilogue warps
   // and the eight weight warps
-  P.epi_split = std::min(kEpiSplitMax, P.NT / (fuse ? 32 : 16));
+  P.epi_split = P.resident ? std::min(kEpiSplitMax, P.NT / (fuse ? 32 : 16)) : P.wgt_groups == 2 ? std::min(2, P.NT / 16) : 1;
   if (fuse && (g.Co & 31) != 0) return pl;          // whole words of the next layer's input
   P.stages = stages; P.npb = npb;
   P.off_tab = 0u;
@@ -1550,7 +1577,9 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse = false) {
 namespace {
 
 // The plan of a variant.  kTcAuto (measured on the AlexNet and ResNet-18 shapes): one CTA per
-// SM unless only a pair, each CTA holding half of a slab, can keep the filters resident.
+// SM unless only a pair, each CTA holding half of a slab, can keep the filters resident.  Neither: pairs
+// where the items are long (each CTA expands half the rows of a slab; 1024 channels, 7x7 kernel: 419 ->
+// 361 us; 1x1 kernel, 16 K-steps: 27.2 -> 30.5 us) and the slabs wide enough to fill a pair.
 Plan plan_variant_uncached(const ConvGeom &g, TcVariant v, bool fuse) {
   switch (v) {
     case kTcSingle: return make_plan(g, 0, false, fuse);
@@ -1561,9 +1590,10 @@ Plan plan_variant_uncached(const ConvGeom &g, TcVariant v, bool fuse) {
   }
   Plan single = make_plan(g, 0, false, fuse);
   if (single.ok && single.P.resident) return single;
+  // a problem of few items is better spread over single CTAs
+  if (single.ok && 2 * single.P.ntiles * single.P.nslabs <= (int)kSms) return single;
   Plan pair = make_plan(g, 0, true, fuse);
-  // neither resident: a pair pays when the slabs are wide (each CTA expands half the rows)
-  if (pair.ok && (pair.P.resident || !single.ok || pair.P.NT > 128)) return pair;
+  if (pair.ok && (pair.P.resident || !single.ok || (pair.P.NT > 64 && pair.P.nsteps >= kLongItem))) return pair;
   return single;
 }
 
@@ -1670,7 +1700,7 @@ cudaError_t launch_binconv_tc(const uint32_t *xp, const uint32_t *wp, const floa
 int tc_fused_parts(const ConvGeom &g, TcVariant variant) {
   const Plan pl = plan_variant(g, variant, true);
   if (!pl.ok) return 0;
-  return pl.P.nslabs * (pl.P.resident ? pl.P.epi_split : 1);
+  return pl.P.nslabs * pl.P.epi_split;
 }
 
 cudaError_t launch_binconv_tc_fused(const uint32_t *xp, const uint32_t *wp, const float *alpha,
