@@ -72,6 +72,14 @@ def test_kbit_pack(oracle, case, kbits):
     assert_close(host(K), oracle.box_filter(A_or, k, k, 1, p), "K")
 
 
+# pixels not a multiple of the 128 of a warp, images ending inside a run; one to five channel words, tails
+@pytest.mark.parametrize("kbits", [1, 2])
+@pytest.mark.parametrize("case", [(83, 100, 28, 29, 1, 0), (83, 33, 29, 28, 1, 0), (70, 130, 30, 32, 3, 1),
+                                  (300, 16, 12, 19, 3, 1), (66, 64, 32, 32, 1, 0)])
+def test_wide_pack(oracle, case, kbits):
+    test_kbit_pack(oracle, case, kbits)
+
+
 @pytest.mark.parametrize("valid", [False, True])
 @pytest.mark.parametrize("case", [(190, 2, 56, 56, 3, 1), (260, 2, 55, 44, 5, 2), (230, 1, 51, 48, 5, 0),
                                   (330, 1, 37, 50, 3, 0)])
