@@ -506,8 +506,12 @@ bwn_conv_kernel(const __grid_constant__ BwnParams P) {
 // HBM bounds it.
 constexpr int kPrepPlanes = 4;                // planes per block: one group of 32 channels
 
+// All 32 loads of a thread are in flight before the first is used: 256 channels, 14x14, 256 images
+// 15.9 -> 14.5 us (HBM: 11.8), 64 channels, 56x56, 128 images 28.9 -> 25.2 (23.6).
+constexpr int kPrepThreads = 128;
+
 template <bool kGrad>
-__global__ void __launch_bounds__(256, 6)
+__global__ void __launch_bounds__(kPrepThreads, 6)
 bwn_prepare_kernel(const float *__restrict__ x, const float *__restrict__ scale,
                    const float *__restrict__ shift, const float *__restrict__ gmax, int C, int H,
                    int W, int s, int Hq, int Wq, int leadY, int leadX, long long L, int Cp, int ngroups,
@@ -521,7 +525,7 @@ bwn_prepare_kernel(const float *__restrict__ x, const float *__restrict__ scale,
     factor[1][threadIdx.x] = !kGrad && ch < C ? __ldg(shift + ch) : 0.0f;
   }
   __syncthreads();
-  const long long m = (long long)blockIdx.x * 256 + threadIdx.x;
+  const long long m = (long long)blockIdx.x * kPrepThreads + threadIdx.x;
   if (m >= L) return;
   const int py = phase / s, px = phase - py * s;
   const uint32_t mu = (uint32_t)m, r = mu / (uint32_t)Wq, c = mu - r * (uint32_t)Wq, n = r / (uint32_t)Hq;   // L < 2^31
@@ -534,14 +538,17 @@ bwn_prepare_kernel(const float *__restrict__ x, const float *__restrict__ scale,
   const float gm = kGrad && real ? __ldg(gmax + n) : 0.0f;    // the scale of this position's image
   uint4 *dst = xs + ((size_t)(phase * (Cp / 8) + grp * kPrepPlanes) * (size_t)L + (size_t)m);
   const bool whole = c0 + 32 <= C;
+  float values[kPrepPlanes][8];
 #pragma unroll
-  for (int q = 0; q < kPrepPlanes; ++q) {
-    float v[8];                               // channels c0 + 4 q + i, then c0 + 16 + 4 q + i
+  for (int q = 0; q < kPrepPlanes; ++q)
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int ch = 4 * q + (j & 3) + 16 * (j >> 2);
-      v[j] = real && (whole || c0 + ch < C) ? __ldg(src + (size_t)ch * plane) : 0.0f;
+      values[q][j] = real && (whole || c0 + ch < C) ? __ldg(src + (size_t)ch * plane) : 0.0f;
     }
+#pragma unroll
+  for (int q = 0; q < kPrepPlanes; ++q) {
+    float (&v)[8] = values[q];                // channels c0 + 4 q + i, then c0 + 16 + 4 q + i
     float sc[8], sh[8];
     if (scale != nullptr) {
 #pragma unroll
@@ -706,8 +713,8 @@ cudaError_t launch_prepare(const float *x, const float *scale, const float *shif
   const StreamGeom q = stream_geom(g);
   const int ngroups = q.Cp / 32;
   if (q.L >= (1ll << 31) || (long long)ngroups * q.phases > 65535) return cudaErrorInvalidValue;
-  const dim3 grid((unsigned)((q.L + 255) / 256), (unsigned)(ngroups * q.phases));
-  return launch_kernel(bwn_prepare_kernel<kGrad>, grid, 256, 0, st, 1, x, scale, shift, gmax, g.C, g.H, g.W, q.s, q.Hq, q.Wq,
+  const dim3 grid((unsigned)((q.L + kPrepThreads - 1) / kPrepThreads), (unsigned)(ngroups * q.phases));
+  return launch_kernel(bwn_prepare_kernel<kGrad>, grid, kPrepThreads, 0, st, 1, x, scale, shift, gmax, g.C, g.H, g.W, q.s, q.Hq, q.Wq,
                        q.leadY, q.leadX, q.L, q.Cp, ngroups, reinterpret_cast<uint4 *>(x_stream));
 }
 

@@ -6,6 +6,7 @@ import pytest
 import torch
 
 import paper_1603_05279_b200 as X
+from test_gpu_bgrad import test_binary_gradient_backward_parity as backward_parity
 from test_gpu_options import _index_of_planes
 from util import GuardSet, assert_close, dev, host
 
@@ -78,6 +79,12 @@ def test_kbit_pack(oracle, case, kbits):
                                   (300, 16, 12, 19, 3, 1), (66, 64, 32, 32, 1, 0)])
 def test_wide_pack(oracle, case, kbits):
     test_kbit_pack(oracle, case, kbits)
+
+
+# max|g| by a cluster per image (74 images and up on 148 SMs), images of odd size and of one chunk per thread
+@pytest.mark.parametrize("shape", [(75, 33, 5, 5, 17, 3, 1), (74, 32, 21, 19, 101, 3, 1)])
+def test_gradient_maximum_of_many_images(oracle, shape):
+    backward_parity(oracle, shape)
 
 
 @pytest.mark.parametrize("valid", [False, True])
