@@ -147,7 +147,9 @@ struct TcParams {
   uint32_t off_tab;            // streaming: descriptor words of the K-steps in shared memory (0: read from here)
   uint32_t off_vec;            // per-filter vectors staged for the epilogue: alpha, then (fused)
   int vec_len;                 // the next layer's scale and shift; vec_len floats each
-  uint32_t raw_bytes;          // size of a raw buffer: the packed input rows a patch can touch
+  uint32_t raw_bytes;          // size of a raw buffer: the packed input rows a patch can touch, of every bit plane
+  uint32_t raw_plane;          // the share of one bit plane
+  const uint32_t *xp2;         // two bit planes in one pass: the upper one (see patch_role)
   int nraw;                    // raw buffers per subgroup of patch warps (1 or 2)
   int pat_group;               // warps that build patches
   int pat_sub;                 // subgroups they form (each builds whole patches): 3 or 1
@@ -790,7 +792,10 @@ __device__ void weight_stream(const TcParams &P, const Smem &S, uint32_t nitems,
 // their way while one is expanded.  Padding and the channel tail become the value 0 through
 // masks folded into the sign mask and the magnitude constants.
 // Streaming: one patch per tile of the CTA's range.  Resident (kRes): one patch per item.
-template <bool kRes>
+// kTwo: two bit planes of a k-bit input in one pass.  Their level code b0 + 2 b1 stands for -3, -1, 1, 3,
+// all of them e2m1 values beside any of the three magnitudes: the upper plane is the sign, and equal bits
+// triple the magnitude.  The convolution then costs what one plane costs.
+template <bool kRes, bool kTwo>
 __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long long i1, int pw,
                            int lane) {
   const ResSched R = res_sched(P.ntiles, P.nslabs, P.pair != 0);
@@ -813,7 +818,7 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
   const int npass = (P.ppix + 31) >> 5;
   const int nunits = npass * phases * ngrp;
 
-  constexpr int kPatUnits = kRes ? 2 : 1;                 // patch units a warp works on together (registers)
+  constexpr int kPatUnits = kRes && !kTwo ? 2 : 1;                 // patch units a warp works on together (registers)
   auto tile_of = [&](uint32_t seq) {
     if (!kRes) return tile0 + (int)seq;
     uint32_t sl, t;
@@ -846,11 +851,15 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
     const size_t a1 = min((b1 + 15) & ~(size_t)15, tensor_bytes & ~(size_t)15);
     const uint32_t bulk = a1 > a0 ? (uint32_t)(a1 - a0) : 0u;
     for (size_t b = a0 + bulk; b < b1; b += 4)           // at most 3 words, at the tensor's end
-      if (in_bounds((uint32_t)(b - a0) + 4u <= P.raw_bytes, 3))
+      if (in_bounds((uint32_t)(b - a0) + 4u <= P.raw_plane, 3))
+      {
         sts32(dst + (uint32_t)(b - a0), __ldg(P.xp + (b >> 2)));
-    if (bulk && in_bounds(bulk <= P.raw_bytes && a0 + bulk <= tensor_bytes, 4)) {
-      mbar_arrive_expect_tx(bar, bulk);
+        if (kTwo) sts32(dst + P.raw_plane + (uint32_t)(b - a0), __ldg(P.xp2 + (b >> 2)));
+      }
+    if (bulk && in_bounds(bulk <= P.raw_plane && a0 + bulk <= tensor_bytes, 4)) {
+      mbar_arrive_expect_tx(bar, kTwo ? 2u * bulk : bulk);
       bulk_copy_g2s(dst, reinterpret_cast<const uint8_t *>(P.xp) + a0, bulk, bar);
+      if (kTwo) bulk_copy_g2s(dst + P.raw_plane, reinterpret_cast<const uint8_t *>(P.xp2) + a0, bulk, bar);
     } else {
       mbar_arrive(bar);
     }
@@ -903,7 +912,7 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
     // warp can overlap, then all are expanded
 #pragma unroll 1
     for (int u0 = (int)mi; u0 < nunits; u0 += kPatUnits * (int)gsize) {
-      uint32_t src[kPatUnits], dst[kPatUnits], sm[kPatUnits], mc[kPatUnits][3], wv[kPatUnits][4];
+      uint32_t src[kPatUnits], dst[kPatUnits], sm[kPatUnits], mc[kPatUnits][3], wv[kPatUnits][4], wu[kTwo ? kPatUnits : 1][4];
       int w0[kPatUnits];
       bool on[kPatUnits], real[kPatUnits];
 #pragma unroll
@@ -933,14 +942,19 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
 #pragma unroll
       for (int b = 0; b < kPatUnits; ++b) {
         wv[b][0] = wv[b][1] = wv[b][2] = wv[b][3] = 0u;
+        if (kTwo) wu[b][0] = wu[b][1] = wu[b][2] = wu[b][3] = 0u;
         if (real[b] && in_bounds(src[b] >= S.raw + rb * P.raw_bytes &&
-                                 src[b] + 4u * (uint32_t)min(4, P.Cw - w0[b]) <= S.raw + (rb + 1u) * P.raw_bytes, 6)) {
+                                 src[b] + 4u * (uint32_t)min(4, P.Cw - w0[b]) <= S.raw + rb * P.raw_bytes + P.raw_plane, 6)) {
           if (vec) {
             lds128(src[b], wv[b]);
+            if (kTwo) lds128(src[b] + P.raw_plane, wu[b]);
           } else {
 #pragma unroll
             for (int i = 0; i < 4; ++i)
-              if (w0[b] + i < P.Cw) wv[b][i] = lds32(src[b] + (uint32_t)i * 4u);
+              if (w0[b] + i < P.Cw) {
+                wv[b][i] = lds32(src[b] + (uint32_t)i * 4u);
+                if (kTwo) wu[b][i] = lds32(src[b] + P.raw_plane + (uint32_t)i * 4u);
+              }
           }
         }
       }
@@ -950,11 +964,18 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             if (w0[b] + i < P.Cw) {
-              const uint32_t w = wv[b][i];
+              const uint32_t w = kTwo ? wu[b][i] : wv[b][i];      // signs
               uint32_t v0 = ((w << 3) & sm[b]) ^ mc[b][0];
               uint32_t v1 = ((w << 2) & sm[b]) ^ mc[b][1];
               uint32_t v2 = ((w << 1) & sm[b]) ^ mc[b][2];
               uint32_t v3 = (w & sm[b]) ^ mc[b][2];
+              if (kTwo) {                                 // magnitudes 2, 1, 0.5 (100, 010, 001) -> 6, 3, 1.5 (111, 101, 011)
+                const uint32_t e = ~(wv[b][i] ^ wu[b][i]), e0 = (e << 3) & sm[b], e1 = (e << 2) & sm[b];
+                v0 ^= (e0 >> 2) | (e0 >> 3);
+                v1 ^= e1 - (e1 >> 3);
+                v2 ^= ((e << 1) & sm[b]) >> 2;
+                v3 ^= (e & sm[b]) >> 2;
+              }
               if (tail && w0[b] + i == P.Cw - 1) {       // channels beyond C_in are 0
                 v0 &= tm[0]; v1 &= tm[1]; v2 &= tm[2]; v3 &= tm[3];
               }
@@ -1240,7 +1261,7 @@ __device__ bool epilogue_role(const TcParams &P, const Smem &S, long long i0, in
   return ok;
 }
 
-template <bool kRes, bool kPair, bool kFuse>
+template <bool kRes, bool kPair, bool kFuse, bool kTwo>
 __global__ void __launch_bounds__(kRes ? kThreadsRes : kThreadsStream, 1)
 binconv_tc_kernel(const __grid_constant__ TcParams P) {
   extern __shared__ __align__(128) uint8_t smem[];
@@ -1340,9 +1361,9 @@ binconv_tc_kernel(const __grid_constant__ TcParams P) {
         if (P.any_swap || (P.row_words & 1)) weight_stream<true>(P, S, (uint32_t)(i1 - i0), slab0, group, t, lane);
         else weight_stream<false>(P, S, (uint32_t)(i1 - i0), slab0, group, t, lane);
       }
-      else if (wi < kPatWarps) patch_role<false>(P, S, i0, i1, wi, lane);
+      else if (wi < kPatWarps) patch_role<false, kTwo>(P, S, i0, i1, wi, lane);
     }
-    else if (warp >= kPatWarp0) patch_role<kRes>(P, S, i0, i1, warp - kPatWarp0, lane);
+    else if (warp >= kPatWarp0) patch_role<kRes, kTwo>(P, S, i0, i1, warp - kPatWarp0, lane);
     else {
       // Slab visits of this CTA in order.  The weight warps expand the slab, then every
       // worker warp drains its share of the visit's items.
@@ -1407,7 +1428,7 @@ int slab_width(int Co, int ns, bool pair) {     // pair: also set for the fused 
 }
 
 // schedule: 0 = resident when the slab fits, 1 = streaming.  pair: CTA pairs (clusters of 2).
-Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse = false) {
+Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes) {
   Plan pl{};
   pl.ok = false;
   TcParams &P = pl.P;
@@ -1435,7 +1456,8 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse = false) {
   const long long raw_rows = ((long long)(P.ppix - 1) / P.Wq + 2) * s;
   const long long raw_bytes = (raw_rows * g.W * g.Cw * 4 + 12 + 15 + 15) / 16 * 16;
   if (raw_bytes > (long long)kSmemMax) return pl;
-  P.raw_bytes = (uint32_t)raw_bytes;
+  P.raw_plane = (uint32_t)raw_bytes;
+  P.raw_bytes = (uint32_t)planes * P.raw_plane;
   P.nplanes = s * s * g.Cw;
   P.patch_bytes = (uint32_t)P.nplanes * (uint32_t)P.ppix * 16u;
   // K-steps
@@ -1580,26 +1602,26 @@ namespace {
 // SM unless only a pair, each CTA holding half of a slab, can keep the filters resident.  Neither: pairs
 // where the items are long (each CTA expands half the rows of a slab; 1024 channels, 7x7 kernel: 419 ->
 // 361 us; 1x1 kernel, 16 K-steps: 27.2 -> 30.5 us) and the slabs wide enough to fill a pair.
-Plan plan_variant_uncached(const ConvGeom &g, TcVariant v, bool fuse) {
+Plan plan_variant_uncached(const ConvGeom &g, TcVariant v, bool fuse, int planes) {
   switch (v) {
-    case kTcSingle: return make_plan(g, 0, false, fuse);
-    case kTcSingleStream: return make_plan(g, 1, false, fuse);
-    case kTcPair: return make_plan(g, 0, true, fuse);
-    case kTcPairStream: return make_plan(g, 1, true, fuse);
+    case kTcSingle: return make_plan(g, 0, false, fuse, planes);
+    case kTcSingleStream: return make_plan(g, 1, false, fuse, planes);
+    case kTcPair: return make_plan(g, 0, true, fuse, planes);
+    case kTcPairStream: return make_plan(g, 1, true, fuse, planes);
     default: break;
   }
-  Plan single = make_plan(g, 0, false, fuse);
+  Plan single = make_plan(g, 0, false, fuse, planes);
   if (single.ok && single.P.resident) return single;
   // a problem of few items is better spread over single CTAs
   if (single.ok && 2 * single.P.ntiles * single.P.nslabs <= (int)kSms) return single;
-  Plan pair = make_plan(g, 0, true, fuse);
+  Plan pair = make_plan(g, 0, true, fuse, planes);
   if (pair.ok && (pair.P.resident || !single.ok || (pair.P.NT > 64 && pair.P.nsteps >= kLongItem))) return pair;
   return single;
 }
 
-template <bool kRes, bool kPair, bool kFuse>
+template <bool kRes, bool kPair, bool kFuse, bool kTwo = false>
 cudaError_t launch_variant(const Plan &pl, unsigned units, cudaStream_t st) {
-  return launch_kernel(binconv_tc_kernel<kRes, kPair, kFuse>, dim3(kPair ? 2 * units : units), kRes ? kThreadsRes : kThreadsStream, pl.smem, st,
+  return launch_kernel(binconv_tc_kernel<kRes, kPair, kFuse, kTwo>, dim3(kPair ? 2 * units : units), kRes ? kThreadsRes : kThreadsStream, pl.smem, st,
                        kPair ? 2u : 1u, pl.P);
 }
 
@@ -1611,27 +1633,27 @@ cudaError_t launch_variant(const Plan &pl, unsigned units, cudaStream_t st) {
 namespace {
 
 struct PlanKey {
-  int N, C, H, W, Co, kh, kw, stride, pad, variant, fuse;
+  int N, C, H, W, Co, kh, kw, stride, pad, variant, fuse, planes;
   bool operator==(const PlanKey &o) const {
     return N == o.N && C == o.C && H == o.H && W == o.W && Co == o.Co && kh == o.kh && kw == o.kw &&
-           stride == o.stride && pad == o.pad && variant == o.variant && fuse == o.fuse;
+           stride == o.stride && pad == o.pad && variant == o.variant && fuse == o.fuse && planes == o.planes;
   }
 };
 
-Plan plan_variant(const ConvGeom &g, TcVariant v, bool fuse = false) {
+Plan plan_variant(const ConvGeom &g, TcVariant v, bool fuse = false, int planes = 1) {
   constexpr int kSlots = 16;
   static std::mutex mu;
   static PlanKey keys[kSlots];
   static Plan plans[kSlots];
   static bool used[kSlots] = {};
   static int next = 0;
-  const PlanKey key{g.N, g.C, g.H, g.W, g.Co, g.kh, g.kw, g.stride, g.pad, (int)v, fuse ? 1 : 0};
+  const PlanKey key{g.N, g.C, g.H, g.W, g.Co, g.kh, g.kw, g.stride, g.pad, (int)v, fuse ? 1 : 0, planes};
   std::lock_guard<std::mutex> lock(mu);
   for (int i = 0; i < kSlots; ++i)
     if (used[i] && keys[i] == key) return plans[i];
   const int slot = next;
   next = (next + 1) % kSlots;
-  plans[slot] = plan_variant_uncached(g, v, fuse);
+  plans[slot] = plan_variant_uncached(g, v, fuse, planes);
   keys[slot] = key;
   used[slot] = true;
   return plans[slot];
@@ -1639,7 +1661,7 @@ Plan plan_variant(const ConvGeom &g, TcVariant v, bool fuse = false) {
 
 }  // namespace
 
-bool umma_tc_supported(const ConvGeom &g, TcVariant v) { return plan_variant(g, v).ok; }
+bool umma_tc_supported(const ConvGeom &g, TcVariant v, int planes) { return plan_variant(g, v, false, planes).ok; }
 
 namespace {
 
@@ -1648,16 +1670,20 @@ cudaError_t launch_plan(Plan &pl, cudaStream_t st, bool fuse) {
   static bool attr_flags[64] = {};
   bool &attr_set = attr_done_for_current_device(attr_flags);
   if (!attr_set) {
-    const void *kernels[8] = {(const void *)binconv_tc_kernel<false, false, false>,
-                              (const void *)binconv_tc_kernel<true, false, false>,
-                              (const void *)binconv_tc_kernel<false, true, false>,
-                              (const void *)binconv_tc_kernel<true, true, false>,
-                              (const void *)binconv_tc_kernel<false, false, true>,
-                              (const void *)binconv_tc_kernel<true, false, true>,
-                              (const void *)binconv_tc_kernel<false, true, true>,
-                              (const void *)binconv_tc_kernel<true, true, true>};
+    const void *kernels[12] = {(const void *)binconv_tc_kernel<false, false, false, false>,
+                               (const void *)binconv_tc_kernel<true, false, false, false>,
+                               (const void *)binconv_tc_kernel<false, true, false, false>,
+                               (const void *)binconv_tc_kernel<true, true, false, false>,
+                               (const void *)binconv_tc_kernel<false, false, true, false>,
+                               (const void *)binconv_tc_kernel<true, false, true, false>,
+                               (const void *)binconv_tc_kernel<false, true, true, false>,
+                               (const void *)binconv_tc_kernel<true, true, true, false>,
+                               (const void *)binconv_tc_kernel<false, false, false, true>,
+                               (const void *)binconv_tc_kernel<true, false, false, true>,
+                               (const void *)binconv_tc_kernel<false, true, false, true>,
+                               (const void *)binconv_tc_kernel<true, true, false, true>};
     cudaError_t e = cudaSuccess;
-    for (int i = 0; i < 8 && e == cudaSuccess; ++i)
+    for (int i = 0; i < 12 && e == cudaSuccess; ++i)
       e = cudaFuncSetAttribute(kernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)kSmemMax);
     if (e != cudaSuccess) { (void)cudaGetLastError(); return e; }
@@ -1671,6 +1697,9 @@ cudaError_t launch_plan(Plan &pl, cudaStream_t st, bool fuse) {
   if (fuse) {
     if (P.pair) e_ = P.resident ? launch_variant<true, true, true>(pl, units, st) : launch_variant<false, true, true>(pl, units, st);
     else e_ = P.resident ? launch_variant<true, false, true>(pl, units, st) : launch_variant<false, false, true>(pl, units, st);
+  } else if (P.xp2 != nullptr) {
+    if (P.pair) e_ = P.resident ? launch_variant<true, true, false, true>(pl, units, st) : launch_variant<false, true, false, true>(pl, units, st);
+    else e_ = P.resident ? launch_variant<true, false, false, true>(pl, units, st) : launch_variant<false, false, false, true>(pl, units, st);
   } else {
     if (P.pair) e_ = P.resident ? launch_variant<true, true, false>(pl, units, st) : launch_variant<false, true, false>(pl, units, st);
     else e_ = P.resident ? launch_variant<true, false, false>(pl, units, st) : launch_variant<false, false, false>(pl, units, st);
@@ -1684,11 +1713,11 @@ cudaError_t launch_plan(Plan &pl, cudaStream_t st, bool fuse) {
 cudaError_t launch_binconv_tc(const uint32_t *xp, const uint32_t *wp, const float *alpha,
                               const float *K, const float *residual, const ConvGeom &g,
                               const EpiOpts &epi, float *out, int32_t *acc_out, TcVariant variant,
-                              cudaStream_t st) {
-  Plan pl = plan_variant(g, variant);
+                              cudaStream_t st, const uint32_t *xp2) {
+  Plan pl = plan_variant(g, variant, false, xp2 != nullptr ? 2 : 1);
   if (!pl.ok) return cudaErrorInvalidValue;
   TcParams &P = pl.P;
-  P.xp = xp; P.wp = wp; P.alpha = alpha; P.K = K; P.residual = residual;
+  P.xp = xp; P.xp2 = xp2; P.wp = wp; P.alpha = alpha; P.K = K; P.residual = residual;
   P.out = out; P.acc_out = acc_out;
   P.relu = epi.relu; P.out_scale = epi.out_scale; P.acc_shift = epi.acc_shift; P.acc_accum = epi.acc_accum;
   P.nscale = nullptr; P.nshift = nullptr; P.xp_next = nullptr; P.A_part = nullptr; P.Cw_next = 0;
@@ -1711,7 +1740,7 @@ cudaError_t launch_binconv_tc_fused(const uint32_t *xp, const uint32_t *wp, cons
   Plan pl = plan_variant(g, variant, true);
   if (!pl.ok) return cudaErrorInvalidValue;
   TcParams &P = pl.P;
-  P.xp = xp; P.wp = wp; P.alpha = alpha; P.K = K; P.residual = residual;
+  P.xp = xp; P.xp2 = nullptr; P.wp = wp; P.alpha = alpha; P.K = K; P.residual = residual;
   P.out = out; P.acc_out = nullptr;
   P.relu = (g.flags & XNOR_FLAG_RELU) ? 1 : 0; P.out_scale = 1.0f; P.acc_shift = 0; P.acc_accum = 0;
   P.nscale = next_scale; P.nshift = next_shift; P.xp_next = xp_next; P.A_part = A_part;

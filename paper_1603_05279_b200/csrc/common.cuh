@@ -137,11 +137,12 @@ inline int sm_count_of_current_device() {
 // (one MMA drives two SMs), each with the filters of a slab resident in shared memory when
 // they fit or always streamed through a ring (re-expanded per work item).
 enum TcVariant { kTcAuto = 0, kTcSingle, kTcSingleStream, kTcPair, kTcPairStream };
-bool umma_tc_supported(const ConvGeom &g, TcVariant v);
+// planes: bit planes of the input that one pass takes, 1 or 2
+bool umma_tc_supported(const ConvGeom &g, TcVariant v, int planes = 1);
 cudaError_t launch_binconv_tc(const uint32_t *xp, const uint32_t *wp, const float *alpha,
                               const float *K, const float *residual, const ConvGeom &g,
                               const EpiOpts &epi, float *out, int32_t *acc_out, TcVariant v,
-                              cudaStream_t st);
+                              cudaStream_t st, const uint32_t *xp2 = nullptr);
 // BinConv with the next layer's BinActiv fused into its epilogue (sign bits packed along the
 // filters, partial sums of |y| per filter slab and epilogue warp); tc_fused_parts = number of
 // partial planes for the shape (0: the fused kernel does not cover it).
