@@ -237,7 +237,8 @@ xnor_status xnor_conv2d_forward(const uint32_t *x_packed, const uint32_t *w_pack
  *                  for kbits = 1 the one plane is xnor_binactiv's x_packed.
  * xnor_conv2d_forward_kbit is xnor_conv2d_forward on those planes:
  *   out = (q_k(I) (*) sign(W)) (.) K alpha (+ residual), one pass of the binary
- *   convolution per plane, each adding D_p K alpha 2^p/(2^k - 1) to the output;
+ *   convolution per two planes (CUDA-core engine: per plane), the pass from plane
+ *   p on adding D K alpha 2^p/(2^k - 1) to the output;
  *   acc_out (nullable) receives the exact integer sum over level codes,
  *   sum_p 2^p D_p = (2^k - 1) (q_k(I) (*) sign(W)).
  * 1 <= kbits <= 7 (INVALID_ARG otherwise); other errors as for the 1-bit calls;

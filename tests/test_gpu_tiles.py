@@ -8,6 +8,7 @@ import torch
 import paper_1603_05279_b200 as X
 from test_gpu_bgrad import test_binary_gradient_backward_parity as backward_parity
 from test_gpu_options import _index_of_planes
+from test_gpu_options import test_kbit_block_parity as kbit_block_parity
 from util import GuardSet, assert_close, dev, host
 
 pytestmark = pytest.mark.gpu
@@ -85,6 +86,15 @@ def test_wide_pack(oracle, case, kbits):
 @pytest.mark.parametrize("shape", [(75, 33, 5, 5, 17, 3, 1), (74, 32, 21, 19, 101, 3, 1)])
 def test_gradient_maximum_of_many_images(oracle, shape):
     backward_parity(oracle, shape)
+
+
+# two bit planes per pass in every schedule, an even and an odd number of passes; channel tails, both phases
+@pytest.mark.parametrize("engine", [X.XNOR_ENGINE_UMMA_SINGLE, X.XNOR_ENGINE_UMMA_STREAM, X.XNOR_ENGINE_UMMA_PAIR,
+                                    X.XNOR_ENGINE_UMMA_PAIR_STREAM])
+@pytest.mark.parametrize("kbits", [2, 4, 5])
+@pytest.mark.parametrize("shape", [(16, 70, 19, 18, 64, 3, 2, 1), (12, 128, 20, 21, 160, 3, 1, 1), (4, 33, 8, 8, 16, 1, 1, 0)])
+def test_kbit_two_planes_per_pass(oracle, shape, kbits, engine):
+    kbit_block_parity(oracle, shape, kbits, engine)
 
 
 @pytest.mark.parametrize("valid", [False, True])
