@@ -464,15 +464,17 @@ __device__ void mma_resident(const TcParams &P, const Smem &S, uint32_t tmem_bas
         const uint32_t first = st == 0 ? 0u : 1u;     // the first MMA of an item overwrites
         if (!mbar_wait(S.wfull + 8u * st, 0u, S.abort_flag, &g_status_tc)) return;
         tc_fence_after();
-        if (nj > 8 && (nj & 3) == 0) {            // small problems (see make_plan)
-          for (int jj = 0; jj < nj; jj += 4)
-            issue_stage<4, kPair>(P, j0 + jj, d_tmem, patch_lo, desc_hi, b_lo + (uint32_t)jj * b_step, desc_hi, b_step, tmem_sf,
-                                  jj == 0 ? first : 1u);
-        } else if (nj == 4) issue_stage<4, kPair>(P, j0, d_tmem, patch_lo, desc_hi, b_lo, desc_hi, b_step, tmem_sf, first);
+        if (nj == 4) issue_stage<4, kPair>(P, j0, d_tmem, patch_lo, desc_hi, b_lo, desc_hi, b_step, tmem_sf, first);
         else if (nj == 2) issue_stage<2, kPair>(P, j0, d_tmem, patch_lo, desc_hi, b_lo, desc_hi, b_step, tmem_sf, first);
         else if (nj == 8) issue_stage<8, kPair>(P, j0, d_tmem, patch_lo, desc_hi, b_lo, desc_hi, b_step, tmem_sf, first);
         else {
-          for (int jj = 0; jj < nj; ++jj)
+          int jj = 0;
+#pragma unroll 1
+          for (; jj + 4 <= nj; jj += 4)              // the large steps of a small problem (see make_plan)
+            issue_stage<4, kPair>(P, j0 + jj, d_tmem, patch_lo, desc_hi, b_lo + (uint32_t)jj * b_step, desc_hi, b_step, tmem_sf,
+                                  jj == 0 ? first : 1u);
+#pragma unroll 1
+          for (; jj < nj; ++jj)
             umma_issue<kPair>(d_tmem, P.adesc_lo[j0 + jj] + patch_lo, desc_hi,
                               b_lo + (uint32_t)jj * b_step, desc_hi, P.idesc, tmem_sf,
                               jj == 0 ? first : 1u);
