@@ -587,8 +587,8 @@ struct WCursor {
 // path without per-step predicates.
 // The role fills the stages of `nitems` consecutive items, the first of slab `slab0` (the
 // slabs then follow cyclically), waiting for the empty barriers with parity `wph0` on the
-// first round.  Streaming: all items of the CTA in one call.  Resident: one call per slab
-// visit with nitems = 1 (the ring then has one stage per stage of the slab).
+// first round: one call per slab visit with nitems = 1 (the ring has one stage per stage of
+// the slab).
 template <int kUnits, bool kSwap>
 __device__ bool weight_role(const TcParams &P, const Smem &S, long long nitems, int slab0,
                             uint32_t wph0, int wt, int lane) {
