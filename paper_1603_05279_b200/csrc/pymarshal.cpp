@@ -4,6 +4,7 @@
 // through this module about 1 us.  The entry points are called by address (bind()), so the module
 // works with whichever build of the library the Python side has loaded.
 #define PY_SSIZE_T_CLEAN
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 #include <c10/cuda/CUDAStream.h>
 
@@ -95,13 +96,7 @@ struct Args {
   void *stream() {
     PyObject *o = a[i++];
     if (!ok) return nullptr;
-    try {
-      if (o == Py_None) return (void *)c10::cuda::getCurrentCUDAStream().stream();
-    } catch (const std::exception &e) {
-      PyErr_SetString(PyExc_RuntimeError, e.what());
-      ok = false;
-      return nullptr;
-    }
+    if (o == Py_None) return (void *)c10::cuda::getCurrentCUDAStream().stream();
     PyObject *v = PyObject_GetAttrString(o, "cuda_stream");
     if (v == nullptr) { PyErr_Clear(); v = Py_NewRef(o); }
     void *s = PyLong_AsVoidPtr(v);
@@ -122,8 +117,7 @@ PyObject *finish(const Args &A, F &&call) {
   return PyLong_FromLong((long)s);
 }
 
-// Sizes of a contiguous tensor argument of `dims` dimensions (0 when it is not one: the pointer
-// conversion or the library then reports the error).
+// Sizes of a tensor argument of `dims` dimensions; anything else is an error.
 void sizes_of(Args &A, PyObject *o, int dims, int *out) {
   if (!A.ok) return;
   if (!THPVariable_Check(o) || THPVariable_Unpack(o).dim() != dims) {
@@ -135,7 +129,16 @@ void sizes_of(Args &A, PyObject *o, int dims, int *out) {
   for (int i = 0; i < dims; ++i) out[i] = (int)t.size(i);
 }
 
-#define XNOR_PY(name) PyObject *name(PyObject *, PyObject *const *args, Py_ssize_t nargs)
+// Torch's accessors throw (a tensor under vmap has no data pointer, one with symbolic sizes no size): an
+// exception must become a Python error before it reaches the interpreter, which is C.
+template <PyObject *(*kCall)(PyObject *const *, Py_ssize_t)>
+PyObject *entry(PyObject *, PyObject *const *args, Py_ssize_t nargs) {
+  HANDLE_TH_ERRORS
+  return kCall(args, nargs);
+  END_HANDLE_TH_ERRORS
+}
+
+#define XNOR_PY(name) PyObject *name(PyObject *const *args, Py_ssize_t nargs)
 
 XNOR_PY(binarize_weights) {          // w, w_packed, alpha, stream
   Args A(args, nargs, 4);
@@ -268,7 +271,7 @@ PyObject *bind(PyObject *, PyObject *seq) {
   Py_RETURN_NONE;
 }
 
-#define XNOR_FAST(name) {#name, (PyCFunction)(void (*)(void))name, METH_FASTCALL, nullptr}
+#define XNOR_FAST(name) {#name, (PyCFunction)(void (*)(void))entry<name>, METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {
     {"bind", bind, METH_O, nullptr},
     XNOR_FAST(binarize_weights), XNOR_FAST(binactiv), XNOR_FAST(conv2d_forward), XNOR_FAST(shortcut_conv1x1),
