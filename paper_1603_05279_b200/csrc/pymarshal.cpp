@@ -92,14 +92,21 @@ struct Args {
     PyBuffer_Release(&b);
     return d;
   }
-  // None: torch's current stream; else a torch stream or a raw cudaStream_t
+  // None: torch's current stream; else a torch stream, or a raw cudaStream_t as anything int() takes
   void *stream() {
     PyObject *o = a[i++];
     if (!ok) return nullptr;
     if (o == Py_None) return (void *)c10::cuda::getCurrentCUDAStream().stream();
     PyObject *v = PyObject_GetAttrString(o, "cuda_stream");
-    if (v == nullptr) { PyErr_Clear(); v = Py_NewRef(o); }
-    void *s = PyLong_AsVoidPtr(v);
+    if (v == nullptr && PyErr_ExceptionMatches(PyExc_AttributeError)) {
+      PyErr_Clear();
+      v = PyNumber_Long(o);
+    }
+    ok = v != nullptr;
+    if (!ok) return nullptr;
+    void *s = nullptr;
+    if (PyLong_Check(v)) s = PyLong_AsVoidPtr(v);
+    else PyErr_Format(PyExc_TypeError, "expected a stream, got %S", (PyObject *)Py_TYPE(o));
     Py_DECREF(v);
     if (s == nullptr && PyErr_Occurred()) ok = false;
     return s;

@@ -27,9 +27,20 @@ def raises(kind, call):
 """
 
 
-def run_child(body):
+# xnor_binarize_weights_transposed replaced by a function that records what the native module passes.
+RECORD = """
+seen = []
+vp, ci = ctypes.c_void_p, ctypes.c_int
+entry = ctypes.CFUNCTYPE(ci, vp, ci, ci, ci, ci, vp, vp)(lambda *a: seen.append(a) or 0)
+addresses = [ctypes.cast(getattr(X.load(), "xnor_" + n), vp).value for n in B._MARSHALLED]
+addresses[B._MARSHALLED.index("binarize_weights_transposed")] = ctypes.cast(entry, vp).value
+B._m.bind(addresses)
+"""
+
+
+def run_child(body, prelude=PRELUDE):
     """In a process of its own: what is tested for is that the interpreter survives."""
-    code = PRELUDE + "with FakeTensorMode(allow_non_fake_inputs=True):\n" + \
+    code = prelude + "with FakeTensorMode(allow_non_fake_inputs=True):\n" + \
         "".join("    %s\n" % line for line in body.strip().splitlines())
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, (r.returncode, r.stdout[-500:], r.stderr[-2000:])
@@ -51,3 +62,23 @@ raises(RuntimeError, lambda: torch.vmap(f)(fake(5, 4, 3)))
 ], ids=["pointer", "size"])
 def test_torch_exceptions_reach_python(body):
     run_child(body)
+
+
+def test_stream_arguments():
+    """A torch stream or what int() takes (cuda-python's handles, numpy's integers); an attribute that
+    fails for another reason than being absent is reported as it is."""
+    run_child("""
+import numpy
+class Torch: cuda_stream = 0x7000
+class Handle:
+    def __int__(self): return 0x8000
+class Broken:
+    @property
+    def cuda_stream(self): raise RuntimeError("lost")
+a, p, al = args()
+for s in (Torch(), Handle(), numpy.int64(0x9000), 0xA000, 0): X.xnor_binarize_weights_transposed(a, p, stream=s)
+assert [x[-1] for x in seen] == [0x7000, 0x8000, 0x9000, 0xA000, None], seen
+raises(RuntimeError, lambda: X.xnor_binarize_weights_transposed(a, p, stream=Broken()))
+raises(TypeError, lambda: X.xnor_binarize_weights_transposed(a, p, stream=object()))
+assert len(seen) == 5
+""", PRELUDE + RECORD)
