@@ -150,7 +150,7 @@ def load():
     except ImportError as e:
         raise ImportError("_pymarshal.so is not built: run `python -m paper_1603_05279_b200.build` "
                           "(%s)" % e) from e
-    _pymarshal.bind([ctypes.cast(getattr(lib, "xnor_" + n), vp).value for n in _MARSHALLED])
+    _pymarshal.bind([ctypes.cast(getattr(lib, "xnor_" + n), vp).value for n in _MARSHALLED], xnor_conv_desc)
     _lib, _m = lib, _pymarshal
     return lib
 

@@ -8,6 +8,9 @@
 #include <torch/csrc/autograd/python_variable.h>
 #include <c10/cuda/CUDAStream.h>
 
+#include <algorithm>
+#include <cstring>
+
 #include "xnor.h"
 
 namespace {
@@ -29,6 +32,7 @@ struct Entry {
   decltype(&xnor_binary_gradient_backward) binary_gradient_backward;
 } E;
 constexpr Py_ssize_t kEntries = sizeof(Entry) / sizeof(void *);
+PyObject *desc_type = nullptr;         // the ctypes structure xnor_conv_desc
 
 // Arguments of one call, converted in order; the first failure sets a Python error and sticks.
 struct Args {
@@ -80,15 +84,16 @@ struct Args {
     else if (v != (long)(int)v) { PyErr_SetString(PyExc_OverflowError, "argument out of int range"); ok = false; }
     return (int)v;
   }
-  // the ctypes structure xnor_conv_desc, read through the buffer protocol
+  // an xnor_conv_desc and nothing else of its size, read through the buffer protocol
   xnor_conv_desc desc() {
     xnor_conv_desc d = {};
     PyObject *o = a[i++];
     if (!ok) return d;
     Py_buffer b;
-    if (PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) != 0) { ok = false; return d; }
-    if (b.len == (Py_ssize_t)sizeof(d)) d = *(const xnor_conv_desc *)b.buf;
-    else { PyErr_SetString(PyExc_TypeError, "expected an xnor_conv_desc"); ok = false; }
+    const int is = PyObject_IsInstance(o, desc_type);
+    if (is == 0) PyErr_Format(PyExc_TypeError, "expected an xnor_conv_desc, got %S", (PyObject *)Py_TYPE(o));
+    if (is != 1 || PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) != 0) { ok = false; return d; }
+    memcpy(&d, b.buf, std::min((size_t)b.len, sizeof(d)));
     PyBuffer_Release(&b);
     return d;
   }
@@ -261,9 +266,11 @@ XNOR_PY(binary_gradient_backward) {  // g, wT_packed, alpha, d, gmax, g_stream, 
   return finish(A, [&] { return E.binary_gradient_backward(g, wT, al, &d, gm, gs, gi, st); });
 }
 
-// bind(addresses): the entry points' addresses, in the order of struct Entry
-PyObject *bind(PyObject *, PyObject *seq) {
-  PyObject *t = PySequence_Tuple(seq);
+// bind(addresses, descriptor): the entry points' addresses, in the order of struct Entry, and the
+// descriptor's class
+PyObject *bind(PyObject *, PyObject *const *args, Py_ssize_t nargs) {
+  if (nargs != 2) return PyErr_Format(PyExc_TypeError, "expected 2 arguments, got %zd", nargs);
+  PyObject *t = PySequence_Tuple(args[0]);
   if (t == nullptr) return nullptr;
   void *p[kEntries];
   bool ok = PyTuple_GET_SIZE(t) == kEntries;
@@ -275,12 +282,13 @@ PyObject *bind(PyObject *, PyObject *seq) {
   Py_DECREF(t);
   if (!ok) return nullptr;
   memcpy((void *)&E, p, sizeof(E));
+  Py_XSETREF(desc_type, Py_NewRef(args[1]));
   Py_RETURN_NONE;
 }
 
 #define XNOR_FAST(name) {#name, (PyCFunction)(void (*)(void))entry<name>, METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {
-    {"bind", bind, METH_O, nullptr},
+    {"bind", (PyCFunction)(void (*)(void))bind, METH_FASTCALL, nullptr},
     XNOR_FAST(binarize_weights), XNOR_FAST(binactiv), XNOR_FAST(conv2d_forward), XNOR_FAST(shortcut_conv1x1),
     XNOR_FAST(conv2d_forward_binactiv), XNOR_FAST(binactiv_finish), XNOR_FAST(maxpool2d), XNOR_FAST(binactiv_kbit),
     XNOR_FAST(conv2d_forward_kbit), XNOR_FAST(bwn_prepare_input), XNOR_FAST(bwn_conv2d_forward),

@@ -34,7 +34,7 @@ vp, ci = ctypes.c_void_p, ctypes.c_int
 entry = ctypes.CFUNCTYPE(ci, vp, ci, ci, ci, ci, vp, vp)(lambda *a: seen.append(a) or 0)
 addresses = [ctypes.cast(getattr(X.load(), "xnor_" + n), vp).value for n in B._MARSHALLED]
 addresses[B._MARSHALLED.index("binarize_weights_transposed")] = ctypes.cast(entry, vp).value
-B._m.bind(addresses)
+B._m.bind(addresses, X.xnor_conv_desc)
 """
 
 
@@ -82,3 +82,15 @@ raises(RuntimeError, lambda: X.xnor_binarize_weights_transposed(a, p, stream=Bro
 raises(TypeError, lambda: X.xnor_binarize_weights_transposed(a, p, stream=object()))
 assert len(seen) == 5
 """, PRELUDE + RECORD)
+
+
+def test_descriptor_arguments():
+    """An xnor_conv_desc (or a subclass): not another structure, or bytes, of its size."""
+    run_child("""
+class Other(ctypes.Structure): _fields_ = X.xnor_conv_desc._fields_
+class Derived(X.xnor_conv_desc): pass
+d = X.make_desc(1, 8, 5, 5, 4, 3, 3, 1, 1)
+call = lambda d: X.xnor_binactiv(fake(1, 8, 5, 5), None, None, d, fake(25, dtype=torch.int32), fake(25), fake(25), stream=0)
+for bad in (bytes(d), bytearray(bytes(d)), Other(), None, 3): raises(TypeError, lambda: call(bad))
+raises(X.XnorError, lambda: call(Derived()))                 # converted; the library refuses its zeros
+""")
