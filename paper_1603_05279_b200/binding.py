@@ -150,7 +150,8 @@ def load():
     except ImportError as e:
         raise ImportError("_pymarshal.so is not built: run `python -m paper_1603_05279_b200.build` "
                           "(%s)" % e) from e
-    _pymarshal.bind([ctypes.cast(getattr(lib, "xnor_" + n), vp).value for n in _MARSHALLED], xnor_conv_desc)
+    _pymarshal.bind([ctypes.cast(getattr(lib, "xnor_" + n), vp).value for n in _MARSHALLED], xnor_conv_desc,
+                    _address)
     _lib, _m = lib, _pymarshal
     return lib
 
@@ -165,6 +166,11 @@ def _ptr(t, dtype=None):
     if dtype is not None and t.dtype != dtype:
         raise ValueError("expected %s, got %s" % (dtype, t.dtype))
     return ctypes.c_void_p(t.data_ptr())
+
+
+def _address(t, dtype):
+    """For the native module: the address of what is not exactly a tensor, by its Python attributes."""
+    return _ptr(t, getattr(torch, dtype)).value or 0
 
 
 def _stream(stream):

@@ -10,6 +10,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <string>
 
 #include "xnor.h"
 
@@ -33,6 +34,7 @@ struct Entry {
 } E;
 constexpr Py_ssize_t kEntries = sizeof(Entry) / sizeof(void *);
 PyObject *desc_type = nullptr;         // the ctypes structure xnor_conv_desc
+PyObject *py_address = nullptr;        // (object, type name) -> its checked address through Python attributes
 
 // Arguments of one call, converted in order; the first failure sets a Python error and sticks.
 struct Args {
@@ -51,13 +53,17 @@ struct Args {
     }
     ok = false;
   }
-  void *ptr(at::ScalarType type, const char *wrong_type) {
+  // Tensors and parameters are read here.  Subclasses and other objects with a tensor's attributes may
+  // define these in Python, so they are asked there.
+  void *ptr(at::ScalarType type, const char *name) {
     PyObject *o = a[i++];
     if (!ok || o == Py_None) return nullptr;
-    if (!THPVariable_Check(o)) {
-      PyErr_Format(PyExc_TypeError, "expected a tensor, got %S", (PyObject *)Py_TYPE(o));
-      ok = false;
-      return nullptr;
+    if (!THPVariable_CheckExact(o)) {
+      PyObject *v = PyObject_CallFunction(py_address, "Os", o, name);
+      void *p = v != nullptr ? PyLong_AsVoidPtr(v) : nullptr;
+      Py_XDECREF(v);
+      ok = !PyErr_Occurred();
+      return p;
     }
     const at::Tensor &t = THPVariable_Unpack(o);
     if (!t.is_cuda()) {
@@ -66,16 +72,17 @@ struct Args {
       PyErr_SetString(PyExc_ValueError, "tensor must be contiguous");
       ok = false;
     } else if (t.scalar_type() != type) {
-      fail_attr(wrong_type, o, "dtype");
+      const std::string fmt = std::string("expected torch.") + name + ", got %S";
+      fail_attr(fmt.c_str(), o, "dtype");
     } else {
       return t.data_ptr();
     }
     return nullptr;
   }
-  float *f32() { return (float *)ptr(at::kFloat, "expected torch.float32, got %S"); }
-  uint32_t *u32() { return (uint32_t *)ptr(at::kInt, "expected torch.int32, got %S"); }
-  int32_t *i32() { return (int32_t *)ptr(at::kInt, "expected torch.int32, got %S"); }
-  uint16_t *bf16() { return (uint16_t *)ptr(at::kBFloat16, "expected torch.bfloat16, got %S"); }
+  float *f32() { return (float *)ptr(at::kFloat, "float32"); }
+  uint32_t *u32() { return (uint32_t *)ptr(at::kInt, "int32"); }
+  int32_t *i32() { return (int32_t *)ptr(at::kInt, "int32"); }
+  uint16_t *bf16() { return (uint16_t *)ptr(at::kBFloat16, "bfloat16"); }
   int num() {
     PyObject *o = a[i++];
     if (!ok) return 0;
@@ -129,16 +136,23 @@ PyObject *finish(const Args &A, F &&call) {
   return PyLong_FromLong((long)s);
 }
 
-// Sizes of a tensor argument of `dims` dimensions; anything else is an error.
+// Sizes of a tensor argument of `dims` dimensions (0: any number, the first size); anything else is an error.
 void sizes_of(Args &A, PyObject *o, int dims, int *out) {
   if (!A.ok) return;
-  if (!THPVariable_Check(o) || THPVariable_Unpack(o).dim() != dims) {
-    PyErr_Format(PyExc_ValueError, "expected a tensor of %d dimensions", dims);
-    A.ok = false;
-    return;
+  const int want = dims > 0 ? dims : 1;
+  if (THPVariable_CheckExact(o)) {
+    const at::Tensor &t = THPVariable_Unpack(o);
+    A.ok = dims > 0 ? t.dim() == dims : t.dim() > 0;
+    for (int i = 0; A.ok && i < want; ++i) out[i] = (int)t.size(i);
+  } else {
+    PyObject *shape = PyObject_GetAttrString(o, "shape"), *s = shape != nullptr ? PySequence_Tuple(shape) : nullptr;
+    Py_XDECREF(shape);
+    if (s != nullptr) A.ok = dims > 0 ? PyTuple_GET_SIZE(s) == dims : PyTuple_GET_SIZE(s) > 0;
+    for (int i = 0; s != nullptr && A.ok && i < want; ++i) out[i] = (int)PyLong_AsLong(PyTuple_GET_ITEM(s, i));
+    Py_XDECREF(s);
+    if (PyErr_Occurred()) { A.ok = false; return; }
   }
-  const at::Tensor &t = THPVariable_Unpack(o);
-  for (int i = 0; i < dims; ++i) out[i] = (int)t.size(i);
+  if (!A.ok) PyErr_Format(PyExc_ValueError, "expected a tensor of %d dimensions", want);
 }
 
 // Torch's accessors throw (a tensor under vmap has no data pointer, one with symbolic sizes no size): an
@@ -226,8 +240,8 @@ XNOR_PY(shortcut_conv1x1) {          // x, w, stride, out, stream
   if (A.ok) sizes_of(A, args[0], 4, z);
   if (!A.ok) return nullptr;
   const float *x = A.f32(), *w = A.f32(); const int s = A.num(); float *out = A.f32(); void *st = A.stream();
-  // filters are [C_out][C_in] or [C_out][C_in][1][1]
-  const int co = A.ok && w && THPVariable_Unpack(args[1]).dim() > 0 ? (int)THPVariable_Unpack(args[1]).size(0) : 0;
+  int co = 0;                        // filters are [C_out][C_in] or [C_out][C_in][1][1]
+  if (args[1] != Py_None) sizes_of(A, args[1], 0, &co);
   return finish(A, [&] { return E.shortcut_conv1x1(x, w, z[0], z[1], z[2], z[3], co, s, out, st); });
 }
 
@@ -266,10 +280,10 @@ XNOR_PY(binary_gradient_backward) {  // g, wT_packed, alpha, d, gmax, g_stream, 
   return finish(A, [&] { return E.binary_gradient_backward(g, wT, al, &d, gm, gs, gi, st); });
 }
 
-// bind(addresses, descriptor): the entry points' addresses, in the order of struct Entry, and the
-// descriptor's class
+// bind(addresses, descriptor, address): the entry points' addresses, in the order of struct Entry, the
+// descriptor's class, and the Python conversion of what is not exactly a tensor
 PyObject *bind(PyObject *, PyObject *const *args, Py_ssize_t nargs) {
-  if (nargs != 2) return PyErr_Format(PyExc_TypeError, "expected 2 arguments, got %zd", nargs);
+  if (nargs != 3) return PyErr_Format(PyExc_TypeError, "expected 3 arguments, got %zd", nargs);
   PyObject *t = PySequence_Tuple(args[0]);
   if (t == nullptr) return nullptr;
   void *p[kEntries];
@@ -283,6 +297,7 @@ PyObject *bind(PyObject *, PyObject *const *args, Py_ssize_t nargs) {
   if (!ok) return nullptr;
   memcpy((void *)&E, p, sizeof(E));
   Py_XSETREF(desc_type, Py_NewRef(args[1]));
+  Py_XSETREF(py_address, Py_NewRef(args[2]));
   Py_RETURN_NONE;
 }
 

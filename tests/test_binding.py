@@ -14,6 +14,7 @@ import paper_1603_05279_b200 as X
 from paper_1603_05279_b200 import binding as B
 from torch._subclasses.fake_tensor import FakeTensorMode
 X.load()
+real = torch.zeros(4, 4, 3, 3)
 fake = lambda *s, dtype=torch.float32: torch.empty(s, device="cuda", dtype=dtype)
 w, wp, al = (4, 4, 3, 3), (9, 4, 2), (4,)
 def args():
@@ -34,7 +35,7 @@ vp, ci = ctypes.c_void_p, ctypes.c_int
 entry = ctypes.CFUNCTYPE(ci, vp, ci, ci, ci, ci, vp, vp)(lambda *a: seen.append(a) or 0)
 addresses = [ctypes.cast(getattr(X.load(), "xnor_" + n), vp).value for n in B._MARSHALLED]
 addresses[B._MARSHALLED.index("binarize_weights_transposed")] = ctypes.cast(entry, vp).value
-B._m.bind(addresses, X.xnor_conv_desc)
+B._m.bind(addresses, X.xnor_conv_desc, B._address)
 """
 
 
@@ -94,3 +95,23 @@ call = lambda d: X.xnor_binactiv(fake(1, 8, 5, 5), None, None, d, fake(25, dtype
 for bad in (bytes(d), bytearray(bytes(d)), Other(), None, 3): raises(TypeError, lambda: call(bad))
 raises(X.XnorError, lambda: call(Derived()))                 # converted; the library refuses its zeros
 """)
+
+
+def test_tensor_subclasses_and_lookalikes():
+    """What a subclass, or an object with a tensor's attributes, says of itself counts."""
+    run_child("""
+class Sub(torch.Tensor):
+    is_cuda = True
+    def data_ptr(self): return 0x1000
+class Like:
+    is_cuda, dtype, device, shape = True, torch.int32, "cuda", (9, 4, 2)
+    def is_contiguous(self): return True
+    def data_ptr(self): return 0x2000
+sub = real.as_subclass(Sub)
+X.xnor_binarize_weights_transposed(sub, Like(), stream=0)
+assert seen == [(0x1000, 4, 4, 3, 3, 0x2000, None)], seen
+raises(ValueError, lambda: X.xnor_binarize_weights_transposed(Like(), sub, stream=0))       # three dimensions
+raises(ValueError, lambda: X.xnor_binarize_weights_transposed(sub, sub, stream=0))          # not int32
+raises(AttributeError, lambda: X.xnor_binarize_weights_transposed(sub, 3, stream=0))
+raises(AttributeError, lambda: X.xnor_binarize_weights_transposed(None, Like(), stream=0))
+""", PRELUDE + RECORD)
