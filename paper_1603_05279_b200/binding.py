@@ -152,7 +152,7 @@ def load():
                           "(%s)" % e) from e
     _pymarshal.bind([ctypes.cast(getattr(lib, "xnor_" + n), vp).value for n in _MARSHALLED], xnor_conv_desc,
                     _address)
-    _lib, _m = lib, _pymarshal
+    _m, _lib = _pymarshal, lib       # in this order: another thread that sees _lib goes on to use _m
     return lib
 
 

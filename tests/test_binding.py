@@ -115,3 +115,20 @@ raises(ValueError, lambda: X.xnor_binarize_weights_transposed(sub, sub, stream=0
 raises(AttributeError, lambda: X.xnor_binarize_weights_transposed(sub, 3, stream=0))
 raises(AttributeError, lambda: X.xnor_binarize_weights_transposed(None, Like(), stream=0))
 """, PRELUDE + RECORD)
+
+
+def test_load_order():
+    """After any instruction of load(), a thread that finds the library loaded finds the native module too."""
+    run_child("""
+B._lib, B._m = None, B._Unloaded()
+states = set()
+def watch(frame, event, arg):
+    if frame.f_code is not B.load.__code__: return None
+    frame.f_trace_opcodes = True
+    states.add((B._lib is not None, not isinstance(B._m, B._Unloaded)))
+    return watch
+sys.settrace(watch)
+X.load()
+sys.settrace(None)
+assert (True, True) in states and (False, False) in states and (True, False) not in states, states
+""")
