@@ -124,7 +124,9 @@ B._lib, B._m = None, B._Unloaded()
 states = set()
 def watch(frame, event, arg):
     if frame.f_code is not B.load.__code__: return None
-    frame.f_trace_opcodes = True
+    if event == "call":
+        frame.f_trace_opcodes = True
+        sys.settrace(watch)                  # Python 3.12 instruments the instructions from here on
     states.add((B._lib is not None, not isinstance(B._m, B._Unloaded)))
     return watch
 sys.settrace(watch)
