@@ -30,12 +30,12 @@ __device__ __forceinline__ float block_abs_max(const float *gi, size_t per_image
     const size_t n4 = per_image / 4;
     size_t i = first;
     for (; i + 3 * step < n4; i += 4 * step) {
-      const float4 a = __ldg(g4 + i), b = __ldg(g4 + i + step), c = __ldg(g4 + i + 2 * step), d = __ldg(g4 + i + 3 * step);
+      const float4 a = load_global(g4 + i), b = load_global(g4 + i + step), c = load_global(g4 + i + 2 * step), d = load_global(g4 + i + 3 * step);
       m = fmaxf(m, fmaxf(fmaxf(abs_max4(a), abs_max4(b)), fmaxf(abs_max4(c), abs_max4(d))));
     }
-    for (; i < n4; i += step) m = fmaxf(m, abs_max4(__ldg(g4 + i)));
+    for (; i < n4; i += step) m = fmaxf(m, abs_max4(load_global(g4 + i)));
   } else {
-    for (size_t i = first; i < per_image; i += step) m = fmaxf(m, fabsf(__ldg(gi + i)));
+    for (size_t i = first; i < per_image; i += step) m = fmaxf(m, fabsf(load_global(gi + i)));
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -48,7 +48,7 @@ __device__ __forceinline__ float block_abs_max(const float *gi, size_t per_image
 }
 
 __global__ void __launch_bounds__(kMaxThreads)
-grad_max_kernel(const float *__restrict__ g, size_t per_image, int vec4, float *__restrict__ gmax) {
+grad_max_kernel(const float *g, size_t per_image, int vec4, float *__restrict__ gmax) {
   stream_order();
   const float m = block_abs_max(g + (size_t)blockIdx.y * per_image, per_image, vec4, blockIdx.x, gridDim.x);
   if (threadIdx.x == 0) atomicMax(reinterpret_cast<unsigned int *>(gmax) + blockIdx.y, __float_as_uint(m));
@@ -58,7 +58,7 @@ grad_max_kernel(const float *__restrict__ g, size_t per_image, int vec4, float *
 // the N values cost 1.3 us and the overlap with the kernel before) nor atomics.  Bound by HBM; the whole
 // backward call at 128 channels, 28x28, 128 images: 67.7 -> 62.4 us with it and the wider preparation.
 __global__ void __launch_bounds__(kMaxThreads)
-grad_max_cluster_kernel(const float *__restrict__ g, size_t per_image, int vec4, float *__restrict__ gmax) {
+grad_max_cluster_kernel(const float *g, size_t per_image, int vec4, float *__restrict__ gmax) {
   __shared__ float part[kMaxCluster];
   stream_order();
   const float m = block_abs_max(g + (size_t)blockIdx.y * per_image, per_image, vec4, blockIdx.x, kMaxCluster);
@@ -78,7 +78,7 @@ grad_max_cluster_kernel(const float *__restrict__ g, size_t per_image, int vec4,
 
 // One warp per packed word: lane = channel co of the word, the word is a ballot.
 __global__ void __launch_bounds__(256)
-binarize_weights_transposed_kernel(const float *__restrict__ w, int Co, int C, int kh, int kw,
+binarize_weights_transposed_kernel(const float *w, int Co, int C, int kh, int kw,
                                    int CwT, uint32_t *__restrict__ wT_packed) {
   stream_order();
   const int lane = threadIdx.x & 31;
@@ -92,7 +92,7 @@ binarize_weights_transposed_kernel(const float *__restrict__ w, int Co, int C, i
       const int ky = tap / kw, kx = tap - ky * kw;
       const int co = cw * 32 + lane;
       const bool in = co < Co;
-      const float v = in ? __ldg(w + (((size_t)co * C + ci) * kh + (kh - 1 - ky)) * kw + (kw - 1 - kx)) : -1.0f;
+      const float v = in ? load_global(w + (((size_t)co * C + ci) * kh + (kh - 1 - ky)) * kw + (kw - 1 - kx)) : -1.0f;
       word = __ballot_sync(0xffffffffu, in && v >= 0.0f);
     }
     if (lane == 0) wT_packed[packed_weight_index(C, ci, f)] = word;

@@ -38,8 +38,8 @@ __host__ __device__ constexpr float decision_point(int j, int kbits) {
 // activations" below.  x_packed is then [kbits][N][H][W][Cw].
 template <bool kHasBN, bool kVec16, int kBits>
 __global__ void __launch_bounds__(32 * kWarps)
-binactiv_pack_kernel(const float *__restrict__ x, const float *__restrict__ scale,
-                     const float *__restrict__ shift, long long total_pix, int C, int HW, int Cw,
+binactiv_pack_kernel(const float *x, const float *scale,
+                     const float *shift, long long total_pix, int C, int HW, int Cw,
                      int G, int PG, int kbits, uint32_t *__restrict__ x_packed, float *__restrict__ A) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   const int nplanes = kBits > 0 ? kBits : kbits;
@@ -59,7 +59,7 @@ binactiv_pack_kernel(const float *__restrict__ x, const float *__restrict__ scal
   stream_order();
   if (kHasBN) {
     for (int c = threadIdx.x; c < Cw * 32; c += 32 * kWarps)
-      bn[c] = c < C ? make_float2(__ldg(scale + c), __ldg(shift + c)) : make_float2(0.0f, 0.0f);
+      bn[c] = c < C ? make_float2(load_global(scale + c), load_global(shift + c)) : make_float2(0.0f, 0.0f);
   }
   __syncthreads();
 
@@ -255,7 +255,7 @@ constexpr int kWideWarps = 12, kWideDepth = 4;
 
 template <bool kHasBN, int kBits>
 __global__ void __launch_bounds__(32 * kWideWarps, 1)
-binactiv_pack_wide_kernel(const float *__restrict__ x, const float *__restrict__ scale, const float *__restrict__ shift,
+binactiv_pack_wide_kernel(const float *x, const float *scale, const float *shift,
                           long long total_pix, int C, int HW, int Cw, uint32_t *__restrict__ x_packed, float *__restrict__ A) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   constexpr int kTile = kWideCh * kWidePix;                // floats
@@ -265,7 +265,7 @@ binactiv_pack_wide_kernel(const float *__restrict__ x, const float *__restrict__
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   stream_order();
   if (kHasBN)
-    for (int c = threadIdx.x; c < C; c += 32 * kWideWarps) bn[c] = make_float2(__ldg(scale + c), __ldg(shift + c));
+    for (int c = threadIdx.x; c < C; c += 32 * kWideWarps) bn[c] = make_float2(load_global(scale + c), load_global(shift + c));
   __syncthreads();
   const int ngroups = (int)((total_pix + kWidePix - 1) / kWidePix);
   const int nsub = (C + kWideCh - 1) / kWideCh;
@@ -511,7 +511,7 @@ binactiv_image_kernel(const __grid_constant__ ImgParams P) {
   // bytes of channels beyond C (C % 32 != 0) are never written by a unit: they stay zero
   for (int i = tid; i < nplanes * HW * P.Cw; i += kImgThreads) reinterpret_cast<uint32_t *>(wbytes)[i] = 0u;
   if (kHasBN)
-    for (int c = tid; c < P.C; c += kImgThreads) bn[c] = make_float2(__ldg(P.scale + c), __ldg(P.shift + c));
+    for (int c = tid; c < P.C; c += kImgThreads) bn[c] = make_float2(load_global(P.scale + c), load_global(P.shift + c));
   __syncthreads();
 
   if (warp == kImgWarps) {
@@ -690,7 +690,7 @@ binactiv_image_kernel(const __grid_constant__ ImgParams P) {
 // run-time bounds issues them one L2 round trip at a time).  KS = 0: any size.
 template <int KS>
 __global__ void __launch_bounds__(256)
-box_filter_kernel(const float *__restrict__ A, int H, int W, int kh, int kw, int stride, int pad,
+box_filter_kernel(const float *A, int H, int W, int kh, int kw, int stride, int pad,
                   int Ho, int Wo, int valid_taps, float *__restrict__ K) {
   stream_order();
   const int i = blockIdx.x * 256 + threadIdx.x;
@@ -707,7 +707,7 @@ box_filter_kernel(const float *__restrict__ A, int H, int W, int kh, int kw, int
       for (int kx = 0; kx < KS; ++kx) {
         const int iy = y0 + ky, ix = x0 + kx;
         const bool in = iy >= 0 && iy < H && ix >= 0 && ix < W;
-        v[ky * KS + kx] = in ? __ldg(a + iy * W + ix) : 0.0f;
+        v[ky * KS + kx] = in ? load_global(a + iy * W + ix) : 0.0f;
       }
 #pragma unroll
     for (int t = 0; t < KS * KS; ++t) s += v[t];
@@ -716,7 +716,7 @@ box_filter_kernel(const float *__restrict__ A, int H, int W, int kh, int kw, int
     const int kx0 = x0 < 0 ? -x0 : 0, kx1 = min(kw, W - x0);
     for (int ky = ky0; ky < ky1; ++ky) {
       const float *row = a + (y0 + ky) * W + x0;
-      for (int kx = kx0; kx < kx1; ++kx) s += __ldg(row + kx);
+      for (int kx = kx0; kx < kx1; ++kx) s += load_global(row + kx);
     }
   }
   // divisor: k_h k_w (zero-padded A), or the number of taps inside the image
@@ -732,7 +732,7 @@ box_filter_kernel(const float *__restrict__ A, int H, int W, int kh, int kw, int
 // is paid once and the taps of neighbouring outputs are loaded once.
 template <int KS>
 __global__ void __launch_bounds__(256)
-box_filter_rows_kernel(const float *__restrict__ A, int H, int W, int pad, int Ho, int Wo, int valid_taps,
+box_filter_rows_kernel(const float *A, int H, int W, int pad, int Ho, int Wo, int valid_taps,
                        float *__restrict__ K) {
   stream_order();
   const int per_row = Wo >> 2, i = blockIdx.x * 256 + threadIdx.x;
@@ -745,7 +745,7 @@ box_filter_rows_kernel(const float *__restrict__ A, int H, int W, int pad, int H
     const bool row = (unsigned)(y0 + ky) < (unsigned)H;
 #pragma unroll
     for (int kx = 0; kx < KS + 3; ++kx)
-      v[ky][kx] = row && (unsigned)(x0 + kx) < (unsigned)W ? __ldg(a + (y0 + ky) * W + x0 + kx) : 0.0f;
+      v[ky][kx] = row && (unsigned)(x0 + kx) < (unsigned)W ? load_global(a + (y0 + ky) * W + x0 + kx) : 0.0f;
   }
   float k[4];
 #pragma unroll
@@ -1011,11 +1011,11 @@ namespace {
 
 // A[i] = (part 0 + part 1 + ...)[i] / C, the parts added in index order.
 __global__ void __launch_bounds__(256)
-sum_parts_kernel(const float *__restrict__ parts, int nparts, size_t n, float C, float *__restrict__ A) {
+sum_parts_kernel(const float *parts, int nparts, size_t n, float C, float *__restrict__ A) {
   stream_order();
   for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (size_t)gridDim.x * 256) {
     float s = 0.0f;
-    for (int p = 0; p < nparts; ++p) s += __ldg(parts + (size_t)p * n + i);
+    for (int p = 0; p < nparts; ++p) s += load_global(parts + (size_t)p * n + i);
     A[i] = s / C;
   }
 }
@@ -1043,8 +1043,8 @@ cudaError_t launch_binactiv_finish(const float *A_part, int parts, const ConvGeo
 namespace {
 
 __global__ void __launch_bounds__(256)
-binactiv_pack_kbit_kernel(const float *__restrict__ x, const float *__restrict__ scale,
-                          const float *__restrict__ shift, long long total_pix, int C, int HW, int Cw,
+binactiv_pack_kbit_kernel(const float *x, const float *scale,
+                          const float *shift, long long total_pix, int C, int HW, int Cw,
                           int kbits, uint32_t *__restrict__ x_planes, float *__restrict__ A) {
   __shared__ float tau[128];                 // tau[j], j = 1 .. 2^k - 1; tau[0] unused
   stream_order();
@@ -1071,13 +1071,13 @@ binactiv_pack_kbit_kernel(const float *__restrict__ x, const float *__restrict__
         float yv[8];                       // eight loads in flight before any is used
 #pragma unroll
         for (int q = 0; q < 8; ++q)
-          yv[q] = j0 + q < nc ? __ldg(src + (size_t)(c0 + j0 + q) * HW) : 0.0f;
+          yv[q] = j0 + q < nc ? load_global(src + (size_t)(c0 + j0 + q) * HW) : 0.0f;
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
           const int j = j0 + q;
           if (j < nc) {
             float y = yv[q];
-            if (scale != nullptr) y = __fmaf_rn(__ldg(scale + c0 + j), y, __ldg(shift + c0 + j));
+            if (scale != nullptr) y = __fmaf_rn(load_global(scale + c0 + j), y, load_global(shift + c0 + j));
             if (q & 1) p1 += fabsf(y); else p0 += fabsf(y);
             // largest index whose decision point is <= y, by bisection over the sorted tau
             int idx = 0;

@@ -9,7 +9,7 @@ namespace {
 constexpr int kThreads = 256;
 
 __global__ void __launch_bounds__(kThreads)
-binarize_weights_kernel(const float *__restrict__ w, int Co, int C, int taps, int Cw,
+binarize_weights_kernel(const float *w, int Co, int C, int taps, int Cw,
                         uint32_t *__restrict__ w_packed, float *__restrict__ alpha) {
   extern __shared__ uint32_t words[];  // [taps][Cw]
   __shared__ double red[kThreads / 32];
@@ -27,7 +27,7 @@ binarize_weights_kernel(const float *__restrict__ w, int Co, int C, int taps, in
   for (int f = warp; f < nwords; f += kThreads / 32) {
     const int ci = cw * 32 + lane;
     const bool in = ci < C;
-    const float v = in ? __ldg(wf + (size_t)ci * taps + tap) : -1.0f;
+    const float v = in ? load_global(wf + (size_t)ci * taps + tap) : -1.0f;
     if (in) l1 += fabs((double)v);
     const uint32_t word = __ballot_sync(0xffffffffu, in && v >= 0.0f);
     if (lane == 0) words[f] = word;

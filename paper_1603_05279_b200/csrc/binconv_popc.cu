@@ -22,8 +22,8 @@ struct PopcParams {
 };
 
 __global__ void __launch_bounds__(kThreads)
-binconv_popc_kernel(const uint32_t *__restrict__ xp, const uint32_t *__restrict__ wp,
-                    const float *__restrict__ alpha, const float *__restrict__ K,
+binconv_popc_kernel(const uint32_t *xp, const uint32_t *wp,
+                    const float *alpha, const float *K,
                     const float *residual, PopcParams P, EpiOpts epi, float *out, int32_t *acc_out) {
   extern __shared__ uint32_t smem[];
   stream_order();
@@ -67,7 +67,7 @@ binconv_popc_kernel(const uint32_t *__restrict__ xp, const uint32_t *__restrict_
       const int iy = iy0 + r, ix = cx - P.pad;
       uint32_t v = 0u;
       if (iy >= 0 && iy < P.H && ix >= 0 && ix < P.W)
-        v = __ldg(xp + (((size_t)n * P.H + iy) * P.W + ix) * P.Cw + cw0 + cw);
+        v = load_global(xp + (((size_t)n * P.H + iy) * P.W + ix) * P.Cw + cw0 + cw);
       patch[cw * P.PP + pix] = v;
     }
     // stage the filter tile
@@ -77,7 +77,7 @@ binconv_popc_kernel(const uint32_t *__restrict__ xp, const uint32_t *__restrict_
       const int f = ft / taps;
       uint32_t v = 0u;
       if (co0 + f < P.Co)
-        v = __ldg(wp + packed_weight_index(P.Co, co0 + f, (ft - f * taps) * P.Cw + cw0 + cw));
+        v = load_global(wp + packed_weight_index(P.Co, co0 + f, (ft - f * taps) * P.Cw + cw0 + cw));
       wts[ft * P.cwc + cw] = v;
     }
     __syncthreads();
@@ -102,14 +102,14 @@ binconv_popc_kernel(const uint32_t *__restrict__ xp, const uint32_t *__restrict_
     }
   }
   if (!live) return;
-  const float kv = __ldg(K + (size_t)n * HoWo + op);
+  const float kv = load_global(K + (size_t)n * HoWo + op);
 #pragma unroll
   for (int f = 0; f < FPT; ++f) {
     const int co = co0 + fg * FPT + f;
     if (co >= P.Co) break;
     const int acc = nvalid * P.C - 2 * pops[f];
     const size_t o = ((size_t)n * P.Co + co) * HoWo + op;
-    float v = __fmul_rn(__fmul_rn((float)acc, kv), __fmul_rn(__ldg(alpha + co), epi.out_scale));
+    float v = __fmul_rn(__fmul_rn((float)acc, kv), __fmul_rn(load_global(alpha + co), epi.out_scale));
     if (residual) v += residual[o];
     if (epi.relu) v = fmaxf(v, 0.0f);
     out[o] = v;

@@ -614,11 +614,11 @@ __device__ bool weight_role(const TcParams &P, const Smem &S, long long nitems, 
     if (on && j0 + gs <= P.nsteps) {
       const uint2 *src = wp2 + ((size_t)j0 * P.Co + co);
 #pragma unroll
-      for (int u = 0; u < kUnits; ++u) dst[u] = __ldg(src + (size_t)u * P.Co);
+      for (int u = 0; u < kUnits; ++u) dst[u] = load_global(src + (size_t)u * P.Co);
     } else {
 #pragma unroll
       for (int u = 0; u < kUnits; ++u)
-        dst[u] = (on && j0 + u < P.nsteps) ? __ldg(wp2 + ((size_t)(j0 + u) * P.Co + co))
+        dst[u] = (on && j0 + u < P.nsteps) ? load_global(wp2 + ((size_t)(j0 + u) * P.Co + co))
                                            : make_uint2(0u, 0u);
     }
   };
@@ -742,7 +742,7 @@ __device__ void weight_stream(const TcParams &P, const Smem &S, uint32_t nitems,
   uint2 w[kU];
   uint32_t off = offset();
 #pragma unroll
-  for (int u = 0; u < kU; ++u) w[u] = __ldg(wp2 + min(off + (uint32_t)u * gstep, last));
+  for (int u = 0; u < kU; ++u) w[u] = load_global(wp2 + min(off + (uint32_t)u * gstep, last));
   uint32_t ws = (uint32_t)group, wph = 1u;           // stages >= groups (host)
 #pragma unroll 1
   while (it < nitems) {
@@ -759,7 +759,7 @@ __device__ void weight_stream(const TcParams &P, const Smem &S, uint32_t nitems,
           uint32_t v0[4], v1[4], sw = 0u;
           expand_signs<false>(w[u].x, v0);
           expand_signs<false>(w[u].y, v1);
-          w[u] = __ldg(wp2 + min(off, last));
+          w[u] = load_global(wp2 + min(off, last));
           if (kSpecial) {
             const int j = j0 + u * subs;
             if ((P.swap_mask[(j >> 5) & 31] >> (j & 31)) & 1u) sw = lbo;
@@ -855,8 +855,8 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
     for (size_t b = a0 + bulk; b < b1; b += 4)           // at most 3 words, at the tensor's end
       if (in_bounds((uint32_t)(b - a0) + 4u <= P.raw_plane, 3))
       {
-        sts32(dst + (uint32_t)(b - a0), __ldg(P.xp + (b >> 2)));
-        if (kTwo) sts32(dst + P.raw_plane + (uint32_t)(b - a0), __ldg(P.xp2 + (b >> 2)));
+        sts32(dst + (uint32_t)(b - a0), load_global(P.xp + (b >> 2)));
+        if (kTwo) sts32(dst + P.raw_plane + (uint32_t)(b - a0), load_global(P.xp2 + (b >> 2)));
       }
     if (bulk && in_bounds(bulk <= P.raw_plane && a0 + bulk <= tensor_bytes, 4)) {
       mbar_arrive_expect_tx(bar, kTwo ? 2u * bulk : bulk);
@@ -1055,7 +1055,7 @@ __device__ bool epilogue_role(const TcParams &P, const Smem &S, long long i0, in
       if (ox < P.Wo && oy < P.Ho) {
         const size_t pix = (size_t)oy * P.Wo + ox;
         px.valid = true;
-        px.kv = __ldg(P.K + (size_t)n * HoWo + pix);
+        px.kv = load_global(P.K + (size_t)n * HoWo + pix);
         px.obase = (size_t)n * P.Co * HoWo + pix;
         px.gpix = (size_t)n * HoWo + pix;
       }
@@ -1328,10 +1328,10 @@ binconv_tc_kernel(const __grid_constant__ TcParams P) {
   if (!kRes && P.off_tab != 0u)
     for (int i = tid; i < P.nsteps; i += kThreads) reinterpret_cast<uint32_t *>(smem + P.off_tab)[i] = P.adesc_lo[i];
   for (int i = tid; i < P.vec_len; i += kThreads) {
-    reinterpret_cast<float *>(smem + P.off_vec)[i] = i < P.Co ? __fmul_rn(__ldg(P.alpha + i), P.out_scale) : 0.0f;
+    reinterpret_cast<float *>(smem + P.off_vec)[i] = i < P.Co ? __fmul_rn(load_global(P.alpha + i), P.out_scale) : 0.0f;
     if (kFuse && P.nscale != nullptr) {
-      reinterpret_cast<float *>(smem + P.off_vec)[P.vec_len + i] = i < P.Co ? __ldg(P.nscale + i) : 0.0f;
-      reinterpret_cast<float *>(smem + P.off_vec)[2 * P.vec_len + i] = i < P.Co ? __ldg(P.nshift + i) : 0.0f;
+      reinterpret_cast<float *>(smem + P.off_vec)[P.vec_len + i] = i < P.Co ? load_global(P.nscale + i) : 0.0f;
+      reinterpret_cast<float *>(smem + P.off_vec)[2 * P.vec_len + i] = i < P.Co ? load_global(P.nshift + i) : 0.0f;
     }
   }
   tc_fence_before();

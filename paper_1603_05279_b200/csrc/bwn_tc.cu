@@ -310,7 +310,7 @@ __device__ void weight_role(const BwnParams &P, const Smem &S, long long i0, lon
 #pragma unroll
     for (int u = 0; u < kU; ++u) {
       const int wl = sub + u * subs, f = c.st * P.wps + wl;
-      w[u] = row < P.NT && wl < P.wps && c.it < i1 && f < P.nwords && co < P.Co ? __ldg(P.wp + packed_weight_index(P.Co, co, f)) : 0u;
+      w[u] = row < P.NT && wl < P.wps && c.it < i1 && f < P.nwords && co < P.Co ? load_global(P.wp + packed_weight_index(P.Co, co, f)) : 0u;
     }
   };
   Cursor c{i0, 0, (int)(i0 % P.nslabs)};
@@ -472,7 +472,7 @@ bwn_conv_kernel(const __grid_constant__ BwnParams P) {
   stream_order();
   for (int i = tid; i < P.vec_len; i += kThreads)
     reinterpret_cast<float *>(smem + P.off_vec)[i] =
-        i < P.Co ? (P.alpha != nullptr ? __ldg(P.alpha + i) : 1.0f) : 0.0f;   // no alpha: unit scale
+        i < P.Co ? (P.alpha != nullptr ? load_global(P.alpha + i) : 1.0f) : 0.0f;   // no alpha: unit scale
   fence_proxy_async();
   tc_fence_before();
   __syncthreads();
@@ -512,8 +512,8 @@ constexpr int kPrepThreads = 128;
 
 template <bool kGrad>
 __global__ void __launch_bounds__(kPrepThreads, 6)
-bwn_prepare_kernel(const float *__restrict__ x, const float *__restrict__ scale,
-                   const float *__restrict__ shift, const float *__restrict__ gmax, int C, int H,
+bwn_prepare_kernel(const float *x, const float *scale,
+                   const float *shift, const float *gmax, int C, int H,
                    int W, int s, int Hq, int Wq, int leadY, int leadX, long long L, int Cp, int ngroups,
                    uint4 *__restrict__ xs) {
   stream_order();
@@ -521,8 +521,8 @@ bwn_prepare_kernel(const float *__restrict__ x, const float *__restrict__ scale,
   __shared__ __align__(16) float factor[2][32];            // scale and shift of the block's channels
   if (threadIdx.x < 32 && scale != nullptr) {
     const int ch = grp * 32 + threadIdx.x;
-    factor[0][threadIdx.x] = ch < C ? __ldg(scale + ch) : 0.0f;
-    factor[1][threadIdx.x] = !kGrad && ch < C ? __ldg(shift + ch) : 0.0f;
+    factor[0][threadIdx.x] = ch < C ? load_global(scale + ch) : 0.0f;
+    factor[1][threadIdx.x] = !kGrad && ch < C ? load_global(shift + ch) : 0.0f;
   }
   __syncthreads();
   const long long m = (long long)blockIdx.x * kPrepThreads + threadIdx.x;
@@ -535,7 +535,7 @@ bwn_prepare_kernel(const float *__restrict__ x, const float *__restrict__ scale,
   const size_t plane = (size_t)H * W;
   const int c0 = grp * 32;
   const float *src = x + ((size_t)n * C + c0) * plane + (size_t)iy * W + ix;
-  const float gm = kGrad && real ? __ldg(gmax + n) : 0.0f;    // the scale of this position's image
+  const float gm = kGrad && real ? load_global(gmax + n) : 0.0f;    // the scale of this position's image
   uint4 *dst = xs + ((size_t)(phase * (Cp / 8) + grp * kPrepPlanes) * (size_t)L + (size_t)m);
   const bool whole = c0 + 32 <= C;
   float values[kPrepPlanes][8];
@@ -544,7 +544,7 @@ bwn_prepare_kernel(const float *__restrict__ x, const float *__restrict__ scale,
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int ch = 4 * q + (j & 3) + 16 * (j >> 2);
-      values[q][j] = real && (whole || c0 + ch < C) ? __ldg(src + (size_t)ch * plane) : 0.0f;
+      values[q][j] = real && (whole || c0 + ch < C) ? load_global(src + (size_t)ch * plane) : 0.0f;
     }
 #pragma unroll
   for (int q = 0; q < kPrepPlanes; ++q) {

@@ -40,9 +40,10 @@ inline ConvGeom make_geom(const xnor_conv_desc &d) {
 }
 
 // Consecutive kernels of a stream overlap their launch and set-up with the end of the kernel before
-// (programmatic dependent launch).  Every kernel of the library is launched through launch_kernel and
-// calls stream_order() before its first access to global memory: it returns when the kernels before
-// it in the stream have completed and their writes are visible, so a kernel still sees everything that
+// (programmatic dependent launch).  Every kernel that reads or writes a caller's memory is launched through
+// launch_kernel, calls stream_order() before its first access to global memory and reads that memory
+// with load_global, asynchronous copies or ordinary loads: stream_order() returns when the kernels before
+// it in the stream have completed and their writes are visible, so a kernel sees everything that
 // was launched before it.  A kernel that leaves SMs free then lets the next one start at once (a batch-1
 // layer's kernels take 2 to 9 us each, a launch gap with the set-up of the tensor-core kernel 3: the
 // 16-layer chain of one image 395 -> 276 us).  A kernel that fills the GPU lets it start as its own
@@ -54,6 +55,32 @@ constexpr unsigned kSms = 148;
 __device__ __forceinline__ void stream_order() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (gridDim.x * gridDim.y < kSms) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// A load of global memory that the kernel before may still have been writing when this one started: coherent,
+// and volatile, which keeps it behind stream_order().  (__ldg, or an ordinary load through a pointer to
+// const that is __restrict__, promises that nobody writes the memory while the kernel lives, and may be
+// moved ahead of the wait.)
+__device__ __forceinline__ float load_global(const float *p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(__cvta_generic_to_global(p)));
+  return v;
+}
+__device__ __forceinline__ float4 load_global(const float4 *p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(__cvta_generic_to_global(p)));
+  return v;
+}
+__device__ __forceinline__ uint32_t load_global(const uint32_t *p) {
+  uint32_t v;
+  asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(__cvta_generic_to_global(p)));
+  return v;
+}
+__device__ __forceinline__ uint2 load_global(const uint2 *p) {
+  uint2 v;
+  asm volatile("ld.global.v2.b32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(__cvta_generic_to_global(p)));
+  return v;
 }
 
 // `cluster`: CTAs per cluster along x (1: none).

@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(kPoolThreads) maxpool_stream_kernel(const Pool
     const long long p0 = place(c) * P.per_chunk, np = min((long long)P.per_chunk, P.planes - p0);
     const uint32_t floats = (uint32_t)np * (uint32_t)HW, bulk = floats & ~3u, dst = base + (uint32_t)b * P.chunk_bytes;
     const float *src = P.x + (size_t)p0 * HW;
-    for (uint32_t i = bulk; i < floats; ++i) reinterpret_cast<float *>(smem + (size_t)b * P.chunk_bytes)[i] = __ldg(src + i);
+    for (uint32_t i = bulk; i < floats; ++i) reinterpret_cast<float *>(smem + (size_t)b * P.chunk_bytes)[i] = load_global(src + i);
     const uint32_t bar = smem_u32(&full[b]);
     if (bulk) {
       mbar_arrive_expect_tx(bar, bulk * 4u);
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(kPoolThreads) maxpool_stream_kernel(const Pool
 // too small to be worth it.
 template <bool kRelu>
 __global__ void __launch_bounds__(kPoolThreads)
-maxpool_kernel(const float *__restrict__ x, long long total_out, int H, int W, int k, int stride,
+maxpool_kernel(const float *x, long long total_out, int H, int W, int k, int stride,
                int pad, int Ho, int Wo, Magic div_howo, Magic div_wo, float *__restrict__ out) {
   stream_order();
   const int HoWo = Ho * Wo;
@@ -149,9 +149,9 @@ maxpool_kernel(const float *__restrict__ x, long long total_out, int H, int W, i
       const int y0 = max(oy * stride - pad, 0), y1 = min(oy * stride - pad + k, H);
       const int x0 = max(ox * stride - pad, 0), x1 = min(ox * stride - pad + k, W);
       const float *t = x + (size_t)(plane0 + pl) * H * W;
-      float m = __ldg(t + (size_t)y0 * W + x0);
+      float m = load_global(t + (size_t)y0 * W + x0);
       for (int iy = y0; iy < y1; ++iy)
-        for (int ix = x0; ix < x1; ++ix) m = fmaxf(m, __ldg(t + (size_t)iy * W + ix));
+        for (int ix = x0; ix < x1; ++ix) m = fmaxf(m, load_global(t + (size_t)iy * W + ix));
       out[base + i] = kRelu ? fmaxf(m, 0.0f) : m;
     }
   }

@@ -41,7 +41,7 @@ __device__ __forceinline__ void copy4(uint32_t dst, const float *src, int bytes)
 // only in a last partial step.
 template <int PT, int FT, int KS, int ST>
 __global__ void __launch_bounds__(kThreads, PT == 8 ? 4 : 8)
-shortcut_conv1x1_kernel(const float *__restrict__ x, const float *__restrict__ w, int C, int H,
+shortcut_conv1x1_kernel(const float *x, const float *w, int C, int H,
                         int W, int Co, int stride, int Ho, int Wo, long long total_pix, int fblocks,
                         float *__restrict__ out) {
   constexpr int TPX = TX * PT, TF = TY * FT, WP = TF + 4;       // pitch of a filter row: staggered banks
