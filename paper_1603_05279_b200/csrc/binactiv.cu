@@ -707,7 +707,7 @@ box_filter_kernel(const float *A, int H, int W, int kh, int kw, int stride, int 
       for (int kx = 0; kx < KS; ++kx) {
         const int iy = y0 + ky, ix = x0 + kx;
         const bool in = iy >= 0 && iy < H && ix >= 0 && ix < W;
-        v[ky * KS + kx] = in ? load_global(a + iy * W + ix) : 0.0f;
+        v[ky * KS + kx] = load_global_if(a + iy * W + ix, in);
       }
 #pragma unroll
     for (int t = 0; t < KS * KS; ++t) s += v[t];
@@ -745,7 +745,7 @@ box_filter_rows_kernel(const float *A, int H, int W, int pad, int Ho, int Wo, in
     const bool row = (unsigned)(y0 + ky) < (unsigned)H;
 #pragma unroll
     for (int kx = 0; kx < KS + 3; ++kx)
-      v[ky][kx] = row && (unsigned)(x0 + kx) < (unsigned)W ? load_global(a + (y0 + ky) * W + x0 + kx) : 0.0f;
+      v[ky][kx] = load_global_if(a + (y0 + ky) * W + x0 + kx, row && (unsigned)(x0 + kx) < (unsigned)W);
   }
   float k[4];
 #pragma unroll
@@ -1071,7 +1071,7 @@ binactiv_pack_kbit_kernel(const float *x, const float *scale,
         float yv[8];                       // eight loads in flight before any is used
 #pragma unroll
         for (int q = 0; q < 8; ++q)
-          yv[q] = j0 + q < nc ? load_global(src + (size_t)(c0 + j0 + q) * HW) : 0.0f;
+          yv[q] = load_global_if(src + (size_t)(c0 + j0 + q) * HW, j0 + q < nc);
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
           const int j = j0 + q;

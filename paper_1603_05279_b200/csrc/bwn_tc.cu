@@ -544,7 +544,7 @@ bwn_prepare_kernel(const float *x, const float *scale,
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int ch = 4 * q + (j & 3) + 16 * (j >> 2);
-      values[q][j] = real && (whole || c0 + ch < C) ? load_global(src + (size_t)ch * plane) : 0.0f;
+      values[q][j] = load_global_if(src + (size_t)ch * plane, real && (whole || c0 + ch < C));
     }
 #pragma unroll
   for (int q = 0; q < kPrepPlanes; ++q) {

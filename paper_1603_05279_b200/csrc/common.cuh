@@ -82,6 +82,18 @@ __device__ __forceinline__ uint2 load_global(const uint2 *p) {
   asm volatile("ld.global.v2.b32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(__cvta_generic_to_global(p)));
   return v;
 }
+// The same where `in`, else 0: one predicated instruction.  (A branch around each volatile load made the
+// 49 taps of the 7x7 box filter 0.7 us slower.)
+__device__ __forceinline__ float load_global_if(const float *p, bool in) {
+  float v;
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "setp.ne.b32 q, %2, 0;\n\t"
+      "mov.f32 %0, 0f00000000;\n\t"
+      "@q ld.global.f32 %0, [%1];\n\t}"
+      : "=&f"(v) : "l"(__cvta_generic_to_global(p)), "r"((int)in));
+  return v;
+}
 
 // `cluster`: CTAs per cluster along x (1: none).
 template <class... Params, class... Args>
