@@ -469,6 +469,9 @@ bwn_conv_kernel(const __grid_constant__ BwnParams P) {
                  ::"r"(smem_u32(S.tmem_slot)), "r"((uint32_t)kTmemCols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  // the tensor memory is taken before any thread lets the next kernel start: a block of that kernel on this
+  // SM could take it first, and then waits for this one
+  __syncthreads();
   stream_order();
   for (int i = tid; i < P.vec_len; i += kThreads)
     reinterpret_cast<float *>(smem + P.off_vec)[i] =

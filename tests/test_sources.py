@@ -30,3 +30,14 @@ def test_memory_is_not_read_before_the_kernel_in_front_is_done(name):
         before, wait, _ = text.partition("stream_order();")
         assert wait, "%s: %s does not wait for the kernels before it" % (name, kernel)
         assert not re.search(r"load_global\(|cp\.async|bulk_copy_g2s\(", before[before.index("{"):].split("auto ")[0]), kernel
+
+
+@pytest.mark.parametrize("name", sorted(n for n in SOURCES if "tcgen05.alloc" in SOURCES[n]))
+def test_tensor_memory_is_taken_before_the_next_kernel_may_start(name):
+    """stream_order() may let the next kernel start.  A block of it that takes an SM's tensor memory before
+    this kernel's block there has would hold it while it waits for this kernel: neither would ever go on."""
+    found = [text for _, text in kernels(SOURCES[name]) if "tcgen05.alloc" in text and "stream_order();" in text]
+    for text in found:
+        before = text.partition("stream_order();")[0]
+        assert "__syncthreads();" in before[before.rindex("tcgen05.alloc"):]
+    assert found or name == "peaks.cu"               # measures with ordinary launches
