@@ -255,6 +255,23 @@ xnor_status xnor_conv2d_forward_kbit(const uint32_t *x_planes, int kbits, const 
                                      void *cuda_stream);
 
 /*
+ * How a convolution call runs a shape under the engine in force: xnor_conv2d_forward (kbits = 1,
+ * fused = 0), xnor_conv2d_forward_kbit (kbits 1 .. 7), xnor_conv2d_forward_binactiv (fused != 0,
+ * kbits = 1).  Nothing is launched.  Status as the call's own for d and kbits; the plan is
+ * written with XNOR_OK only.  resident, pair, slabs and slab_filters describe the first pass on
+ * the tensor cores and are 0 on the CUDA cores.
+ */
+typedef struct xnor_conv_plan {
+  int tensor_cores;   /* 1: tensor cores, 0: CUDA cores */
+  int launches;       /* kernels, one per pass */
+  int resident;       /* 1: a block keeps its slab's filters in shared memory, 0: they stream through it */
+  int pair;           /* 1: blocks work in pairs */
+  int slabs;          /* filter slabs */
+  int slab_filters;   /* filters per slab (the last may have fewer) */
+} xnor_conv_plan;
+xnor_status xnor_conv2d_plan(const xnor_conv_desc *d, int kbits, int fused, xnor_conv_plan *plan);
+
+/*
  * Binary-Weight-Network convolution -- Section 3.1, Eq. 1:
  *   I * W ~ (I (+) B) alpha,
  * real-valued inputs, B = sign(W) and alpha from xnor_binarize_weights; (+) is a

@@ -41,7 +41,7 @@ EXPORTS = [
     "xnor_binarize_weights", "xnor_binactiv", "xnor_binactiv_static", "xnor_conv2d_forward", "xnor_shortcut_conv1x1",
     "xnor_set_engine", "xnor_get_engine", "xnor_check_device", "xnor_selftest_wait_timeout",
     "xnor_maxpool2d", "xnor_binactiv_launches", "xnor_binactiv_kbit_launches", "xnor_conv2d_binactiv_parts", "xnor_conv2d_forward_binactiv", "xnor_binactiv_finish",
-    "xnor_binactiv_kbit", "xnor_conv2d_forward_kbit",
+    "xnor_binactiv_kbit", "xnor_conv2d_forward_kbit", "xnor_conv2d_plan",
     "xnor_bwn_input_elems", "xnor_bwn_prepare_input", "xnor_bwn_conv2d_forward",
     "xnor_bgrad_stream_elems", "xnor_binarize_weights_transposed", "xnor_binary_gradient_backward", "xnor_measure_peaks",
 ]
@@ -50,6 +50,11 @@ EXPORTS = [
 class xnor_conv_desc(ctypes.Structure):
     _fields_ = [(n, ctypes.c_int) for n in
                 ("N", "C_in", "H", "W", "C_out", "k_h", "k_w", "stride", "pad", "flags")]
+
+
+class xnor_conv_plan(ctypes.Structure):
+    _fields_ = [(n, ctypes.c_int) for n in
+                ("tensor_cores", "launches", "resident", "pair", "slabs", "slab_filters")]
 
 
 class XnorError(RuntimeError):
@@ -131,6 +136,8 @@ def load():
     lib.xnor_conv2d_forward_kbit.restype = ci
     lib.xnor_conv2d_forward_kbit.argtypes = [vp, ci, vp, vp, vp, vp, ctypes.POINTER(xnor_conv_desc),
                                              vp, vp, vp]
+    lib.xnor_conv2d_plan.restype = ci
+    lib.xnor_conv2d_plan.argtypes = [ctypes.POINTER(xnor_conv_desc), ci, ci, ctypes.POINTER(xnor_conv_plan)]
     lib.xnor_bwn_input_elems.restype = ctypes.c_size_t
     lib.xnor_bwn_input_elems.argtypes = [ctypes.POINTER(xnor_conv_desc)]
     lib.xnor_bwn_prepare_input.restype = ci
@@ -234,6 +241,14 @@ def xnor_binactiv_launches(d, has_bn=False):
 def xnor_binactiv_kbit_launches(d, kbits, has_bn=False):
     """Kernels xnor_binactiv_kbit launches for this shape (1 or 2; 0 = bad arguments)."""
     return int(load().xnor_binactiv_kbit_launches(ctypes.byref(d), int(kbits), int(bool(has_bn))))
+
+
+def xnor_conv2d_plan(d, kbits=1, fused=False):
+    """How a convolution call runs this shape under the engine in force (an xnor_conv_plan)."""
+    plan = xnor_conv_plan()
+    _check(load().xnor_conv2d_plan(ctypes.byref(d), int(kbits), int(bool(fused)), ctypes.byref(plan)),
+           "xnor_conv2d_plan")
+    return plan
 
 
 def xnor_conv2d_binactiv_parts(d):

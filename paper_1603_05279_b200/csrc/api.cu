@@ -128,6 +128,15 @@ int pick_engine(const xnor::ConvGeom &g, xnor_engine e) {
   return xnor::binconv_popc_supported(g) ? 0 : -1;
 }
 
+// Shapes the BinConv calls take, whatever the engine.
+xnor_status check_conv_shape(const xnor_conv_desc *d) {
+  xnor_status s = check_desc(d, true);
+  if (s != XNOR_OK) return s;
+  if (d->k_h > 11 || d->k_w > 11) return XNOR_ERR_UNSUPPORTED;
+  if ((long long)d->C_in * d->k_h * d->k_w >= (1LL << 24)) return XNOR_ERR_UNSUPPORTED;
+  return XNOR_OK;
+}
+
 xnor_status check_conv_args(const uint32_t *x_packed, const uint32_t *w_packed, const float *alpha,
                             const float *K, const float *residual, const xnor_conv_desc *d,
                             const float *out, const int32_t *acc_out) {
@@ -137,10 +146,19 @@ xnor_status check_conv_args(const uint32_t *x_packed, const uint32_t *w_packed, 
     return XNOR_ERR_INVALID_ARG;
   if ((residual && misaligned(residual)) || (acc_out && misaligned(acc_out)))
     return XNOR_ERR_INVALID_ARG;
-  if (d->k_h > 11 || d->k_w > 11) return XNOR_ERR_UNSUPPORTED;
-  if ((long long)d->C_in * d->k_h * d->k_w >= (1LL << 24)) return XNOR_ERR_UNSUPPORTED;
-  return XNOR_OK;
+  return check_conv_shape(d);
 }
+
+// Words of a bit plane; planes stay 16-byte aligned, or there is only one.
+size_t plane_words_of(const xnor_conv_desc *d) { return (size_t)d->N * d->H * d->W * ((d->C_in + 31) / 32); }
+bool planes_aligned(const xnor_conv_desc *d, int kbits) { return kbits == 1 || (plane_words_of(d) & 3u) == 0; }
+
+// Bit planes that the pass from plane p on takes: two on the tensor cores where their rows fit beside each
+// other (see xnor_conv2d_forward_kbit).
+bool planes_in_pairs(const xnor::ConvGeom &g, int engine, xnor_engine choice) {
+  return engine == 1 && xnor::umma_tc_supported(g, variant_of(choice), 2);
+}
+int planes_of_pass(bool pairs, int p, int kbits) { return pairs && p + 1 < kbits ? 2 : 1; }
 
 xnor_status run_conv(int engine, xnor_engine choice, const uint32_t *x_packed,
                      const uint32_t *w_packed, const float *alpha, const float *K,
@@ -190,8 +208,8 @@ xnor_status xnor_conv2d_forward_kbit(const uint32_t *x_planes, int kbits, const 
   xnor_status s = check_conv_args(x_planes, w_packed, alpha, K, residual, d, out, acc_out);
   if (s != XNOR_OK) return s;
   if (kbits < 1 || kbits > 7) return XNOR_ERR_INVALID_ARG;
-  const size_t plane_words = (size_t)d->N * d->H * d->W * ((d->C_in + 31) / 32);
-  if (kbits > 1 && (plane_words & 3u)) return XNOR_ERR_UNSUPPORTED;   // planes stay 16-byte aligned
+  if (!planes_aligned(d, kbits)) return XNOR_ERR_UNSUPPORTED;
+  const size_t plane_words = plane_words_of(d);
   const xnor::ConvGeom g = xnor::make_geom(*d);
   const xnor_engine choice = current_engine();
   const int engine = pick_engine(g, choice);
@@ -202,9 +220,9 @@ xnor_status xnor_conv2d_forward_kbit(const uint32_t *x_planes, int kbits, const 
   // images, k = 2: one convolution of 45 us instead of two), else one; the pass from plane p on adds
   // D K alpha 2^p / (2^k - 1) to what the passes before it wrote (the output is its own residual).
   const double levels = (double)((1 << kbits) - 1);
-  const bool pairs = engine == 1 && xnor::umma_tc_supported(g, variant_of(choice), 2);
+  const bool pairs = planes_in_pairs(g, engine, choice);
   for (int p = 0; p < kbits;) {
-    const int planes = pairs && p + 1 < kbits ? 2 : 1;
+    const int planes = planes_of_pass(pairs, p, kbits);
     const uint32_t *x = x_planes + (size_t)p * plane_words;
     xnor::EpiOpts epi = xnor::default_epi(g);
     epi.relu = epi.relu && p + planes == kbits;
@@ -248,6 +266,24 @@ int xnor_conv2d_binactiv_parts(const xnor_conv_desc *d) {
       (long long)d->C_in * d->k_h * d->k_w >= (1LL << 24))
     return 0;
   return xnor::tc_fused_parts(xnor::make_geom(*d), current_variant());
+}
+
+xnor_status xnor_conv2d_plan(const xnor_conv_desc *d, int kbits, int fused, xnor_conv_plan *plan) {
+  if (plan == nullptr || kbits < 1 || kbits > 7 || (fused && kbits != 1)) return XNOR_ERR_INVALID_ARG;
+  const xnor_status s = check_conv_shape(d);
+  if (s != XNOR_OK) return s;
+  if (!planes_aligned(d, kbits)) return XNOR_ERR_UNSUPPORTED;
+  const xnor::ConvGeom g = xnor::make_geom(*d);
+  const xnor_engine choice = current_engine();
+  const int engine = fused ? (choice == XNOR_ENGINE_POPC ? -1 : 1) : pick_engine(g, choice);
+  if (engine < 0) return XNOR_ERR_UNSUPPORTED;
+  xnor_conv_plan r = {};
+  const bool pairs = kbits > 1 && planes_in_pairs(g, engine, choice);
+  if (engine == 1 && !xnor::tc_plan_info(g, variant_of(choice), fused != 0, planes_of_pass(pairs, 0, kbits), &r))
+    return XNOR_ERR_UNSUPPORTED;
+  for (int p = 0; p < kbits; p += planes_of_pass(pairs, p, kbits)) ++r.launches;
+  *plan = r;
+  return XNOR_OK;
 }
 
 xnor_status xnor_conv2d_forward_binactiv(const uint32_t *x_packed, const uint32_t *w_packed,

@@ -1665,6 +1665,14 @@ Plan plan_variant(const ConvGeom &g, TcVariant v, bool fuse = false, int planes 
 
 bool umma_tc_supported(const ConvGeom &g, TcVariant v, int planes) { return plan_variant(g, v, false, planes).ok; }
 
+bool tc_plan_info(const ConvGeom &g, TcVariant v, bool fuse, int planes, xnor_conv_plan *out) {
+  const Plan pl = plan_variant(g, v, fuse, planes);
+  if (!pl.ok) return false;
+  out->tensor_cores = 1;
+  out->resident = pl.P.resident; out->pair = pl.P.pair; out->slabs = pl.P.nslabs; out->slab_filters = pl.P.NT;
+  return true;
+}
+
 namespace {
 
 cudaError_t launch_plan(Plan &pl, cudaStream_t st, bool fuse) {

@@ -89,13 +89,12 @@ class LayerBuffers:
 
     def launches(self):
         """Kernels one forward() launches: binarize 1, BinActiv 1 or 2 (pack + A, box filter; one
-        kernel where a block streams whole images), BinConv 1 (k-bit: one per two planes on the
-        tensor cores, one per plane on the CUDA cores)."""
+        kernel where a block streams whole images), BinConv 1 (k-bit: one per pass)."""
         if self.variant == "bgrad":
             return 2 + 3             # two weight packings; maximum, gradient stream, convolution
         conv = 1
         if self.variant == "kbit":
-            conv = self.kbits if B.xnor_get_engine() == B.XNOR_ENGINE_POPC else (self.kbits + 1) // 2
+            conv = B.xnor_conv2d_plan(self.desc, self.kbits).launches
         return 1 + self.binactiv_launches() + conv
 
     def binactiv_bytes(self):

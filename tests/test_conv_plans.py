@@ -1,0 +1,46 @@
+"""How the convolution calls run a shape (xnor_conv2d_plan): host logic, no GPU needed."""
+import pytest
+
+import paper_1603_05279_b200 as X
+from paper_1603_05279_b200 import binding as B
+from paper_1603_05279_b200 import workloads as wl
+from paper_1603_05279_b200.runner import LayerBuffers
+
+
+def plan(N, C, H, W, Co, k, stride=1, pad=None, kbits=1, fused=False):
+    return X.xnor_conv2d_plan(X.make_desc(N, C, H, W, Co, k, k, stride, k // 2 if pad is None else pad), kbits, fused)
+
+
+@pytest.fixture(autouse=True)
+def default_engine():
+    yield
+    X.xnor_set_engine(B.XNOR_ENGINE_AUTO)
+
+
+# kernels for 1 .. 7 bit planes: in pairs on the tensor cores; one by one where the rows of two do not fit
+# beside each other, and on the CUDA cores (stride 3, or by choice)
+@pytest.mark.parametrize("shape,engine,tensor,launches", [
+    ((4, 128, 28, 28, 128, 3, 1, 1), B.XNOR_ENGINE_AUTO, 1, [1, 1, 2, 2, 3, 3, 4]),
+    ((32, 897, 36, 40, 135, 5, 1, 1), B.XNOR_ENGINE_AUTO, 1, [1, 2, 3, 4, 5, 6, 7]),
+    ((4, 128, 28, 28, 128, 3, 3, 1), B.XNOR_ENGINE_AUTO, 0, [1, 2, 3, 4, 5, 6, 7]),
+    ((4, 128, 28, 28, 128, 3, 1, 1), B.XNOR_ENGINE_POPC, 0, [1, 2, 3, 4, 5, 6, 7]),
+])
+def test_launches_of_a_kbit_convolution(shape, engine, tensor, launches):
+    X.xnor_set_engine(engine)
+    plans = [plan(*shape, kbits=k) for k in range(1, 8)]
+    assert [p.launches for p in plans] == launches
+    assert all(p.tensor_cores == tensor for p in plans)
+    N, C, H, W, Co, k, stride, pad = shape
+    for kbits in (2, 3):
+        L = LayerBuffers(wl.ConvShape("s", N, C, H, W, Co, k, stride, pad, 1.0), device="meta", variant="kbit", kbits=kbits)
+        assert L.launches() == 1 + L.binactiv_launches() + launches[kbits - 1]
+
+
+def test_plan_refuses_what_the_calls_refuse():
+    for bad in (dict(kbits=0), dict(kbits=8), dict(kbits=2, fused=True)):
+        with pytest.raises(X.XnorError):
+            plan(4, 64, 8, 8, 64, 3, **bad)
+    with pytest.raises(X.XnorError):
+        plan(1, 8, 5, 5, 4, 3, kbits=2)               # 25 words per plane
+    with pytest.raises(X.XnorError):
+        plan(1, 8, 5, 5, 40, 3, fused=True)           # the next layer's words are not whole
