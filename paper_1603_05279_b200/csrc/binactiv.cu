@@ -1015,7 +1015,13 @@ sum_parts_kernel(const float *parts, int nparts, size_t n, float C, float *__res
   stream_order();
   for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (size_t)gridDim.x * 256) {
     float s = 0.0f;
-    for (int p = 0; p < nparts; ++p) s += load_global(parts + (size_t)p * n + i);
+    for (int p0 = 0; p0 < nparts; p0 += 8) {     // eight loads in flight, added in order
+      float v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = load_global_if(parts + (size_t)(p0 + k) * n + i, p0 + k < nparts);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) s += v[k];
+    }
     A[i] = s / C;
   }
 }

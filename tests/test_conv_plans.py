@@ -44,3 +44,7 @@ def test_plan_refuses_what_the_calls_refuse():
         plan(1, 8, 5, 5, 4, 3, kbits=2)               # 25 words per plane
     with pytest.raises(X.XnorError):
         plan(1, 8, 5, 5, 40, 3, fused=True)           # the next layer's words are not whole
+
+
+def schedule(p):
+    return ("pair " if p.pair else "") + ("resident" if p.resident else "streaming"), p.slabs, p.slab_filters
