@@ -1501,12 +1501,14 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
     // patch per tile and narrow MMAs re-read the pixel operand more often.  So (measured) several slabs
     // pay only from 128 filters (a pair: 96; 512 channels, 7x7, residual: 45.6 -> 34.1 us) and with two
     // K-steps or more per plane of the patch: kernels of 3x3 and up with stride 1 (128 channels, 28x28,
-    // stride 2: 29.5 us resident, 27.0 streaming).
+    // stride 2: 29.5 us resident, 27.0 streaming).  The fused epilogue, half as long again, outweighs the
+    // patches whatever the kernel: resident wherever it fits (16 channels, 34x34, 768 filters 1x1, 58 images:
+    // 136 us streaming, 64 resident; 0.68 of the time in the median of 68 drawn shapes of several slabs).
     for (int ns = min_slabs; ns <= 16 && !P.resident; ++ns) {
       P.NT = slab_width(g.Co, ns, pair || fuse);
       P.nslabs = (g.Co + P.NT - 1) / P.NT;
       P.NTh = pair ? P.NT / 2 : P.NT;
-      if (P.nslabs > 1 && !few && (P.NT < (pair ? 96 : 128) || P.nsteps < 2 * P.nplanes)) break;
+      if (P.nslabs > 1 && !few && (P.NT < (pair ? 96 : 128) || (!fuse && P.nsteps < 2 * P.nplanes))) break;
       // (Lending four of the weight warps to the patch builders where a pixel has many channel
       // words was the better split while the drain loop was longer; since its trimming twelve
       // draining warps win on every layer measured: conv4 50.4 -> 48.1 us, conv5 39.4 -> 37.3.)

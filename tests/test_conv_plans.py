@@ -48,3 +48,9 @@ def test_plan_refuses_what_the_calls_refuse():
 
 def schedule(p):
     return ("pair " if p.pair else "") + ("resident" if p.resident else "streaming"), p.slabs, p.slab_filters
+
+
+def test_fused_slabs_stay_resident():
+    """The fused epilogue outweighs a patch per slab, however few K-steps a slab has."""
+    assert schedule(plan(58, 16, 34, 34, 768, 1, fused=True)) == ("resident", 4, 192)
+    assert schedule(plan(60, 64, 55, 53, 384, 3, stride=2, fused=True)) == ("resident", 2, 192)
