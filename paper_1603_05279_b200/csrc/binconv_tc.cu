@@ -105,7 +105,7 @@ constexpr int kWgtWarp0 = 5, kWgtWarps = 8;
 constexpr int kPatWarp0 = 13, kPatWarps = 3;
 constexpr int kThreadsRes = 32 * (kPatWarp0 + kPatWarps);   // 512: 16 warps, 128 registers each
 // streaming: weight warps in groups of four, patch warps behind them (see the kernel's role table)
-constexpr int kLongItem = 64;         // streaming: K-steps of an item that count as many
+constexpr int kLongItem = 64, kLongFused = 96;   // streaming: K-steps of an item that count as many
 constexpr int kGroupWarps = 4, kThreadsStream = 768;   // 24 warps, 80 registers each
 constexpr int kTileM = 128;          // stream positions per tile = tensor-memory lanes
 constexpr int kTmemCols = 512;
@@ -1540,8 +1540,9 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
     while (P.mps > 4 && P.nsteps < 3 * P.mps) P.mps /= 2;   // short items: smaller stages start sooner
     // Long items are bound by the expansion, short ones by the epilogue: two warps per quarter of the
     // lanes in place of a weight group (1024 channels, 1x1: 27.2 -> 25.6 us; 512 channels, 3x3, 72 K-steps:
-    // 32.8 -> 34.7 us).
-    P.wgt_groups = P.nsteps < kLongItem && !fuse ? 2 : 3;
+    // 32.8 -> 34.7 us).  The fused epilogue is the longer one (245 channels, 52x52, 640 filters 3x3 stride 2,
+    // 16 images: 49 -> 40 us with two; 976 channels, 192 filters, 140 K-steps: 96 -> 114).
+    P.wgt_groups = P.nsteps < (fuse ? kLongFused : kLongItem) ? 2 : 3;
     auto stage = [&](int mps) { P.mps = mps; P.stage_bytes = (uint32_t)mps * (uint32_t)P.NTh * 32u; };
     stage(P.mps);
     while (P.mps > 1 && !fits(P.wgt_groups, 1, 1)) stage(P.mps / 2);
@@ -1557,7 +1558,7 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
   P.nacc = std::max(1, std::min(kMaxAcc, kMaxAccCols / P.NT));
   // worker warps per quarter of the lanes in the resident schedule: the four epilogue warps
   // and the eight weight warps
-  P.epi_split = P.resident ? std::min(kEpiSplitMax, P.NT / (fuse ? 32 : 16)) : P.wgt_groups == 2 ? std::min(2, P.NT / 16) : 1;
+  P.epi_split = P.resident ? std::min(kEpiSplitMax, P.NT / (fuse ? 32 : 16)) : P.wgt_groups == 2 ? std::min(2, P.NT / (fuse ? 32 : 16)) : 1;
   if (fuse && (g.Co & 31) != 0) return pl;          // whole words of the next layer's input
   P.stages = stages; P.npb = npb;
   P.off_tab = 0u;
