@@ -1405,6 +1405,7 @@ struct Plan {
   TcParams P;
   size_t smem;
   bool ok;
+  bool by_time;                // streaming although the resident schedule would fit: estimated to be faster
 };
 
 // Weight-thread mapping and stage size for slabs of NT filters: rows_mod threads cover the
@@ -1496,19 +1497,37 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
   }
   int stages = 0, npb = 0;
   P.resident = 0;
+  const int units = (int)kSms / (pair ? 2 : 1);
+  const int stream_slabs = std::max(min_slabs, (g.Co + 127) / 128);
+  // Several slabs of few K-steps: the resident schedule drains with three warps per quarter of the lanes and
+  // builds a patch per item, the streaming one drains with two and builds a patch per tile.  The time of the
+  // fullest CTA from what was measured: per 16 columns drained 6 and 9, per plane and 32 positions of a patch
+  // 1 (0.055 us).  Within a sixth of each other streaming wins.  79 images, 80 channels, 49x49, 912 filters
+  // 3x3 stride 2: 98 us streaming, 60 resident; 128 channels, 28x28, 256 filters, 256 images: 27.0 and 29.5.
+  // Over 210 drawn 1x1 and stride-2 shapes of 256 to 1024 filters 0.95 of the time of streaming alone in
+  // the median (0.52 to 1.05); a residual, unknown here, favours the resident schedule a little more.
+  auto streams_faster = [&]() {
+    const int snt = slab_width(g.Co, stream_slabs, pair || fuse), sns = (g.Co + snt - 1) / snt;
+    const int patch = P.nplanes * ((P.ppix + 31) / 32), group = units / P.nslabs;
+    auto time = [&](long long items, int drain, int patch_per_item) {
+      return patch + drain + (items - 1) * std::max(drain, patch_per_item);
+    };
+    const long long res = time((P.ntiles + group - 1) / group, 6 * P.NT / 16, patch);
+    const long long str = time(((long long)P.ntiles * sns + units - 1) / units, 9 * snt / 16, (patch + sns - 1) / sns);
+    return 5 * str < 6 * res;
+  };
   if (schedule == 0) {
     // Resident: the widest slab whose expanded rows fit beside two patches.  Every slab needs its own
     // patch per tile and narrow MMAs re-read the pixel operand more often.  So (measured) several slabs
-    // pay only from 128 filters (a pair: 96; 512 channels, 7x7, residual: 45.6 -> 34.1 us) and with two
-    // K-steps or more per plane of the patch: kernels of 3x3 and up with stride 1 (128 channels, 28x28,
-    // stride 2: 29.5 us resident, 27.0 streaming).  The fused epilogue, half as long again, outweighs the
+    // pay only from 128 filters (a pair: 96; 512 channels, 7x7, residual: 45.6 -> 34.1 us) and, with fewer
+    // than two K-steps per plane of the patch, where streams_faster() says no.  The fused epilogue, half as long again, outweighs the
     // patches whatever the kernel: resident wherever it fits (16 channels, 34x34, 768 filters 1x1, 58 images:
     // 136 us streaming, 64 resident; 0.68 of the time in the median of 68 drawn shapes of several slabs).
     for (int ns = min_slabs; ns <= 16 && !P.resident; ++ns) {
       P.NT = slab_width(g.Co, ns, pair || fuse);
       P.nslabs = (g.Co + P.NT - 1) / P.NT;
       P.NTh = pair ? P.NT / 2 : P.NT;
-      if (P.nslabs > 1 && !few && (P.NT < (pair ? 96 : 128) || (!fuse && P.nsteps < 2 * P.nplanes))) break;
+      if (P.nslabs > 1 && !few && (P.NT < (pair ? 96 : 128) || (!fuse && P.nsteps < 2 * P.nplanes && (pl.by_time = streams_faster())))) break;
       // (Lending four of the weight warps to the patch builders where a pixel has many channel
       // words was the better split while the drain loop was longer; since its trimming twelve
       // draining warps win on every layer measured: conv4 50.4 -> 48.1 us, conv5 39.4 -> 37.3.)
@@ -1525,7 +1544,7 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
     }
   }
   if (!P.resident) {
-    P.NT = slab_width(g.Co, std::max(min_slabs, (g.Co + 127) / 128), pair || fuse);
+    P.NT = slab_width(g.Co, stream_slabs, pair || fuse);
     P.nslabs = (g.Co + P.NT - 1) / P.NT;
     P.NTh = pair ? P.NT / 2 : P.NT;
     P.wgt_warps = kWgtWarps;
@@ -1619,7 +1638,7 @@ Plan plan_variant_uncached(const ConvGeom &g, TcVariant v, bool fuse, int planes
   if (single.ok && single.P.resident) return single;
   // a problem of few items is better spread over single CTAs
   if (single.ok && 2 * single.P.ntiles * single.P.nslabs <= (int)kSms) return single;
-  Plan pair = make_plan(g, 0, true, fuse, planes);
+  Plan pair = make_plan(g, single.by_time ? 1 : 0, true, fuse, planes);
   if (pair.ok && (pair.P.resident || !single.ok || (pair.P.NT > 64 && pair.P.nsteps >= kLongItem))) return pair;
   return single;
 }

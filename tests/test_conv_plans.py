@@ -63,3 +63,14 @@ def test_fused_streaming_drains_short_items_with_two_warps(shape, warps):
     assert not p.resident
     N, C, H, W, Co, k, stride, pad = shape
     assert X.xnor_conv2d_binactiv_parts(X.make_desc(N, C, H, W, Co, k, k, stride, pad)) == p.slabs * warps
+
+
+@pytest.mark.parametrize("shape,expected", [
+    ((190, 67, 51, 51, 428, 1, 2, 0), ("resident", 2, 224)),          # the drain is the longest part: three warps
+    ((79, 80, 49, 49, 912, 3, 2, 1), ("resident", 4, 240)),
+    ((255, 272, 7, 7, 768, 1, 2, 0), ("resident", 4, 192)),           # one patch each either way
+    ((256, 128, 28, 28, 256, 3, 2, 1), ("streaming", 2, 128)),        # the patch is: built once per tile
+    ((136, 944, 8, 19, 512, 1, 1, 0), ("streaming", 4, 128)),
+    ((155, 432, 9, 9, 513, 1, 1, 0), ("streaming", 5, 112))])         # and pairs do not change that
+def test_slabs_of_few_steps_are_resident_where_that_is_faster(shape, expected):
+    assert schedule(plan(*shape)) == expected
