@@ -1488,11 +1488,15 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
   // Items for fewer than half the SMs: narrower slabs on up to half of them, a CTA then expands and
   // drains less (512 channels, 7x7, one image: 15.6 -> 9.4 us; 64 channels, 14x14: 6.7 -> 6.5 us).  With
   // few K-steps the drain counts most and 16 filters win, else 32.  A small problem fills its one item's
-  // stages in few, large steps (`few` in plan_stage): the latency per stage is what it waits for.
+  // stages in few, large steps (`few` in plan_stage): the latency per stage is what it waits for.  Fused, 64
+  // filters: every slab adds planes of partial sums (352 channels, 9x9, 224 filters 3x3: 21.4 us in slabs of
+  // 128, 13.3 of 64, 15.8 of 32; 0.87 of the time in the median of 68 drawn shapes of up to four images).
+  // Beyond 16 slabs the resident search below gives up and the shape streams, which is the faster there
+  // (16 channels, 5x5, 832 filters 3x3, two images: 7.0 us, 9.1 resident; 1.04 to 1.30 over 19 drawn shapes).
   const int spread = (int)kSms / 2 / P.ntiles;
-  const bool few = !pair && !fuse && min_slabs <= spread;
+  const bool few = !pair && min_slabs <= spread;
   if (few) {
-    const int width = P.nsteps < 16 ? 16 : 32;
+    const int width = fuse ? 64 : P.nsteps < 16 ? 16 : 32;
     min_slabs = std::max(min_slabs, std::min(spread, (g.Co + width - 1) / width));
   }
   int stages = 0, npb = 0;
@@ -1527,7 +1531,7 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
       P.NT = slab_width(g.Co, ns, pair || fuse);
       P.nslabs = (g.Co + P.NT - 1) / P.NT;
       P.NTh = pair ? P.NT / 2 : P.NT;
-      if (P.nslabs > 1 && !few && (P.NT < (pair ? 96 : 128) || (!fuse && P.nsteps < 2 * P.nplanes && (pl.by_time = streams_faster())))) break;
+      if (P.nslabs > 1 && (!few || (fuse && ns > spread)) && (P.NT < (pair ? 96 : 128) || (!fuse && P.nsteps < 2 * P.nplanes && (pl.by_time = streams_faster())))) break;
       // (Lending four of the weight warps to the patch builders where a pixel has many channel
       // words was the better split while the drain loop was longer; since its trimming twelve
       // draining warps win on every layer measured: conv4 50.4 -> 48.1 us, conv5 39.4 -> 37.3.)

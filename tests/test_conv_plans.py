@@ -74,3 +74,10 @@ def test_fused_streaming_drains_short_items_with_two_warps(shape, warps):
     ((155, 432, 9, 9, 513, 1, 1, 0), ("streaming", 5, 112))])         # and pairs do not change that
 def test_slabs_of_few_steps_are_resident_where_that_is_faster(shape, expected):
     assert schedule(plan(*shape)) == expected
+
+
+@pytest.mark.parametrize("shape,expected", [
+    ((1, 352, 9, 9, 224, 3, 1, 1), ("resident", 4, 64)), ((2, 33, 7, 5, 96, 3, 1, 1), ("resident", 2, 64)),
+    ((2, 448, 46, 46, 416, 3, 1, 1), ("pair resident", 5, 96))])       # no slabs beyond the two that spread it
+def test_small_fused_problems_are_spread(shape, expected):
+    assert schedule(plan(*shape, fused=True)) == expected
