@@ -1548,7 +1548,25 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
     }
   }
   if (!P.resident) {
-    P.NT = slab_width(g.Co, stream_slabs, pair || fuse);
+    int ns = stream_slabs;
+    if (pair) {
+      // Up to 224 filters per slab: the expansion, the longest part of an item, takes the same time for the
+      // rows between two powers of two, so wider slabs pay where they save rounds of the pairs over the items
+      // (928 channels, 38x38, 912 filters 5x5, two images: 92.6 us in 8 slabs of 128, 60.8 in 5 of 192) and
+      // at equal estimates (544 channels, 22x53, 176 filters 3x3, 8 images: 23.5 -> 21.2).  Only where stages
+      // of four K-steps still fit.  Of 175 drawn shapes of 64 K-steps and more 29 change, to 0.66 .. 1.07.
+      auto rows = [&](int n) {
+        int r = 16;
+        while (2 * r < slab_width(g.Co, n, true)) r *= 2;
+        return r;
+      };
+      auto time = [&](int n) { return ((long long)P.ntiles * n + units - 1) / units * rows(n); };
+      for (int n = stream_slabs - 1; n >= min_slabs; --n) {
+        const size_t ring = (size_t)3 * 4 * 32 * (slab_width(g.Co, n, true) / 2);
+        if (time(n) <= time(ns) && ring + P.patch_bytes + P.raw_bytes <= avail) ns = n;
+      }
+    }
+    P.NT = slab_width(g.Co, ns, pair || fuse);
     P.nslabs = (g.Co + P.NT - 1) / P.NT;
     P.NTh = pair ? P.NT / 2 : P.NT;
     P.wgt_warps = kWgtWarps;

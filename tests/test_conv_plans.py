@@ -81,3 +81,11 @@ def test_slabs_of_few_steps_are_resident_where_that_is_faster(shape, expected):
     ((2, 448, 46, 46, 416, 3, 1, 1), ("pair resident", 5, 96))])       # no slabs beyond the two that spread it
 def test_small_fused_problems_are_spread(shape, expected):
     assert schedule(plan(*shape, fused=True)) == expected
+
+
+@pytest.mark.parametrize("shape,expected", [
+    ((2, 928, 38, 38, 912, 5, 1, 2), ("pair streaming", 5, 192)),      # 65 items for 74 pairs instead of 104
+    ((12, 544, 22, 53, 176, 3, 1, 1), ("pair streaming", 1, 192)),     # as long, and half the items
+    ((113, 544, 27, 5, 576, 5, 1, 2), ("pair streaming", 5, 128))])    # seven short rounds beat four long ones
+def test_pairs_stream_the_slabs_that_save_rounds(shape, expected):
+    assert schedule(plan(*shape)) == expected
