@@ -1542,7 +1542,8 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
       if (nst <= kMaxBarStages && fits(nst, 2, 1)) {
         P.resident = 1;
         stages = nst; npb = 2;
-        if (fits(stages, 3, 1)) npb = 3;
+        // (one item per block, one patch: a third buffer would have each patch warp build patches by itself)
+        if (!few && fits(stages, 3, 1)) npb = 3;
         if (npb == 3 && fits(stages, 4, 2)) npb = 4;     // a second raw buffer comes first
       }
     }
