@@ -257,7 +257,7 @@ xnor_status xnor_conv2d_forward_kbit(const uint32_t *x_planes, int kbits, const 
 /*
  * How a convolution call runs a shape under the engine in force: xnor_conv2d_forward (kbits = 1,
  * fused = 0), xnor_conv2d_forward_kbit (kbits 1 .. 7), xnor_conv2d_forward_binactiv (fused != 0,
- * kbits = 1).  Nothing is launched.  Status as the call's own for d and kbits; the plan is
+ * kbits = 1), with a residual (residual != 0) or without.  Nothing is launched.  Status as the call's own for d and kbits; the plan is
  * written with XNOR_OK only.  resident, pair, slabs and slab_filters describe the first pass on
  * the tensor cores and are 0 on the CUDA cores.
  */
@@ -269,7 +269,8 @@ typedef struct xnor_conv_plan {
   int slabs;          /* filter slabs */
   int slab_filters;   /* filters per slab (the last may have fewer) */
 } xnor_conv_plan;
-xnor_status xnor_conv2d_plan(const xnor_conv_desc *d, int kbits, int fused, xnor_conv_plan *plan);
+xnor_status xnor_conv2d_plan(const xnor_conv_desc *d, int kbits, int fused, int residual,
+                             xnor_conv_plan *plan);
 
 /*
  * Binary-Weight-Network convolution -- Section 3.1, Eq. 1:

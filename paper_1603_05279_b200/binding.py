@@ -137,7 +137,7 @@ def load():
     lib.xnor_conv2d_forward_kbit.argtypes = [vp, ci, vp, vp, vp, vp, ctypes.POINTER(xnor_conv_desc),
                                              vp, vp, vp]
     lib.xnor_conv2d_plan.restype = ci
-    lib.xnor_conv2d_plan.argtypes = [ctypes.POINTER(xnor_conv_desc), ci, ci, ctypes.POINTER(xnor_conv_plan)]
+    lib.xnor_conv2d_plan.argtypes = [ctypes.POINTER(xnor_conv_desc), ci, ci, ci, ctypes.POINTER(xnor_conv_plan)]
     lib.xnor_bwn_input_elems.restype = ctypes.c_size_t
     lib.xnor_bwn_input_elems.argtypes = [ctypes.POINTER(xnor_conv_desc)]
     lib.xnor_bwn_prepare_input.restype = ci
@@ -243,10 +243,11 @@ def xnor_binactiv_kbit_launches(d, kbits, has_bn=False):
     return int(load().xnor_binactiv_kbit_launches(ctypes.byref(d), int(kbits), int(bool(has_bn))))
 
 
-def xnor_conv2d_plan(d, kbits=1, fused=False):
+def xnor_conv2d_plan(d, kbits=1, fused=False, residual=False):
     """How a convolution call runs this shape under the engine in force (an xnor_conv_plan)."""
     plan = xnor_conv_plan()
-    _check(load().xnor_conv2d_plan(ctypes.byref(d), int(kbits), int(bool(fused)), ctypes.byref(plan)),
+    _check(load().xnor_conv2d_plan(ctypes.byref(d), int(kbits), int(bool(fused)), int(bool(residual)),
+                                   ctypes.byref(plan)),
            "xnor_conv2d_plan")
     return plan
 

@@ -268,7 +268,8 @@ int xnor_conv2d_binactiv_parts(const xnor_conv_desc *d) {
   return xnor::tc_fused_parts(xnor::make_geom(*d), current_variant());
 }
 
-xnor_status xnor_conv2d_plan(const xnor_conv_desc *d, int kbits, int fused, xnor_conv_plan *plan) {
+xnor_status xnor_conv2d_plan(const xnor_conv_desc *d, int kbits, int fused, int residual,
+                             xnor_conv_plan *plan) {
   if (plan == nullptr || kbits < 1 || kbits > 7 || (fused && kbits != 1)) return XNOR_ERR_INVALID_ARG;
   const xnor_status s = check_conv_shape(d);
   if (s != XNOR_OK) return s;
@@ -279,7 +280,7 @@ xnor_status xnor_conv2d_plan(const xnor_conv_desc *d, int kbits, int fused, xnor
   if (engine < 0) return XNOR_ERR_UNSUPPORTED;
   xnor_conv_plan r = {};
   const bool pairs = kbits > 1 && planes_in_pairs(g, engine, choice);
-  if (engine == 1 && !xnor::tc_plan_info(g, variant_of(choice), fused != 0, planes_of_pass(pairs, 0, kbits), &r))
+  if (engine == 1 && !xnor::tc_plan_info(g, variant_of(choice), fused != 0, planes_of_pass(pairs, 0, kbits), residual != 0, &r))
     return XNOR_ERR_UNSUPPORTED;
   for (int p = 0; p < kbits; p += planes_of_pass(pairs, p, kbits)) ++r.launches;
   *plan = r;

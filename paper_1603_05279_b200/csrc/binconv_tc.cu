@@ -1431,7 +1431,7 @@ int slab_width(int Co, int ns, bool pair) {     // pair: also set for the fused 
 }
 
 // schedule: 0 = resident when the slab fits, 1 = streaming.  pair: CTA pairs (clusters of 2).
-Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes) {
+Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes, bool residual) {
   Plan pl{};
   pl.ok = false;
   TcParams &P = pl.P;
@@ -1505,20 +1505,21 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
   const int stream_slabs = std::max(min_slabs, (g.Co + 127) / 128);
   // Several slabs of few K-steps: the resident schedule drains with three warps per quarter of the lanes and
   // builds a patch per item, the streaming one drains with two and builds a patch per tile.  The time of the
-  // fullest CTA from what was measured: per 16 columns drained 6 and 9, per plane and 32 positions of a patch
-  // 1 (0.055 us).  Within a sixth of each other streaming wins.  79 images, 80 channels, 49x49, 912 filters
-  // 3x3 stride 2: 98 us streaming, 60 resident; 128 channels, 28x28, 256 filters, 256 images: 27.0 and 29.5.
-  // Over 210 drawn 1x1 and stride-2 shapes of 256 to 1024 filters 0.95 of the time of streaming alone in
-  // the median (0.52 to 1.05); a residual, unknown here, favours the resident schedule a little more.
+  // fullest CTA from what was measured: per 16 columns drained 6 and 9 (with a residual 11 and 16), per plane
+  // and 32 positions of a patch 1 (0.055 us).  79 images, 80 channels, 49x49, 912 filters 3x3 stride 2: 98 us
+  // streaming, 60 resident; 37 images, 544 channels, 51x47, 256 filters 1x1 with a residual: 70 and 52; 128
+  // channels, 28x28, 256 filters 3x3 stride 2, 256 images: 27.0 and 29.5.  Without a residual streaming also wins
+  // within a sixth: there it is ahead of the estimate by up to 1.16 (170 images, 146 channels, 24x8, 800 filters
+  // 1x1 stride 2: 17.4 and 20.1 us).
   auto streams_faster = [&]() {
     const int snt = slab_width(g.Co, stream_slabs, pair || fuse), sns = (g.Co + snt - 1) / snt;
     const int patch = P.nplanes * ((P.ppix + 31) / 32), group = units / P.nslabs;
     auto time = [&](long long items, int drain, int patch_per_item) {
       return patch + drain + (items - 1) * std::max(drain, patch_per_item);
     };
-    const long long res = time((P.ntiles + group - 1) / group, 6 * P.NT / 16, patch);
-    const long long str = time(((long long)P.ntiles * sns + units - 1) / units, 9 * snt / 16, (patch + sns - 1) / sns);
-    return 5 * str < 6 * res;
+    const long long res = time((P.ntiles + group - 1) / group, (residual ? 11 : 6) * P.NT / 16, patch);
+    const long long str = time(((long long)P.ntiles * sns + units - 1) / units, (residual ? 16 : 9) * snt / 16, (patch + sns - 1) / sns);
+    return (residual ? 6 : 5) * str < 6 * res;
   };
   if (schedule == 0) {
     // Resident: the widest slab whose expanded rows fit beside two patches.  Every slab needs its own
@@ -1649,19 +1650,19 @@ namespace {
 // SM unless only a pair, each CTA holding half of a slab, can keep the filters resident.  Neither: pairs
 // where the items are long (each CTA expands half the rows of a slab; 1024 channels, 7x7 kernel: 419 ->
 // 361 us; 1x1 kernel, 16 K-steps: 27.2 -> 30.5 us) and the slabs wide enough to fill a pair.
-Plan plan_variant_uncached(const ConvGeom &g, TcVariant v, bool fuse, int planes) {
+Plan plan_variant_uncached(const ConvGeom &g, TcVariant v, bool fuse, int planes, bool residual) {
   switch (v) {
-    case kTcSingle: return make_plan(g, 0, false, fuse, planes);
-    case kTcSingleStream: return make_plan(g, 1, false, fuse, planes);
-    case kTcPair: return make_plan(g, 0, true, fuse, planes);
-    case kTcPairStream: return make_plan(g, 1, true, fuse, planes);
+    case kTcSingle: return make_plan(g, 0, false, fuse, planes, residual);
+    case kTcSingleStream: return make_plan(g, 1, false, fuse, planes, residual);
+    case kTcPair: return make_plan(g, 0, true, fuse, planes, residual);
+    case kTcPairStream: return make_plan(g, 1, true, fuse, planes, residual);
     default: break;
   }
-  Plan single = make_plan(g, 0, false, fuse, planes);
+  Plan single = make_plan(g, 0, false, fuse, planes, residual);
   if (single.ok && single.P.resident) return single;
   // a problem of few items is better spread over single CTAs
   if (single.ok && 2 * single.P.ntiles * single.P.nslabs <= (int)kSms) return single;
-  Plan pair = make_plan(g, single.by_time ? 1 : 0, true, fuse, planes);
+  Plan pair = make_plan(g, single.by_time ? 1 : 0, true, fuse, planes, residual);
   if (pair.ok && (pair.P.resident || !single.ok || (pair.P.NT > 64 && pair.P.nsteps >= kLongItem))) return pair;
   return single;
 }
@@ -1674,33 +1675,33 @@ cudaError_t launch_variant(const Plan &pl, unsigned units, cudaStream_t st) {
 
 }  // namespace
 
-// The last plans made, by (geometry, variant, fused): one call of the library plans its shape
+// The last plans made, by (geometry, variant, fused, bit planes, residual): one call of the library plans its shape
 // two or three times (support check, then launch), and a network repeats a few shapes; planning
 // evaluates up to 800 descriptor words.  Plans hold no pointers until a launcher fills them in.
 namespace {
 
 struct PlanKey {
-  int N, C, H, W, Co, kh, kw, stride, pad, variant, fuse, planes;
+  int N, C, H, W, Co, kh, kw, stride, pad, variant, fuse, planes, residual;
   bool operator==(const PlanKey &o) const {
     return N == o.N && C == o.C && H == o.H && W == o.W && Co == o.Co && kh == o.kh && kw == o.kw &&
-           stride == o.stride && pad == o.pad && variant == o.variant && fuse == o.fuse && planes == o.planes;
+           stride == o.stride && pad == o.pad && variant == o.variant && fuse == o.fuse && planes == o.planes && residual == o.residual;
   }
 };
 
-Plan plan_variant(const ConvGeom &g, TcVariant v, bool fuse = false, int planes = 1) {
+Plan plan_variant(const ConvGeom &g, TcVariant v, bool fuse, int planes, bool residual) {
   constexpr int kSlots = 16;
   static std::mutex mu;
   static PlanKey keys[kSlots];
   static Plan plans[kSlots];
   static bool used[kSlots] = {};
   static int next = 0;
-  const PlanKey key{g.N, g.C, g.H, g.W, g.Co, g.kh, g.kw, g.stride, g.pad, (int)v, fuse ? 1 : 0, planes};
+  const PlanKey key{g.N, g.C, g.H, g.W, g.Co, g.kh, g.kw, g.stride, g.pad, (int)v, fuse ? 1 : 0, planes, residual ? 1 : 0};
   std::lock_guard<std::mutex> lock(mu);
   for (int i = 0; i < kSlots; ++i)
     if (used[i] && keys[i] == key) return plans[i];
   const int slot = next;
   next = (next + 1) % kSlots;
-  plans[slot] = plan_variant_uncached(g, v, fuse, planes);
+  plans[slot] = plan_variant_uncached(g, v, fuse, planes, residual);
   keys[slot] = key;
   used[slot] = true;
   return plans[slot];
@@ -1708,10 +1709,10 @@ Plan plan_variant(const ConvGeom &g, TcVariant v, bool fuse = false, int planes 
 
 }  // namespace
 
-bool umma_tc_supported(const ConvGeom &g, TcVariant v, int planes) { return plan_variant(g, v, false, planes).ok; }
+bool umma_tc_supported(const ConvGeom &g, TcVariant v, int planes) { return plan_variant(g, v, false, planes, false).ok; }
 
-bool tc_plan_info(const ConvGeom &g, TcVariant v, bool fuse, int planes, xnor_conv_plan *out) {
-  const Plan pl = plan_variant(g, v, fuse, planes);
+bool tc_plan_info(const ConvGeom &g, TcVariant v, bool fuse, int planes, bool residual, xnor_conv_plan *out) {
+  const Plan pl = plan_variant(g, v, fuse, planes, residual);
   if (!pl.ok) return false;
   out->tensor_cores = 1;
   out->resident = pl.P.resident; out->pair = pl.P.pair; out->slabs = pl.P.nslabs; out->slab_filters = pl.P.NT;
@@ -1769,7 +1770,7 @@ cudaError_t launch_binconv_tc(const uint32_t *xp, const uint32_t *wp, const floa
                               const float *K, const float *residual, const ConvGeom &g,
                               const EpiOpts &epi, float *out, int32_t *acc_out, TcVariant variant,
                               cudaStream_t st, const uint32_t *xp2) {
-  Plan pl = plan_variant(g, variant, false, xp2 != nullptr ? 2 : 1);
+  Plan pl = plan_variant(g, variant, false, xp2 != nullptr ? 2 : 1, residual != nullptr);
   if (!pl.ok) return cudaErrorInvalidValue;
   TcParams &P = pl.P;
   P.xp = xp; P.xp2 = xp2; P.wp = wp; P.alpha = alpha; P.K = K; P.residual = residual;
@@ -1782,7 +1783,7 @@ cudaError_t launch_binconv_tc(const uint32_t *xp, const uint32_t *wp, const floa
 // Partial planes of |y| sums that the fused kernel writes for this shape: one per filter slab
 // and, in the resident schedule, per warp that shares a quarter of the lanes.  0: not supported.
 int tc_fused_parts(const ConvGeom &g, TcVariant variant) {
-  const Plan pl = plan_variant(g, variant, true);
+  const Plan pl = plan_variant(g, variant, true, 1, false);
   if (!pl.ok) return 0;
   return pl.P.nslabs * pl.P.epi_split;
 }
@@ -1792,7 +1793,7 @@ cudaError_t launch_binconv_tc_fused(const uint32_t *xp, const uint32_t *wp, cons
                                     float *out, const float *next_scale, const float *next_shift,
                                     uint32_t *xp_next, float *A_part, TcVariant variant,
                                     cudaStream_t st) {
-  Plan pl = plan_variant(g, variant, true);
+  Plan pl = plan_variant(g, variant, true, 1, false);
   if (!pl.ok) return cudaErrorInvalidValue;
   TcParams &P = pl.P;
   P.xp = xp; P.xp2 = nullptr; P.wp = wp; P.alpha = alpha; P.K = K; P.residual = residual;

@@ -179,7 +179,7 @@ enum TcVariant { kTcAuto = 0, kTcSingle, kTcSingleStream, kTcPair, kTcPairStream
 // planes: bit planes of the input that one pass takes, 1 or 2
 bool umma_tc_supported(const ConvGeom &g, TcVariant v, int planes = 1);
 // Fills the tensor-core fields of *out; false: the shape is not covered.
-bool tc_plan_info(const ConvGeom &g, TcVariant v, bool fuse, int planes, xnor_conv_plan *out);
+bool tc_plan_info(const ConvGeom &g, TcVariant v, bool fuse, int planes, bool residual, xnor_conv_plan *out);
 cudaError_t launch_binconv_tc(const uint32_t *xp, const uint32_t *wp, const float *alpha,
                               const float *K, const float *residual, const ConvGeom &g,
                               const EpiOpts &epi, float *out, int32_t *acc_out, TcVariant v,

@@ -7,8 +7,9 @@ from paper_1603_05279_b200 import workloads as wl
 from paper_1603_05279_b200.runner import LayerBuffers
 
 
-def plan(N, C, H, W, Co, k, stride=1, pad=None, kbits=1, fused=False):
-    return X.xnor_conv2d_plan(X.make_desc(N, C, H, W, Co, k, k, stride, k // 2 if pad is None else pad), kbits, fused)
+def plan(N, C, H, W, Co, k, stride=1, pad=None, kbits=1, fused=False, residual=False):
+    return X.xnor_conv2d_plan(X.make_desc(N, C, H, W, Co, k, k, stride, k // 2 if pad is None else pad), kbits, fused,
+                              residual)
 
 
 @pytest.fixture(autouse=True)
@@ -70,10 +71,15 @@ def test_fused_streaming_drains_short_items_with_two_warps(shape, warps):
     ((79, 80, 49, 49, 912, 3, 2, 1), ("resident", 4, 240)),
     ((255, 272, 7, 7, 768, 1, 2, 0), ("resident", 4, 192)),           # one patch each either way
     ((256, 128, 28, 28, 256, 3, 2, 1), ("streaming", 2, 128)),        # the patch is: built once per tile
-    ((136, 944, 8, 19, 512, 1, 1, 0), ("streaming", 4, 128)),
-    ((155, 432, 9, 9, 513, 1, 1, 0), ("streaming", 5, 112))])         # and pairs do not change that
+    ((136, 944, 8, 19, 512, 1, 1, 0), ("streaming", 4, 128)),          # (pairs, where they fit, do not change that)
+    ((155, 432, 9, 9, 513, 1, 1, 0), ("streaming", 5, 112))])
 def test_slabs_of_few_steps_are_resident_where_that_is_faster(shape, expected):
     assert schedule(plan(*shape)) == expected
+
+
+def test_a_residual_favours_the_three_draining_warps():
+    assert schedule(plan(37, 544, 51, 47, 256, 1)) == ("streaming", 2, 128)
+    assert schedule(plan(37, 544, 51, 47, 256, 1, residual=True)) == ("resident", 2, 128)
 
 
 @pytest.mark.parametrize("shape,expected", [
