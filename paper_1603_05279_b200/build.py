@@ -48,9 +48,8 @@ def build_pyext(force=False):
     return PYEXT
 
 
-def build(force=False, verbose=False, bounds_check=False):
-    """Builds libxnor.so, or with bounds_check the checking build libxnor_check.so."""
-    build_pyext(force and not bounds_check)
+def build_library(force=False, verbose=False, bounds_check=False):
+    """Builds libxnor.so, or with bounds_check the checking build libxnor_check.so: nvcc alone."""
     lib = LIB_CHECK if bounds_check else LIB
     if not force and up_to_date(lib):
         return lib
@@ -58,6 +57,14 @@ def build(force=False, verbose=False, bounds_check=False):
     cmd = [nvcc] + NVCC_FLAGS + (["-DXNOR_BOUNDS_CHECK"] if bounds_check else []) + \
         (["-Xptxas", "-v"] if verbose else []) + ["-o", lib] + SOURCES
     subprocess.run(cmd, check=True)
+    return lib
+
+
+def build(force=False, verbose=False, bounds_check=False):
+    """The library, and then the Python binding's native half: the C library needs neither torch's headers
+    nor a host C++ compiler set up for them, and is there when building the other fails."""
+    lib = build_library(force, verbose, bounds_check)
+    build_pyext(force and not bounds_check)
     return lib
 
 
