@@ -285,7 +285,7 @@ xnor_status xnor_conv2d_plan(const xnor_conv_desc *d, int kbits, int fused, int 
  *       affine y = fmaf(bn_scale[c], x, bn_shift[c])) -> x_stream, the bfloat16 values
  *       in the order the convolution reads them: for each of the stride^2 phases of the
  *       input, the pixels as one stream with zero pixels where the filter overhangs the
- *       image, C_in padded with zeros to a multiple of 16.  xnor_bwn_input_elems(d)
+ *       image, C_in padded with zeros to a multiple of 32.  xnor_bwn_input_elems(d)
  *       gives the number of 16-bit elements of x_stream for the geometry (0: bad
  *       descriptor); the layout is private to the two calls.
  *   xnor_bwn_conv2d_forward  x_stream, w_packed u32 [P][C_out][2], alpha fp32 [C_out],
@@ -293,8 +293,9 @@ xnor_status xnor_conv2d_plan(const xnor_conv_desc *d, int kbits, int fused, int 
  *       out fp32 [N][C_out][H_out][W_out].
  * INVALID_ARG as for the other calls.  UNSUPPORTED (nothing launched): stride > 2,
  * more than 121 filter taps, a tile's input window of more than 256 stream positions
- * (roughly (k_h - 1) * (W + k_w) > 120 at stride 1), or a window that does not fit
- * shared memory beside two weight stages (C_in above ~600 at 3x3 on small images).
+ * (roughly (k_h - 1) * (W + k_w) > 120 at stride 1; no wider window was ever taken or
+ * measured), or a window that does not fit shared memory beside three weight stages of
+ * one packed word per filter (C_in above ~600 at 3x3 on small images).
  * Device-side waits are bounded as in xnor_conv2d_forward (xnor_check_device).
  */
 size_t xnor_bwn_input_elems(const xnor_conv_desc *d);

@@ -15,13 +15,12 @@ namespace {
 
 constexpr int kMaxThreads = 256, kMaxCluster = 8;
 
-// Non-negative floats order like their bit patterns, so the maximum over blocks is an
-// integer atomicMax: exact and independent of the order of arrival.  NaN is skipped.
 __device__ __forceinline__ float abs_max4(float4 v) {
   return fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
 }
 
-// max|g| over the block's share of an image: part `part` of `parts`, four 16-byte loads in flight
+// max|g| over the block's share of an image: part `part` of `parts`, four 16-byte loads in flight.  NaN is
+// skipped.
 __device__ __forceinline__ float block_abs_max(const float *gi, size_t per_image, int vec4, unsigned part, unsigned parts) {
   const size_t step = (size_t)parts * kMaxThreads, first = (size_t)part * kMaxThreads + threadIdx.x;
   float m = 0.0f;
@@ -47,6 +46,8 @@ __device__ __forceinline__ float block_abs_max(const float *gi, size_t per_image
   return m;
 }
 
+// Blocks of an image meet in its element of gmax, cleared before: non-negative floats order like their bit
+// patterns, so an integer atomicMax is exact and independent of the order of arrival.
 __global__ void __launch_bounds__(kMaxThreads)
 grad_max_kernel(const float *g, size_t per_image, int vec4, float *__restrict__ gmax) {
   stream_order();

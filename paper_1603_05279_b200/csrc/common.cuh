@@ -51,6 +51,8 @@ inline ConvGeom make_geom(const xnor_conv_desc &d) {
 // waiting blocks keep other streams' kernels off the SMs (the four AlexNet layers on parallel branches
 // 224 -> 238 us) and its own split of L1 and shared memory is the one of the kernel it waits for (a pool
 // that reads through L1 92 -> 113 us).
+// (Plans and this rule take a B200's SM count for a constant, so that they can be made without a device;
+// grids go by the device's.)
 constexpr unsigned kSms = 148;
 __device__ __forceinline__ void stream_order() {
   asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -7,11 +7,17 @@ import torch
 
 import paper_1603_05279_b200 as X
 from test_gpu_bgrad import test_binary_gradient_backward_parity as backward_parity
+from test_gpu_fused import test_fused_binactiv_parity as fused_parity
 from test_gpu_options import _index_of_planes
 from test_gpu_options import test_kbit_block_parity as kbit_block_parity
+from test_gpu_parity import test_block_parity as block_parity
 from util import GuardSet, assert_close, dev, host
 
 pytestmark = pytest.mark.gpu
+
+
+def sms():
+    return torch.cuda.get_device_properties(0).multi_processor_count
 
 
 def rng(seed):
@@ -98,10 +104,12 @@ def test_kbit_two_planes_per_pass(oracle, shape, kbits, engine):
 
 
 @pytest.mark.parametrize("valid", [False, True])
-@pytest.mark.parametrize("case", [(190, 2, 56, 56, 3, 1), (260, 2, 55, 44, 5, 2), (230, 1, 51, 48, 5, 0),
-                                  (330, 1, 37, 50, 3, 0)])
+@pytest.mark.parametrize("case", [(190, 2, 56, 56, 3, 1), (260, 2, 55, 44, 5, 2), (300, 1, 51, 48, 5, 0),
+                                  (360, 1, 37, 50, 3, 0)])
 def test_box_filter_rows(oracle, case, valid):
     N, C, H, W, k, p = case
+    Ho, Wo = H + 2 * p - k + 1, W + 2 * p - k + 1
+    assert Wo % 4 == 0 and (Ho * Wo + 255) // 256 * N > 16 * sms()         # four outputs per thread from here on
     x = rng(sum(case)).standard_normal((N, C, H, W)).astype(np.float32)
     d = X.make_desc(N, C, H, W, 8, k, k, 1, p, X.XNOR_FLAG_K_VALID_TAPS if valid else 0)
     gs = GuardSet()
@@ -112,3 +120,34 @@ def test_box_filter_rows(oracle, case, valid):
     assert_close(host(A), A_or, "A")
     want = oracle.box_filter_valid_taps(A_or, k, k, 1, p) if valid else oracle.box_filter(A_or, k, k, 1, p)
     assert_close(host(K), want, "K")
+
+
+# fused, the schedule the planner takes: resident in several slabs of few K-steps, streaming with two warps per
+# quarter of the lanes, small problems in slabs of 64
+@pytest.mark.parametrize("case,resident,slabs,filters,parts", [
+    ((40, 16, 14, 14, 544, 1, 1, 0, 3, 1, 1, True), 1, 3, 192, 9),
+    ((30, 16, 9, 19, 288, 3, 2, 1, 1, 1, 0, False), 1, 3, 96, 9),
+    ((60, 416, 14, 13, 384, 1, 2, 0, 3, 1, 1, True), 0, 3, 128, 6),
+    ((1, 352, 9, 9, 224, 3, 1, 1, 3, 1, 1, False), 1, 4, 64, 8),
+    ((2, 33, 7, 5, 96, 3, 1, 1, 3, 2, 1, True), 1, 2, 64, 4)])
+def test_fused_schedules(oracle, case, resident, slabs, filters, parts):
+    N, C, H, W, Co, k, s, p = case[:8]
+    d = X.make_desc(N, C, H, W, Co, k, k, s, p)
+    plan = X.xnor_conv2d_plan(d, fused=True)
+    assert (plan.resident, plan.slabs, plan.slab_filters) == (resident, slabs, filters)
+    assert X.xnor_conv2d_binactiv_parts(d) == parts
+    fused_parity(oracle, case, X.XNOR_ENGINE_AUTO)
+
+
+# the plain convolution: several resident slabs of few K-steps, streaming because it is faster, pairs streaming
+# slabs of more than 128 filters, and both sides of the 16 slabs that a small problem may keep resident
+@pytest.mark.parametrize("shape,resident,pair,slabs,filters", [
+    ((30, 33, 31, 30, 428, 1, 1, 2, 0), 1, 0, 2, 224), ((16, 128, 28, 28, 256, 3, 3, 2, 1), 1, 0, 2, 128),
+    ((136, 944, 8, 19, 512, 1, 1, 1, 0), 0, 0, 4, 128), ((11, 544, 22, 37, 178, 3, 3, 1, 1), 0, 1, 1, 192),
+    ((1, 256, 7, 7, 256, 1, 1, 1, 0), 1, 0, 16, 16), ((1, 256, 7, 7, 272, 1, 1, 1, 0), 0, 0, 17, 16),
+    ((1, 512, 7, 7, 512, 3, 3, 1, 1), 1, 0, 16, 32), ((1, 512, 7, 7, 528, 3, 3, 1, 1), 0, 0, 17, 32)])
+def test_plain_schedules(oracle, shape, resident, pair, slabs, filters):
+    N, C, H, W, Co, kh, kw, s, p = shape
+    plan = X.xnor_conv2d_plan(X.make_desc(N, C, H, W, Co, kh, kw, s, p))
+    assert (plan.resident, plan.pair, plan.slabs, plan.slab_filters) == (resident, pair, slabs, filters)
+    block_parity(oracle, shape, X.XNOR_ENGINE_AUTO)
