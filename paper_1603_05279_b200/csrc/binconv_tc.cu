@@ -38,9 +38,10 @@
 //  Roles (one CTA per SM, CTAs loop over work items = (pixel tile, filter slab)): warps 0-3 epilogue
 //  (tensor memory -> registers -> coalesced NCHW stores of D * K * alpha (+ residual)), warp 4 issues the
 //  MMAs.  Resident schedule (512 threads): warps 5-12 expand weights, warps 13-15 expand activation
-//  patches.  Streaming schedule (768 threads): twelve warps expand weights and three patches, none of
-//  them on scheduler 0 (warp w runs on scheduler w % 4), whose instruction cache then holds the loop of
-//  the issuing thread, the path everything waits for.
+//  patches.  Streaming schedule (768 threads): twelve warps expand weights, or eight with four more
+//  draining (items of few K-steps, see make_plan), and three patches; neither weights nor patches are on
+//  scheduler 0 (warp w runs on scheduler w % 4), whose instruction cache then holds the loop of the
+//  issuing thread, the path everything waits for.
 //  Accumulators are multi-buffered in tensor memory so the epilogue of one
 //  item overlaps the MMAs of the next.  Every wait is bounded: on expiry the
 //  CTA records XNOR_ERR_TIMEOUT in a device status word, stops, frees its
@@ -1491,6 +1492,8 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
   // stages in few, large steps (`few` in plan_stage): the latency per stage is what it waits for.  Fused, 64
   // filters: every slab adds planes of partial sums (352 channels, 9x9, 224 filters 3x3: 21.4 us in slabs of
   // 128, 13.3 of 64, 15.8 of 32; 0.87 of the time in the median of 68 drawn shapes of up to four images).
+  // Narrower slabs than those that spread the problem stay one item per SM (480 channels, 51x51, 192 filters
+  // 3x3, three images, in 12 resident slabs of 16: 28.7 us, streaming 14.8).
   // Beyond 16 slabs the resident search below gives up and the shape streams, which is the faster there
   // (16 channels, 5x5, 832 filters 3x3, two images: 7.0 us, 9.1 resident; 1.04 to 1.30 over 19 drawn shapes).
   const int spread = (int)kSms / 2 / P.ntiles;
@@ -1532,7 +1535,7 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
       P.NT = slab_width(g.Co, ns, pair || fuse);
       P.nslabs = (g.Co + P.NT - 1) / P.NT;
       P.NTh = pair ? P.NT / 2 : P.NT;
-      if (P.nslabs > 1 && (!few || (fuse && ns > spread)) && (P.NT < (pair ? 96 : 128) || (!fuse && P.nsteps < 2 * P.nplanes && (pl.by_time = streams_faster())))) break;
+      if (P.nslabs > 1 && (!few || P.ntiles * ns > (int)kSms) && (P.NT < (pair ? 96 : 128) || (!fuse && P.nsteps < 2 * P.nplanes && (pl.by_time = streams_faster())))) break;
       // (Lending four of the weight warps to the patch builders where a pixel has many channel
       // words was the better split while the drain loop was longer; since its trimming twelve
       // draining warps win on every layer measured: conv4 50.4 -> 48.1 us, conv5 39.4 -> 37.3.)
