@@ -1511,9 +1511,10 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
   // fullest CTA from what was measured: per 16 columns drained 6 and 9 (with a residual 11 and 16), per plane
   // and 32 positions of a patch 1 (0.055 us).  79 images, 80 channels, 49x49, 912 filters 3x3 stride 2: 98 us
   // streaming, 60 resident; 37 images, 544 channels, 51x47, 256 filters 1x1 with a residual: 70 and 52; 128
-  // channels, 28x28, 256 filters 3x3 stride 2, 256 images: 27.0 and 29.5.  Without a residual streaming also wins
-  // within a sixth: there it is ahead of the estimate by up to 1.16 (170 images, 146 channels, 24x8, 800 filters
-  // 1x1 stride 2: 17.4 and 20.1 us).
+  // channels, 28x28, 256 filters 3x3 stride 2, 256 images: 27.0 and 29.5.  Without a residual streaming also
+  // wins within a tenth: of 14 drawn shapes where the sides differ by that or the choice was wrong, those up to
+  // 1.09 were faster streaming (72 images, 192 channels, 48x48, 400 filters 1x1 stride 2: 29.3 and 32.6 us),
+  // those from 1.12 resident (84 images, 720 channels, 17x53, 448 filters 1x1: 70 and 50 us).
   auto streams_faster = [&]() {
     const int snt = slab_width(g.Co, stream_slabs, pair || fuse), sns = (g.Co + snt - 1) / snt;
     const int patch = P.nplanes * ((P.ppix + 31) / 32), group = units / P.nslabs;
@@ -1522,7 +1523,7 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
     };
     const long long res = time((P.ntiles + group - 1) / group, (residual ? 11 : 6) * P.NT / 16, patch);
     const long long str = time(((long long)P.ntiles * sns + units - 1) / units, (residual ? 16 : 9) * snt / 16, (patch + sns - 1) / sns);
-    return (residual ? 6 : 5) * str < 6 * res;
+    return (residual ? 11 : 10) * str < 11 * res;
   };
   if (schedule == 0) {
     // Resident: the widest slab whose expanded rows fit beside two patches.  Every slab needs its own

@@ -72,7 +72,8 @@ def test_fused_streaming_drains_short_items_with_two_warps(shape, warps):
     ((255, 272, 7, 7, 768, 1, 2, 0), ("resident", 4, 192)),           # one patch each either way
     ((256, 128, 28, 28, 256, 3, 2, 1), ("streaming", 2, 128)),        # the patch is: built once per tile
     ((136, 944, 8, 19, 512, 1, 1, 0), ("streaming", 4, 128)),          # (pairs, where they fit, do not change that)
-    ((155, 432, 9, 9, 513, 1, 1, 0), ("streaming", 5, 112))])
+    ((155, 432, 9, 9, 513, 1, 1, 0), ("resident", 3, 176)),
+    ((61, 112, 28, 28, 272, 3, 2, 1), ("resident", 2, 144)), ((72, 192, 48, 48, 400, 1, 2, 0), ("streaming", 4, 112))])
 def test_slabs_of_few_steps_are_resident_where_that_is_faster(shape, expected):
     assert schedule(plan(*shape)) == expected
 
