@@ -24,6 +24,25 @@ __host__ __device__ constexpr float decision_point(int j, int kbits) {
   return (float)((double)(2 * j - 1) / (double)((1 << kbits) - 1) - 1.0);
 }
 
+// The decision point that settles bit L of the index once the bits above it are known: a tree of selects over
+// constants.  Bits TOP .. L + 1 remain to be looked at, BASE is what the bits above TOP add up to.
+template <int K, int L, int TOP, int BASE>
+__device__ __forceinline__ float bit_threshold(const bool (&b)[K]) {
+  if constexpr (TOP == L) {
+    constexpr float t = decision_point(BASE + (1 << L), K);
+    return t;
+  } else {
+    return b[TOP] ? bit_threshold<K, L, TOP - 1, BASE + (1 << TOP)>(b) : bit_threshold<K, L, TOP - 1, BASE>(b);
+  }
+}
+// Bits of the level index of y, K <= 4 planes: bit `bit` of words[p] is set where bit p of the index is.
+template <int K, int L = K - 1>
+__device__ __forceinline__ void set_index_bits(float y, uint32_t bit, bool (&b)[K], uint32_t (&words)[K]) {
+  b[L] = y >= bit_threshold<K, L, K - 1, 0>(b);
+  if (b[L]) words[L] |= bit;
+  if constexpr (L > 0) set_index_bits<K, L - 1>(y, bit, b, words);
+}
+
 // Persistent blocks of 8 warps.  A task is (group of 32 consecutive pixels, flat over n,h,w;
 // 32-channel word): lane = pixel, so one channel of a task is a contiguous 128-byte run of
 // x.  The G warps of a pixel group take words g, g + G, ...; a block works on 8 / G pixel
@@ -33,9 +52,12 @@ __host__ __device__ constexpr float decision_point(int j, int kbits) {
 // bandwidth needs) do not depend on how the compiler schedules loads against their uses.
 // Packed words are staged and written as contiguous runs; A is reduced over the warps of a
 // pixel group in a fixed order.
-// kBits: 1 = sign bits; 2 = two bit planes of the level index (decision points in registers); 0 = any
-// number of planes (bisection over the decision points in shared memory); see "BinActiv with k-bit
-// activations" below.  x_packed is then [kbits][N][H][W][Cw].
+// kBits: 1 = sign bits; 2 .. 4 = bit planes of the level index (decision points are constants); 0 = up to
+// seven planes (bisection over the decision points in shared memory); see "BinActiv with k-bit
+// activations" below.  x_packed is then [kbits][N][H][W][Cw].  The words of a pixel are built in registers:
+// in shared memory (a load and a store per value and plane) three and four planes were bound by that, slower
+// than the simple kernel below on many pixels (487 channels, 52x52, 32 images, k = 4: 664 us, 292 the simple
+// kernel, 98 now; 512 channels, 40x57, 40 images, k = 3: 559, 303, 47; half the time over 119 drawn shapes).
 template <bool kHasBN, bool kVec16, int kBits>
 __global__ void __launch_bounds__(32 * kWarps)
 binactiv_pack_kernel(const float *x, const float *scale,
@@ -46,7 +68,7 @@ binactiv_pack_kernel(const float *x, const float *scale,
   const int plane_words = PG * kPix * Cw;                  // staged words of a bit plane
   const size_t out_words = (size_t)total_pix * Cw;         // words of a bit plane of the tensor
   __shared__ float tau[kBits == 0 ? 128 : 1];
-  constexpr float t1 = decision_point(1, 2), t2 = decision_point(2, 2), t3 = decision_point(3, 2);
+  constexpr int kB = kBits > 0 ? kBits : 7;
   if (kBits == 0)
     for (int j = 1 + threadIdx.x; j < (1 << kbits); j += 32 * kWarps) tau[j] = decision_point(j, kbits);
   float *stage = reinterpret_cast<float *>(smem_raw);                      // [warp][buf][32][32]
@@ -139,27 +161,25 @@ binactiv_pack_kernel(const float *x, const float *scale,
       const int cw = g + k * G;
       const int c0 = cw * 32;
       const float *t = my_stage + buf * kTileFloats + lane;
-      uint32_t word = 0u, word2 = 0u;
+      uint32_t word[kB];
+#pragma unroll
+      for (int pl = 0; pl < kB; ++pl) word[pl] = 0u;
       float part = 0.0f;
-      if (kBits == 0) {
-        // any number of planes: the words are built in shared memory
-        float p0 = 0.0f, p1 = 0.0f;
-        uint32_t *w = words + (pgl * kPix + lane) * Cw + cw;
-        for (int pl = 0; pl < nplanes; ++pl) w[pl * plane_words] = 0u;
-        if (live) {
-          const int nc = min(32, C - c0);
-          for (int j = 0; j < nc; ++j) {
-            float y = t[j * kPix];
-            if (kHasBN) y = __fmaf_rn(bn[c0 + j].x, y, bn[c0 + j].y);
-            if (j & 1) p1 += fabsf(y); else p0 += fabsf(y);
-            int idx = 0;                       // the largest index whose decision point is <= y
-            for (int b = nplanes - 1; b >= 0; --b)
-              if (y >= tau[idx + (1 << b)]) idx += 1 << b;
-            for (int pl = 0; pl < nplanes; ++pl) w[pl * plane_words] |= (uint32_t)((idx >> pl) & 1) << j;
-          }
-          part = p0 + p1;
+      // channel j of the word: its bits, its |y|
+      auto take = [&](float y, int j, float &sum) {
+        sum += fabsf(y);
+        if constexpr (kBits > 0) {
+          bool b[kB];
+          set_index_bits<kB>(y, 1u << j, b, word);
+        } else {
+          int idx = 0;                         // the largest index whose decision point is <= y
+          for (int b = nplanes - 1; b >= 0; --b)
+            if (y >= tau[idx + (1 << b)]) idx += 1 << b;
+#pragma unroll
+          for (int pl = 0; pl < kB; ++pl) word[pl] |= (uint32_t)((idx >> pl) & 1) << j;   // bits beyond the planes are 0
         }
-      } else if (live) {
+      };
+      if (live) {
         const float2 *ss = bn + c0;
         if (c0 + 32 <= C) {
           // two interleaved sums keep the additions from forming one long dependent chain
@@ -171,39 +191,24 @@ binactiv_pack_kernel(const float *x, const float *scale,
               y0 = __fmaf_rn(ss[j].x, y0, ss[j].y);
               y1 = __fmaf_rn(ss[j + 1].x, y1, ss[j + 1].y);
             }
-            if (kBits == 1) {
-              if (y0 >= 0.0f) word |= 1u << j;
-              if (y1 >= 0.0f) word |= 2u << j;
-            } else {
-              // bit 1 of the index: y >= tau_2; bit 0: the parity of how many comparisons hold
-              const bool b0 = y0 >= t2, b1 = y1 >= t2;
-              if (b0 ? y0 >= t3 : y0 >= t1) word |= 1u << j;
-              if (b1 ? y1 >= t3 : y1 >= t1) word |= 2u << j;
-              if (b0) word2 |= 1u << j;
-              if (b1) word2 |= 2u << j;
-            }
-            p0 += fabsf(y0);
-            p1 += fabsf(y1);
+            take(y0, j, p0);
+            take(y1, j + 1, p1);
           }
           part = p0 + p1;
         } else {
+          float odd = 0.0f;                    // three planes and more: two sums here too
           for (int j = 0; c0 + j < C; ++j) {
             float y = t[j * kPix];
             if (kHasBN) y = __fmaf_rn(ss[j].x, y, ss[j].y);
-            if (kBits == 1) {
-              if (y >= 0.0f) word |= 1u << j;
-            } else {
-              const bool b = y >= t2;
-              if (b ? y >= t3 : y >= t1) word |= 1u << j;
-              if (b) word2 |= 1u << j;
-            }
-            part += fabsf(y);
+            take(y, j, kBits != 1 && kBits != 2 && (j & 1) ? odd : part);
           }
+          part += odd;
         }
       }
       asum += part;
-      if (kBits > 0) words[(pgl * kPix + lane) * Cw + cw] = word;
-      if (kBits == 2) words[plane_words + (pgl * kPix + lane) * Cw + cw] = word2;
+#pragma unroll
+      for (int pl = 0; pl < kB; ++pl)
+        if (kBits > 0 || pl < nplanes) words[pl * plane_words + (pgl * kPix + lane) * Cw + cw] = word[pl];
       __syncwarp();                      // every lane is done reading the tile before it is refilled
       issue(fb, fk, buf); advance_fetch();                   // refill the tile just consumed
       buf ^= 1;
@@ -249,7 +254,7 @@ binactiv_pack_kernel(const float *x, const float *scale,
 // only what it copied itself.  Tiles of 8 channels, kWideDepth in flight per warp: a few warps per SM
 // are enough to keep HBM busy, which evens out the last wave.  Bound by HBM; sums, bits and results as
 // above (G = 1).  With the box filter after it, 64x56x56: 256 images 45 -> 42 us, 64 images 14.0 -> 11.0;
-// 128x28x28, 256 images: 25.7 -> 23.0, two bit planes 32.9 -> 25.5.
+// 128x28x28, 256 images: 25.7 -> 23.0, two bit planes 32.9 -> 23.
 constexpr int kWidePix = 128, kWideCh = 8;
 constexpr int kWideWarps = 12, kWideDepth = 4;
 
@@ -958,7 +963,7 @@ template <int kBits>
 cudaError_t launch_pack(const float *x, const float *scale, const float *shift, const ConvGeom &g, const PackPlan &pl,
                         int kbits, uint32_t *x_packed, float *A, cudaStream_t st) {
   const bool v16 = ((g.H * g.W) & 3) == 0;
-  if constexpr (kBits > 0) {
+  if constexpr (kBits == 1 || kBits == 2) {
     if (v16 && pl.G == 1 && pack_wide_smem(g.C, scale != nullptr) <= kWideSmemMax)
       return scale ? launch_pack_wide<true, kBits>(x, scale, shift, g, x_packed, A, st)
                    : launch_pack_wide<false, kBits>(x, scale, shift, g, x_packed, A, st);
@@ -1120,12 +1125,14 @@ cudaError_t launch_binactiv_kbit(const float *x, const float *scale, const float
       return launch_binactiv_image(ip, scale != nullptr, sms, st);
     }
   }
-  // The pipelined pack kernel with k bit planes per tile (128x28x28, 256 images, k = 2: 30 us, the
-  // simple kernel below 127); the simple one where the staged words do not fit shared memory.
+  // The pipelined pack kernels with k bit planes per tile (128x28x28, 256 images, k = 2: 23 us with the box
+  // filter, the simple kernel below 127); the simple one where the staged words do not fit shared memory.
   PackPlan pl;
   if (pack_plan(g, scale != nullptr, &pl, kbits)) {
     cudaError_t e = kbits == 1 ? launch_pack<1>(x, scale, shift, g, pl, 1, x_planes, A, st)
                     : kbits == 2 ? launch_pack<2>(x, scale, shift, g, pl, 2, x_planes, A, st)
+                    : kbits == 3 ? launch_pack<3>(x, scale, shift, g, pl, 3, x_planes, A, st)
+                    : kbits == 4 ? launch_pack<4>(x, scale, shift, g, pl, 4, x_planes, A, st)
                                  : launch_pack<0>(x, scale, shift, g, pl, kbits, x_planes, A, st);
     if (e != cudaSuccess) return e;
     return launch_box_filter(A, g, K, st);

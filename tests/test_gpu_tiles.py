@@ -57,7 +57,7 @@ def test_shortcut_tiles(oracle, case):
 
 
 # one warp per pixel group and groups shared by warps; channel tails; 16- and 4-byte copies
-@pytest.mark.parametrize("kbits", [2, 3, 7])
+@pytest.mark.parametrize("kbits", [2, 3, 4, 5, 7])
 @pytest.mark.parametrize("case", [(90, 40, 28, 28, 3, 1), (2, 300, 10, 14, 5, 2), (3, 70, 9, 11, 3, 1)])
 def test_kbit_pack(oracle, case, kbits):
     N, C, H, W, k, p = case
@@ -78,6 +78,25 @@ def test_kbit_pack(oracle, case, kbits):
     A_or = oracle.channel_abs_mean(y)
     assert_close(host(A), A_or, "A")
     assert_close(host(K), oracle.box_filter(A_or, k, k, 1, p), "K")
+
+
+# the decision points themselves and their neighbours, whole and partial channel words
+@pytest.mark.parametrize("kbits", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("C,H", [(64, 8), (43, 8), (64, 7)])
+def test_kbit_decision_points(oracle, kbits, C, H):
+    levels = 2 ** kbits - 1
+    tau = np.array([(2 * j - 1) / levels - 1 for j in range(1, levels + 1)], np.float32)
+    edges = np.concatenate([tau, np.nextafter(tau, np.float32(-9)), np.nextafter(tau, np.float32(9)),
+                            np.array([0.0, -0.0, 1, -1, 3, -3, np.inf, -np.inf], np.float32)])
+    x = rng(kbits + C).choice(edges, (2, C, H, H)).astype(np.float32)
+    d = X.make_desc(2, C, H, H, 8, 1, 1, 1, 0)
+    gs = GuardSet()
+    planes = gs.new("x_planes", (kbits, 2, H, H, (C + 31) // 32), torch.int32)
+    _, A, K = X.alloc_binactiv(d)
+    X.xnor_binactiv_kbit(dev(x), None, None, d, kbits, planes, A, K)
+    gs.check()
+    codes = 2 * _index_of_planes(host(planes), C) - levels
+    assert np.array_equal(codes, oracle.quantize_k(x, kbits).astype(np.int64))
 
 
 # pixels not a multiple of the 128 of a warp, images ending inside a run; one to five channel words, tails
