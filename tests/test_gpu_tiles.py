@@ -27,7 +27,10 @@ def rng(seed):
 # (N, C, H, W, k, stride, pad): a last chunk of one plane and a tensor that is not a multiple of four
 # floats; several planes per chunk; clipped windows; the largest planes that are streamed
 @pytest.mark.parametrize("relu", [False, True])
-@pytest.mark.parametrize("case", [(197, 193, 9, 7, 2, 2, 0), (150, 256, 13, 13, 3, 2, 0),
+@pytest.mark.parametrize("case", [(11, 256, 36, 34, 3, 2, 1), (9, 301, 30, 37, 2, 3, 1), (24, 128, 35, 35, 4, 3, 3),
+                                  (40, 90, 21, 23, 5, 2, 4), (7, 400, 30, 31, 7, 2, 3), (40, 90, 21, 23, 6, 2, 3),
+                                  (90, 129, 11, 12, 1, 2, 0),
+                                  (197, 193, 9, 7, 2, 2, 0), (150, 256, 13, 13, 3, 2, 0),
                                   (10, 256, 27, 27, 3, 2, 1), (3, 805, 38, 40, 5, 3, 2)])
 def test_streamed_maxpool_is_exact(oracle, case, relu):
     N, C, H, W, k, s, p = case
@@ -41,8 +44,10 @@ def test_streamed_maxpool_is_exact(oracle, case, relu):
     assert np.array_equal(host(out), want)
 
 
-# large, middle and small tiles; channel, filter and pixel tails; planes of odd size
-@pytest.mark.parametrize("case", [(64, 64, 28, 28, 130, 1), (40, 70, 57, 55, 96, 2), (16, 128, 28, 28, 256, 2),
+# tiles of 64 x 32 (the first two, with tails of pixels, channels and filters, and the fifth), 128 x 64 (the two
+# between) and 32 x 16 by the rule of launch_shortcut_conv1x1 on 148 SMs; planes of odd size
+@pytest.mark.parametrize("case", [(14, 131, 29, 29, 250, 2), (13, 45, 17, 14, 230, 1),
+                                  (64, 64, 28, 28, 130, 1), (40, 70, 57, 55, 96, 2), (16, 128, 28, 28, 256, 2),
                                   (5, 70, 15, 13, 90, 1), (2, 256, 14, 14, 512, 2), (1, 33, 9, 9, 40, 2)])
 def test_shortcut_tiles(oracle, case):
     N, C, H, W, Co, s = case
