@@ -152,9 +152,7 @@ struct TcParams {
   uint32_t raw_plane;          // the share of one bit plane
   const uint32_t *xp2;         // two bit planes in one pass: the upper one (see patch_role)
   int nraw;                    // raw buffers per subgroup of patch warps (1 or 2)
-  int pat_group;               // warps that build patches
-  int pat_sub;                 // subgroups they form (each builds whole patches): 3 or 1
-  int wgt_warps;               // warps that expand weights: 8, or 4
+  int pat_sub;                 // subgroups of the patch warps (each builds whole patches): 3 or 1
   uint32_t idesc;
   uint32_t tail_mask;          // bits of real channels in the last word
   // Low word of the A-operand descriptor of every K-step (start address relative to the
@@ -328,34 +326,25 @@ __device__ __forceinline__ uint32_t fast_div(uint32_t n, uint32_t m, int s) {
 // together lie together in memory (measured on 27x27 planes: 3.9 TB/s of stores against
 // 2.85 TB/s when every CTA owns a contiguous range of tiles).
 struct ResSched {
-  uint32_t ntiles, nslabs;
+  uint32_t ntiles;
   uint32_t slab, g, G;           // this unit's slab, its index in the slab's group, the group's size
-  __device__ __forceinline__ uint32_t first(uint32_t s) const { return g; }
-  __device__ __forceinline__ uint32_t step() const { return G; }
-  __device__ __forceinline__ uint32_t count(uint32_t s) const {
-    return (s == slab && g < ntiles) ? (ntiles - g + G - 1u) / G : 0u;
-  }
-  __device__ __forceinline__ uint32_t total() const { return count(slab); }
-  // the seq-th item of the unit (seq < total()): its slab and tile
-  __device__ __forceinline__ void item(uint32_t seq, uint32_t &sl, uint32_t &tile) const {
-    sl = slab;
-    tile = g + seq * G;
-  }
+  __device__ __forceinline__ uint32_t total() const { return g < ntiles ? (ntiles - g + G - 1u) / G : 0u; }
+  __device__ __forceinline__ uint32_t tile(uint32_t seq) const { return g + seq * G; }    // seq < total()
 };
 
 __device__ __forceinline__ ResSched res_sched(int ntiles, int nslabs, bool pair) {
   ResSched R;
   const uint32_t unit = pair ? blockIdx.x >> 1 : blockIdx.x;
   const uint32_t units = pair ? gridDim.x >> 1 : gridDim.x;    // >= nslabs (host)
+  const uint32_t ns = (uint32_t)nslabs;
   R.ntiles = (uint32_t)ntiles;
-  R.nslabs = (uint32_t)nslabs;
   // group s = units [s U / nslabs, (s + 1) U / nslabs)
-  R.slab = unit * R.nslabs / units;
-  while ((R.slab + 1u) * units / R.nslabs <= unit) ++R.slab;
-  while (R.slab * units / R.nslabs > unit) --R.slab;
-  const uint32_t g0 = R.slab * units / R.nslabs;
+  R.slab = unit * ns / units;
+  while ((R.slab + 1u) * units / ns <= unit) ++R.slab;
+  while (R.slab * units / ns > unit) --R.slab;
+  const uint32_t g0 = R.slab * units / ns;
   R.g = unit - g0;
-  R.G = (R.slab + 1u) * units / R.nslabs - g0;
+  R.G = (R.slab + 1u) * units / ns - g0;
   return R;
 }
 
@@ -577,23 +566,13 @@ __device__ __forceinline__ void mma_role(const TcParams &P, const Smem &S, long 
 // The packed words of kPrefetch stages are in flight in registers.
 constexpr int kPrefetch = 3;
 
-struct WCursor {
-  long long item;
-  int st, slab;
-};
-
 // kUnits = grp_steps: K-steps a thread expands per stage.  kSwap: some K-step has its two
 // pieces in descending address order (odd Cw or stride 2); otherwise the swap test is compiled
 // out.  The common stage (all its K-steps exist, none is the row's lone last word) takes a
 // path without per-step predicates.
-// The role fills the stages of `nitems` consecutive items, the first of slab `slab0` (the
-// slabs then follow cyclically), waiting for the empty barriers with parity `wph0` on the
-// first round: one call per slab visit with nitems = 1 (the ring has one stage per stage of
-// the slab).
+// The role fills the ring once: it has one stage per stage of the slab, so nothing is waited for.
 template <int kUnits, bool kSwap>
-__device__ bool weight_role(const TcParams &P, const Smem &S, long long nitems, int slab0,
-                            uint32_t wph0, int wt, int lane) {
-  const long long i0 = 0, i1 = nitems;
+__device__ void weight_role(const TcParams &P, const Smem &S, int slab, int wt, int lane) {
   const int nst = (P.nsteps + P.mps - 1) / P.mps;
   const int row = wt % P.rows_mod, grp = wt / P.rows_mod;
   constexpr int gs = kUnits;
@@ -602,16 +581,12 @@ __device__ bool weight_role(const TcParams &P, const Smem &S, long long nitems, 
   const int row_co = (int)S.rank * P.NTh + row;          // this thread's filter inside a slab
   const int jj0 = grp * gs;                         // first K-step of this thread inside a stage
   const int nplain = (P.row_words >> 1);            // K-steps j < nplain have both words
-  WCursor fc{i0, 0, slab0}, cc{i0, 0, slab0};
-  auto advance = [&](WCursor &c) {
-    if (++c.st == nst) { c.st = 0; ++c.item; if (++c.slab == P.nslabs) c.slab = 0; }
-  };
+  const int co = slab * P.NT + row_co;
+  const bool on = grp_on && co < P.Co;
   const uint2 *wp2 = reinterpret_cast<const uint2 *>(P.wp);
   uint2 pf[kPrefetch][kUnits];
-  auto fetch = [&](uint2 dst[kUnits], const WCursor &c) {
-    const int co = c.slab * P.NT + row_co;
-    const bool on = grp_on && c.item < i1 && co < P.Co;
-    const int j0 = c.st * P.mps + jj0;
+  auto fetch = [&](uint2 dst[kUnits], int st) {
+    const int j0 = st * P.mps + jj0;                // beyond the last stage every K-step is beyond nsteps
     if (on && j0 + gs <= P.nsteps) {
       const uint2 *src = wp2 + ((size_t)j0 * P.Co + co);
 #pragma unroll
@@ -624,21 +599,14 @@ __device__ bool weight_role(const TcParams &P, const Smem &S, long long nitems, 
     }
   };
 #pragma unroll
-  for (int d = 0; d < kPrefetch; ++d) { fetch(pf[d], fc); advance(fc); }
-  int ws = 0;
-  uint32_t wph = wph0;        // parity to wait for on the empty barriers
-  bool ok = true;
+  for (int d = 0; d < kPrefetch; ++d) fetch(pf[d], d);
   const uint32_t row_off = (uint32_t)row * 16u + (uint32_t)(2 * jj0) * b_lbo;
   const uint32_t ring_end = S.ring + (uint32_t)P.stages * P.stage_bytes;
   (void)ring_end;
 #pragma unroll 1
-  while (cc.item < i1 && ok) {
-    ok = mbar_wait_relaxed(S.wempty + 8u * ws, wph, S.abort_flag, &g_status_tc, XNOR_SLEEP_WGT);
-    if (!ok) break;
-    const uint32_t stage = S.ring + (uint32_t)ws * P.stage_bytes + row_off;
-    const int co = cc.slab * P.NT + row_co;
-    const int j0 = cc.st * P.mps + jj0;
-    const bool on = grp_on && co < P.Co;
+  for (int st = 0; st < nst; ++st) {
+    const uint32_t stage = S.ring + (uint32_t)st * P.stage_bytes + row_off;
+    const int j0 = st * P.mps + jj0;
     if (on && j0 + gs <= nplain) {
       // plain stage: every K-step of this thread exists and has both of its words
       uint32_t sbits = 0u;                      // swap bits of K-steps j0 .. j0 + gs - 1
@@ -679,36 +647,29 @@ __device__ bool weight_role(const TcParams &P, const Smem &S, long long nitems, 
     }
     fence_proxy_async();
     __syncwarp();
-    if (lane == 0) { if (P.pair) mbar_arrive_cluster(S.wfull + 8u * ws, 0u); else mbar_arrive(S.wfull + 8u * ws); }
-    if (++ws == P.stages) { ws = 0; wph ^= 1u; }
-    advance(cc);
+    if (lane == 0) { if (P.pair) mbar_arrive_cluster(S.wfull + 8u * st, 0u); else mbar_arrive(S.wfull + 8u * st); }
     // the queue of packed words moves up one stage; the freed slot is refilled
 #pragma unroll
     for (int d = 0; d + 1 < kPrefetch; ++d)
 #pragma unroll
       for (int u = 0; u < kUnits; ++u) pf[d][u] = pf[d + 1][u];
-    fetch(pf[kPrefetch - 1], fc);
-    advance(fc);
+    fetch(pf[kPrefetch - 1], st + kPrefetch);
   }
-  return ok;
 }
 
 template <int kUnits>
-__device__ __forceinline__ bool weight_role_swap(const TcParams &P, const Smem &S,
-                                                 long long nitems, int slab0, uint32_t wph0,
-                                                 int wt, int lane) {
-  return P.any_swap ? weight_role<kUnits, true>(P, S, nitems, slab0, wph0, wt, lane)
-                    : weight_role<kUnits, false>(P, S, nitems, slab0, wph0, wt, lane);
+__device__ __forceinline__ void weight_role_swap(const TcParams &P, const Smem &S, int slab, int wt, int lane) {
+  if (P.any_swap) weight_role<kUnits, true>(P, S, slab, wt, lane);
+  else weight_role<kUnits, false>(P, S, slab, wt, lane);
 }
 
-__device__ __forceinline__ bool weight_dispatch(const TcParams &P, const Smem &S, long long nitems,
-                                                int slab0, uint32_t wph0, int wt, int lane) {
-  if (P.grp_steps == 4) return weight_role_swap<4>(P, S, nitems, slab0, wph0, wt, lane);
-  if (P.grp_steps == 2) return weight_role_swap<2>(P, S, nitems, slab0, wph0, wt, lane);
-  return weight_role_swap<1>(P, S, nitems, slab0, wph0, wt, lane);
+__device__ __forceinline__ void weight_dispatch(const TcParams &P, const Smem &S, int slab, int wt, int lane) {
+  if (P.grp_steps == 4) weight_role_swap<4>(P, S, slab, wt, lane);
+  else if (P.grp_steps == 2) weight_role_swap<2>(P, S, slab, wt, lane);
+  else weight_role_swap<1>(P, S, slab, wt, lane);
 }
 
-// ---- streaming schedule: twelve warps
+// ---- streaming schedule: three groups of four warps, or two
 // The groups of four warps fill the stages of the sequence over all items in turn: with every warp on
 // every stage the expansion was bound by its latency (one instruction in 10 to 15 cycles per warp next
 // to the other roles, barriers and bookkeeping per stage).  A thread expands up to four K-steps of one
@@ -784,7 +745,7 @@ __device__ void weight_stream(const TcParams &P, const Smem &S, uint32_t nitems,
 }
 
 // ------------------------------------------------------------------ patch producers
-// A group of P.pat_group warps (the three patch warps) builds the CTA's patches one after the
+// The group of the three patch warps builds the CTA's patches one after the
 // other, all warps on the same patch: units of (32 stream positions, phase plane, up to 4 channel words) are dealt round
 // robin.  The packed pixels a patch touches are ONE contiguous range of x_packed: input rows
 // g0 .. g1 - 1 of the N*H rows (images follow one another in memory, the zero rows and
@@ -822,12 +783,7 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
   const int nunits = npass * phases * ngrp;
 
   constexpr int kPatUnits = kRes && !kTwo ? 2 : 1;                 // patch units a warp works on together (registers)
-  auto tile_of = [&](uint32_t seq) {
-    if (!kRes) return tile0 + (int)seq;
-    uint32_t sl, t;
-    R.item(seq, sl, t);
-    return (int)t;
-  };
+  auto tile_of = [&](uint32_t seq) { return kRes ? (int)R.tile(seq) : tile0 + (int)seq; };
   // input rows [g0, g1) (of the N*H rows of the tensor) that the patch of a tile reads
   auto row_range = [&](int tile, int &g0, int &g1) {
     const uint32_t m0 = ((uint32_t)tile * tmul + S.rank) * kTileM;
@@ -871,7 +827,7 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
   // The group works as `nsub` subgroups of equal size; subgroup sg builds patches sg,
   // sg + nsub, ... (nsub <= npb: a barrier's parity tells apart only two consecutive uses of
   // a buffer, so no subgroup may run more than one use ahead of the consumer).
-  const uint32_t nsub = (uint32_t)P.pat_sub, gsize = (uint32_t)P.pat_group / nsub;
+  const uint32_t nsub = (uint32_t)P.pat_sub, gsize = (uint32_t)kPatWarps / nsub;
   const uint32_t sg = (uint32_t)pw % nsub, mi = (uint32_t)pw / nsub;
   // The subgroup's k-th patch (patch sg + k nsub of the CTA) expands from the subgroup's raw
   // buffer k % nraw; its rows are fetched as soon as the subgroup is done with patch k - nraw.
@@ -1011,16 +967,15 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
 // Warp w reads tensor-memory lanes 32 w .. +31 (pixels), all the slab's columns (filters).
 // Lane = pixel, so for one filter a warp stores 32 consecutive stream pixels: a contiguous
 // run of the NCHW output row.
-// Drains `nitems` items, the k0-th and following of the CTA: streaming, items i0, i0 + 1, ...
+// Drains the CTA's `nitems` items: streaming, items i0, i0 + 1, ...
 // (item = tile * nslabs + slab); resident, tiles tile0, tile0 + tstep, ... of slab `slab0`.
 // Of every item this warp takes
 // the 16-column groups e, e + esplit, ... (esplit warps share a quarter of the lanes).
 // kFuse: the groups a warp takes come in pairs (32 consecutive filters = one packed word of the
 // next layer's input); see the fused emit below.
 template <bool kRes, bool kFuse>
-__device__ bool epilogue_role(const TcParams &P, const Smem &S, long long i0, int slab0, int tile0,
-                              int tstep, uint32_t nitems, long long k0, uint32_t tmem_base,
-                              int quarter, int e, int lane) {
+__device__ void epilogue_role(const TcParams &P, const Smem &S, long long i0, int slab0, int tile0,
+                              int tstep, uint32_t nitems, uint32_t tmem_base, int quarter, int e, int lane) {
   const int b_end = P.NT / 16;
   const int esplit = P.epi_split;
   // the k-th group of this warp: groups e, e + esplit, ... or, fused, the two groups of the
@@ -1064,8 +1019,8 @@ __device__ bool epilogue_role(const TcParams &P, const Smem &S, long long i0, in
     return px;
   };
   Pix px = decode(tile);
-  int ab = (int)(k0 % P.nacc);            // accumulator buffer of the next item and the parity
-  uint32_t fph = (uint32_t)(k0 / P.nacc) & 1u;   // of its full barrier
+  int ab = 0;                             // accumulator buffer of the next item and the parity
+  uint32_t fph = 0u;                      // of its full barrier
   for (uint32_t it = 0; it < nitems && ok; ++it) {
     const bool valid = px.valid;
     const float kv = px.kv;
@@ -1261,7 +1216,6 @@ __device__ bool epilogue_role(const TcParams &P, const Smem &S, long long i0, in
     slab = nslab;
     if (++ab == P.nacc) { ab = 0; fph ^= 1u; }
   }
-  return ok;
 }
 
 template <bool kRes, bool kPair, bool kFuse, bool kTwo>
@@ -1277,16 +1231,16 @@ binconv_tc_kernel(const __grid_constant__ TcParams P) {
     // waits for them); the MMA warp's commits reach the consumer barriers of both CTAs.
     constexpr uint32_t kCtas = kPair ? 2u : 1u;
     for (int i = 0; i < kMaxBarStages; ++i) {
-      mbar_init(S.wfull + 8u * i, (uint32_t)(kRes ? P.wgt_warps : kGroupWarps) * kCtas);
+      mbar_init(S.wfull + 8u * i, (uint32_t)(kRes ? kWgtWarps : kGroupWarps) * kCtas);
       mbar_init(S.wempty + 8u * i, 1);
     }
     for (int i = 0; i < kMaxPatchBufs; ++i) {
-      mbar_init(S.pfull + 8u * i, (uint32_t)(P.pat_group / P.pat_sub) * kCtas);
+      mbar_init(S.pfull + 8u * i, (uint32_t)(kPatWarps / P.pat_sub) * kCtas);
       mbar_init(S.pempty + 8u * i, 1);
     }
     for (int i = 0; i < kMaxRaw; ++i) {
       mbar_init(S.rawfull + 8u * i, 1);
-      mbar_init(S.rawdone + 8u * i, (uint32_t)(P.pat_group / P.pat_sub));
+      mbar_init(S.rawdone + 8u * i, (uint32_t)(kPatWarps / P.pat_sub));
     }
     for (int i = 0; i < kMaxAcc; ++i) {
       mbar_init(S.afull + 8u * i, 1);
@@ -1357,7 +1311,7 @@ binconv_tc_kernel(const __grid_constant__ TcParams P) {
       const int wi = ((warp >> 2) - 1) * 3 + (warp & 3) - 1 - kGroupWarps * P.wgt_groups;
       const bool last = warp >= kThreadsStream / 32 - kEpiWarps && P.epi_split == 2;
       if (warp < kEpiWarps || last)
-        epilogue_role<false, kFuse>(P, S, i0, 0, 0, 0, (uint32_t)(i1 - i0), 0, tmem_base, warp & 3, last ? 1 : 0, lane);
+        epilogue_role<false, kFuse>(P, S, i0, 0, 0, 0, (uint32_t)(i1 - i0), tmem_base, warp & 3, last ? 1 : 0, lane);
       else if ((warp & 3) == 0) {}
       else if (wi < 0) {
         const int group = (wi >> 2) + P.wgt_groups, t = 32 * (wi & 3) + lane, slab0 = (int)(i0 % P.nslabs);
@@ -1368,22 +1322,12 @@ binconv_tc_kernel(const __grid_constant__ TcParams P) {
     }
     else if (warp >= kPatWarp0) patch_role<kRes, kTwo>(P, S, i0, i1, warp - kPatWarp0, lane);
     else {
-      // Slab visits of this CTA in order.  The weight warps expand the slab, then every
-      // worker warp drains its share of the visit's items.
+      // The weight warps expand the slab, then every worker warp drains its share of the items.
       const bool wgt = warp >= kWgtWarp0;
       const int e = wgt ? 1 + (warp - kWgtWarp0) / 4 : 0;
-      uint32_t visit = 0, done = 0;
-      bool ok = true;
-      for (uint32_t slab = 0; slab < R.nslabs && ok; ++slab) {
-        const uint32_t n = R.count(slab);
-        if (n == 0u) continue;
-        if (wgt) ok = weight_dispatch(P, S, 1, (int)slab, (visit & 1u) ^ 1u, wt, lane);
-        if (ok && e < P.epi_split)
-          ok = epilogue_role<true, kFuse>(P, S, 0, (int)slab, (int)R.first(slab), (int)R.step(), n,
-                                          done, tmem_base, warp & 3, e, lane);
-        done += n;
-        ++visit;
-      }
+      if (wgt) weight_dispatch(P, S, (int)R.slab, wt, lane);
+      if (e < P.epi_split)
+        epilogue_role<true, kFuse>(P, S, 0, (int)R.slab, (int)R.g, (int)R.G, R.total(), tmem_base, warp & 3, e, lane);
     }
   }
   tc_fence_before();
@@ -1416,7 +1360,7 @@ void plan_stage(TcParams &P, bool few) {
   int ntp = 16;
   while (ntp < P.NTh) ntp *= 2;                         // 16 .. 256
   P.rows_mod = ntp;
-  const int groups = std::max(1, 32 * P.wgt_warps / P.rows_mod);   // 1 .. 16
+  const int groups = std::max(1, 32 * kWgtWarps / P.rows_mod);   // 1 .. 16
   P.mps = std::max(2, std::min(few ? 32 : 8, 1024 / ntp));
   while (P.mps > 4 && P.nsteps < (few ? 2 : 3) * P.mps) P.mps /= 2;   // short items: smaller stages start sooner
   if (P.mps > 4 * groups) P.mps = 4 * groups;           // a thread expands at most 4 K-steps of a stage
@@ -1476,13 +1420,11 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
   if (P.off_ring + 4096 > kSmemMax) return pl;
   const size_t avail = kSmemMax - P.off_ring;
   // st weight stages, pb patch buffers, nraw raw buffers for each subgroup of patch warps
-  auto subgroups = [&](int pb) { return (P.pat_group == kPatWarps && pb >= kPatWarps) ? kPatWarps : 1; };
+  auto subgroups = [&](int pb) { return pb >= kPatWarps ? kPatWarps : 1; };
   auto fits = [&](int st, int pb, int nraw) {
     return (size_t)st * P.stage_bytes + (size_t)pb * P.patch_bytes +
            (size_t)(subgroups(pb) * nraw) * P.raw_bytes <= avail;
   };
-  P.wgt_warps = kWgtWarps;
-  P.pat_group = kPatWarps;
   // as few slabs as fit two accumulators in the tensor-memory columns
   const int max_nt = pair ? 224 : 240;
   int min_slabs = (g.Co + max_nt - 1) / max_nt;
@@ -1540,8 +1482,6 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
       // (Lending four of the weight warps to the patch builders where a pixel has many channel
       // words was the better split while the drain loop was longer; since its trimming twelve
       // draining warps win on every layer measured: conv4 50.4 -> 48.1 us, conv5 39.4 -> 37.3.)
-      P.wgt_warps = kWgtWarps;
-      P.pat_group = kPatWarps;
       plan_stage(P, few);
       const int nst = (P.nsteps + P.mps - 1) / P.mps;
       if (nst <= kMaxBarStages && fits(nst, 2, 1)) {
@@ -1575,8 +1515,6 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
     P.NT = slab_width(g.Co, ns, pair || fuse);
     P.nslabs = (g.Co + P.NT - 1) / P.NT;
     P.NTh = pair ? P.NT / 2 : P.NT;
-    P.wgt_warps = kWgtWarps;
-    P.pat_group = kPatWarps;
     // stages of four units per thread of a group of warps (see weight_stream), shorter ones where the
     // patch leaves little room; a stage per group at least
     if (P.NTh > 32 * kGroupWarps) return pl;             // a thread expands one row
