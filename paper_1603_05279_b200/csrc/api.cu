@@ -217,7 +217,7 @@ xnor_status xnor_conv2d_forward_kbit(const uint32_t *x_planes, int kbits, const 
   // With index bits b_p the level code is sum_p 2^p (2 b_p - 1), so the sum over codes is
   // sum_p 2^p (sum over plane p).  A pass of the tensor-core engine takes two planes where their rows fit
   // beside each other (the codes -3, -1, 1, 3 are values of its operand type; 128 channels, 28x28, 256
-  // images, k = 2: one convolution of 45 us instead of two), else one; the pass from plane p on adds
+  // images, k = 2: one convolution of 35 us instead of two), else one; the pass from plane p on adds
   // D K alpha 2^p / (2^k - 1) to what the passes before it wrote (the output is its own residual).
   const double levels = (double)((1 << kbits) - 1);
   const bool pairs = planes_in_pairs(g, engine, choice);

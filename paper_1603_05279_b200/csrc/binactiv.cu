@@ -254,7 +254,7 @@ binactiv_pack_kernel(const float *x, const float *scale,
 // only what it copied itself.  Tiles of 8 channels, kWideDepth in flight per warp: a few warps per SM
 // are enough to keep HBM busy, which evens out the last wave.  Bound by HBM; sums, bits and results as
 // above (G = 1).  With the box filter after it, 64x56x56: 256 images 45 -> 42 us, 64 images 14.0 -> 11.0;
-// 128x28x28, 256 images: 25.7 -> 23.0, two bit planes 32.9 -> 23.
+// 128x28x28, 256 images: 25.7 -> 23.0, two bit planes 32.9 -> 24.
 constexpr int kWidePix = 128, kWideCh = 8;
 constexpr int kWideWarps = 12, kWideDepth = 4;
 
@@ -1125,7 +1125,7 @@ cudaError_t launch_binactiv_kbit(const float *x, const float *scale, const float
       return launch_binactiv_image(ip, scale != nullptr, sms, st);
     }
   }
-  // The pipelined pack kernels with k bit planes per tile (128x28x28, 256 images, k = 2: 23 us with the box
+  // The pipelined pack kernels with k bit planes per tile (128x28x28, 256 images, k = 2: 24 us with the box
   // filter, the simple kernel below 127); the simple one where the staged words do not fit shared memory.
   PackPlan pl;
   if (pack_plan(g, scale != nullptr, &pl, kbits)) {

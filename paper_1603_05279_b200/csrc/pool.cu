@@ -187,7 +187,7 @@ cudaError_t launch_maxpool2d(const float *x, int N, int C, int H, int W, int k, 
   const Magic dh = magic((uint32_t)(Ho * Wo)), dw = magic((uint32_t)Wo);
   // Streamed when chunks of at least four planes and at most 24 KB exist, enough of them for several
   // rounds of every block (as many blocks per SM as fit, four chunks each).  AlexNet's 3x3/2 pool of conv2's
-  // output (235 MB): 92 us with a thread per output, bounded by its nine global loads, 44 us streamed (5.3 TB/s).
+  // output (235 MB): 92 us with a thread per output, bounded by its nine global loads, 47 us streamed (5 TB/s).
   const size_t four = 16 * (size_t)H * W;
   if (four <= 24 * 1024 && (k <= 5 || k == 7)) {
     PoolParams P;
