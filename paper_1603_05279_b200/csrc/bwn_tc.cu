@@ -628,6 +628,8 @@ BwnPlan make_plan(const ConvGeom &g) {
   P.ntaps = g.kh * g.kw;
   P.nwords = P.ntaps * g.Cw;
   const int halo = (q.dymax - q.dymin) * q.Wq + (q.dxmax - q.dxmin);
+  // the window of one tile: 256 positions was the most a tiled copy took; the bulk copies do not need the limit,
+  // which stays because no wider window has been tested or timed
   if ((kTileM + halo + 7) / 8 * 8 > 256) return pl;
   if (q.L + 4 * kTileM + 256 >= (1ll << 31)) return pl;
   // filter slabs: as few as fit two accumulators into the tensor-memory columns
