@@ -1435,7 +1435,8 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
   // filters: every slab adds planes of partial sums (352 channels, 9x9, 224 filters 3x3: 21.4 us in slabs of
   // 128, 13.3 of 64, 15.8 of 32; 0.87 of the time in the median of 68 drawn shapes of up to four images).
   // Narrower slabs than those that spread the problem stay one item per SM (480 channels, 51x51, 192 filters
-  // 3x3, three images, in 12 resident slabs of 16: 28.7 us, streaming 14.8).
+  // 3x3, three images, in 12 resident slabs of 16: 28.7 us, streaming 14.8); with two bit planes, whose patches
+  // cost more, two items (256 channels, 23x23, 120 filters 5x5, 12 images, k = 2: 16.3 us, streaming 22.1).
   // Beyond 16 slabs the resident search below gives up and the shape streams, which is the faster there
   // (16 channels, 5x5, 832 filters 3x3, two images: 7.0 us, 9.1 resident; 1.04 to 1.30 over 19 drawn shapes).
   const int spread = (int)kSms / 2 / P.ntiles;
@@ -1478,7 +1479,7 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
       P.NT = slab_width(g.Co, ns, pair || fuse);
       P.nslabs = (g.Co + P.NT - 1) / P.NT;
       P.NTh = pair ? P.NT / 2 : P.NT;
-      if (P.nslabs > 1 && (!few || P.ntiles * ns > (int)kSms) && (P.NT < (pair ? 96 : 128) || (!fuse && P.nsteps < 2 * P.nplanes && (pl.by_time = streams_faster())))) break;
+      if (P.nslabs > 1 && (!few || P.ntiles * ns > (int)kSms * planes) && (P.NT < (pair ? 96 : 128) || (!fuse && P.nsteps < 2 * P.nplanes && (pl.by_time = streams_faster())))) break;
       // (Lending four of the weight warps to the patch builders where a pixel has many channel
       // words was the better split while the drain loop was longer; since its trimming twelve
       // draining warps win on every layer measured: conv4 50.4 -> 48.1 us, conv5 39.4 -> 37.3.)

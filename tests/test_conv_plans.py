@@ -96,3 +96,10 @@ def test_small_fused_problems_are_spread(shape, expected):
     ((113, 544, 27, 5, 576, 5, 1, 2), ("pair streaming", 5, 128))])    # seven short rounds beat four long ones
 def test_pairs_stream_the_slabs_that_save_rounds(shape, expected):
     assert schedule(plan(*shape)) == expected
+
+
+def test_a_small_problem_keeps_one_item_per_sm():
+    """59 tiles: slabs of 32 filters are two items per SM, which two bit planes are worth and one is not."""
+    shape = (12, 256, 23, 23, 120, 5, 1, 2)
+    assert plan(*shape, kbits=2).resident and not plan(*shape).resident
+    assert not plan(3, 480, 51, 51, 192, 3).resident
