@@ -61,7 +61,7 @@
 //  shared memory beside two patches, the slab is expanded ONCE per CTA and the
 //  CTA then walks the pixel tiles of that slab (items in slab-major order, one
 //  patch per item); the weight warps, idle after the fill, join the epilogue
-//  (three warps per quarter of the lanes, splitting the columns).  "Streaming":
+//  (three warps per quarter of the lanes, taking chunks of the items in turn).  "Streaming":
 //  otherwise the weights of every item pass through a ring of stages (items in
 //  tile-major order, so that a patch serves all slabs of its tile).
 #include <algorithm>
@@ -170,11 +170,12 @@ struct TcParams {
   // layer's channels) and sums |y| over the filters it handles.
   const float *nscale, *nshift;      // [C_out], both null = identity
   uint32_t *xp_next;                 // u32 [N][Ho][Wo][Cw_next]
-  float *A_part;                     // fp32 [nslabs * epi_split][N][Ho][Wo]: partial sums of |y|
+  float *A_part;                     // fp32 [nslabs * epi_chunks][N][Ho][Wo]: partial sums of |y|
   int Cw_next;                       // ceil(C_out / 32)
   int resident;                // 1: resident schedule (stages = all stages of a slab)
   int wgt_groups;              // streaming: groups of four warps that expand weights, 3 or 2
-  int epi_split;               // warps per lane quarter that drain an accumulator
+  int epi_split;               // warps per lane quarter that drain accumulators
+  int epi_chunk, epi_chunks;   // groups of 16 columns that a warp drains in one go; such chunks of an item
   int any_swap;                // some bit of swap_mask is set
   uint32_t div_wq_m, div_hq_m; // multipliers and shifts of the exact divisions by Wq and Hq
   int div_wq_s, div_hq_s;      // (dividends below 2^31)
@@ -969,22 +970,16 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
 // run of the NCHW output row.
 // Drains the CTA's `nitems` items: streaming, items i0, i0 + 1, ...
 // (item = tile * nslabs + slab); resident, tiles tile0, tile0 + tstep, ... of slab `slab0`.
-// Of every item this warp takes
-// the 16-column groups e, e + esplit, ... (esplit warps share a quarter of the lanes).
-// kFuse: the groups a warp takes come in pairs (32 consecutive filters = one packed word of the
-// next layer's input); see the fused emit below.
+// An item is cut into chunks of epi_chunk groups of 16 columns, and the chunks of all items in sequence are
+// dealt to the esplit warps that share a quarter of the lanes: a warp's work per item (decoding its pixel,
+// the waits) is then spread over a whole chunk.
+// kFuse: a chunk is an even number of groups (a pair = 32 consecutive filters = one packed word of the
+// next layer's input) and has a plane of partial sums of its own; see the fused emit below.
 template <bool kRes, bool kFuse>
 __device__ void epilogue_role(const TcParams &P, const Smem &S, long long i0, int slab0, int tile0,
                               int tstep, uint32_t nitems, uint32_t tmem_base, int quarter, int e, int lane) {
   const int b_end = P.NT / 16;
-  const int esplit = P.epi_split;
-  // the k-th group of this warp: groups e, e + esplit, ... or, fused, the two groups of the
-  // pairs e, e + esplit, ...
-  const int units = kFuse ? b_end / 2 : b_end;
-  const int nk = ((units - e + esplit - 1) / esplit) * (kFuse ? 2 : 1);
-  auto group_of = [&](int k) {
-    return kFuse ? 2 * (e + esplit * (k >> 1)) + (k & 1) : e + esplit * k;
-  };
+  const int esplit = P.epi_split, chunks = P.epi_chunks;
   const size_t HoWo = (size_t)P.Ho * P.Wo;
   const uint32_t howo = (uint32_t)HoWo;
   const size_t out_elems = (size_t)P.N * P.Co * HoWo;
@@ -994,14 +989,26 @@ __device__ void epilogue_role(const TcParams &P, const Smem &S, long long i0, in
   const bool relu = P.relu != 0;
   const bool plain = small && P.residual == nullptr, with_res = small && P.residual != nullptr;
   const uint32_t t_lane = tmem_base + ((uint32_t)(quarter * 32) << 16);
-  int tile, slab;
-  if (kRes) { slab = slab0; tile = tile0; }
-  else { tile = (int)(i0 / P.nslabs); slab = (int)(i0 - (long long)tile * P.nslabs); }
-  bool ok = true;
+  // the chunk at hand: chunk c of item it; its accumulator buffer and the parity of that one's full barrier
+  struct At { uint32_t it; int c, tile, slab, ab; uint32_t fph; };
+  At at{0u, e, 0, 0, 0, 0u};
+  if (kRes) { at.slab = slab0; at.tile = tile0; }
+  else { at.tile = (int)(i0 / P.nslabs); at.slab = (int)(i0 - (long long)at.tile * P.nslabs); }
+  auto settle = [&](At &a) {
+    while (a.c >= chunks) {
+      a.c -= chunks;
+      ++a.it;
+      if (++a.ab == P.nacc) { a.ab = 0; a.fph ^= 1u; }
+      if (kRes) a.tile += tstep;
+      else if (++a.slab == P.nslabs) { a.slab = 0; ++a.tile; }
+    }
+  };
+  settle(at);
+  constexpr uint32_t kNoPixel = 0xFFFFFFFFu;
   // this lane's output pixel in a tile: whether it exists, its K, offset of (image, filter 0, pixel)
-  struct Pix { bool valid; float kv; size_t obase; size_t gpix; };   // gpix: pixel index over all images
+  struct Pix { float kv; size_t obase; uint32_t gpix; };   // gpix: pixel index over all images (below the stream's length)
   auto decode = [&](int t) {
-    Pix px{false, 0.0f, 0, 0};
+    Pix px{0.0f, 0, kNoPixel};
     const uint32_t m = ((uint32_t)t * (P.pair ? 2u : 1u) + S.rank) * kTileM + (uint32_t)(quarter * 32 + lane);
     if (m < (uint32_t)P.L) {
       const uint32_t r = fast_div(m, P.div_wq_m, P.div_wq_s);
@@ -1010,57 +1017,53 @@ __device__ void epilogue_role(const TcParams &P, const Smem &S, long long i0, in
       const int oy = (int)(r - n * (uint32_t)P.Hq);
       if (ox < P.Wo && oy < P.Ho) {
         const size_t pix = (size_t)oy * P.Wo + ox;
-        px.valid = true;
         px.kv = load_global(P.K + (size_t)n * HoWo + pix);
         px.obase = (size_t)n * P.Co * HoWo + pix;
-        px.gpix = (size_t)n * HoWo + pix;
+        px.gpix = n * howo + (uint32_t)pix;
       }
     }
     return px;
   };
-  Pix px = decode(tile);
-  int ab = 0;                             // accumulator buffer of the next item and the parity
-  uint32_t fph = 0u;                      // of its full barrier
-  for (uint32_t it = 0; it < nitems && ok; ++it) {
-    const bool valid = px.valid;
+  // The residual of a chunk is pulled into L2 while the warp drains the chunk before: the loads in the
+  // drain loop then see L2 latency only, and the bytes in flight are not bounded by registers.  The warp's
+  // pixels are one run of a filter's plane (at most 128 bytes: two lines), so a lane takes a filter and touches
+  // the two ends of its run: a handful of instructions instead of one prefetch per filter and lane.
+  auto prefetch_residual = [&](const At &a, const Pix &px) {
+    const unsigned vm = __ballot_sync(0xffffffffu, px.gpix != kNoPixel);
+    if (vm == 0u) return;
+    const unsigned long long o0 = __shfl_sync(0xffffffffu, (unsigned long long)px.obase, __ffs(vm) - 1);
+    const unsigned long long o1 = __shfl_sync(0xffffffffu, (unsigned long long)px.obase, 31 - __clz(vm));
+    const int f0 = a.slab * P.NT + a.c * P.epi_chunk * 16, f1 = min(P.Co, min(f0 + P.epi_chunk * 16, (a.slab + 1) * P.NT));
+    for (int j = f0 + lane; j < f1; j += 32) {
+      const float *rp = P.residual + (size_t)j * HoWo;
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(rp + o0));
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(rp + o1));
+    }
+  };
+  Pix px{0.0f, 0, kNoPixel};
+  if (at.it < nitems) {
+    px = decode(at.tile);
+    if (P.residual != nullptr) prefetch_residual(at, px);
+  }
+  while (at.it < nitems) {
+    const bool valid = px.gpix != kNoPixel;
     const float kv = px.kv;
     const size_t obase = px.obase;
-    const size_t obase_pix = px.gpix;
-    // the item after this one; its pixel is decoded (and its K loaded) while this one drains
-    int ntile = tile, nslab = slab;
-    bool next_new;
-    if (kRes) {
-      next_new = true;
-      ntile += tstep;
-    } else {
-      next_new = false;
-      if (++nslab == P.nslabs) { nslab = 0; ++ntile; next_new = true; }
-    }
-    if (P.residual != nullptr && e == 0) {
-      // The residual tile of this item is pulled into L2 while its MMAs run: the loads in the
-      // drain loop then see L2 latency only, and the bytes in flight are not bounded by registers.
-      // The warp's pixels are one run of a filter's plane (at most 128 bytes: two lines), so a
-      // lane takes a filter and touches the two ends of its run: a handful of instructions per
-      // item instead of one prefetch per filter and lane.
-      const unsigned vm = __ballot_sync(0xffffffffu, valid);
-      if (vm != 0u) {
-        const unsigned long long o0 = __shfl_sync(0xffffffffu, (unsigned long long)obase, __ffs(vm) - 1);
-        const unsigned long long o1 = __shfl_sync(0xffffffffu, (unsigned long long)obase, 31 - __clz(vm));
-        const int nf = min(P.NT, P.Co - slab * P.NT);
-        const float *rp = P.residual + (size_t)(slab * P.NT) * HoWo;
-        for (int j = lane; j < nf; j += 32) {
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(rp + o0 + (size_t)j * HoWo));
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(rp + o1 + (size_t)j * HoWo));
-        }
-      }
-    }
-    ok = mbar_wait_relaxed(S.afull + 8u * ab, fph, S.abort_flag, &g_status_tc, XNOR_SLEEP_EPI);
-    if (!ok) break;
-    tc_fence_after();
-    const uint32_t t_acc = t_lane + (uint32_t)(ab * P.NT);
-    const int co0 = slab * P.NT;
+    const uint32_t obase_pix = px.gpix;
+    // the chunk after this one; its pixel is decoded (and its K and residual on their way) while this one drains
+    At nx = at;
+    nx.c += esplit;
+    settle(nx);
     Pix npx = px;
-    if (next_new && it + 1 < nitems) npx = decode(ntile);
+    if (nx.it < nitems) {
+      if (nx.tile != at.tile) npx = decode(nx.tile);
+      if (P.residual != nullptr) prefetch_residual(nx, npx);
+    }
+    const int slab = at.slab;
+    if (!mbar_wait_relaxed(S.afull + 8u * at.ab, at.fph, S.abort_flag, &g_status_tc, XNOR_SLEEP_EPI)) break;
+    tc_fence_after();
+    const uint32_t t_acc = t_lane + (uint32_t)(at.ab * P.NT);
+    const int co0 = slab * P.NT;
 
     // Store addresses step from filter to filter by one multiply-add each (forming every
     // address from the group's base takes two instructions per store and measured slower).
@@ -1185,24 +1188,24 @@ __device__ void epilogue_role(const TcParams &P, const Smem &S, long long i0, in
     // stores of the current ones saves the ~50 cycles of a tensor-memory load per group but
     // costs 16 register copies, which take longer here.)
     int32_t cur[16];
+    const int b1 = min((at.c + 1) * P.epi_chunk, b_end);      // groups of the chunk
 #pragma unroll 1
-    for (int k = 0; k < nk; ++k) {
-      const int b = group_of(k);
+    for (int b = at.c * P.epi_chunk; b < b1; ++b) {
       tmem_ld16(t_acc + (uint32_t)(b * 16), cur);
       tmem_wait16(cur);
-      if (k + 1 == nk) {                         // that was the last load: release the buffer
+      if (b + 1 == b1) {                         // that was the last load: release the buffer
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) { if (P.pair) mbar_arrive_cluster(S.aempty + 8u * ab, 0u); else mbar_arrive(S.aempty + 8u * ab); }
+        if (lane == 0) { if (P.pair) mbar_arrive_cluster(S.aempty + 8u * at.ab, 0u); else mbar_arrive(S.aempty + 8u * at.ab); }
       }
       if (kFuse) {
         // C_out is a multiple of 32, so a pair of groups lies inside the filters or (last slab)
         // wholly beyond them
         if (co0 + b * 16 >= P.Co) continue;
         emit_fused(b, cur);
-        if ((k & 1) && valid) {                  // the pair is complete: its word of the next input
+        if ((b & 1) && valid) {                  // the pair is complete: its word of the next input
           if (in_bounds(obase_pix < (size_t)P.N * HoWo && ((co0 + b * 16) >> 5) < P.Cw_next, 11))
-            P.xp_next[(obase_pix) * (size_t)P.Cw_next + (size_t)((co0 + b * 16) >> 5)] = word;
+            P.xp_next[(size_t)obase_pix * (size_t)P.Cw_next + (size_t)((co0 + b * 16) >> 5)] = word;
           word = 0u;
         }
       } else {
@@ -1210,11 +1213,9 @@ __device__ void epilogue_role(const TcParams &P, const Smem &S, long long i0, in
       }
     }
     if (kFuse && valid && in_bounds(obase_pix < (size_t)P.N * HoWo, 12))
-      P.A_part[(size_t)(slab * esplit + e) * ((size_t)P.N * HoWo) + obase_pix] = (as0 + as1) + (as2 + as3);
+      P.A_part[(size_t)(slab * chunks + at.c) * ((size_t)P.N * HoWo) + obase_pix] = (as0 + as1) + (as2 + as3);
     px = npx;
-    tile = ntile;
-    slab = nslab;
-    if (++ab == P.nacc) { ab = 0; fph ^= 1u; }
+    at = nx;
   }
 }
 
@@ -1244,7 +1245,7 @@ binconv_tc_kernel(const __grid_constant__ TcParams P) {
     }
     for (int i = 0; i < kMaxAcc; ++i) {
       mbar_init(S.afull + 8u * i, 1);
-      mbar_init(S.aempty + 8u * i, (uint32_t)(kEpiWarps * P.epi_split * kCtas));
+      mbar_init(S.aempty + 8u * i, (uint32_t)(kEpiWarps * P.epi_chunks) * kCtas);
     }
     *S.abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1545,6 +1546,18 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
   // worker warps per quarter of the lanes in the resident schedule: the four epilogue warps
   // and the eight weight warps
   P.epi_split = P.resident ? std::min(kEpiSplitMax, P.NT / (fuse ? 32 : 16)) : P.wgt_groups == 2 ? std::min(2, P.NT / (fuse ? 32 : 16)) : 1;
+  // Chunks of an item that the draining warps take in turn (see epilogue_role).  What a warp does per item
+  // (its pixel, K, the waits: some 150 instructions) was a third of all instructions while every warp took a
+  // share of every item: 64 channels, 56x56, 64 filters 3x3, 256 images 71.8 -> 63.1 us, with a residual 107.0 ->
+  // 90.5 (four groups over three warps had also left one with two); 128 channels, 28x28: 36.2 -> 32.7 and 51.4 -> 49.0;
+  // fused, the same two layers 102 -> 82 and 50 -> 41.  With fewer items than warps take turns over, all of them
+  // share an item, whose latency then counts (fused, one image: 7.4 us, in chunks of 64 filters 7.7).
+  const int epi_groups = P.NT / 16;
+  const long long unit_items = ((long long)P.ntiles * P.nslabs + units - 1) / units;
+  P.epi_chunk = (epi_groups + P.epi_split - 1) / P.epi_split;
+  if (fuse) P.epi_chunk = std::max(unit_items >= 4 ? 4 : 2, (P.epi_chunk + 1) / 2 * 2);
+  else if (unit_items >= 4) P.epi_chunk = 4;
+  P.epi_chunks = (epi_groups + P.epi_chunk - 1) / P.epi_chunk;
   if (fuse && (g.Co & 31) != 0) return pl;          // whole words of the next layer's input
   P.stages = stages; P.npb = npb;
   P.off_tab = 0u;
@@ -1724,11 +1737,11 @@ cudaError_t launch_binconv_tc(const uint32_t *xp, const uint32_t *wp, const floa
 }
 
 // Partial planes of |y| sums that the fused kernel writes for this shape: one per filter slab
-// and, in the resident schedule, per warp that shares a quarter of the lanes.  0: not supported.
+// and chunk of its columns.  0: not supported.
 int tc_fused_parts(const ConvGeom &g, TcVariant variant) {
   const Plan pl = plan_variant(g, variant, true, 1, false);
   if (!pl.ok) return 0;
-  return pl.P.nslabs * pl.P.epi_split;
+  return pl.P.nslabs * pl.P.epi_chunks;
 }
 
 cudaError_t launch_binconv_tc_fused(const uint32_t *xp, const uint32_t *wp, const float *alpha,

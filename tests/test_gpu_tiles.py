@@ -175,3 +175,31 @@ def test_plain_schedules(oracle, shape, resident, pair, slabs, filters):
     plan = X.xnor_conv2d_plan(X.make_desc(N, C, H, W, Co, kh, kw, s, p))
     assert (plan.resident, plan.pair, plan.slabs, plan.slab_filters) == (resident, pair, slabs, filters)
     block_parity(oracle, shape, X.XNOR_ENGINE_AUTO)
+
+
+# several items per CTA, drained in chunks of 64 filters that the warps of a lane quarter take in turn: one to
+# four chunks, a short last chunk, filters beyond C_out, warps that skip items; every schedule
+@pytest.mark.parametrize("engine", [X.XNOR_ENGINE_AUTO, X.XNOR_ENGINE_UMMA_STREAM, X.XNOR_ENGINE_UMMA_PAIR])
+@pytest.mark.parametrize("residual", [False, True])
+@pytest.mark.parametrize("Co,k", [(16, 1), (48, 3), (70, 1), (112, 3), (200, 1), (240, 1)])
+def test_drained_chunks(oracle, Co, k, residual, engine):
+    N, C, H, W = 160, 16, 23, 24
+    d = X.make_desc(N, C, H, W, Co, k, k, 1, k // 2)
+    g = rng(Co + k)
+    x = g.standard_normal((N, C, H, W)).astype(np.float32)
+    w = g.standard_normal((Co, C, k, k)).astype(np.float32)
+    res = g.standard_normal((N, Co, H, W)).astype(np.float32) if residual else None
+    wp, alpha = X.alloc_weights(Co, C, k, k)
+    xp, A, K = X.alloc_binactiv(d)
+    gs = GuardSet()
+    out = gs.like("out", X.alloc_out(d))
+    X.xnor_binarize_weights(dev(w), wp, alpha)
+    X.xnor_binactiv(dev(x), None, None, d, xp, A, K)
+    X.xnor_set_engine(engine)
+    try:
+        X.xnor_conv2d_forward(xp, wp, alpha, K, None if res is None else dev(res), d, out)
+    finally:
+        X.xnor_set_engine(X.XNOR_ENGINE_AUTO)
+    X.xnor_check_device()
+    gs.check()
+    assert_close(host(out), oracle.xnor_block(x, w, 1, k // 2, None, None, res).out, "out")
