@@ -66,6 +66,7 @@
 //  tile-major order, so that a patch serves all slabs of its tile).
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "umma_common.cuh"
@@ -181,6 +182,8 @@ struct TcParams {
   int div_wq_s, div_hq_s;      // (dividends below 2^31)
   uint32_t div_pg_m, div_g_m;  // the same for the patch units: by phases * ngrp and by ngrp
   int div_pg_s, div_g_s;       // (ngrp = groups of four channel words)
+  uint32_t wq_rcp;             // 2^32 / Wq, rounded up: exact quotients of a patch's positions
+  int pat_table;               // a patch touches at most 32 rows of the stream
 };
 
 // One MMA.  The issuing warp elects one lane, and that lane alone runs the whole issue loop:
@@ -747,8 +750,7 @@ __device__ void weight_stream(const TcParams &P, const Smem &S, uint32_t nitems,
 
 // ------------------------------------------------------------------ patch producers
 // The group of the three patch warps builds the CTA's patches one after the
-// other, all warps on the same patch: units of (32 stream positions, phase plane, up to 4 channel words) are dealt round
-// robin.  The packed pixels a patch touches are ONE contiguous range of x_packed: input rows
+// other, all warps on the same patch, or each builds patches of its own.  The packed pixels a patch touches are ONE contiguous range of x_packed: input rows
 // g0 .. g1 - 1 of the N*H rows (images follow one another in memory, the zero rows and
 // columns of the stream exist only in the patch).  Every patch buffer has a raw buffer; the
 // group's first warp brings a patch's range into it with one bulk copy (an aligned superset
@@ -769,54 +771,44 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
                                  : (uint32_t)((i1 - 1) / P.nslabs) - (uint32_t)tile0 + 1u;
   const int s = P.stride, phases = s * s;
   const uint32_t plane_bytes = (uint32_t)P.ppix * 16u;
-  const bool vec = (P.Cw & 3) == 0;
   // nibble masks of the channel tail, one per expanded register
   uint32_t tm[4];
 #pragma unroll
   for (int r = 0; r < 4; ++r) tm[r] = ((P.tail_mask >> r) & 0x11111111u) * 0xFu;
   const bool tail = P.tail_mask != 0xFFFFFFFFu;
-  const uint32_t row_bytes = (uint32_t)P.W * (uint32_t)P.Cw * 4u;
-  const size_t tensor_bytes = (size_t)P.N * P.H * row_bytes;
+  const uint32_t word_bytes = (uint32_t)P.Cw * 4u, row_bytes = (uint32_t)P.W * word_bytes;   // of a pixel, a row
   // pairs: work tile t is stream tiles 2t (rank 0) and 2t + 1 (rank 1)
   const uint32_t tmul = P.pair ? 2u : 1u;
   const int ngrp = (P.Cw + 3) >> 2;                       // groups of 4 channel words
-  const int npass = (P.ppix + 31) >> 5;
-  const int nunits = npass * phases * ngrp;
 
-  constexpr int kPatUnits = kRes && !kTwo ? 2 : 1;                 // patch units a warp works on together (registers)
-  auto tile_of = [&](uint32_t seq) { return kRes ? (int)R.tile(seq) : tile0 + (int)seq; };
-  // input rows [g0, g1) (of the N*H rows of the tensor) that the patch of a tile reads
-  auto row_range = [&](int tile, int &g0, int &g1) {
-    const uint32_t m0 = ((uint32_t)tile * tmul + S.rank) * kTileM;
-    const uint32_t mlast = min(m0 + (uint32_t)P.ppix - 1u, (uint32_t)P.L - 1u);
-    const uint32_t r0 = fast_div(m0, P.div_wq_m, P.div_wq_s);
-    const uint32_t r1 = fast_div(mlast, P.div_wq_m, P.div_wq_s);
-    const uint32_t n0 = fast_div(r0, P.div_hq_m, P.div_hq_s);
-    const uint32_t n1 = fast_div(r1, P.div_hq_m, P.div_hq_s);
-    const int ry0 = (int)(r0 - n0 * (uint32_t)P.Hq), ry1 = (int)(r1 - n1 * (uint32_t)P.Hq);
-    const int t0 = min(max((ry0 - P.leadY) * s, 0), P.H);
-    const int t1 = min(max((ry1 - P.leadY) * s + s, 0), P.H);
-    g0 = (int)n0 * P.H + t0;
-    g1 = (int)n1 * P.H + t1;
+  auto first_pos = [&](uint32_t seq) {                    // of patch seq, in the stream
+    return ((kRes ? R.tile(seq) : (uint32_t)tile0 + seq) * tmul + S.rank) * kTileM;
+  };
+  // the input row (of the N*H rows of the tensor) that stream row r stands for, clamped to its image;
+  // add = 0: the first of its rows, s: the one behind the last
+  auto input_row = [&](uint32_t r, int add) {
+    const uint32_t n = fast_div(r, P.div_hq_m, P.div_hq_s);
+    return (int)n * P.H + min(max(((int)(r - n * (uint32_t)P.Hq) - P.leadY) * s + add, 0), P.H);
   };
   // a subgroup's first warp, lane 0: starts the copy of a patch's rows into raw buffer rb
   auto start_copy = [&](uint32_t seq, uint32_t rb) {
-    int g0, g1;
-    row_range(tile_of(seq), g0, g1);
+    const uint32_t m0 = first_pos(seq), mlast = min(m0 + (uint32_t)P.ppix - 1u, (uint32_t)P.L - 1u);
+    const int g0 = input_row(fast_div(m0, P.div_wq_m, P.div_wq_s), 0);
+    const int g1 = input_row(fast_div(mlast, P.div_wq_m, P.div_wq_s), s);
     const uint32_t bar = S.rawfull + 8u * rb;
     const uint32_t dst = S.raw + rb * P.raw_bytes;
     if (g1 <= g0) { mbar_arrive(bar); return; }          // nothing but padding
-    const size_t b0 = (size_t)g0 * row_bytes, b1 = (size_t)g1 * row_bytes;
-    const size_t a0 = b0 & ~(size_t)15;
-    const size_t a1 = min((b1 + 15) & ~(size_t)15, tensor_bytes & ~(size_t)15);
-    const uint32_t bulk = a1 > a0 ? (uint32_t)(a1 - a0) : 0u;
-    for (size_t b = a0 + bulk; b < b1; b += 4)           // at most 3 words, at the tensor's end
-      if (in_bounds((uint32_t)(b - a0) + 4u <= P.raw_plane, 3))
+    const size_t b0 = (size_t)g0 * row_bytes, a0 = b0 & ~(size_t)15, left = (size_t)P.N * P.H * row_bytes - a0;
+    const uint32_t need = ((uint32_t)b0 & 15u) + (uint32_t)(g1 - g0) * row_bytes;    // from the 16-byte boundary a0
+    uint32_t bulk = (need + 15u) & ~15u;
+    if (bulk > left) bulk = (uint32_t)left & ~15u;
+    for (uint32_t b = bulk; b < need; b += 4u)           // at most 3 words, at the tensor's end
+      if (in_bounds(b + 4u <= P.raw_plane, 3))
       {
-        sts32(dst + (uint32_t)(b - a0), load_global(P.xp + (b >> 2)));
-        if (kTwo) sts32(dst + P.raw_plane + (uint32_t)(b - a0), load_global(P.xp2 + (b >> 2)));
+        sts32(dst + b, load_global(P.xp + ((a0 + b) >> 2)));
+        if (kTwo) sts32(dst + P.raw_plane + b, load_global(P.xp2 + ((a0 + b) >> 2)));
       }
-    if (bulk && in_bounds(bulk <= P.raw_plane && a0 + bulk <= tensor_bytes, 4)) {
+    if (bulk && in_bounds(bulk <= P.raw_plane && bulk <= left, 4)) {
       mbar_arrive_expect_tx(bar, kTwo ? 2u * bulk : bulk);
       bulk_copy_g2s(dst, reinterpret_cast<const uint8_t *>(P.xp) + a0, bulk, bar);
       if (kTwo) bulk_copy_g2s(dst + P.raw_plane, reinterpret_cast<const uint8_t *>(P.xp2) + a0, bulk, bar);
@@ -830,6 +822,126 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
   // a buffer, so no subgroup may run more than one use ahead of the consumer).
   const uint32_t nsub = (uint32_t)P.pat_sub, gsize = (uint32_t)kPatWarps / nsub;
   const uint32_t sg = (uint32_t)pw % nsub, mi = (uint32_t)pw / nsub;
+
+  // Expands this warp's share of a patch: raw buffer rb holds input rows g0 .. from address `raw` on, m0 is the
+  // patch's first position.  Units, in this order of nesting: kPos x 32 positions, phase plane, kWords channel
+  // words (0: up to four, word by word); every warp of the subgroup takes a contiguous share.  A lane keeps
+  // the address of one row of the patch, so that locating a position costs a multiplication and a shuffle; the
+  // work on the kPos positions is independent, and the innermost part does not branch.  What bounds a patch is
+  // the latency of its one warp: two divisions per position and unit, as before, took 4500 cycles for the patch of
+  // 64 channels, 56x56, where an item takes 2300 and three warps build patches (256 images, 64 filters 3x3: 63.1 ->
+  // 55.7 us; stride 2, 128 filters 38.1 -> 32.4; 256 channels, 14x14, stride 2, one image 8.7 -> 7.5).  The same steps with
+  // the place of a unit kept by branches in one flat loop were slower than the divisions (67.5).
+  auto build = [&](auto kpos_, auto kwords_, uint32_t m0, int g0, uint32_t raw, uint32_t rb, uint32_t patch) {
+    constexpr int kPos = decltype(kpos_)::value, kWords = decltype(kwords_)::value, kLoop = kWords ? kWords : 4;
+    const uint32_t r0 = fast_div(m0, P.div_wq_m, P.div_wq_s), c0 = m0 - r0 * (uint32_t)P.Wq;
+    // addresses of the input rows of stream row r, one per row phase; 0: padding
+    auto row_address = [&](uint32_t r, uint32_t &a0, uint32_t &a1) {
+      const uint32_t n = fast_div(r, P.div_hq_m, P.div_hq_s);
+      const int y = ((int)(r - n * (uint32_t)P.Hq) - P.leadY) * s;
+      const uint32_t a = raw + (uint32_t)((int)n * P.H + y - g0) * row_bytes;
+      const bool in = n < (uint32_t)P.N && y >= 0;
+      a0 = in && y < P.H ? a : 0u;
+      a1 = in && y + 1 < P.H ? a + row_bytes : 0u;
+    };
+    uint32_t tab0, tab1;
+    row_address(r0 + (uint32_t)lane, tab0, tab1);
+    const int nunits = (P.ppix + 32 * kPos - 1) / (32 * kPos) * phases * ngrp;
+    const int share = (nunits + (int)gsize - 1) / (int)gsize;
+    int u = (int)mi * share;
+    const int u1 = min(u + share, nunits);
+    int block = 0, phase = 0, w0 = 0;
+    if (u > 0) {
+      block = (int)fast_div((uint32_t)u, P.div_pg_m, P.div_pg_s);
+      const int rem = u - block * (phases * ngrp);
+      phase = (int)fast_div((uint32_t)rem, P.div_g_m, P.div_g_s);
+      w0 = (rem - phase * ngrp) * 4;
+    }
+#pragma unroll 1
+    for (; u < u1; ++block, phase = 0) {
+      int col[kPos];
+      uint32_t row0[kPos], row1[kPos], pdst[kPos];
+      bool on[kPos];
+#pragma unroll
+      for (int b = 0; b < kPos; ++b) {
+        const int q = (block * kPos + b) * 32 + lane;
+        const uint32_t x = c0 + (uint32_t)q;
+        on[b] = q < P.ppix;
+        pdst[b] = patch + (uint32_t)q * 16u;
+        if (P.pat_table) {
+          const uint32_t i = __umulhi(x, P.wq_rcp);
+          col[b] = ((int)(x - i * (uint32_t)P.Wq) - P.leadX) * s;
+          row0[b] = __shfl_sync(0xffffffffu, tab0, (int)i);
+          row1[b] = s == 2 ? __shfl_sync(0xffffffffu, tab1, (int)i) : 0u;
+        } else {
+          const uint32_t i = fast_div(x, P.div_wq_m, P.div_wq_s);
+          col[b] = ((int)(x - i * (uint32_t)P.Wq) - P.leadX) * s;
+          row_address(r0 + i, row0[b], row1[b]);
+        }
+      }
+#pragma unroll 1
+      for (; phase < phases && u < u1; ++phase, w0 = 0) {
+        const int py = phase >> (s - 1), px = phase & (s - 1);     // stride 1 or 2
+        uint32_t src[kPos], dst[kPos], sm[kPos], mc[kPos][3];
+#pragma unroll
+        for (int b = 0; b < kPos; ++b) {
+          const uint32_t row = py ? row1[b] : row0[b];
+          const bool real = on[b] && row != 0u && col[b] >= 0 && col[b] + px < P.W;
+          const uint32_t keep = real ? 0xFFFFFFFFu : 0u;           // padding expands to 0, whatever its word is
+          sm[b] = 0x88888888u & keep;
+          mc[b][0] = 0xCCCCCCCCu & keep; mc[b][1] = 0xAAAAAAAAu & keep; mc[b][2] = 0x99999999u & keep;
+          src[b] = (real ? row + (uint32_t)(col[b] + px) * word_bytes : S.raw + rb * P.raw_bytes) + (uint32_t)w0 * 4u;
+          dst[b] = pdst[b] + (uint32_t)(phase * P.Cw + w0) * plane_bytes;
+        }
+#pragma unroll 1
+        for (; w0 < P.Cw && u < u1; w0 += 4, ++u) {
+          uint32_t wv[kPos][4], wu[kTwo ? kPos : 1][4];
+          auto load = [&](uint32_t a, uint32_t (&v)[4]) {
+            if constexpr (kWords == 4) lds128(a, v);
+            else if constexpr (kWords == 2) lds64(a, v[0], v[1]);
+            else {
+#pragma unroll
+              for (int i = 0; i < kLoop; ++i) v[i] = kWords || w0 + i < P.Cw ? lds32(a + (uint32_t)i * 4u) : 0u;
+            }
+          };
+#pragma unroll
+          for (int b = 0; b < kPos; ++b) {
+            if (in_bounds(src[b] >= S.raw + rb * P.raw_bytes &&
+                          src[b] + 4u * (uint32_t)min(4, P.Cw - w0) <= S.raw + rb * P.raw_bytes + P.raw_plane, 6)) {
+              load(src[b], wv[b]);
+              if constexpr (kTwo) load(src[b] + P.raw_plane, wu[b]);
+            }
+            src[b] += 16u;
+          }
+#pragma unroll
+          for (int i = 0; i < kLoop; ++i) {
+            if (kWords || w0 + i < P.Cw) {
+              const bool cut = tail && w0 + i == P.Cw - 1;       // channels beyond C_in are 0
+#pragma unroll
+              for (int b = 0; b < kPos; ++b) {
+                const uint32_t w = kTwo ? wu[b][i] : wv[b][i];      // signs
+                uint32_t v0 = ((w << 3) & sm[b]) ^ mc[b][0];
+                uint32_t v1 = ((w << 2) & sm[b]) ^ mc[b][1];
+                uint32_t v2 = ((w << 1) & sm[b]) ^ mc[b][2];
+                uint32_t v3 = (w & sm[b]) ^ mc[b][2];
+                if constexpr (kTwo) {                     // magnitudes 2, 1, 0.5 (100, 010, 001) -> 6, 3, 1.5 (111, 101, 011)
+                  const uint32_t e = ~(wv[b][i] ^ wu[b][i]), e0 = (e << 3) & sm[b], e1 = (e << 2) & sm[b];
+                  v0 ^= (e0 >> 2) | (e0 >> 3);
+                  v1 ^= e1 - (e1 >> 3);
+                  v2 ^= ((e << 1) & sm[b]) >> 2;
+                  v3 ^= (e & sm[b]) >> 2;
+                }
+                if (cut) { v0 &= tm[0]; v1 &= tm[1]; v2 &= tm[2]; v3 &= tm[3]; }
+                if (on[b] && in_bounds(dst[b] >= patch && dst[b] + 16u <= patch + P.patch_bytes, 5)) sts128(dst[b], v0, v1, v2, v3);
+                dst[b] += plane_bytes;
+              }
+            }
+          }
+        }
+      }
+    }
+  };
+
   // The subgroup's k-th patch (patch sg + k nsub of the CTA) expands from the subgroup's raw
   // buffer k % nraw; its rows are fetched as soon as the subgroup is done with patch k - nraw.
   const uint32_t nraw = (uint32_t)P.nraw, rb0 = sg * nraw;
@@ -842,7 +954,6 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
   uint32_t k = 0;
 #pragma unroll 1
   for (uint32_t seq = sg; seq < npatches && ok; seq += nsub, ++k) {
-    const int tile = tile_of(seq);
     const uint32_t pb = seq % (uint32_t)P.npb;
     const uint32_t use = seq / (uint32_t)P.npb;
     const uint32_t rb = rb0 + k % nraw, ruse = k / nraw;
@@ -857,96 +968,25 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
       if (lane == 0) start_copy(sg + kc * nsub, crb);
       ++kc;
     }
-    int g0, g1;
-    row_range(tile, g0, g1);
+    const uint32_t m0 = first_pos(seq);
+    const int g0 = input_row(fast_div(m0, P.div_wq_m, P.div_wq_s), 0);
     ok = mbar_wait_relaxed(S.rawfull + 8u * rb, ruse & 1u, S.abort_flag, &g_status_tc, XNOR_SLEEP_PAT);
     if (!ok) break;
     ok = mbar_wait_relaxed(S.pempty + 8u * pb, (use & 1u) ^ 1u, S.abort_flag, &g_status_tc,
                            XNOR_SLEEP_PAT);
     if (!ok) break;
     const uint32_t patch = S.patch + pb * P.patch_bytes;
-    const uint32_t m0 = ((uint32_t)tile * tmul + S.rank) * kTileM;
     const uint32_t raw = S.raw + rb * P.raw_bytes +
                          (uint32_t)(((size_t)g0 * row_bytes) & 15u);   // where row g0 starts
-    // kPatUnits units at a time: their index arithmetic and loads are independent chains the
-    // warp can overlap, then all are expanded
-#pragma unroll 1
-    for (int u0 = (int)mi; u0 < nunits; u0 += kPatUnits * (int)gsize) {
-      uint32_t src[kPatUnits], dst[kPatUnits], sm[kPatUnits], mc[kPatUnits][3], wv[kPatUnits][4], wu[kTwo ? kPatUnits : 1][4];
-      int w0[kPatUnits];
-      bool on[kPatUnits], real[kPatUnits];
-#pragma unroll
-      for (int b = 0; b < kPatUnits; ++b) {
-        const int u = u0 + b * (int)gsize;
-        const int pass = (int)fast_div((uint32_t)u, P.div_pg_m, P.div_pg_s);
-        const int rem = u - pass * (phases * ngrp);
-        const int phase = (int)fast_div((uint32_t)rem, P.div_g_m, P.div_g_s);
-        w0[b] = (rem - phase * ngrp) * 4;
-        const int q = pass * 32 + lane;
-        on[b] = u < nunits && q < P.ppix;
-        const uint32_t sq = m0 + (uint32_t)q;
-        const uint32_t r = fast_div(sq, P.div_wq_m, P.div_wq_s);
-        const int c = (int)(sq - r * (uint32_t)P.Wq);
-        const uint32_t n = fast_div(r, P.div_hq_m, P.div_hq_s);
-        const int ry = (int)(r - n * (uint32_t)P.Hq);
-        const int py = phase >> (s - 1), px = phase & (s - 1);     // stride 1 or 2
-        const int rrow = (ry - P.leadY) * s + py, rcol = (c - P.leadX) * s + px;
-        real[b] = on[b] && sq < (uint32_t)P.L && ry >= P.leadY && c >= P.leadX && rrow < P.H &&
-                  rcol < P.W;
-        const uint32_t keep = real[b] ? 0xFFFFFFFFu : 0u;        // padding expands to 0
-        sm[b] = 0x88888888u & keep;
-        mc[b][0] = 0xCCCCCCCCu & keep; mc[b][1] = 0xAAAAAAAAu & keep; mc[b][2] = 0x99999999u & keep;
-        src[b] = raw + (uint32_t)((((int)n * P.H + rrow - g0) * P.W + rcol) * P.Cw + w0[b]) * 4u;
-        dst[b] = patch + (uint32_t)(phase * P.Cw + w0[b]) * plane_bytes + (uint32_t)q * 16u;
-      }
-#pragma unroll
-      for (int b = 0; b < kPatUnits; ++b) {
-        wv[b][0] = wv[b][1] = wv[b][2] = wv[b][3] = 0u;
-        if (kTwo) wu[b][0] = wu[b][1] = wu[b][2] = wu[b][3] = 0u;
-        if (real[b] && in_bounds(src[b] >= S.raw + rb * P.raw_bytes &&
-                                 src[b] + 4u * (uint32_t)min(4, P.Cw - w0[b]) <= S.raw + rb * P.raw_bytes + P.raw_plane, 6)) {
-          if (vec) {
-            lds128(src[b], wv[b]);
-            if (kTwo) lds128(src[b] + P.raw_plane, wu[b]);
-          } else {
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-              if (w0[b] + i < P.Cw) {
-                wv[b][i] = lds32(src[b] + (uint32_t)i * 4u);
-                if (kTwo) wu[b][i] = lds32(src[b] + P.raw_plane + (uint32_t)i * 4u);
-              }
-          }
-        }
-      }
-#pragma unroll
-      for (int b = 0; b < kPatUnits; ++b) {
-        if (on[b]) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            if (w0[b] + i < P.Cw) {
-              const uint32_t w = kTwo ? wu[b][i] : wv[b][i];      // signs
-              uint32_t v0 = ((w << 3) & sm[b]) ^ mc[b][0];
-              uint32_t v1 = ((w << 2) & sm[b]) ^ mc[b][1];
-              uint32_t v2 = ((w << 1) & sm[b]) ^ mc[b][2];
-              uint32_t v3 = (w & sm[b]) ^ mc[b][2];
-              if (kTwo) {                                 // magnitudes 2, 1, 0.5 (100, 010, 001) -> 6, 3, 1.5 (111, 101, 011)
-                const uint32_t e = ~(wv[b][i] ^ wu[b][i]), e0 = (e << 3) & sm[b], e1 = (e << 2) & sm[b];
-                v0 ^= (e0 >> 2) | (e0 >> 3);
-                v1 ^= e1 - (e1 >> 3);
-                v2 ^= ((e << 1) & sm[b]) >> 2;
-                v3 ^= (e & sm[b]) >> 2;
-              }
-              if (tail && w0[b] + i == P.Cw - 1) {       // channels beyond C_in are 0
-                v0 &= tm[0]; v1 &= tm[1]; v2 &= tm[2]; v3 &= tm[3];
-              }
-              if (in_bounds(dst[b] + (uint32_t)i * plane_bytes >= patch &&
-                            dst[b] + (uint32_t)i * plane_bytes + 16u <= patch + P.patch_bytes, 5))
-                sts128(dst[b] + (uint32_t)i * plane_bytes, v0, v1, v2, v3);
-            }
-          }
-        }
-      }
-    }
+    using std::integral_constant;
+    constexpr int kWide = kRes ? 2 : 1;           // (registers)
+    const integral_constant<int, kWide> few;
+    const integral_constant<int, 2 * kWide> many;
+    if ((P.Cw & 3) == 0) build(few, integral_constant<int, 4>{}, m0, g0, raw, rb, patch);
+    else if (P.Cw == 1) build(many, integral_constant<int, 1>{}, m0, g0, raw, rb, patch);
+    else if (P.Cw == 2) build(many, integral_constant<int, 2>{}, m0, g0, raw, rb, patch);
+    else if (P.Cw == 3) build(few, integral_constant<int, 3>{}, m0, g0, raw, rb, patch);
+    else build(few, integral_constant<int, 0>{}, m0, g0, raw, rb, patch);
     fence_proxy_async();
     __syncwarp();
     if (lane == 0) {
@@ -1594,6 +1634,8 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
   const uint32_t ngrp = (uint32_t)(P.Cw + 3) / 4u;
   magic((uint32_t)(s * s) * ngrp, &P.div_pg_m, &P.div_pg_s);
   magic(ngrp, &P.div_g_m, &P.div_g_s);
+  P.wq_rcp = (uint32_t)((((unsigned long long)1 << 32) + P.Wq - 1) / P.Wq);    // (0 for a width of 1: no table then)
+  P.pat_table = (P.ppix + P.Wq - 2) / P.Wq + 1 <= 32 && P.Wq > 1;
   pl.ok = true;
   return pl;
 }
