@@ -24,15 +24,39 @@ binarize_weights_kernel(const float *w, int Co, int C, int taps, int Cw,
   double l1 = 0.0;
   int tap = 0, cw = warp;                      // word f = tap * Cw + cw, visited in steps of 8
   while (cw >= Cw) { cw -= Cw; ++tap; }
-  for (int f = warp; f < nwords; f += kThreads / 32) {
+  // whole batches of words with all their loads in flight together, then the rest one by one (256 filters of 1024
+  // channels 7x7: 87.6 -> 62.5 us, 256 of 96 channels 5x5 4.0 -> 3.0; a batch in every case costs small filters 0.2)
+  constexpr int kStep = kThreads / 32, kBatch = 4;
+  int f = warp;
+  auto next = [&]() {
+    cw += kStep;
+    while (cw >= Cw) { cw -= Cw; ++tap; }
+  };
+  for (; f + (kBatch - 1) * kStep < nwords; f += kBatch * kStep) {
+    float v[kBatch];
+    bool in[kBatch];
+#pragma unroll
+    for (int i = 0; i < kBatch; ++i) {
+      const int ci = cw * 32 + lane;
+      in[i] = ci < C;
+      v[i] = load_global_if(wf + (size_t)(in[i] ? ci : 0) * taps + tap, in[i]);
+      next();
+    }
+#pragma unroll
+    for (int i = 0; i < kBatch; ++i) {
+      if (in[i]) l1 += fabs((double)v[i]);
+      const uint32_t word = __ballot_sync(0xffffffffu, in[i] && v[i] >= 0.0f);
+      if (lane == 0) words[f + i * kStep] = word;
+    }
+  }
+  for (; f < nwords; f += kStep) {
     const int ci = cw * 32 + lane;
     const bool in = ci < C;
     const float v = in ? load_global(wf + (size_t)ci * taps + tap) : -1.0f;
     if (in) l1 += fabs((double)v);
     const uint32_t word = __ballot_sync(0xffffffffu, in && v >= 0.0f);
     if (lane == 0) words[f] = word;
-    cw += kThreads / 32;
-    while (cw >= Cw) { cw -= Cw; ++tap; }
+    next();
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) l1 += __shfl_xor_sync(0xffffffffu, l1, o);

@@ -11,7 +11,7 @@ from test_gpu_fused import test_fused_binactiv_parity as fused_parity
 from test_gpu_options import _index_of_planes
 from test_gpu_options import test_kbit_block_parity as kbit_block_parity
 from test_gpu_parity import test_block_parity as block_parity
-from util import GuardSet, assert_close, dev, host
+from util import GuardSet, assert_close, dev, host, unpack_weights
 
 pytestmark = pytest.mark.gpu
 
@@ -217,3 +217,17 @@ def test_drained_chunks(oracle, Co, k, residual, engine):
     (37, 100, 15, 17, 77, 5, 5, 1, 2), (60, 40, 29, 30, 64, 3, 3, 2, 1), (36, 64, 27, 28, 100, 3, 3, 1, 1)])
 def test_patches(oracle, shape, engine):
     block_parity(oracle, shape, engine)
+
+
+# words of a filter around whole batches of 32 (8 warps, four words each), tails of channels
+@pytest.mark.parametrize("C,k", [(32, 5), (768, 1), (800, 1), (980, 1), (1024, 1), (1030, 1), (45, 4), (200, 3), (225, 3), (1, 7)])
+def test_weight_words(oracle, C, k):
+    w = rng(C + k).standard_normal((5, C, k, k)).astype(np.float32)
+    wp0, alpha0 = X.alloc_weights(5, C, k, k)
+    gs = GuardSet()
+    wp, alpha = gs.like("w_packed", wp0), gs.like("alpha", alpha0)
+    X.xnor_binarize_weights(dev(w), wp, alpha)
+    gs.check()
+    B, want = oracle.binarize_weights(w)
+    assert np.array_equal(unpack_weights(host(wp), C, k, k), B)
+    assert_close(host(alpha), want, "alpha")
