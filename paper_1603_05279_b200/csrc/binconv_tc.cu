@@ -108,6 +108,7 @@ constexpr int kPatWarp0 = 13, kPatWarps = 3;
 constexpr int kThreadsRes = 32 * (kPatWarp0 + kPatWarps);   // 512: 16 warps, 128 registers each
 // streaming: weight warps in groups of four, patch warps behind them (see the kernel's role table)
 constexpr int kLongItem = 64, kLongFused = 96;   // streaming: K-steps of an item that count as many
+constexpr int kPairSteps = 32;       // K-steps from which a pair issues them better (see plan_variant_uncached)
 constexpr int kGroupWarps = 4, kThreadsStream = 768;   // 24 warps, 80 registers each
 constexpr int kTileM = 128;          // stream positions per tile = tensor-memory lanes
 constexpr int kTmemCols = 512;
@@ -1664,11 +1665,22 @@ Plan plan_variant_uncached(const ConvGeom &g, TcVariant v, bool fuse, int planes
     default: break;
   }
   Plan single = make_plan(g, 0, false, fuse, planes, residual);
-  if (single.ok && single.P.resident) return single;
+  // From 32 K-steps on the MMAs bound an item, and one thread of a pair issues those of two SMs at the cost of one's.
+  // Two resident slabs and several items per CTA: 0.87 .. 0.99 of the time over 14 drawn shapes (AlexNet conv2 58.6 -> 54.9
+  // us; 96 channels, 50x50, 256 filters 5x5, 51 images 0.87); fewer items 0.99 .. 1.03, three slabs (conv3) 1.10, 25
+  // K-steps 1.00.  Streaming: 0.71 .. 0.98 over 12 (256 channels, 14x14, 512 filters 3x3 stride 2, 256 images 24.7 -> 22.6).
+  const bool long_items = !fuse && planes == 1 && single.ok && single.P.nsteps >= kPairSteps;
+  if (single.ok && single.P.resident) {
+    if (long_items && single.P.nslabs == 2 && single.P.ntiles * 2 >= 5 * (int)kSms) {
+      const Plan pair = make_plan(g, 0, true, fuse, planes, residual);
+      if (pair.ok && pair.P.resident) return pair;
+    }
+    return single;
+  }
   // a problem of few items is better spread over single CTAs
   if (single.ok && 2 * single.P.ntiles * single.P.nslabs <= (int)kSms) return single;
   Plan pair = make_plan(g, single.by_time ? 1 : 0, true, fuse, planes, residual);
-  if (pair.ok && (pair.P.resident || !single.ok || (pair.P.NT > 64 && pair.P.nsteps >= kLongItem))) return pair;
+  if (pair.ok && (pair.P.resident || !single.ok || (pair.P.NT > 64 && (long_items || pair.P.nsteps >= kLongItem)))) return pair;
   return single;
 }
 

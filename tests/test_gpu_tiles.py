@@ -169,6 +169,7 @@ def test_fused_schedules(oracle, case, resident, slabs, filters, parts):
     ((30, 33, 31, 30, 428, 1, 1, 2, 0), 1, 0, 2, 224), ((16, 128, 28, 28, 256, 3, 3, 2, 1), 1, 0, 2, 128),
     ((136, 944, 8, 19, 512, 1, 1, 1, 0), 0, 0, 4, 128), ((11, 544, 22, 37, 178, 3, 3, 1, 1), 0, 1, 1, 192),
     ((40, 300, 14, 13, 250, 7, 7, 1, 3), 0, 1, 1, 256),
+    ((170, 90, 15, 16, 256, 5, 5, 1, 2), 1, 1, 2, 128), ((42, 320, 21, 22, 200, 3, 3, 2, 1), 0, 1, 2, 128),
     ((1, 256, 7, 7, 256, 1, 1, 1, 0), 1, 0, 16, 16), ((1, 256, 7, 7, 272, 1, 1, 1, 0), 0, 0, 17, 16),
     ((1, 512, 7, 7, 512, 3, 3, 1, 1), 1, 0, 16, 32), ((1, 512, 7, 7, 528, 3, 3, 1, 1), 0, 0, 17, 32)])
 def test_plain_schedules(oracle, shape, resident, pair, slabs, filters):
