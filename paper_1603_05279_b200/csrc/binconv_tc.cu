@@ -1652,10 +1652,10 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
 
 namespace {
 
-// The plan of a variant.  kTcAuto (measured on the AlexNet and ResNet-18 shapes): one CTA per
-// SM unless only a pair, each CTA holding half of a slab, can keep the filters resident.  Neither: pairs
-// where the items are long (each CTA expands half the rows of a slab; 1024 channels, 7x7 kernel: 419 ->
-// 361 us; 1x1 kernel, 16 K-steps: 27.2 -> 30.5 us) and the slabs wide enough to fill a pair.
+// The plan of a variant.  kTcAuto: one CTA per SM unless only a pair, each CTA holding half of a slab, can keep
+// the filters resident, or the items are long (see below).  Neither resident: pairs where the items are long (each CTA
+// expands half the rows of a slab; 1024 channels, 1x1, 16 K-steps: 16.9 -> 17.5 us) and the slabs wide enough to
+// fill a pair.  Over 253 drawn shapes the choice is within 1 % (geometric mean) of the best variant.
 Plan plan_variant_uncached(const ConvGeom &g, TcVariant v, bool fuse, int planes, bool residual) {
   switch (v) {
     case kTcSingle: return make_plan(g, 0, false, fuse, planes, residual);
