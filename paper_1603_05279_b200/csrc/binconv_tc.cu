@@ -69,6 +69,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "drain.cuh"
 #include "umma_common.cuh"
 
 namespace xnor {
@@ -172,12 +173,11 @@ struct TcParams {
   // layer's channels) and sums |y| over the filters it handles.
   const float *nscale, *nshift;      // [C_out], both null = identity
   uint32_t *xp_next;                 // u32 [N][Ho][Wo][Cw_next]
-  float *A_part;                     // fp32 [nslabs * epi_chunks][N][Ho][Wo]: partial sums of |y|
+  float *A_part;                     // fp32 [nslabs * drain.chunks][N][Ho][Wo]: partial sums of |y|
   int Cw_next;                       // ceil(C_out / 32)
   int resident;                // 1: resident schedule (stages = all stages of a slab)
   int wgt_groups;              // streaming: groups of four warps that expand weights, 3 or 2
-  int epi_split;               // warps per lane quarter that drain accumulators
-  int epi_chunk, epi_chunks;   // groups of 16 columns that a warp drains in one go; such chunks of an item
+  Drain drain;                 // how the warps of a lane quarter drain accumulators
   int any_swap;                // some bit of swap_mask is set
   uint32_t div_wq_m, div_hq_m; // multipliers and shifts of the exact divisions by Wq and Hq
   int div_wq_s, div_hq_s;      // (dividends below 2^31)
@@ -1011,16 +1011,15 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
 // run of the NCHW output row.
 // Drains the CTA's `nitems` items: streaming, items i0, i0 + 1, ...
 // (item = tile * nslabs + slab); resident, tiles tile0, tile0 + tstep, ... of slab `slab0`.
-// An item is cut into chunks of epi_chunk groups of 16 columns, and the chunks of all items in sequence are
-// dealt to the esplit warps that share a quarter of the lanes: a warp's work per item (decoding its pixel,
-// the waits) is then spread over a whole chunk.
+// An item is cut into chunks, and the chunks of all items in sequence are dealt to the warps that share a quarter
+// of the lanes (Drain): a warp's work per item (decoding its pixel, the waits) is then spread over a whole chunk.
 // kFuse: a chunk is an even number of groups (a pair = 32 consecutive filters = one packed word of the
 // next layer's input) and has a plane of partial sums of its own; see the fused emit below.
 template <bool kRes, bool kFuse>
 __device__ void epilogue_role(const TcParams &P, const Smem &S, long long i0, int slab0, int tile0,
                               int tstep, uint32_t nitems, uint32_t tmem_base, int quarter, int e, int lane) {
   const int b_end = P.NT / 16;
-  const int esplit = P.epi_split, chunks = P.epi_chunks;
+  const Drain D = P.drain;
   const size_t HoWo = (size_t)P.Ho * P.Wo;
   const uint32_t howo = (uint32_t)HoWo;
   const size_t out_elems = (size_t)P.N * P.Co * HoWo;
@@ -1036,8 +1035,8 @@ __device__ void epilogue_role(const TcParams &P, const Smem &S, long long i0, in
   if (kRes) { at.slab = slab0; at.tile = tile0; }
   else { at.tile = (int)(i0 / P.nslabs); at.slab = (int)(i0 - (long long)at.tile * P.nslabs); }
   auto settle = [&](At &a) {
-    while (a.c >= chunks) {
-      a.c -= chunks;
+    while (a.c >= D.chunks) {
+      a.c = D.carry(a.c);
       ++a.it;
       if (++a.ab == P.nacc) { a.ab = 0; a.fph ^= 1u; }
       if (kRes) a.tile += tstep;
@@ -1048,9 +1047,10 @@ __device__ void epilogue_role(const TcParams &P, const Smem &S, long long i0, in
   constexpr uint32_t kNoPixel = 0xFFFFFFFFu;
   // this lane's output pixel in a tile: whether it exists, its K, offset of (image, filter 0, pixel)
   struct Pix { float kv; size_t obase; uint32_t gpix; };   // gpix: pixel index over all images (below the stream's length)
+  const uint32_t tile_len = P.pair ? 2u * kTileM : kTileM, pos0 = S.rank * kTileM + (uint32_t)(quarter * 32 + lane);
   auto decode = [&](int t) {
     Pix px{0.0f, 0, kNoPixel};
-    const uint32_t m = ((uint32_t)t * (P.pair ? 2u : 1u) + S.rank) * kTileM + (uint32_t)(quarter * 32 + lane);
+    const uint32_t m = (uint32_t)t * tile_len + pos0;
     if (m < (uint32_t)P.L) {
       const uint32_t r = fast_div(m, P.div_wq_m, P.div_wq_s);
       const int ox = (int)(m - r * (uint32_t)P.Wq);
@@ -1074,7 +1074,7 @@ __device__ void epilogue_role(const TcParams &P, const Smem &S, long long i0, in
     if (vm == 0u) return;
     const unsigned long long o0 = __shfl_sync(0xffffffffu, (unsigned long long)px.obase, __ffs(vm) - 1);
     const unsigned long long o1 = __shfl_sync(0xffffffffu, (unsigned long long)px.obase, 31 - __clz(vm));
-    const int f0 = a.slab * P.NT + a.c * P.epi_chunk * 16, f1 = min(P.Co, min(f0 + P.epi_chunk * 16, (a.slab + 1) * P.NT));
+    const int f0 = a.slab * P.NT + a.c * D.chunk * 16, f1 = min(P.Co, min(f0 + D.chunk * 16, (a.slab + 1) * P.NT));
     for (int j = f0 + lane; j < f1; j += 32) {
       const float *rp = P.residual + (size_t)j * HoWo;
       asm volatile("prefetch.global.L2 [%0];" ::"l"(rp + o0));
@@ -1093,7 +1093,7 @@ __device__ void epilogue_role(const TcParams &P, const Smem &S, long long i0, in
     const uint32_t obase_pix = px.gpix;
     // the chunk after this one; its pixel is decoded (and its K and residual on their way) while this one drains
     At nx = at;
-    nx.c += esplit;
+    nx.c += D.split;
     settle(nx);
     Pix npx = px;
     if (nx.it < nitems) {
@@ -1229,9 +1229,9 @@ __device__ void epilogue_role(const TcParams &P, const Smem &S, long long i0, in
     // stores of the current ones saves the ~50 cycles of a tensor-memory load per group but
     // costs 16 register copies, which take longer here.)
     int32_t cur[16];
-    const int b1 = min((at.c + 1) * P.epi_chunk, b_end);      // groups of the chunk
+    const int b1 = min((at.c + 1) * D.chunk, b_end);      // groups of the chunk
 #pragma unroll 1
-    for (int b = at.c * P.epi_chunk; b < b1; ++b) {
+    for (int b = at.c * D.chunk; b < b1; ++b) {
       tmem_ld16(t_acc + (uint32_t)(b * 16), cur);
       tmem_wait16(cur);
       if (b + 1 == b1) {                         // that was the last load: release the buffer
@@ -1254,7 +1254,7 @@ __device__ void epilogue_role(const TcParams &P, const Smem &S, long long i0, in
       }
     }
     if (kFuse && valid && in_bounds(obase_pix < (size_t)P.N * HoWo, 12))
-      P.A_part[(size_t)(slab * chunks + at.c) * ((size_t)P.N * HoWo) + obase_pix] = (as0 + as1) + (as2 + as3);
+      P.A_part[(size_t)(slab * D.chunks + at.c) * ((size_t)P.N * HoWo) + obase_pix] = (as0 + as1) + (as2 + as3);
     px = npx;
     at = nx;
   }
@@ -1286,7 +1286,7 @@ binconv_tc_kernel(const __grid_constant__ TcParams P) {
     }
     for (int i = 0; i < kMaxAcc; ++i) {
       mbar_init(S.afull + 8u * i, 1);
-      mbar_init(S.aempty + 8u * i, (uint32_t)(kEpiWarps * P.epi_chunks) * kCtas);
+      mbar_init(S.aempty + 8u * i, (uint32_t)(kEpiWarps * P.drain.chunks) * kCtas);
     }
     *S.abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1351,7 +1351,7 @@ binconv_tc_kernel(const __grid_constant__ TcParams P) {
       // warps 5-7, 9-11, ... in this order: weight groups, patch warps; the last four warps drain too
       // where the epilogue is split
       const int wi = ((warp >> 2) - 1) * 3 + (warp & 3) - 1 - kGroupWarps * P.wgt_groups;
-      const bool last = warp >= kThreadsStream / 32 - kEpiWarps && P.epi_split == 2;
+      const bool last = warp >= kThreadsStream / 32 - kEpiWarps && P.drain.split == 2;
       if (warp < kEpiWarps || last)
         epilogue_role<false, kFuse>(P, S, i0, 0, 0, 0, (uint32_t)(i1 - i0), tmem_base, warp & 3, last ? 1 : 0, lane);
       else if ((warp & 3) == 0) {}
@@ -1368,7 +1368,7 @@ binconv_tc_kernel(const __grid_constant__ TcParams P) {
       const bool wgt = warp >= kWgtWarp0;
       const int e = wgt ? 1 + (warp - kWgtWarp0) / 4 : 0;
       if (wgt) weight_dispatch(P, S, (int)R.slab, wt, lane);
-      if (e < P.epi_split)
+      if (e < P.drain.split)
         epilogue_role<true, kFuse>(P, S, 0, (int)R.slab, (int)R.g, (int)R.G, R.total(), tmem_base, warp & 3, e, lane);
     }
   }
@@ -1591,21 +1591,10 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
   }
   P.nraw = fits(stages, npb, 2) ? 2 : 1;
   P.nacc = std::max(1, std::min(kMaxAcc, kMaxAccCols / P.NT));
-  // worker warps per quarter of the lanes in the resident schedule: the four epilogue warps
-  // and the eight weight warps
-  P.epi_split = P.resident ? std::min(kEpiSplitMax, P.NT / (fuse ? 32 : 16)) : P.wgt_groups == 2 ? std::min(2, P.NT / (fuse ? 32 : 16)) : 1;
-  // Chunks of an item that the draining warps take in turn (see epilogue_role).  What a warp does per item
-  // (its pixel, K, the waits: some 150 instructions) was a third of all instructions while every warp took a
-  // share of every item: 64 channels, 56x56, 64 filters 3x3, 256 images 71.8 -> 63.1 us, with a residual 107.0 ->
-  // 90.5 (four groups over three warps had also left one with two); 128 channels, 28x28: 36.2 -> 32.7 and 51.4 -> 49.0;
-  // fused, the same two layers 102 -> 82 and 50 -> 41.  With fewer items than warps take turns over, all of them
-  // share an item, whose latency then counts (fused, one image: 7.4 us, in chunks of 64 filters 7.7).
-  const int epi_groups = P.NT / 16;
+  // warps per quarter of the lanes: resident, the four epilogue warps and the eight weight warps
+  const int drain_warps = P.resident ? kEpiSplitMax : P.wgt_groups == 2 ? 2 : 1;
   const long long unit_items = ((long long)P.ntiles * P.nslabs + units - 1) / units;
-  P.epi_chunk = (epi_groups + P.epi_split - 1) / P.epi_split;
-  if (fuse) P.epi_chunk = std::max(unit_items >= 4 ? 4 : 2, (P.epi_chunk + 1) / 2 * 2);
-  else if (unit_items >= 4) P.epi_chunk = 4;
-  P.epi_chunks = (epi_groups + P.epi_chunk - 1) / P.epi_chunk;
+  P.drain = plan_drain(P.NT / 16, std::min(drain_warps, P.NT / (fuse ? 32 : 16)), unit_items >= 4, fuse);
   if (fuse && (g.Co & 31) != 0) return pl;          // whole words of the next layer's input
   P.stages = stages; P.npb = npb;
   P.off_tab = 0u;
@@ -1802,7 +1791,7 @@ cudaError_t launch_binconv_tc(const uint32_t *xp, const uint32_t *wp, const floa
 int tc_fused_parts(const ConvGeom &g, TcVariant variant) {
   const Plan pl = plan_variant(g, variant, true, 1, false);
   if (!pl.ok) return 0;
-  return pl.P.nslabs * pl.P.epi_chunks;
+  return pl.P.nslabs * pl.P.drain.chunks;
 }
 
 cudaError_t launch_binconv_tc_fused(const uint32_t *xp, const uint32_t *wp, const float *alpha,

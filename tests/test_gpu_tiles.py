@@ -183,7 +183,7 @@ def test_plain_schedules(oracle, shape, resident, pair, slabs, filters):
 # four chunks, a short last chunk, filters beyond C_out, warps that skip items; every schedule
 @pytest.mark.parametrize("engine", [X.XNOR_ENGINE_AUTO, X.XNOR_ENGINE_UMMA_STREAM, X.XNOR_ENGINE_UMMA_PAIR])
 @pytest.mark.parametrize("residual", [False, True])
-@pytest.mark.parametrize("Co,k", [(16, 1), (48, 3), (70, 1), (112, 3), (200, 1), (240, 1)])
+@pytest.mark.parametrize("Co,k", [(16, 1), (48, 3), (70, 1), (80, 1), (112, 3), (144, 3), (200, 1), (240, 1)])
 def test_drained_chunks(oracle, Co, k, residual, engine):
     N, C, H, W = 160, 16, 23, 24
     d = X.make_desc(N, C, H, W, Co, k, k, 1, k // 2)
