@@ -1013,6 +1013,7 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
 // (item = tile * nslabs + slab); resident, tiles tile0, tile0 + tstep, ... of slab `slab0`.
 // An item is cut into chunks, and the chunks of all items in sequence are dealt to the warps that share a quarter
 // of the lanes (Drain): a warp's work per item (decoding its pixel, the waits) is then spread over a whole chunk.
+// A warp may have no chunk in an item and skips it; plan_drain keeps such steps within what parities can tell.
 // kFuse: a chunk is an even number of groups (a pair = 32 consecutive filters = one packed word of the
 // next layer's input) and has a plane of partial sums of its own; see the fused emit below.
 template <bool kRes, bool kFuse>
@@ -1594,7 +1595,7 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
   // warps per quarter of the lanes: resident, the four epilogue warps and the eight weight warps
   const int drain_warps = P.resident ? kEpiSplitMax : P.wgt_groups == 2 ? 2 : 1;
   const long long unit_items = ((long long)P.ntiles * P.nslabs + units - 1) / units;
-  P.drain = plan_drain(P.NT / 16, std::min(drain_warps, P.NT / (fuse ? 32 : 16)), unit_items >= 4, fuse);
+  P.drain = plan_drain(P.NT / 16, std::min(drain_warps, P.NT / (fuse ? 32 : 16)), unit_items >= 4, fuse, P.nacc);
   if (fuse && (g.Co & 31) != 0) return pl;          // whole words of the next layer's input
   P.stages = stages; P.npb = npb;
   P.off_tab = 0u;

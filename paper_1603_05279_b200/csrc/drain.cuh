@@ -24,7 +24,14 @@ struct Drain {
   }
 };
 
-// many: four and more items per CTA (pair).
+// many: four and more items per CTA (pair).  accumulators: buffers that the items take in turn.
+//
+// A draining warp may have no chunk in some items.  It finds an item's accumulator full by the parity of that
+// buffer's barrier, which tells apart two consecutive uses only.  So when it waits for an item it must know that the
+// buffer's use before is over, that is, have seen an item no more than `accumulators` back (they are committed
+// in order): ceil(split / chunks) <= accumulators.  Beyond that it would take an earlier item's accumulator
+// for the one it waits for, with wrong sums and no expired wait.  Fewer warps take turns then.  (No plan needs that
+// today: one chunk is at most 64 filters, which leave four accumulators for three warps.)
 //
 // What a warp does per item (its pixel, K, the waits: some 150 instructions) was a third of all instructions while
 // every warp took a share of every item: 64 channels, 56x56, 64 filters 3x3, 256 images 71.8 -> 63.1 us in chunks
@@ -40,13 +47,14 @@ struct Drain {
 // Without need: 160 filters 22.1 -> 22.5, 176 24.0 -> 24.4.
 //
 // Fused, a chunk is an even number of groups (a pair is a packed word of the next layer's input).
-inline Drain plan_drain(int groups, int warps, bool many, bool fused) {
+inline Drain plan_drain(int groups, int warps, bool many, bool fused, int accumulators) {
   Drain d{};
   d.split = warps;
   d.chunk = (groups + warps - 1) / warps;
   if (fused) d.chunk = (d.chunk + 1) / 2 * 2;
   if (many && (!fused || d.chunk < 4)) d.chunk = 4;
   d.chunks = (groups + d.chunk - 1) / d.chunk;
+  if ((warps + d.chunks - 1) / d.chunks > accumulators) return plan_drain(groups, warps - 1, many, fused, accumulators);
   const int unit = fused ? 2 : 1, share = (groups / unit + warps - 1) / warps * unit;
   d.rotate = d.chunks % warps == 0 && d.chunks / warps * d.chunk > share;
   return d;
