@@ -652,7 +652,7 @@ __device__ void weight_role(const TcParams &P, const Smem &S, int slab, int wt, 
     }
     fence_proxy_async();
     __syncwarp();
-    if (lane == 0) { if (P.pair) mbar_arrive_cluster(S.wfull + 8u * st, 0u); else mbar_arrive(S.wfull + 8u * st); }
+    if (lane == 0) { if (P.pair) mbar_arrive_peer_mma(S.wfull + 8u * st, 0u); else mbar_arrive(S.wfull + 8u * st); }
     // the queue of packed words moves up one stage; the freed slot is refilled
 #pragma unroll
     for (int d = 0; d + 1 < kPrefetch; ++d)
@@ -743,7 +743,7 @@ __device__ void weight_stream(const TcParams &P, const Smem &S, uint32_t nitems,
     }
     fence_proxy_async();
     __syncwarp();
-    if (lane == 0) { if (P.pair) mbar_arrive_cluster(S.wfull + 8u * ws, 0u); else mbar_arrive(S.wfull + 8u * ws); }
+    if (lane == 0) { if (P.pair) mbar_arrive_peer_mma(S.wfull + 8u * ws, 0u); else mbar_arrive(S.wfull + 8u * ws); }
     ws += (uint32_t)P.wgt_groups;
     if (ws >= (uint32_t)P.stages) { ws -= (uint32_t)P.stages; wph ^= 1u; }
   }
@@ -992,7 +992,7 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
     __syncwarp();
     if (lane == 0) {
       mbar_arrive(S.rawdone + 8u * rb);
-      if (P.pair) mbar_arrive_cluster(S.pfull + 8u * pb, 0u); else mbar_arrive(S.pfull + 8u * pb);
+      if (P.pair) mbar_arrive_peer_mma(S.pfull + 8u * pb, 0u); else mbar_arrive(S.pfull + 8u * pb);
     }
   }
   if (!ok && mi == 0) {
@@ -1238,7 +1238,7 @@ __device__ void epilogue_role(const TcParams &P, const Smem &S, long long i0, in
       if (b + 1 == b1) {                         // that was the last load: release the buffer
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) { if (P.pair) mbar_arrive_cluster(S.aempty + 8u * at.ab, 0u); else mbar_arrive(S.aempty + 8u * at.ab); }
+        if (lane == 0) { if (P.pair) mbar_arrive_peer_mma(S.aempty + 8u * at.ab, 0u); else mbar_arrive(S.aempty + 8u * at.ab); }
       }
       if (kFuse) {
         // C_out is a multiple of 32, so a pair of groups lies inside the filters or (last slab)

@@ -53,12 +53,21 @@ __device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) {
   asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
-// Arrival on the barrier at the same shared-memory offset in CTA `cta` of this cluster.  Released at the
-// scope of the CTA, as the open-source CUTLASS barriers do: what it stands for is shared memory that this CTA's own
-// tensor core reads (behind fence_proxy_async()) or tensor memory that this CTA has read.  A release at the scope of
-// the cluster waits for all memory operations of the thread, some 1000 cycles, which was half of a weight
-// stage's time (1024 channels, 7x7, 256 filters, 64 images on CTA pairs: 101.8 -> 79.7 us).
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar, uint32_t cta) {
+// Arrival of a producer or draining warp on the barrier at the same shared-memory offset in CTA `cta` of its pair,
+// for the thread there that issues the pair's MMAs.  It stands for shared memory of THIS CTA that this SM's own
+// tensor core reads (written ahead of fence_proxy_async()) or for tensor memory of this CTA that has been read
+// (tcgen05.wait::ld has returned).
+//
+// It is released at the scope of the CTA (the default).  The PTX memory model does not make that an order between
+// this thread's writes and what a thread of the other CTA does after its wait; that the MMA finds them rests on
+// their being complete in this SM before the arrival leaves it, and on the open-source CUTLASS kernels for CTA pairs,
+// whose barriers are signalled in this form.  So it must NOT announce data that the peer's threads read themselves,
+// by loads from shared or global memory: that takes a release at the scope of the cluster.
+//
+// A release at that scope waits for the memory operations in flight: 1024 channels, 7x7, 256 filters, 64 images
+// 101.8 us with one in every arrival, 122.5 with arrivals inside each CTA passed on by a thread of its own, 70.2
+// in this form; 384 channels, 13x13, 384 filters 3x3, 256 images 36.2, 40.0 and 32.0.
+__device__ __forceinline__ void mbar_arrive_peer_mma(uint32_t bar, uint32_t cta) {
   asm volatile(
       "{\n\t.reg .b32 ra;\n\t"
       "mapa.shared::cluster.u32 ra, %0, %1;\n\t"

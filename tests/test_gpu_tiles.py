@@ -207,6 +207,44 @@ def test_drained_chunks(oracle, Co, k, residual, engine):
     assert_close(host(out), oracle.xnor_block(x, w, 1, k // 2, None, None, res).out, "out")
 
 
+# CTA pairs: what the warps of one CTA announce to the issuing thread of the other is there when the MMA reads it.  Many
+# launches of many items, resident (one and several slabs) and streaming, the inputs changing from launch to launch
+# so that nothing left over from the one before can pass: bit for bit what the CUDA cores give
+@pytest.mark.parametrize("engine", [X.XNOR_ENGINE_UMMA_PAIR, X.XNOR_ENGINE_UMMA_PAIR_STREAM])
+@pytest.mark.parametrize("shape", [(40, 384, 13, 13, 384, 3, 1), (64, 64, 28, 28, 96, 3, 1), (24, 512, 14, 14, 224, 3, 2),
+                                   (64, 128, 14, 14, 512, 1, 1)])
+def test_pairs_are_repeatably_exact(shape, engine):
+    N, C, H, W, Co, k, s = shape
+    d = X.make_desc(N, C, H, W, Co, k, k, s, k // 2)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(sum(shape))
+
+    def normal(*size):
+        return torch.randn(size, generator=g, device="cuda")
+
+    layers = []
+    for _ in range(3):
+        wp, alpha = X.alloc_weights(Co, C, k, k)
+        xp, A, K = X.alloc_binactiv(d)
+        X.xnor_binarize_weights(normal(Co, C, k, k), wp, alpha)
+        X.xnor_binactiv(normal(N, C, H, W), None, None, d, xp, A, K)
+        layers.append((xp, wp, alpha, K, X.alloc_out(d)))
+    outs = [X.alloc_out(d) for _ in range(30)]
+    try:
+        X.xnor_set_engine(X.XNOR_ENGINE_POPC)
+        for xp, wp, alpha, K, want in layers:
+            X.xnor_conv2d_forward(xp, wp, alpha, K, None, d, want)
+        X.xnor_set_engine(engine)
+        assert X.xnor_conv2d_plan(d).pair
+        for i, out in enumerate(outs):
+            xp, wp, alpha, K, _ = layers[i % 3]
+            X.xnor_conv2d_forward(xp, wp, alpha, K, None, d, out)
+    finally:
+        X.xnor_set_engine(X.XNOR_ENGINE_AUTO)
+    X.xnor_check_device()
+    assert all(torch.equal(out, layers[i % 3][4]) for i, out in enumerate(outs))
+
+
 # how a patch is built: one to six channel words, both strides, planes of more and of less than four columns (a
 # patch then touches more rows than a warp has lanes), the ragged end of the packed tensor; patches of one or two
 # items per CTA, which all patch warps build
