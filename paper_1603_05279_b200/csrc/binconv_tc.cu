@@ -182,7 +182,7 @@ struct TcParams {
   uint32_t div_wq_m, div_hq_m; // multipliers and shifts of the exact divisions by Wq and Hq
   int div_wq_s, div_hq_s;      // (dividends below 2^31)
   uint32_t div_pg_m, div_g_m;  // the same for the patch units: by phases * ngrp and by ngrp
-  int div_pg_s, div_g_s;       // (ngrp = groups of four channel words)
+  int div_pg_s, div_g_s;       // (ngrp = patch_groups())
   uint32_t wq_rcp;             // 2^32 / Wq, rounded up: exact quotients of a patch's positions
   int pat_table;               // a patch touches at most 32 rows of the stream
 };
@@ -317,6 +317,15 @@ inline uint32_t kstep_desc(const TcParams &P, int j, bool *swap) {
     lbo = o2 - o1;
   }
   return (o1 >> 4) | ((lbo >> 4) << 16);
+}
+
+// Units of channel words at one position of a patch.  Four words come together where they can be loaded as one, and in
+// the resident schedule.  Streaming, with fewer registers, other counts of five words and more go one by one, for
+// twice as many positions at a time: guarding each of four words for one position was slower than the two
+// divisions per unit before it (26.2 us for 218 images, 477 channels, 14x14, 400 filters 1x1 stride 2, 25.2 before,
+// 20.6 now; 0.98 to 1.08 of the time before over 28 drawn shapes, 0.80 to 1.0 now).  Resident, one by one is as often slower.
+__host__ __device__ inline int patch_groups(int Cw, bool resident) {
+  return !resident && Cw > 4 && (Cw & 3) != 0 ? Cw : (Cw + 3) / 4;
 }
 
 // Exact n / d for n < 2^31: q = (n * m) >> (31 + s) with m = ceil(2^(31+s) / d), s = ceil(log2 d).
@@ -780,7 +789,7 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
   const uint32_t word_bytes = (uint32_t)P.Cw * 4u, row_bytes = (uint32_t)P.W * word_bytes;   // of a pixel, a row
   // pairs: work tile t is stream tiles 2t (rank 0) and 2t + 1 (rank 1)
   const uint32_t tmul = P.pair ? 2u : 1u;
-  const int ngrp = (P.Cw + 3) >> 2;                       // groups of 4 channel words
+  const int ngrp = patch_groups(P.Cw, kRes);
 
   auto first_pos = [&](uint32_t seq) {                    // of patch seq, in the stream
     return ((kRes ? R.tile(seq) : (uint32_t)tile0 + seq) * tmul + S.rank) * kTileM;
@@ -826,7 +835,7 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
 
   // Expands this warp's share of a patch: raw buffer rb holds input rows g0 .. from address `raw` on, m0 is the
   // patch's first position.  Units, in this order of nesting: kPos x 32 positions, phase plane, kWords channel
-  // words (0: up to four, word by word); every warp of the subgroup takes a contiguous share.  A lane keeps
+  // words (0: up to four, one after the other); every warp of the subgroup takes a contiguous share.  A lane keeps
   // the address of one row of the patch, so that locating a position costs a multiplication and a shuffle; the
   // work on the kPos positions is independent, and the innermost part does not branch.  What bounds a patch is
   // the latency of its one warp: two divisions per position and unit, as before, took 4500 cycles for the patch of
@@ -835,6 +844,7 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
   // the place of a unit kept by branches in one flat loop were slower than the divisions (67.5).
   auto build = [&](auto kpos_, auto kwords_, uint32_t m0, int g0, uint32_t raw, uint32_t rb, uint32_t patch) {
     constexpr int kPos = decltype(kpos_)::value, kWords = decltype(kwords_)::value, kLoop = kWords ? kWords : 4;
+    constexpr int kStep = kWords == 1 ? 1 : 4;            // channel words of a unit
     const uint32_t r0 = fast_div(m0, P.div_wq_m, P.div_wq_s), c0 = m0 - r0 * (uint32_t)P.Wq;
     // addresses of the input rows of stream row r, one per row phase; 0: padding
     auto row_address = [&](uint32_t r, uint32_t &a0, uint32_t &a1) {
@@ -856,7 +866,7 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
       block = (int)fast_div((uint32_t)u, P.div_pg_m, P.div_pg_s);
       const int rem = u - block * (phases * ngrp);
       phase = (int)fast_div((uint32_t)rem, P.div_g_m, P.div_g_s);
-      w0 = (rem - phase * ngrp) * 4;
+      w0 = (rem - phase * ngrp) * kStep;
     }
 #pragma unroll 1
     for (; u < u1; ++block, phase = 0) {
@@ -895,7 +905,7 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
           dst[b] = pdst[b] + (uint32_t)(phase * P.Cw + w0) * plane_bytes;
         }
 #pragma unroll 1
-        for (; w0 < P.Cw && u < u1; w0 += 4, ++u) {
+        for (; w0 < P.Cw && u < u1; w0 += kStep, ++u) {
           uint32_t wv[kPos][4], wu[kTwo ? kPos : 1][4];
           auto load = [&](uint32_t a, uint32_t (&v)[4]) {
             if constexpr (kWords == 4) lds128(a, v);
@@ -908,11 +918,11 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
 #pragma unroll
           for (int b = 0; b < kPos; ++b) {
             if (in_bounds(src[b] >= S.raw + rb * P.raw_bytes &&
-                          src[b] + 4u * (uint32_t)min(4, P.Cw - w0) <= S.raw + rb * P.raw_bytes + P.raw_plane, 6)) {
+                          src[b] + 4u * (uint32_t)min(kStep, P.Cw - w0) <= S.raw + rb * P.raw_bytes + P.raw_plane, 6)) {
               load(src[b], wv[b]);
               if constexpr (kTwo) load(src[b] + P.raw_plane, wu[b]);
             }
-            src[b] += 16u;
+            src[b] += 4u * kStep;
           }
 #pragma unroll
           for (int i = 0; i < kLoop; ++i) {
@@ -987,7 +997,8 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
     else if (P.Cw == 1) build(many, integral_constant<int, 1>{}, m0, g0, raw, rb, patch);
     else if (P.Cw == 2) build(many, integral_constant<int, 2>{}, m0, g0, raw, rb, patch);
     else if (P.Cw == 3) build(few, integral_constant<int, 3>{}, m0, g0, raw, rb, patch);
-    else build(few, integral_constant<int, 0>{}, m0, g0, raw, rb, patch);
+    else if constexpr (kRes) build(few, integral_constant<int, 0>{}, m0, g0, raw, rb, patch);
+    else build(many, integral_constant<int, 1>{}, m0, g0, raw, rb, patch);
     fence_proxy_async();
     __syncwarp();
     if (lane == 0) {
@@ -1629,7 +1640,7 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
   };
   magic((uint32_t)P.Wq, &P.div_wq_m, &P.div_wq_s);
   magic((uint32_t)P.Hq, &P.div_hq_m, &P.div_hq_s);
-  const uint32_t ngrp = (uint32_t)(P.Cw + 3) / 4u;
+  const uint32_t ngrp = (uint32_t)patch_groups(P.Cw, P.resident != 0);
   magic((uint32_t)(s * s) * ngrp, &P.div_pg_m, &P.div_pg_s);
   magic(ngrp, &P.div_g_m, &P.div_g_s);
   P.wq_rcp = (uint32_t)((((unsigned long long)1 << 32) + P.Wq - 1) / P.Wq);    // (0 for a width of 1: no table then)

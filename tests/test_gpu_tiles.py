@@ -245,7 +245,8 @@ def test_pairs_are_repeatably_exact(shape, engine):
     assert all(torch.equal(out, layers[i % 3][4]) for i, out in enumerate(outs))
 
 
-# how a patch is built: one to six channel words, both strides, planes of more and of less than four columns (a
+# how a patch is built: one to thirteen channel words (five and more that are no multiple of four go one by one when
+# streaming), both strides, planes of more and of less than four columns (a
 # patch then touches more rows than a warp has lanes), the ragged end of the packed tensor; patches of one or two
 # items per CTA, which all patch warps build
 @pytest.mark.parametrize("engine", [X.XNOR_ENGINE_AUTO, X.XNOR_ENGINE_UMMA_STREAM, X.XNOR_ENGINE_UMMA_PAIR])
@@ -253,7 +254,8 @@ def test_pairs_are_repeatably_exact(shape, engine):
     (70, 20, 9, 1, 16, 1, 1, 1, 0), (70, 33, 5, 2, 16, 3, 3, 1, 1), (150, 70, 3, 3, 24, 3, 3, 1, 1),
     (90, 128, 7, 4, 16, 3, 3, 2, 1), (41, 161, 5, 3, 32, 3, 2, 1, 1), (3, 64, 41, 33, 20, 3, 3, 2, 1),
     (5, 96, 17, 19, 40, 5, 5, 2, 2), (3, 31, 29, 40, 16, 3, 3, 2, 0), (7, 190, 13, 11, 48, 1, 1, 2, 0),
-    (37, 100, 15, 17, 77, 5, 5, 1, 2), (60, 40, 29, 30, 64, 3, 3, 2, 1), (36, 64, 27, 28, 100, 3, 3, 1, 1)])
+    (37, 100, 15, 17, 77, 5, 5, 1, 2), (60, 40, 29, 30, 64, 3, 3, 2, 1), (36, 64, 27, 28, 100, 3, 3, 1, 1),
+    (9, 167, 35, 35, 288, 1, 1, 1, 0), (2, 392, 23, 24, 112, 3, 3, 2, 1), (4, 352, 9, 2, 48, 3, 3, 1, 1), (1, 200, 21, 3, 32, 1, 1, 2, 0)])
 def test_patches(oracle, shape, engine):
     block_parity(oracle, shape, engine)
 
