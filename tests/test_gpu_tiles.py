@@ -164,7 +164,8 @@ def test_fused_schedules(oracle, case, resident, slabs, filters, parts):
 
 
 # the plain convolution: several resident slabs of few K-steps, streaming because it is faster, pairs streaming
-# slabs of more than 128 filters (and of 256, with one accumulator, where a pair has one item), and both sides of the 16 slabs that a small problem may keep resident
+# slabs of more than 128 filters (and of 256, with one accumulator, where a pair has one item), and both sides
+# of the 16 slabs that a small problem may keep resident
 @pytest.mark.parametrize("shape,resident,pair,slabs,filters", [
     ((30, 33, 31, 30, 428, 1, 1, 2, 0), 1, 0, 2, 224), ((16, 128, 28, 28, 256, 3, 3, 2, 1), 1, 0, 2, 128),
     ((136, 944, 8, 19, 512, 1, 1, 1, 0), 0, 0, 4, 128), ((11, 544, 22, 37, 178, 3, 3, 1, 1), 0, 1, 1, 192),
@@ -180,7 +181,8 @@ def test_plain_schedules(oracle, shape, resident, pair, slabs, filters):
 
 
 # several items per CTA, drained in chunks of 64 filters that the warps of a lane quarter take in turn: one to
-# four chunks, a short last chunk, filters beyond C_out, warps that skip items; every schedule
+# four chunks, a short last chunk, turns that move on from item to item, filters beyond C_out, warps that skip items.
+# Items of few K-steps: resident with three warps per quarter (single CTAs, pairs), streaming with two
 @pytest.mark.parametrize("engine", [X.XNOR_ENGINE_AUTO, X.XNOR_ENGINE_UMMA_STREAM, X.XNOR_ENGINE_UMMA_PAIR])
 @pytest.mark.parametrize("residual", [False, True])
 @pytest.mark.parametrize("Co,k", [(16, 1), (48, 3), (70, 1), (80, 1), (112, 3), (144, 3), (200, 1), (240, 1)])
@@ -205,6 +207,58 @@ def test_drained_chunks(oracle, Co, k, residual, engine):
     X.xnor_check_device()
     gs.check()
     assert_close(host(out), oracle.xnor_block(x, w, 1, k // 2, None, None, res).out, "out")
+
+
+# The remaining schedules of the drain, through both lean store branches (acc_out absent, with and without a
+# residual), against the CUDA cores bit for bit and the oracle on the outer images: streaming and streaming pairs with one
+# draining warp per quarter (64 K-steps and more), two and three chunks per item, four items per CTA; pairs
+# streaming short items, two chunks of 4 + 2 groups; one slab of 256 filters with one accumulator
+@pytest.mark.parametrize("residual", [False, True])
+@pytest.mark.parametrize("shape,engine,resident,pair,slabs,filters", [
+    ((100, 256, 28, 28, 128, 3, 1, 1), X.XNOR_ENGINE_UMMA_STREAM, 0, 0, 1, 128),
+    ((100, 256, 28, 28, 128, 3, 1, 1), X.XNOR_ENGINE_UMMA_PAIR_STREAM, 0, 1, 1, 128),
+    ((60, 490, 35, 30, 190, 3, 1, 1), X.XNOR_ENGINE_AUTO, 0, 1, 1, 192),
+    ((100, 64, 28, 28, 96, 3, 1, 1), X.XNOR_ENGINE_UMMA_PAIR_STREAM, 0, 1, 1, 96),
+    ((40, 300, 14, 13, 256, 7, 1, 3), X.XNOR_ENGINE_AUTO, 0, 1, 1, 256)])
+def test_drain_of_streamed_items(oracle, shape, engine, resident, pair, slabs, filters, residual):
+    N, C, H, W, Co, k, s, p = shape
+    d = X.make_desc(N, C, H, W, Co, k, k, s, p)
+    g = rng(Co + k)
+    x = g.standard_normal((N, C, H, W)).astype(np.float32)
+    w = g.standard_normal((Co, C, k, k)).astype(np.float32)
+    wp, alpha = X.alloc_weights(Co, C, k, k)
+    xp, A, K = X.alloc_binactiv(d)
+    gs = GuardSet()
+    want = X.alloc_out(d)
+    out = gs.like("out", want)
+    res = dev(g.standard_normal(tuple(out.shape)).astype(np.float32)) if residual else None
+    X.xnor_binarize_weights(dev(w), wp, alpha)
+    X.xnor_binactiv(dev(x), None, None, d, xp, A, K)
+    try:
+        X.xnor_set_engine(engine)
+        plan = X.xnor_conv2d_plan(d, residual=residual)
+        assert (plan.resident, plan.pair, plan.slabs, plan.slab_filters) == (resident, pair, slabs, filters)
+        X.xnor_conv2d_forward(xp, wp, alpha, K, res, d, out)
+        X.xnor_set_engine(X.XNOR_ENGINE_POPC)
+        X.xnor_conv2d_forward(xp, wp, alpha, K, res, d, want)
+    finally:
+        X.xnor_set_engine(X.XNOR_ENGINE_AUTO)
+    X.xnor_check_device()
+    gs.check()
+    assert torch.equal(out, want)
+    for n in (0, N - 1):
+        r = oracle.xnor_block(x[n:n + 1], w, s, p, residual=None if res is None else host(res[n:n + 1]))
+        assert_close(host(out[n:n + 1]), r.out, "out, image %d" % n)
+
+
+# fused, four items and more per CTA: chunks of 4 + 2 groups over three warps (resident, single CTAs and pairs) and
+# two (streaming), 4 + 4 + 2 and 6 + 4; from 96 K-steps one warp per quarter with a chunk of six groups
+@pytest.mark.parametrize("engine", [X.XNOR_ENGINE_UMMA_SINGLE, X.XNOR_ENGINE_UMMA_STREAM, X.XNOR_ENGINE_UMMA_PAIR,
+                                    X.XNOR_ENGINE_UMMA_PAIR_STREAM])
+@pytest.mark.parametrize("case", [(100, 64, 28, 28, 96, 3, 1, 1, 3, 1, 1, True), (100, 40, 28, 27, 160, 1, 1, 0, 1, 1, 0, False),
+                                  (50, 704, 28, 28, 192, 3, 1, 1, 1, 1, 0, False)])
+def test_fused_drain_of_many_items(oracle, case, engine):
+    fused_parity(oracle, case, engine)
 
 
 # CTA pairs: what the warps of one CTA announce to the issuing thread of the other is there when the MMA reads it.  Many

@@ -28,6 +28,8 @@ def test_parity_suite_on_the_checking_build():
                            cwd=ROOT, env=env, capture_output=True, text=True)
     assert probe.returncode == 0 and probe.stdout.strip() == "1", probe.stderr
     files = ["tests/test_gpu_parity.py", "tests/test_gpu_fused.py", "tests/test_gpu_options.py",
+             "tests/test_gpu_tiles.py::test_patches", "tests/test_gpu_tiles.py::test_drained_chunks",
+             "tests/test_gpu_tiles.py::test_drain_of_streamed_items", "tests/test_gpu_tiles.py::test_fused_drain_of_many_items",
              "tests/test_gpu_timed_paths.py::test_every_sweep_point",
              "tests/test_gpu_timed_paths.py::test_layers_at_full_batch_without_acc_out"]
     r = subprocess.run([sys.executable, "-m", "pytest", "-x", "-q", "-m", "gpu", "-p", "no:cacheprovider"] + files,
