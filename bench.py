@@ -47,7 +47,7 @@ NCU_TRAFFIC = {"kernel_sha1": "029c4ca259d103806041fd60e2a27329bf1c7de4", "bytes
 def kernel_sha1():
     import hashlib
     h = hashlib.sha1()
-    for f in ("binconv_tc.cu", "umma_common.cuh", "common.cuh"):
+    for f in ("binconv_tc.cu", "drain.cuh", "umma_common.cuh", "common.cuh"):
         h.update(open(os.path.join(ROOT, "paper_1603_05279_b200", "csrc", f), "rb").read())
     return h.hexdigest()
 

@@ -760,7 +760,8 @@ __device__ void weight_stream(const TcParams &P, const Smem &S, uint32_t nitems,
 
 // ------------------------------------------------------------------ patch producers
 // The group of the three patch warps builds the CTA's patches one after the
-// other, all warps on the same patch, or each builds patches of its own.  The packed pixels a patch touches are ONE contiguous range of x_packed: input rows
+// other, all warps on the same patch, or each builds patches of its own.  The
+// packed pixels a patch touches are ONE contiguous range of x_packed: input rows
 // g0 .. g1 - 1 of the N*H rows (images follow one another in memory, the zero rows and
 // columns of the stream exist only in the patch).  Every patch buffer has a raw buffer; the
 // group's first warp brings a patch's range into it with one bulk copy (an aligned superset
@@ -1017,7 +1018,7 @@ __device__ void patch_role(const TcParams &P, const Smem &S, long long i0, long 
 }
 
 // ------------------------------------------------------------------ epilogue (4 warps)
-// Warp w reads tensor-memory lanes 32 w .. +31 (pixels), all the slab's columns (filters).
+// Warp w reads tensor-memory lanes 32 (w % 4) .. +31 (pixels), of every item the columns (filters) of some chunks.
 // Lane = pixel, so for one filter a warp stores 32 consecutive stream pixels: a contiguous
 // run of the NCHW output row.
 // Drains the CTA's `nitems` items: streaming, items i0, i0 + 1, ...
@@ -1526,14 +1527,18 @@ Plan make_plan(const ConvGeom &g, int schedule, bool pair, bool fuse, int planes
     // Resident: the widest slab whose expanded rows fit beside two patches.  Every slab needs its own
     // patch per tile and narrow MMAs re-read the pixel operand more often.  So (measured) several slabs
     // pay only from 128 filters (a pair: 96; 512 channels, 7x7, residual: 45.6 -> 34.1 us) and, with fewer
-    // than two K-steps per plane of the patch, where streams_faster() says no.  The fused epilogue, half as long again, outweighs the
-    // patches whatever the kernel: resident wherever it fits (16 channels, 34x34, 768 filters 1x1, 58 images:
-    // 136 us streaming, 64 resident; 0.68 of the time in the median of 68 drawn shapes of several slabs).
+    // than two K-steps per plane of the patch, where streams_faster() says no.  The fused epilogue, half as long
+    // again, outweighs the patches whatever the kernel: resident wherever it fits (16 channels, 34x34, 768
+    // filters 1x1, 58 images: 136 us streaming, 64 resident; 0.68 of the time in the median of 68 drawn shapes of
+    // several slabs).
     for (int ns = min_slabs; ns <= 16 && !P.resident; ++ns) {
       P.NT = slab_width(g.Co, ns, pair || fuse);
       P.nslabs = (g.Co + P.NT - 1) / P.NT;
       P.NTh = pair ? P.NT / 2 : P.NT;
-      if (P.nslabs > 1 && (!few || P.ntiles * ns > (int)kSms * planes) && (P.NT < (pair ? 96 : 128) || (!fuse && P.nsteps < 2 * P.nplanes && (pl.by_time = streams_faster())))) break;
+      if (P.nslabs > 1 && (!few || P.ntiles * ns > (int)kSms * planes)) {
+        if (P.NT < (pair ? 96 : 128)) break;
+        if (!fuse && P.nsteps < 2 * P.nplanes && (pl.by_time = streams_faster())) break;
+      }
       // (Lending four of the weight warps to the patch builders where a pixel has many channel
       // words was the better split while the drain loop was longer; since its trimming twelve
       // draining warps win on every layer measured: conv4 50.4 -> 48.1 us, conv5 39.4 -> 37.3.)
@@ -1656,7 +1661,8 @@ namespace {
 // The plan of a variant.  kTcAuto: one CTA per SM unless only a pair, each CTA holding half of a slab, can keep
 // the filters resident, or the items are long (see below).  Neither resident: pairs where the items are long (each CTA
 // expands half the rows of a slab; 1024 channels, 1x1, 16 K-steps: 16.9 -> 17.5 us) and the slabs wide enough to
-// fill a pair.  Over 253 drawn shapes the choice is within 1 % (geometric mean) of the best variant.
+// fill a pair.  Over 255 drawn shapes the choice takes 1.010 of the time of the best variant (geometric mean;
+// 234 of them within 2 %, 245 within 5 %).
 Plan plan_variant_uncached(const ConvGeom &g, TcVariant v, bool fuse, int planes, bool residual) {
   switch (v) {
     case kTcSingle: return make_plan(g, 0, false, fuse, planes, residual);
@@ -1666,10 +1672,14 @@ Plan plan_variant_uncached(const ConvGeom &g, TcVariant v, bool fuse, int planes
     default: break;
   }
   Plan single = make_plan(g, 0, false, fuse, planes, residual);
-  // From 32 K-steps on the MMAs bound an item, and one thread of a pair issues those of two SMs at the cost of one's.
-  // Two resident slabs and several items per CTA: 0.87 .. 0.99 of the time over 14 drawn shapes (AlexNet conv2 58.6 -> 54.9
-  // us; 96 channels, 50x50, 256 filters 5x5, 51 images 0.87); fewer items 0.99 .. 1.03, three slabs (conv3) 1.10, 25
-  // K-steps 1.00.  Streaming: 0.71 .. 0.98 over 12 (256 channels, 14x14, 512 filters 3x3 stride 2, 256 images 24.7 -> 22.6).
+  // From 32 K-steps on the MMAs bound an item, and one thread of a pair issues those of two SMs at the cost of
+  // one's; against that the two CTAs wait for each other's patches and accumulators at every item.  Measured, pair
+  // against single CTAs, both resident, 26 to 75 K-steps: two slabs and five items and more per CTA 0.90 from 32
+  // K-steps (AlexNet conv2 58.6 -> 54.9 us; 219 channels, 20x20, 256 filters 3x3, 160 images 0.903), 0.95 .. 0.98
+  // at 27, with fewer items 0.98 .. 1.29.  One slab, where a single CTA has every filter and each patch is built
+  // once, 1.03 over 88 shapes (0.90 .. 1.19, no size tells the better ones apart); three slabs of 128, which
+  // a pair makes two of 192, 1.00 and 1.05, conv3 1.10.  Streaming: 0.71 .. 0.98 over 12 (256 channels, 14x14,
+  // 512 filters 3x3 stride 2, 256 images 24.7 -> 22.6).
   const bool long_items = !fuse && planes == 1 && single.ok && single.P.nsteps >= kPairSteps;
   if (single.ok && single.P.resident) {
     if (long_items && single.P.nslabs == 2 && single.P.ntiles * 2 >= 5 * (int)kSms) {

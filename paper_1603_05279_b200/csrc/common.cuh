@@ -187,7 +187,7 @@ cudaError_t launch_binconv_tc(const uint32_t *xp, const uint32_t *wp, const floa
                               const EpiOpts &epi, float *out, int32_t *acc_out, TcVariant v,
                               cudaStream_t st, const uint32_t *xp2 = nullptr);
 // BinConv with the next layer's BinActiv fused into its epilogue (sign bits packed along the
-// filters, partial sums of |y| per filter slab and epilogue warp); tc_fused_parts = number of
+// filters, partial sums of |y| per filter slab and chunk of its columns); tc_fused_parts = number of
 // partial planes for the shape (0: the fused kernel does not cover it).
 int tc_fused_parts(const ConvGeom &g, TcVariant v);
 cudaError_t launch_binconv_tc_fused(const uint32_t *xp, const uint32_t *wp, const float *alpha,
