@@ -1662,7 +1662,7 @@ namespace {
 // the filters resident, or the items are long (see below).  Neither resident: pairs where the items are long (each CTA
 // expands half the rows of a slab; 1024 channels, 1x1, 16 K-steps: 16.9 -> 17.5 us) and the slabs wide enough to
 // fill a pair.  Over 255 drawn shapes the choice takes 1.010 of the time of the best variant (geometric mean;
-// 234 of them within 2 %, 245 within 5 %).
+// 233 of them within 2 %, 245 within 5 %).
 Plan plan_variant_uncached(const ConvGeom &g, TcVariant v, bool fuse, int planes, bool residual) {
   switch (v) {
     case kTcSingle: return make_plan(g, 0, false, fuse, planes, residual);
@@ -1675,11 +1675,11 @@ Plan plan_variant_uncached(const ConvGeom &g, TcVariant v, bool fuse, int planes
   // From 32 K-steps on the MMAs bound an item, and one thread of a pair issues those of two SMs at the cost of
   // one's; against that the two CTAs wait for each other's patches and accumulators at every item.  Measured, pair
   // against single CTAs, both resident, 26 to 75 K-steps: two slabs and five items and more per CTA 0.90 from 32
-  // K-steps (AlexNet conv2 58.6 -> 54.9 us; 219 channels, 20x20, 256 filters 3x3, 160 images 0.903), 0.95 .. 0.98
-  // at 27, with fewer items 0.98 .. 1.29.  One slab, where a single CTA has every filter and each patch is built
-  // once, 1.03 over 88 shapes (0.90 .. 1.19, no size tells the better ones apart); three slabs of 128, which
-  // a pair makes two of 192, 1.00 and 1.05, conv3 1.10.  Streaming: 0.71 .. 0.98 over 12 (256 channels, 14x14,
-  // 512 filters 3x3 stride 2, 256 images 24.7 -> 22.6).
+  // K-steps (AlexNet conv2 58.6 -> 54.9 us; 219 channels, 20x20, 256 filters 3x3, 160 images 0.91), 0.96 .. 0.98
+  // at 27, with fewer items 0.99 .. 1.29.  One slab, where a single CTA has every filter and each patch is built
+  // once, 1.03 over 88 shapes (0.89 .. 1.19; with five items and more from 32 K-steps 0.99 over 20, no size tells
+  // the better ones apart); three slabs of 128, which a pair makes two of 192, 0.99 and 1.04, conv3 1.10.
+  // Streaming: 0.71 .. 0.98 over 12 (256 channels, 14x14, 512 filters 3x3 stride 2, 256 images 24.7 -> 22.6).
   const bool long_items = !fuse && planes == 1 && single.ok && single.P.nsteps >= kPairSteps;
   if (single.ok && single.P.resident) {
     if (long_items && single.P.nslabs == 2 && single.P.ntiles * 2 >= 5 * (int)kSms) {
