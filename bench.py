@@ -41,7 +41,7 @@ POPC_PER_CLK_PER_SM = 16
 # DRAM traffic of the dominant kernel from one ncu capture: dram__bytes_read.sum +
 # dram__bytes_write.sum summed over the four BinConv launches of one step of the default
 # workload.  Valid only for the kernel source it was taken from (hash below); null otherwise.
-NCU_TRAFFIC = {"kernel_sha1": "940fa80f38eb1174c8f534e0c5100e1bd1372a54", "bytes_per_step": 161.0e6}
+NCU_TRAFFIC = {"kernel_sha1": "42f9ac10947e86acd2f6fa3f54f54e611dda9587", "bytes_per_step": 161.0e6}
 
 
 def kernel_sha1():

@@ -322,8 +322,9 @@ inline uint32_t kstep_desc(const TcParams &P, int j, bool *swap) {
 // Units of channel words at one position of a patch.  Four words come together where they can be loaded as one, and in
 // the resident schedule.  Streaming, with fewer registers, other counts of five words and more go one by one, for
 // twice as many positions at a time: guarding each of four words for one position was slower than the two
-// divisions per unit before it (26.2 us for 218 images, 477 channels, 14x14, 400 filters 1x1 stride 2, 25.2 before,
-// 20.6 now; 0.98 to 1.08 of the time before over 28 drawn shapes, 0.80 to 1.0 now).  Resident, one by one is as often slower.
+// divisions per unit before it (218 images, 477 channels, 14x14, 400 filters 1x1 stride 2: 25.1 us with the
+// divisions, 26.2 guarded, 20.4 now; over 16 drawn shapes 0.97 to 1.10 of the time with the divisions, now 0.81
+// to 0.98).  Resident, one by one takes 0.85 to 1.05 of the time; small problems lose.
 __host__ __device__ inline int patch_groups(int Cw, bool resident) {
   return !resident && Cw > 4 && (Cw & 3) != 0 ? Cw : (Cw + 3) / 4;
 }
@@ -1679,7 +1680,8 @@ Plan plan_variant_uncached(const ConvGeom &g, TcVariant v, bool fuse, int planes
   // at 27, with fewer items 0.99 .. 1.29.  One slab, where a single CTA has every filter and each patch is built
   // once, 1.03 over 88 shapes (0.89 .. 1.19; with five items and more from 32 K-steps 0.99 over 20, no size tells
   // the better ones apart); three slabs of 128, which a pair makes two of 192, 0.99 and 1.04, conv3 1.10.
-  // Streaming: 0.71 .. 0.98 over 12 (256 channels, 14x14, 512 filters 3x3 stride 2, 256 images 24.7 -> 22.6).
+  // Streaming, slabs wider than 64: 0.87 (0.74 .. 1.02) over 9 shapes of 32 to 63 K-steps, 0.82 (0.58 .. 1.02) over 25
+  // of more (256 channels, 14x14, 512 filters 3x3 stride 2, 256 images 24.7 -> 22.6 us).
   const bool long_items = !fuse && planes == 1 && single.ok && single.P.nsteps >= kPairSteps;
   if (single.ok && single.P.resident) {
     if (long_items && single.P.nslabs == 2 && single.P.ntiles * 2 >= 5 * (int)kSms) {
